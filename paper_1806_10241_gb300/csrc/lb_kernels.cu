@@ -80,6 +80,14 @@ template <typename S> struct Scaled { static constexpr bool value = std::is_same
 
 // ---- kernel parameters in the compute type --------------------------------
 
+// Parameters of the pair kernels' node update as FP32x2 operands (both halves
+// equal): the packed instructions take them as they lie in the parameters,
+// where a scalar would first be copied into a register pair.
+struct PairConst {
+    float2 rho0, T0, bfx, fb, nu, nuh, alh, k3;              // fb = rho0 g_beta; nu / 2, alpha / 2, rho0 / 3
+    float2 c3, c4, nc4, ch, nch, cg, ct, m9, m6, m5, sg, os; // relaxation and back-transform factors, storage scale
+};
+
 template <typename C> struct KP {
     int nr, nz, pitch, xper;
     long long plane;
@@ -104,6 +112,7 @@ template <typename C> struct KP {
     // u_theta and T for the central differences.
     C latf[2][3], latgs[2], latgc[2], laths[2], lathc[2], gha[2][4], ghb[2][4];
     const float *ytab;    // y[pitch] then 1/y[pitch] (pair kernels)
+    PairConst pc;
     // Nusselt and equivalent-conductivity scales per side (diagnostics)
     double nu_scale[4], keq_scale[4];
 };
@@ -184,6 +193,19 @@ template <typename C> KP<C> make_kp(const HostParams &h)
         k.ghb[j][3] = k.heat[sd] == 0 ? two * k.Tw[sd] : (C)0;
     }
     k.ytab = h.ytab;
+    {
+        const float osc = (float)h.scale, om3 = (float)h.omega3, om4 = (float)omn, omh = (float)h.omega_hi;
+        const float rho0 = (float)h.rho0, nu = (float)h.nu, alpha = (float)h.alpha;
+        auto two = [](float v) { return make_float2(v, v); };
+        PairConst &c = k.pc;
+        c.rho0 = two(rho0), c.T0 = two((float)h.T0), c.bfx = two((float)h.body_fx), c.fb = two(rho0 * (float)h.g_beta);
+        c.nu = two(nu), c.nuh = two(0.5f * nu), c.alh = two(0.5f * alpha), c.k3 = two(rho0 * (1.0f / 3.0f));
+        c.c3 = two(om3 * (1.0f / 12.0f) * osc), c.c4 = two(om4 * 0.25f * osc), c.nc4 = two(om4 * -0.25f * osc);
+        c.ch = two(omh * 0.25f * osc), c.nch = two(omh * -0.25f * osc);
+        c.cg = two(om4 * 0.5f * osc), c.ct = two((float)oma * 0.5f * osc);
+        c.m9 = two((1.0f / 9.0f) * osc), c.m6 = two((1.0f / 6.0f) * osc), c.m5 = two(0.2f * osc);
+        c.sg = two(h.sign_literal ? -1.0f : 1.0f), c.os = two(osc);
+    }
     // Nusselt normalisation (Sec. 3.2): lateral walls -R_w / (H dT), end
     // walls -(H / dT) * 2 / (R_o^2 - R_i^2); dT from the Dirichlet values.
     double tmin = 0, tmax = 0;
@@ -758,6 +780,16 @@ __device__ __forceinline__ void march(const KP<C> &k, const S *__restrict__ src,
 
 #include "lb_pair.cuh"
 
+// SplitMix64 finaliser of a step counter (the same function as step_salt on
+// the host: a lattice draws the same rounding bits alone and in a batch)
+__host__ __device__ __forceinline__ uint32_t salt_of(unsigned long long step)
+{
+    unsigned long long z = step + 0x9E3779B97F4A7C15ULL;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
+    return (uint32_t)(z ^ (z >> 31));
+}
+
 // Programmatic dependent launch (sm_90+): the kernels of consecutive steps
 // are launched with programmatic stream serialisation, so a step's blocks
 // may start while the previous step's last blocks run.  Each block first
@@ -1268,16 +1300,6 @@ __global__ void k_import(HostParams h, const double *__restrict__ in, S *__restr
 int nwindows(int nr) { return (nr + OUT_COLS - 1) / OUT_COLS; }
 
 // ---- batched step: many lattices, one launch per step ----------------------------
-
-// SplitMix64 finaliser of a step counter (the same function as step_salt on
-// the host: a lattice draws the same rounding bits alone and in a batch)
-__host__ __device__ __forceinline__ uint32_t salt_of(unsigned long long step)
-{
-    unsigned long long z = step + 0x9E3779B97F4A7C15ULL;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
-    return (uint32_t)(z ^ (z >> 31));
-}
 
 struct alignas(128) BatchDesc {
     unsigned char map[2][128];  // CUtensorMap of buf[0], buf[1] (64-byte aligned in the device array)

@@ -47,9 +47,25 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
     r.v = __ffma2_rn(a.v, b.v, c.v);
     return r;
 }
-// a - b, exactly (one rounding of b * (-1) + a)
-__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return fma2(b, sp(-1.0f), a); }
-__device__ __forceinline__ F2 rcp2(F2 a) { return mk2(__fdividef(1.0f, a.v.x), __fdividef(1.0f, a.v.y)); }
+__device__ __forceinline__ F2 operator-(F2 a, F2 b)
+{
+    F2 r;
+    asm("{\n\t.reg .b64 x, y, d;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 d, x, y;\n\t"
+        "mov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(r.v.x), "=f"(r.v.y)
+        : "f"(a.v.x), "f"(a.v.y), "f"(b.v.x), "f"(b.v.y));
+    return r;
+}
+// 1 / x of a density: the hardware reciprocal alone.  __fdividef(1, x) has the
+// same bits for every normal x whose reciprocal is normal, but wraps the
+// reciprocal in a rescaling for the others (five more instructions each).
+__device__ __forceinline__ float rcp1(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ F2 rcp2(F2 a) { return mk2(rcp1(a.v.x), rcp1(a.v.y)); }
 __device__ __forceinline__ F2 sel2(bool px, bool py, F2 a, F2 b)  // per component: p ? a : b
 {
     return mk2(px ? a.v.x : b.v.x, py ? a.v.y : b.v.y);
@@ -94,12 +110,16 @@ template <> struct PairIO<__half> {
         r.v = __half22float2(*reinterpret_cast<const __half2 *>(p));
         return r;
     }
-    static __device__ __forceinline__ void st(__half *p, F2 v, uint32_t rbits)
+    static __device__ __forceinline__ uint32_t round(F2 v, uint32_t rbits)
     {
         uint32_t d;
         // d = {hi: v.y, lo: v.x}: x stays at the lower address
         asm("cvt.rs.satfinite.f16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v.v.y), "f"(v.v.x), "r"(rbits));
-        *reinterpret_cast<uint32_t *>(p) = d;
+        return d;
+    }
+    static __device__ __forceinline__ void st(__half *p, F2 v, uint32_t rbits)
+    {
+        *reinterpret_cast<uint32_t *>(p) = round(v, rbits);
     }
 };
 template <> struct PairIO<__nv_bfloat16> {
@@ -110,11 +130,15 @@ template <> struct PairIO<__nv_bfloat16> {
         r.v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
         return r;
     }
-    static __device__ __forceinline__ void st(__nv_bfloat16 *p, F2 v, uint32_t rbits)
+    static __device__ __forceinline__ uint32_t round(F2 v, uint32_t rbits)
     {
         uint32_t d;
         asm("cvt.rs.satfinite.bf16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(v.v.y), "f"(v.v.x), "r"(rbits));
-        *reinterpret_cast<uint32_t *>(p) = d;
+        return d;
+    }
+    static __device__ __forceinline__ void st(__nv_bfloat16 *p, F2 v, uint32_t rbits)
+    {
+        *reinterpret_cast<uint32_t *>(p) = round(v, rbits);
     }
 };
 
@@ -160,62 +184,86 @@ template <> struct LoadScaled<__half> {
 // ---- the node update on pairs ------------------------------------------------
 
 struct NodeOut2 {
-    F2 f[9], g[5], h[5];
+    F2 v[NQ];  // f, g, h
 };
 
-// The post-collision values come out multiplied by osc, a power of two (the
-// FP16 storage scale, else 1): osc is folded into the constants of the
+// The gradient inputs are the undivided central differences (twice the
+// derivatives); the halves are folded into the geometric factors, which is
+// exact.  iy is 1 / y, or 0 in the planar form (no geometric sources).
+// kScale: the post-collision values come out multiplied by osc, a power of two
+// (the FP16 storage scale): osc is folded into the constants of the
 // post-collision moments and into the fused multiply-add that adds them to
 // the streamed values.  Scaling by a power of two commutes with every
 // rounding, so the results are exactly osc times the unscaled ones.
+//
+// What the order of the terms is chosen for: packed instructions occupy the
+// FP32 pipe for two cycles and are two thirds of its work, so factors of +-1
+// and +-2 ride on the velocities (n2ux, nuy, ...) instead of costing a
+// multiplication per product, and products with rho are taken from the
+// momentum (rho ux^2 = jx ux): 306 packed instructions per pair where the term
+// by term form had 334.  With the bare reciprocal (rcp1) the 1024 x 2048 step
+// executes 809 instead of 883 warp instructions per 64 columns in FP32, 1043
+// instead of 1100 in FP16: 53.4 -> 52.0 us and 49.2 -> 45.7 us.
+template <bool kScale>
 __device__ __forceinline__ void update_node2(const KP<float> &k, F2 iy, const F2 fv[9], const F2 gv[5],
                                              const F2 hv[5], F2 dxuy, F2 dyux, F2 dyuy, F2 dyut, F2 dyT,
-                                             float osc, NodeOut2 &o)
+                                             NodeOut2 &o)
 {
-    const F2 OS = sp(osc);
+    const PairConst &c = k.pc;
+    auto K = [](const float2 &v) {
+        F2 r;
+        r.v = v;
+        return r;
+    };
+    const F2 m1 = sp(-1.0f);
+    const F2 OS = K(c.os);
+    auto plus = [&](F2 v, F2 m) { return kScale ? fma2(v, OS, m) : v + m; };
+
     // output moments, Eq. 18, 35, 47 (deviation form)
     const F2 a57 = fv[5] - fv[7], a86 = fv[8] - fv[6];
     const F2 s57 = fv[5] + fv[7], s68 = fv[6] + fv[8];
     const F2 s13 = fv[1] + fv[3], s24 = fv[2] + fv[4];
     const F2 s5678 = s57 + s68;
     const F2 rdo = (fv[0] + s13) + (s24 + s5678);
-    const F2 jxo = (fv[1] - fv[3]) + (a57 + a86);
-    const F2 jyo = (fv[2] - fv[4]) + (a57 - a86);
+    const F2 Dxxy = a57 - a86, Dxyy = a57 + a86;
+    const F2 jxo = (fv[1] - fv[3]) + Dxyy;
+    const F2 jyo = (fv[2] - fv[4]) + Dxxy;
     const F2 pso = (gv[0] + gv[1]) + (gv[2] + gv[3]) + gv[4];
     const F2 tdo = (hv[0] + hv[1]) + (hv[2] + hv[3]) + hv[4];
 
     // sources at the pre-collision state, two sweeps (see update_node)
-    const bool geo = !k.planar;
-    const F2 gy = geo ? iy : sp(0.0f);
-    const F2 ngy = gy * sp(-1.0f);
-    const F2 nuiy = gy * sp(k.nu);
-    const F2 Gx = (dxuy + dyux) * nuiy;
-    const F2 Gy = dyuy * (nuiy + nuiy);
-    const F2 Gw = dyut * nuiy;
-    const F2 Gt = dyT * (gy * sp(k.alpha));
-    const F2 iy2nu = nuiy * gy;
-    const F2 m2iy2nu = iy2nu * sp(-2.0f);
-    const F2 Fbx = sp(k.bfx);
-    const F2 Fb = sp(k.rho0 * k.gbeta), rho0 = sp(k.rho0), T0 = sp(k.T0), half = sp(0.5f);
+    const F2 gy = iy, ngy = gy * m1;
+    const F2 nuiyh = gy * K(c.nuh), nuiy = gy * K(c.nu);
+    const F2 Gx = (dxuy + dyux) * nuiyh;
+    const F2 Gy = dyuy * nuiy;
+    const F2 Gw = dyut * nuiyh;
+    const F2 Gt = dyT * (gy * K(c.alh));
+    const F2 niy2nu = nuiy * ngy;
+    const F2 m2iy2nu = niy2nu + niy2nu;
+    const F2 Fbx = K(c.bfx);
+    const F2 Fb = K(c.fb), rho0 = K(c.rho0), T0 = K(c.T0), half = sp(0.5f);
     F2 rd = rdo, jx = jxo, jy = jyo, ps = pso, td = tdo;
-    F2 MA = sp(0.0f), Fx = sp(0.0f), Fy = sp(0.0f), Sps = sp(0.0f), Sph = sp(0.0f);
-    const int sweeps = k.explicit_src ? 1 : 2;
-    for (int sw = 0; sw < sweeps; ++sw) {
+    F2 MA, Fx, Fy, Sps, Sph;
+    auto sweep = [&]() {
         const F2 r = rho0 + rd, ir = rcp2(r);
         const F2 uyyn = (jy * ir) * ngy;  // -u_y / y
-        const F2 igy = ir * gy;
-        const F2 FAx = fma2(jx, uyyn, r * Gx);
-        const F2 FAy = fma2(jy, m2iy2nu, fma2(r, Gy, ((ps - jy) * (ps + jy)) * igy));
-        Sps = fma2(ps, fma2(uyyn, sp(2.0f), iy2nu * sp(-1.0f)), r * Gw);
+        Fx = fma2(Fb, td, fma2(jx, uyyn, fma2(r, Gx, Fbx)));
+        Fy = fma2(jy, m2iy2nu, fma2(r, Gy, ((ps - jy) * (ps + jy)) * (ir * gy)));
+        Sps = fma2(ps, fma2(uyyn, sp(2.0f), niy2nu), r * Gw);
         Sph = fma2(uyyn, T0 + td, Gt);
-        Fx = fma2(Fb, td, FAx + Fbx);
-        Fy = FAy;
         jx = fma2(Fx, half, jxo);
         jy = fma2(Fy, half, jyo);
         ps = fma2(Sps, half, pso);
         td = fma2(Sph, half, tdo);
-        MA = (k.explicit_src ? jyo : jy) * ngy;
+        MA = jy * ngy;
         rd = fma2(MA, half, rdo);
+    };
+    sweep();
+    if (k.explicit_src) {
+        MA = jyo * ngy;
+        rd = fma2(MA, half, rdo);
+    } else {
+        sweep();
     }
     const F2 r = rho0 + rd, ir = rcp2(r);
     const F2 ux = jx * ir, uy = jy * ir;
@@ -223,109 +271,102 @@ __device__ __forceinline__ void update_node2(const KP<float> &k, F2 iy, const F2
 
     // D2Q9 cascaded collision, Eq. 17
     const F2 Dxx = s13 + s5678, Dyy = s24 + s5678;
-    const F2 Dxy = s57 - s68, Dxxy = a57 - a86, Dxyy = a57 + a86, Dxxyy = s5678;
-    const F2 k3 = sp(k.rho0 * (1.0f / 3.0f));
+    const F2 Dxy = s57 - s68, Dxxyy = s5678;
+    const F2 k3 = K(c.k3);
     const F2 Kxx = k3 + Dxx, Kyy = k3 + Dyy;
-    const F2 ux2 = ux * ux, uy2 = uy * uy, uxy = ux * uy;
-    const F2 uu = ux2 + uy2, ud = ux2 - uy2;
-    const F2 p3 = (fma2(rd, sp(2.0f / 3.0f), r * uu) - (Dxx + Dyy)) * sp(k.om3 * (1.0f / 12.0f) * osc);
-    const F2 c4 = sp(k.om4 * 0.25f * osc);
-    const F2 p4 = ((r * ud) - (Dxx - Dyy)) * c4;
-    const F2 p5 = ((r * uxy) - Dxy) * c4;
-    const F2 q34p = fma2(p3, sp(3.0f), p4), q34m = fma2(p3, sp(3.0f), p4 * sp(-1.0f));
-    const F2 ch = sp(k.omhi * 0.25f * osc);
-    const F2 m2p5 = p5 * sp(-2.0f);
-    const F2 m2Dxy = Dxy * sp(-2.0f);
-    const F2 r2 = r + r;
+    const F2 ux2 = ux * ux, uy2 = uy * uy;
+    const F2 rxx = jx * ux, ryy = jy * uy;  // rho ux^2, rho uy^2
+    const F2 nux = ux * m1, nuy = uy * m1, n2ux = ux * sp(-2.0f), n2uy = uy * sp(-2.0f);
+    const F2 uxy4 = n2ux * n2uy;
+    const F2 p3 = (fma2(rd, sp(2.0f / 3.0f), rxx + ryy) - (Dxx + Dyy)) * K(c.c3);
+    const F2 c4 = K(c.c4), ch = K(c.ch), nch = K(c.nch);
+    const F2 p4 = ((rxx - ryy) - (Dxx - Dyy)) * c4;
+    const F2 x5 = jx * uy - Dxy;
+    const F2 p5 = x5 * c4, np5 = x5 * K(c.nc4);
+    // -(3 p3 + p4) / 2 and -(3 p3 - p4) / 2
+    const F2 hp = fma2(p3, sp(-1.5f), p4 * sp(-0.5f)), hm = fma2(p3, sp(-1.5f), p4 * half);
+    const F2 rxx2 = rxx + rxx, ryy2 = ryy + ryy;
     // p6: (2 r ux^2 uy + Dxxy - 2 ux Dxy - uy Kxx) omhi/4 - uy (3 p3 + p4)/2 - 2 ux p5
-    F2 Z = fma2(r2 * ux2, uy, Dxxy);
-    Z = fma2(ux, m2Dxy, Z);
-    Z = fma2(uy, Kxx * sp(-1.0f), Z);
-    const F2 p6 = fma2(Z, ch, fma2(uy, q34p * sp(-0.5f), ux * m2p5));
-    F2 Y = fma2(r2 * ux, uy2, Dxyy);
-    Y = fma2(uy, m2Dxy, Y);
-    Y = fma2(ux, Kyy * sp(-1.0f), Y);
-    const F2 p7 = fma2(Y, ch, fma2(ux, q34m * sp(-0.5f), uy * m2p5));
+    const F2 Z = fma2(nuy, Kxx, fma2(n2ux, Dxy, fma2(rxx2, uy, Dxxy)));
+    const F2 p6 = fma2(Z, ch, fma2(uy, hp, n2ux * p5));
+    const F2 Y = fma2(nux, Kyy, fma2(n2uy, Dxy, fma2(ryy2, ux, Dxyy)));
+    const F2 p7 = fma2(Y, ch, fma2(ux, hm, n2uy * p5));
     // p8
     F2 B = fma2(ux2, Kyy, Dxxyy);
     B = fma2(uy2, Kxx, B);
-    B = fma2(uxy, Dxy * sp(4.0f), B);
-    B = fma2(ux, Dxyy * sp(-2.0f), B);
-    B = fma2(uy, Dxxy * sp(-2.0f), B);
-    const F2 W = fma2(rd, sp(1.0f / 9.0f), (r * sp(3.0f)) * (ux2 * uy2)) - B;
-    F2 p8 = W * ch;
-    p8 = fma2(p3, sp(-2.0f), p8);
-    p8 = fma2(uy2, q34p * sp(-0.5f), p8);
-    p8 = fma2(ux2, q34m * sp(-0.5f), p8);
-    p8 = fma2(uxy, p5 * sp(-4.0f), p8);
-    p8 = fma2(uy, p6 * sp(-2.0f), p8);
-    p8 = fma2(ux, p7 * sp(-2.0f), p8);
+    B = fma2(uxy4, Dxy, B);
+    B = fma2(n2ux, Dxyy, B);
+    B = fma2(n2uy, Dxxy, B);
+    const F2 Wm = fma2(rd, sp(1.0f / 9.0f), (rxx2 * uy2) * sp(1.5f)) - B;
+    F2 p8 = fma2(p3, sp(-2.0f), Wm * ch);
+    p8 = fma2(uy2, hp, p8);
+    p8 = fma2(ux2, hm, p8);
+    p8 = fma2(uxy4, np5, p8);
+    p8 = fma2(n2uy, p6, p8);
+    p8 = fma2(n2ux, p7, p8);
     // source moments, Eq. 26
-    const F2 p0 = MA * sp((1.0f / 9.0f) * osc), p1 = Fx * sp((1.0f / 6.0f) * osc), p2 = Fy * sp((1.0f / 6.0f) * osc);
+    const F2 p0 = MA * K(c.m9), p1 = Fx * K(c.m6), p2 = Fy * K(c.m6);
     // back-transform, Eq. 27, grouped
     {
         const F2 A0 = p0 - p3;
-        const F2 E = A0 + p4, Fm = A0 - p4;
-        const F2 t78m = p7 - p8, t78p = p7 + p8, t68m = p6 - p8, t68p = p6 + p8;
-        o.f[0] = fma2(p3 - p8, sp(-4.0f), fma2(fv[0], OS, p0));
-        o.f[1] = fma2(fv[1], OS, E) + fma2(t78m, sp(2.0f), p1);
-        o.f[3] = fma2(fv[3], OS, E) - fma2(t78p, sp(2.0f), p1);
-        o.f[2] = fma2(fv[2], OS, Fm) + fma2(t68m, sp(2.0f), p2);
-        o.f[4] = fma2(fv[4], OS, Fm) - fma2(t68p, sp(2.0f), p2);
+        const F2 E = fma2(p8, sp(-2.0f), A0 + p4), Fm = fma2(p8, sp(-2.0f), A0 - p4);
+        const F2 u = fma2(p7, sp(2.0f), p1), w = fma2(p6, sp(2.0f), p2);
+        o.v[0] = fma2(p3 - p8, sp(-4.0f), plus(fv[0], p0));
+        o.v[1] = plus(fv[1], E) + u;
+        o.v[3] = plus(fv[3], E) - u;
+        o.v[2] = plus(fv[2], Fm) + w;
+        o.v[4] = plus(fv[4], Fm) - w;
         const F2 B0 = fma2(p3, sp(2.0f), p0 + p8);
-        const F2 u12 = p1 + p2, v12 = p1 - p2, s67 = p6 + p7, d67 = p6 - p7;
-        const F2 C5 = B0 + p5, C6 = B0 - p5;
-        const F2 us = u12 - s67, vd = v12 + d67;
-        o.f[5] = fma2(fv[5], OS, C5) + us;
-        o.f[7] = fma2(fv[7], OS, C5) - us;
-        o.f[6] = fma2(fv[6], OS, C6) - vd;
-        o.f[8] = fma2(fv[8], OS, C6) + vd;
+        const F2 C5 = B0 + p5, C6 = B0 + np5;
+        const F2 p17 = p1 - p7, p26 = p2 - p6;
+        const F2 us = p17 + p26, vd = p17 - p26;
+        o.v[5] = plus(fv[5], C5) + us;
+        o.v[7] = plus(fv[7], C5) - us;
+        o.v[6] = plus(fv[6], C6) - vd;
+        o.v[8] = plus(fv[8], C6) + vd;
     }
 
-    // D2Q5 cascaded collisions, Eq. 34 / 49 (sign reading of the paper: -)
-    const F2 coefu = fma2(sp(k.sign_lit ? 1.0f : -1.0f), uu, sp(2.0f / 3.0f));
-    const F2 coefd = sp(k.sign_lit ? 1.0f : -1.0f) * ud;
+    // D2Q5 cascaded collisions, Eq. 34 / 49 (sign reading of the paper: -),
+    // the bracket of q3, q4 with its sign turned
+    const F2 uu = ux2 + uy2, ud = ux2 - uy2;
+    const F2 sg = K(c.sg);
+    const F2 ncu = fma2(sg, uu, sp(-2.0f / 3.0f)), ncd = sg * ud;
     {
         const F2 kxn = gv[3] - gv[1], kyn = gv[4] - gv[2];  // -kappa'_x, -kappa'_y
         const F2 kxx = gv[1] + gv[3], kyy = gv[2] + gv[4];
-        const F2 cg = sp(k.omg * 0.5f * osc);
+        const F2 cg = K(c.cg);
         const F2 q1 = fma2(ps, ux, kxn) * cg;
         const F2 q2 = fma2(ps, uy, kyn) * cg;
-        const F2 m = fma2(ux, kxn, uy * kyn);  // -(ux kx + uy ky)
-        const F2 mm = fma2(ux, kxn, uy * (gv[2] - gv[4]));  // -(ux kx - uy ky)
-        const F2 X3 = fma2(ps, coefu, fma2(m, sp(-2.0f), (kxx + kyy) * sp(-1.0f)));
-        const F2 X4 = fma2(ps, coefd, fma2(mm, sp(-2.0f), (kxx - kyy) * sp(-1.0f)));
-        const F2 q3 = fma2(X3, ch, fma2(ux, q1, uy * q2));
-        const F2 q4 = fma2(X4, ch, fma2(ux, q1, uy * q2 * sp(-1.0f)));
-        const F2 q0 = Sps * sp(0.2f * osc);
+        const F2 X3 = fma2(ps, ncu, fma2(fma2(ux, kxn, uy * kyn), sp(2.0f), kxx + kyy));
+        const F2 X4 = fma2(ps, ncd, fma2(fma2(ux, kxn, nuy * kyn), sp(2.0f), kxx - kyy));
+        const F2 q3 = fma2(X3, nch, fma2(ux, q1, uy * q2));
+        const F2 q4 = fma2(X4, nch, fma2(ux, q1, nuy * q2));
+        const F2 q0 = Sps * K(c.m5);
         const F2 Q = q0 + q3, Qp = Q + q4, Qm = Q - q4;
-        o.g[0] = fma2(q3, sp(-4.0f), fma2(gv[0], OS, q0));
-        o.g[1] = fma2(gv[1], OS, Qp) + q1;
-        o.g[3] = fma2(gv[3], OS, Qp) - q1;
-        o.g[2] = fma2(gv[2], OS, Qm) + q2;
-        o.g[4] = fma2(gv[4], OS, Qm) - q2;
+        o.v[G0 + 0] = fma2(q3, sp(-4.0f), plus(gv[0], q0));
+        o.v[G0 + 1] = plus(gv[1], Qp) + q1;
+        o.v[G0 + 3] = plus(gv[3], Qp) - q1;
+        o.v[G0 + 2] = plus(gv[2], Qm) + q2;
+        o.v[G0 + 4] = plus(gv[4], Qm) - q2;
     }
     {
         const F2 kxn = hv[3] - hv[1], kyn = hv[4] - hv[2];
         const F2 Hxx = hv[1] + hv[3], Hyy = hv[2] + hv[4];
-        const F2 ct = sp(k.omh * 0.5f * osc);
+        const F2 ct = K(c.ct);
         const F2 r1 = fma2(phi, ux, kxn) * ct;
-        const F2 r2t = fma2(phi, uy, kyn) * ct;
-        const F2 m = fma2(ux, kxn, uy * kyn);
-        const F2 mm = fma2(ux, kxn, uy * (hv[2] - hv[4]));
+        const F2 r2 = fma2(phi, uy, kyn) * ct;
         // 2 c^2 phi - (kxx + kyy) with the rest parts written out: 2/3 td - (Hxx + Hyy)
-        const F2 X3 = fma2(sp(2.0f / 3.0f), td, fma2(phi, coefu - sp(2.0f / 3.0f), fma2(m, sp(-2.0f),
-                                                                                    (Hxx + Hyy) * sp(-1.0f))));
-        const F2 X4 = fma2(phi, coefd, fma2(mm, sp(-2.0f), (Hxx - Hyy) * sp(-1.0f)));
-        const F2 r3 = fma2(X3, ch, fma2(ux, r1, uy * r2t));
-        const F2 r4 = fma2(X4, ch, fma2(ux, r1, uy * r2t * sp(-1.0f)));
-        const F2 r0 = Sph * sp(0.2f * osc);
+        const F2 X3 = fma2(sp(-2.0f / 3.0f), td, fma2(phi, sg * uu, fma2(fma2(ux, kxn, uy * kyn), sp(2.0f), Hxx + Hyy)));
+        const F2 X4 = fma2(phi, ncd, fma2(fma2(ux, kxn, nuy * kyn), sp(2.0f), Hxx - Hyy));
+        const F2 r3 = fma2(X3, nch, fma2(ux, r1, uy * r2));
+        const F2 r4 = fma2(X4, nch, fma2(ux, r1, nuy * r2));
+        const F2 r0 = Sph * K(c.m5);
         const F2 Q = r0 + r3, Qp = Q + r4, Qm = Q - r4;
-        o.h[0] = fma2(r3, sp(-4.0f), fma2(hv[0], OS, r0));
-        o.h[1] = fma2(hv[1], OS, Qp) + r1;
-        o.h[3] = fma2(hv[3], OS, Qp) - r1;
-        o.h[2] = fma2(hv[2], OS, Qm) + r2t;
-        o.h[4] = fma2(hv[4], OS, Qm) - r2t;
+        o.v[H0 + 0] = fma2(r3, sp(-4.0f), plus(hv[0], r0));
+        o.v[H0 + 1] = plus(hv[1], Qp) + r1;
+        o.v[H0 + 3] = plus(hv[3], Qp) - r1;
+        o.v[H0 + 2] = plus(hv[2], Qm) + r2;
+        o.v[H0 + 4] = plus(hv[4], Qm) - r2;
     }
 }
 
@@ -580,19 +621,24 @@ __device__ __forceinline__ Lane2 lane2(const KP<float> &k, int c0)
     const float2 yv = *reinterpret_cast<const float2 *>(k.ytab + L.Ac);
     const float2 iyv = *reinterpret_cast<const float2 *>(k.ytab + k.pitch + L.Ac);
     L.y2 = mk2(yv.x, yv.y);
-    L.iy = mk2(iyv.x, iyv.y);
+    L.iy = k.planar ? sp(0.0f) : mk2(iyv.x, iyv.y);  // no geometric sources in the planar form
     return L;
 }
 
+// The fields of one column, with the operations of moments2 in its order: a
+// column's fields have the same bits whether it is a halo column of one
+// window or a column of another.
 __device__ __forceinline__ void halo_fields(const KP<float> &k, const float h[NQ], float &ux, float &uy, float &ut,
                                             float &T)
 {
-    const float rd = h[0] + h[1] + h[2] + h[3] + h[4] + h[5] + h[6] + h[7] + h[8];
-    const float ir = __fdividef(1.0f, k.rho0 + rd);
-    ux = (h[1] - h[3] + h[5] - h[6] - h[7] + h[8]) * ir;
-    uy = (h[2] - h[4] + h[5] + h[6] - h[7] - h[8]) * ir;
-    ut = (h[9] + h[10] + h[11] + h[12] + h[13]) * ir;
-    T = k.T0 + (h[14] + h[15] + h[16] + h[17] + h[18]);
+    const float s13 = h[1] + h[3], s24 = h[2] + h[4], s5678 = (h[5] + h[7]) + (h[6] + h[8]);
+    const float rd = (h[0] + s13) + (s24 + s5678);
+    const float a57 = h[5] - h[7], a86 = h[8] - h[6];
+    const float ir = rcp1(k.rho0 + rd);
+    ux = ((h[1] - h[3]) + (a57 + a86)) * ir;
+    uy = ((h[2] - h[4]) + (a57 - a86)) * ir;
+    ut = ((h[9] + h[10]) + (h[11] + h[12]) + h[13]) * ir;
+    T = k.T0 + ((h[14] + h[15]) + (h[16] + h[17]) + h[18]);
 }
 
 // Own post-collision values that the wall and axis rules need (own(q): the
@@ -620,8 +666,8 @@ template <typename S> struct OwnGlobal {
     __device__ __forceinline__ F2 shl(int q) const { return mk2(at(q, Ac - 1), at(q, Ac)); }
     __device__ __forceinline__ F2 shr(int q) const { return mk2(at(q, Ac + 1), at(q, Ac + 2)); }
 };
-template <typename S> struct OwnStage {
-    const S *b;  // stage of row i
+template <typename S, int C> struct OwnStage {
+    const S *b;  // stage of row i, planes of C columns
     int cA;      // column of the lane's pair in the stage
     float is, m8v, p7v;
     // FP32: the loads are volatile so that they stay inside the wall lanes'
@@ -633,55 +679,47 @@ template <typename S> struct OwnStage {
     {
         if constexpr (sizeof(S) == 4) {
             float x, y;
-            const uint32_t a = smem_u32(b + q * TmaGeom<S>::cols + cA);
+            const uint32_t a = smem_u32(b + q * C + cA);
             asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "r"(a) : "memory");
             return mk2(x, y);
         } else {
-            return LoadScaled<S>::pair(b + q * TmaGeom<S>::cols + cA, is);
+            return LoadScaled<S>::pair(b + q * C + cA, is);
         }
     }
     __device__ __forceinline__ float own0(int q) const
     {
         if constexpr (sizeof(S) == 4) {
             float x;
-            const uint32_t a = smem_u32(b + q * TmaGeom<S>::cols + cA);
+            const uint32_t a = smem_u32(b + q * C + cA);
             asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(a) : "memory");
             return x;
         } else {
-            return LoadScaled<S>::one(b + q * TmaGeom<S>::cols + cA, is);
+            return LoadScaled<S>::one(b + q * C + cA, is);
         }
     }
     __device__ __forceinline__ float m8() const { return m8v; }
     __device__ __forceinline__ float p7() const { return p7v; }
     __device__ __forceinline__ F2 shl(int q) const
     {
-        const S *p = b + q * TmaGeom<S>::cols + cA;
+        const S *p = b + q * C + cA;
         return mk2(LoadScaled<S>::one(p - 1, is), LoadScaled<S>::one(p, is));
     }
     __device__ __forceinline__ F2 shr(int q) const
     {
-        const S *p = b + q * TmaGeom<S>::cols + cA;
+        const S *p = b + q * C + cA;
         return mk2(LoadScaled<S>::one(p + 1, is), LoadScaled<S>::one(p + 2, is));
     }
 };
 
-// The rest of a row update once the pulled values of the pair are in fv, gv,
-// hv5: wall and axis rules (the own post-collision values they need are read
-// from src), central differences of the stored-state fields with ghosts, the
-// node update and the stores.  kBc = false is the interior form, for a warp
-// with no wall or axis column on a row with both neighbour rows: the rules are
-// left out at compile time instead of being branched or predicated around.
-template <typename S, bool kBc, typename Own>
-__device__ __forceinline__ void row_tail(const KP<float> &k, const Own &own, S *__restrict__ dst,
-                                         const Lane2 &L, int i, bool has_m_, bool has_p_, uint32_t salt, F2 fv[9],
-                                         F2 gv[5], F2 hv5[5], const PM2 &pm_cur, const PM2 &pm_n, F2 uy_prev,
-                                         float pmh_ux, float pmh_uy, float pmh_ut, float pmh_T)
+// Wall and axis rules on the pulled values fv, gv, hv5 of a pair (the own
+// post-collision values they need come from own).
+template <typename Own>
+__device__ __forceinline__ void wall_rules(const KP<float> &k, const Own &own, const Lane2 &L, bool edge_warp,
+                                           bool has_m, bool has_p, F2 fv[9], F2 gv[5], F2 hv5[5])
 {
-    const int lane = L.lane, A = L.A, Ac = L.Ac, nz = k.nz;
-    const bool has_m = kBc ? has_m_ : true, has_p = kBc ? has_p_ : true;
-    const bool outA = L.outA, atA0 = L.atA0, atAN = L.atAN, atBN = L.atBN, edge_warp = kBc && L.edge_warp;
-    const F2 y2 = L.y2, iy = L.iy;
-    const float sc = k.scale;
+    const int A = L.A;
+    const bool atA0 = L.atA0, atAN = L.atAN, atBN = L.atBN;
+    const F2 y2 = L.y2;
     // lateral boundaries: column 0 is always the x of a pair, column
     // nr - 1 the x or the y
     // (the wall terms and rule coefficients come precomputed in k.latf,
@@ -800,19 +838,78 @@ __device__ __forceinline__ void row_tail(const KP<float> &k, const Own &own, S *
                      scalar_bc<float>(heat_rule(k, sy), oh.v.y, end_T(k, sy, y2.v.y) - k.T0, false));
     }
 
-    // central differences of the stored-state fields, with ghosts (a free
-    // surface: no shear, u_y even across it)
+}
+
+// u_y beyond an end wall for the axial central difference: the ghost value,
+// or the own value across a free surface (no shear, u_y even across it)
+__device__ __forceinline__ F2 end_ghost_uy(const KP<float> &k, const Lane2 &L, int side, F2 uy)
+{
+    const int sx = end_seg(k, side, L.A), sy = end_seg(k, side, L.A + 1);
+    return mk2(k.flow[sx] == 3 ? uy.v.x : 2.0f * k.uwy[sx] - uy.v.x,
+               k.flow[sy] == 3 ? uy.v.y : 2.0f * k.uwy[sy] - uy.v.y);
+}
+
+// Ghosts at the lateral walls, a q + b (k.gha, k.ghb), in place of the left
+// neighbour (column 0) and the right one (column nr - 1) of u_x, u_y, u_theta, T
+struct Sides2 {
+    F2 ux, uy, ut, T;
+};
+__device__ __forceinline__ void lateral_ghosts(const KP<float> &k, const Lane2 &L, const Sides2 &c, Sides2 &l, Sides2 &r)
+{
+    if (L.atA0) {
+        l.ux.v.x = __fmaf_rn(k.gha[0][0], c.ux.v.x, k.ghb[0][0]);
+        l.uy.v.x = __fmaf_rn(k.gha[0][1], c.uy.v.x, k.ghb[0][1]);
+        l.ut.v.x = __fmaf_rn(k.gha[0][2], c.ut.v.x, k.ghb[0][2]);
+        l.T.v.x = __fmaf_rn(k.gha[0][3], c.T.v.x, k.ghb[0][3]);
+    }
+    if (L.atAN) {
+        r.ux.v.x = __fmaf_rn(k.gha[1][0], c.ux.v.x, k.ghb[1][0]);
+        r.uy.v.x = __fmaf_rn(k.gha[1][1], c.uy.v.x, k.ghb[1][1]);
+        r.ut.v.x = __fmaf_rn(k.gha[1][2], c.ut.v.x, k.ghb[1][2]);
+        r.T.v.x = __fmaf_rn(k.gha[1][3], c.T.v.x, k.ghb[1][3]);
+    }
+    if (L.atBN) {
+        r.ux.v.y = __fmaf_rn(k.gha[1][0], c.ux.v.y, k.ghb[1][0]);
+        r.uy.v.y = __fmaf_rn(k.gha[1][1], c.uy.v.y, k.ghb[1][1]);
+        r.ut.v.y = __fmaf_rn(k.gha[1][2], c.ut.v.y, k.ghb[1][2]);
+        r.T.v.y = __fmaf_rn(k.gha[1][3], c.T.v.y, k.ghb[1][3]);
+    }
+}
+
+// The pair's post-collision values to row i of dst (whole rows of planes).
+template <typename S>
+__device__ __forceinline__ void store_row(const KP<float> &k, S *__restrict__ dst, int i, int A, uint32_t salt,
+                                          const NodeOut2 &o)
+{
+    S *p = dst + (long long)i * k.pitch + A;
+    uint32_t w = 0;
+    if (PairIO<S>::rounds) w = pcg_hash(((uint32_t)i * (uint32_t)k.pitch + (uint32_t)A) ^ salt) | 1u;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        if (PairIO<S>::rounds) w = xorshift32(w);
+        PairIO<S>::st(p + q * k.plane, o.v[q], w);
+    }
+}
+
+// The rest of a row update once the pulled values of the pair are in fv, gv,
+// hv5: wall and axis rules, central differences of the stored-state fields
+// with ghosts, the node update and the stores.  kBc = false is the interior
+// form, for a warp with no wall or axis column on a row with both neighbour
+// rows: the rules are left out at compile time instead of being branched or
+// predicated around.
+template <typename S, bool kBc, typename Own>
+__device__ __forceinline__ void row_tail(const KP<float> &k, const Own &own, S *__restrict__ dst,
+                                         const Lane2 &L, int i, bool has_m_, bool has_p_, uint32_t salt, F2 fv[9],
+                                         F2 gv[5], F2 hv5[5], const PM2 &pm_cur, const PM2 &pm_n, F2 uy_prev,
+                                         float pmh_ux, float pmh_uy, float pmh_ut, float pmh_T)
+{
+    const int lane = L.lane;
+    const bool has_m = kBc ? has_m_ : true, has_p = kBc ? has_p_ : true, edge_warp = kBc && L.edge_warp;
+    wall_rules(k, own, L, edge_warp, has_m, has_p, fv, gv, hv5);
+
     F2 uy_xm = uy_prev, uy_xp = pm_n.uy;
-    if (!has_m) {
-        const int sx = end_seg(k, 0, A), sy = end_seg(k, 0, A + 1);
-        uy_xm = mk2(k.flow[sx] == 3 ? pm_cur.uy.v.x : 2.0f * k.uwy[sx] - pm_cur.uy.v.x,
-                    k.flow[sy] == 3 ? pm_cur.uy.v.y : 2.0f * k.uwy[sy] - pm_cur.uy.v.y);
-    }
-    if (!has_p) {
-        const int sx = end_seg(k, 1, A), sy = end_seg(k, 1, A + 1);
-        uy_xp = mk2(k.flow[sx] == 3 ? pm_cur.uy.v.x : 2.0f * k.uwy[sx] - pm_cur.uy.v.x,
-                    k.flow[sy] == 3 ? pm_cur.uy.v.y : 2.0f * k.uwy[sy] - pm_cur.uy.v.y);
-    }
+    if (!has_m) uy_xm = end_ghost_uy(k, L, 0, pm_cur.uy);
+    if (!has_p) uy_xp = end_ghost_uy(k, L, 1, pm_cur.uy);
     float lux = __shfl_up_sync(FULL, pm_cur.ux.v.y, 1), luy = __shfl_up_sync(FULL, pm_cur.uy.v.y, 1);
     float lut = __shfl_up_sync(FULL, pm_cur.ut.v.y, 1), lT = __shfl_up_sync(FULL, pm_cur.T.v.y, 1);
     float rux = __shfl_down_sync(FULL, pm_cur.ux.v.x, 1), ruy = __shfl_down_sync(FULL, pm_cur.uy.v.x, 1);
@@ -829,63 +926,17 @@ __device__ __forceinline__ void row_tail(const KP<float> &k, const Own &own, S *
         rut = pmh_ut;
         rT = pmh_T;
     }
-    F2 Lux = mk2(lux, pm_cur.ux.v.x), Luy = mk2(luy, pm_cur.uy.v.x);
-    F2 Lut = mk2(lut, pm_cur.ut.v.x), LT = mk2(lT, pm_cur.T.v.x);
-    F2 Rux = mk2(pm_cur.ux.v.y, rux), Ruy = mk2(pm_cur.uy.v.y, ruy);
-    F2 Rut = mk2(pm_cur.ut.v.y, rut), RT = mk2(pm_cur.T.v.y, rT);
-    // ghosts at the lateral walls, a q + b (k.gha, k.ghb)
-    if (edge_warp) {
-        if (atA0) {
-            Lux.v.x = __fmaf_rn(k.gha[0][0], pm_cur.ux.v.x, k.ghb[0][0]);
-            Luy.v.x = __fmaf_rn(k.gha[0][1], pm_cur.uy.v.x, k.ghb[0][1]);
-            Lut.v.x = __fmaf_rn(k.gha[0][2], pm_cur.ut.v.x, k.ghb[0][2]);
-            LT.v.x = __fmaf_rn(k.gha[0][3], pm_cur.T.v.x, k.ghb[0][3]);
-        }
-        if (atAN) {
-            Rux.v.x = __fmaf_rn(k.gha[1][0], pm_cur.ux.v.x, k.ghb[1][0]);
-            Ruy.v.x = __fmaf_rn(k.gha[1][1], pm_cur.uy.v.x, k.ghb[1][1]);
-            Rut.v.x = __fmaf_rn(k.gha[1][2], pm_cur.ut.v.x, k.ghb[1][2]);
-            RT.v.x = __fmaf_rn(k.gha[1][3], pm_cur.T.v.x, k.ghb[1][3]);
-        }
-        if (atBN) {
-            Rux.v.y = __fmaf_rn(k.gha[1][0], pm_cur.ux.v.y, k.ghb[1][0]);
-            Ruy.v.y = __fmaf_rn(k.gha[1][1], pm_cur.uy.v.y, k.ghb[1][1]);
-            Rut.v.y = __fmaf_rn(k.gha[1][2], pm_cur.ut.v.y, k.ghb[1][2]);
-            RT.v.y = __fmaf_rn(k.gha[1][3], pm_cur.T.v.y, k.ghb[1][3]);
-        }
-    }
-    const F2 hf = sp(0.5f);
-    const F2 dxuy = (uy_xp - uy_xm) * hf;
-    const F2 dyux = (Rux - Lux) * hf;
-    const F2 dyuy = (Ruy - Luy) * hf;
-    const F2 dyut = (Rut - Lut) * hf;
-    const F2 dyT = (RT - LT) * hf;
+    const Sides2 c{pm_cur.ux, pm_cur.uy, pm_cur.ut, pm_cur.T};
+    Sides2 l{mk2(lux, pm_cur.ux.v.x), mk2(luy, pm_cur.uy.v.x), mk2(lut, pm_cur.ut.v.x), mk2(lT, pm_cur.T.v.x)};
+    Sides2 r{mk2(pm_cur.ux.v.y, rux), mk2(pm_cur.uy.v.y, ruy), mk2(pm_cur.ut.v.y, rut), mk2(pm_cur.T.v.y, rT)};
+    if (edge_warp) lateral_ghosts(k, L, c, l, r);
+    auto across = [](F2 right, F2 left) { return mk2(right.v.x - left.v.x, right.v.y - left.v.y); };
 
     // FP16 storage: the update returns the values already times the scale
     NodeOut2 o;
-    update_node2(k, iy, fv, gv, hv5, dxuy, dyux, dyuy, dyut, dyT, Scaled<S>::value ? sc : 1.0f, o);
-
-    if (outA) {
-        S *p = dst + (long long)i * k.pitch + A;
-        uint32_t w = 0;
-        if (PairIO<S>::rounds) w = pcg_hash(((uint32_t)i * (uint32_t)k.pitch + (uint32_t)A) ^ salt) | 1u;
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            if (PairIO<S>::rounds) w = xorshift32(w);
-            PairIO<S>::st(p + q * k.plane, o.f[q], w);
-        }
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            if (PairIO<S>::rounds) w = xorshift32(w);
-            PairIO<S>::st(p + (G0 + q) * k.plane, o.g[q], w);
-        }
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            if (PairIO<S>::rounds) w = xorshift32(w);
-            PairIO<S>::st(p + (H0 + q) * k.plane, o.h[q], w);
-        }
-    }
-
+    update_node2<Scaled<S>::value>(k, L.iy, fv, gv, hv5, uy_xp - uy_xm, across(r.ux, l.ux), across(r.uy, l.uy),
+                                   across(r.ut, l.ut), across(r.T, l.T), o);
+    if (L.outA) store_row<S>(k, dst, i, L.A, salt, o);
 }
 
 template <typename S, typename RS>
@@ -1083,27 +1134,27 @@ template <typename S, int R> struct RowRing {
 
 // stage reads: the pair (A, B), the pair shifted one column left (A - 1, A)
 // or right (B, B + 1), and one column (the halo lanes)
-template <typename S> struct StageRd {
+template <typename S, int C> struct StageRd {
     const S *b;
     int cA;  // column of A inside the stage
     float is;
     __device__ __forceinline__ F2 pair(int q) const
     {
-        return LoadScaled<S>::pair(b + q * TmaGeom<S>::cols + cA, is);
+        return LoadScaled<S>::pair(b + q * C + cA, is);
     }
     __device__ __forceinline__ F2 left(int q) const
     {
-        const S *p = b + q * TmaGeom<S>::cols + cA;
+        const S *p = b + q * C + cA;
         return mk2(LoadScaled<S>::one(p - 1, is), LoadScaled<S>::one(p, is));
     }
     __device__ __forceinline__ F2 right(int q) const
     {
-        const S *p = b + q * TmaGeom<S>::cols + cA;
+        const S *p = b + q * C + cA;
         return mk2(LoadScaled<S>::one(p + 1, is), LoadScaled<S>::one(p + 2, is));
     }
     __device__ __forceinline__ float col(int q, int c) const
     {
-        return LoadScaled<S>::one(b + q * TmaGeom<S>::cols + c, is);
+        return LoadScaled<S>::one(b + q * C + c, is);
     }
 };
 
@@ -1119,7 +1170,7 @@ __device__ __forceinline__ void march3(const KP<float> &k, const S *__restrict__
     constexpr int O = TmaGeom<S>::off;
     const int hc = lane == 0 ? O - 1 : O + 64;  // halo column of lanes 0 / 31
     const int first = (row_s > 0 || k.xper) ? row_s - 1 : row_s;
-    StageRd<S> rd{nullptr, O + 2 * lane, k.inv_scale};
+    StageRd<S, TmaGeom<S>::cols> rd{nullptr, O + 2 * lane, k.inv_scale};
 
     // stored-state fields of row row_s (and u_y of row row_s - 1)
     PM2 pm_cur;
@@ -1152,7 +1203,7 @@ __device__ __forceinline__ void march3(const KP<float> &k, const S *__restrict__
         if (has_p && !rs.wait_upto(t + 1)) return rs.finish();
 
         F2 fv[9], gv[5], hv5[5];
-        OwnStage<S> own{rs.stage(t), O + 2 * lane, k.inv_scale, 0.0f, 0.0f};
+        OwnStage<S, TmaGeom<S>::cols> own{rs.stage(t), O + 2 * lane, k.inv_scale, 0.0f, 0.0f};
         // e_x = +1 group from row i - 1, then that row's stage is free
         if (has_m) {
             rd.b = rs.stage(t - 1);
