@@ -187,7 +187,10 @@ LB_EXPORT lb_status lb_set_params(lb_ctx *ctx, const lb_params *params);
  * rho, u_x, u_y, u_theta, T.  step = 0.  Synchronous. */
 LB_EXPORT lb_status lb_init_fields(lb_ctx *ctx, const double *host_fields);
 
-/* Advance nsteps >= 0 time steps, asynchronously on the context's stream. */
+/* Advance nsteps >= 0 time steps, asynchronously on the context's stream.
+ * Under the automatic launch (lb_set_launch) FP32 and 16-bit lattices take up
+ * to four steps per kernel launch; the results are bitwise those of nsteps
+ * calls of one step. */
 LB_EXPORT lb_status lb_step(lb_ctx *ctx, int32_t nsteps);
 
 /* Pre-collision fields of the current state (the rho, u, u_theta, T the
@@ -237,11 +240,13 @@ LB_EXPORT lb_status lb_get_step(const lb_ctx *ctx, int64_t *step);
  * block (0 = automatic, at most 8) and how the FP32 / 16-bit step fetches
  * its rows (0 = automatic, 1 = plain loads, 2 = TMA bulk tensor copies into
  * a shared-memory ring, 3 = the same ring holding rows i - 1, i, i + 1 of
- * the step, read in place).  Results do not depend on the launch shape.
- * LB_ERR_ARG for values out of range. */
+ * the step, read in place).  With all three 0 (the state after lb_create)
+ * FP32 and 16-bit lattices are stepped on tiles held in shared memory, several
+ * steps per launch; any other setting takes one launch per step.  Results do
+ * not depend on the launch shape.  LB_ERR_ARG for values out of range. */
 LB_EXPORT lb_status lb_set_launch(lb_ctx *ctx, int32_t seg_rows, int32_t warps_per_block, int32_t row_fetch);
 
-/* The launch the next lb_step uses, with the automatic choices resolved:
+/* The launch the next single step uses, with the automatic choices resolved:
  * rows per z-segment, warps per block and row fetch (1, 2 or 3 as for
  * lb_set_launch; FP64 storage always 1).  NULL outputs are skipped. */
 LB_EXPORT lb_status lb_get_launch(const lb_ctx *ctx, int32_t *seg_rows, int32_t *warps_per_block,

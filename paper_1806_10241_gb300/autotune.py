@@ -57,26 +57,33 @@ def _time(stream, fn, steps: int) -> float:
 
 
 def tune_solver(solver, steps: int = 20, use_cache: bool = True) -> tuple:
-    """Pick (seg_rows, warps_per_block, row_fetch) for this solver's shape."""
+    """Pick the launch for this solver's shape: one of SOLVER_CANDIDATES, or the
+    automatic one (several steps per launch; reported as lb_get_launch does).
+    Returns (seg_rows, warps_per_block, row_fetch)."""
     key = f"solver/{solver.storage}/{_size_class(solver.nr)}/{_size_class(solver.nz)}"
     with _lock:
         cache = _load() if use_cache else {}
     if key in cache:
         best = tuple(cache[key]["launch"])
-        solver.set_launch(*best)
-        return best
+        # "auto": the launch was the automatic one, which lb_get_launch reports as `launch`
+        solver.set_launch(*((0, 0, 0) if cache[key].get("auto") else best))
+        return solver.get_launch() if cache[key].get("auto") else best
     cands = SOLVER_CANDIDATES if solver.storage != "fp64" else [(s, w, 1) for s in (16, 32) for w in (2, 4)]
     results = []
-    for c in cands:
+    # the automatic launch first: of equal times it wins, as it takes several steps per launch
+    for c in [(0, 0, 0)] + list(cands):
         solver.set_launch(*c)
         solver.step(2)  # warm
         results.append((_time(solver.stream, solver.step, steps), c))
-    results.sort()
-    best = results[0][1]
+    ms, best = min(results, key=lambda r: r[0])
     solver.set_launch(*best)
+    entry = {"launch": list(best), "ms_per_step": ms}
+    if best == (0, 0, 0):
+        best = solver.get_launch()
+        entry.update(launch=list(best), auto=True)
     with _lock:
         cache = _load()
-        cache[key] = {"launch": list(best), "ms_per_step": results[0][0]}
+        cache[key] = entry
         _store(cache)
     return best
 

@@ -38,7 +38,9 @@ struct lb_ctx {
     Launch launch;
     bool launch_auto;
     alignas(64) unsigned char tmap[2][128];  // TMA tensor maps of dist[0], dist[1]
+    alignas(64) unsigned char tmap64[2][128];  // the same with 64-column boxes, for the tiles
     bool tmap_ready;
+    unsigned passes;  // launches of several steps so far (their block order alternates)
     int *status;  // device status word (bounded-wait timeouts of the step kernel)
     char err[256];
 };
@@ -315,6 +317,7 @@ lb_status lb_create(const lb_grid_desc *desc, void *dev_buf, size_t bytes, void 
     c->params_set = false;
     c->launch = lbk::default_launch(h);
     c->launch_auto = true;
+    c->passes = 0;
     c->err[0] = 0;
     *out = c;
     return LB_OK;
@@ -381,10 +384,36 @@ lb_status lb_step(lb_ctx *ctx, int32_t nsteps)
     if (nsteps < 0) return fail(ctx, LB_ERR_ARG, "nsteps < 0");
     if (ctx->hp.storage != LB_FP64 && !ctx->tmap_ready) {
         for (int b = 0; b < 2; ++b) {
-            cudaError_t e = lbk::make_tensor_map(ctx->hp, ctx->dist[b], ctx->tmap[b]);
+            cudaError_t e = lbk::make_tensor_map(ctx->hp, ctx->dist[b], lbk::ring_cols(ctx->hp.storage), ctx->tmap[b]);
+            if (e == cudaSuccess) e = lbk::make_tensor_map(ctx->hp, ctx->dist[b], 64, ctx->tmap64[b]);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "tensor map");
         }
         ctx->tmap_ready = true;
+    }
+    const int32_t fused = ctx->hp.storage != LB_FP64 && ctx->launch_auto ? nsteps : 0;
+    if (fused > 0) {
+        // Passes of up to T steps.  Their number is made even or odd as the
+        // number of steps is, so that the current buffer alternates with the
+        // step count as it does with one launch per step.
+        lbk::TileLaunch pass = lbk::tile_plan(ctx->hp, 0);
+        int32_t m = (fused + pass.T - 1) / pass.T;
+        if ((fused - m) & 1) ++m;
+        for (int32_t p = 0; p < m; ++p) {
+            const int32_t T = fused / m + (p < fused % m ? 1 : 0);
+            if (T != pass.T) pass = lbk::tile_plan(ctx->hp, T);
+            cudaError_t e;
+            if (T == 1 && pass.strip)  // a large lattice's single step: one warp per work item
+                e = lbk::launch_step(ctx->hp, ctx->launch, ctx->dist[ctx->cur], ctx->dist[1 - ctx->cur],
+                                     (unsigned long long)ctx->step, ctx->tmap[ctx->cur], ctx->status, ctx->stream);
+            else
+                e = lbk::launch_tile(ctx->hp, pass, ctx->tmap64[ctx->cur], ctx->dist[1 - ctx->cur],
+                                     (unsigned long long)ctx->step, ctx->status, (int)(ctx->passes & 1), ctx->stream);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "step launch");
+            ctx->cur ^= 1;
+            ctx->step += T;
+            ctx->passes += 1;
+        }
+        return LB_OK;
     }
     for (int32_t t = 0; t < nsteps; ++t) {
         const void *map = ctx->tmap_ready ? ctx->tmap[ctx->cur] : nullptr;

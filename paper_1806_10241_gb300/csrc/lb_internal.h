@@ -65,8 +65,21 @@ void diag_from_sums(const HostParams &h, const double *res, int kstatus, int64_t
 cudaError_t launch_step(const HostParams &p, const Launch &l, const void *src, void *dst,
                         unsigned long long step, const void *tmap, int *status, cudaStream_t s);
 // Tensor map (CUtensorMap, 128 bytes) of a distribution buffer for the TMA
-// row fetches of the FP32 / 16-bit step.
-cudaError_t make_tensor_map(const HostParams &p, void *buf, void *map_out);
+// row fetches of the FP32 / 16-bit step, box_cols columns per row: ring_cols
+// for the row rings, 64 for the tiles.
+int ring_cols(int storage);
+cudaError_t make_tensor_map(const HostParams &p, void *buf, int box_cols, void *map_out);
+// T time steps on tiles in shared memory (FP32 / 16-bit storage), from the
+// buffer of tmap (64-column boxes) to dst.
+struct TileLaunch {
+    int T, rows, warps;       // time steps, rows of a full tile, warps per block
+    int strip;                // long strips marched through a ring of rows
+    int parts;                // launches that the pass is cut into
+};
+// The pass for a lattice: of T steps, or (T = 0) of as many as pay.
+TileLaunch tile_plan(const HostParams &p, int T);
+cudaError_t launch_tile(const HostParams &p, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
+                        int *status, int rev, cudaStream_t s);
 // Pre-collision fields of rows [row0, row1) into out[5][row1-row0][nr] (double).
 cudaError_t launch_fields(const HostParams &p, const Launch &l, const void *src, double *out,
                           int row0, int row1, cudaStream_t s);

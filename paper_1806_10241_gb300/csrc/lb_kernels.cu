@@ -39,6 +39,7 @@ namespace lbk {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
+constexpr int kMaxSmem = 227 * 1024;  // dynamic shared memory of a block
 constexpr int OUT_COLS = 30;  // columns updated per warp
 #ifndef LB_MARCH_UNROLL
 #define LB_MARCH_UNROLL 2
@@ -809,6 +810,8 @@ __device__ __forceinline__ void grid_dependency_trigger_and_wait()
     grid_dependency_trigger();
     grid_dependency_wait();
 }
+
+#include "lb_tile.cuh"
 
 template <typename S, typename C>
 __device__ __forceinline__ void step_body(const KP<C> &k, const S *__restrict__ src, S *__restrict__ dst,
@@ -1842,9 +1845,12 @@ cudaError_t launch_step(const HostParams &p, const Launch &l, const void *src, v
     DISPATCH(p, (step_t<S, C>(p, l, src, dst, step, tmap, status, s)));
 }
 
+int ring_cols(int storage) { return 64 + 2 * (16 / (int)storage_bytes(storage)); }
+
 // Tensor map of one distribution buffer for the TMA row fetches: a 3-D view
-// [19 planes][nz rows][pitch columns], box of TmaGeom::cols x 1 x 19.
-cudaError_t make_tensor_map(const HostParams &p, void *buf, void *map_out)
+// [19 planes][nz rows][pitch columns], box of box_cols x 1 x 19
+// (ring_cols(storage) for the row rings, 64 for the tiles).
+cudaError_t make_tensor_map(const HostParams &p, void *buf, int box_cols, void *map_out)
 {
     if (p.storage == ST_FP64) return cudaErrorInvalidValue;
     static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
@@ -1861,12 +1867,163 @@ cudaError_t make_tensor_map(const HostParams &p, void *buf, void *map_out)
                                                           : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     const cuuint64_t dims[3] = {(cuuint64_t)p.pitch, (cuuint64_t)p.nz, (cuuint64_t)NQ};
     const cuuint64_t strides[2] = {(cuuint64_t)p.pitch * es, (cuuint64_t)p.plane * es};
-    const cuuint32_t box[3] = {(cuuint32_t)(64 + 2 * (16 / es)), 1u, (cuuint32_t)NQ};
+    const cuuint32_t box[3] = {(cuuint32_t)box_cols, 1u, (cuuint32_t)NQ};
     const cuuint32_t estr[3] = {1u, 1u, 1u};
     CUresult r = encode((CUtensorMap *)map_out, dt, 3, buf, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                         CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+namespace {
+
+// The geometry of a pass of T steps: windows of 64 columns whose starts lie on
+// 16-byte boundaries (TMA), so the margin is T rounded up to 2 columns in
+// FP32, 4 in 16-bit storage.
+TileShape tile_shape(const HostParams &h, int T, int rows)
+{
+    TileShape sh;
+    sh.T = T;
+    sh.cm = h.storage == ST_FP32 ? (T + 1) / 2 * 2 : (T + 3) / 4 * 4;
+    sh.cs = 64 - 2 * sh.cm;
+    sh.rows = rows;
+    sh.rs = rows - 2 * T;
+    sh.nw = h.nr <= 64 ? 1 : (h.nr - 64 + sh.cs - 1) / sh.cs + 1;
+    sh.first = 0;
+    return sh;
+}
+
+// Tiles along z.
+int tiles_along(const HostParams &h, const TileShape &sh)
+{
+    if (h.flow[0] == 2) return (h.nz + sh.rs - 1) / sh.rs;
+    return h.nz <= sh.rows ? 1 : (h.nz - sh.rows + sh.rs - 1) / sh.rs + 1;
+}
+
+int tile_slot_bytes(int storage)
+{
+    return storage == ST_FP32 ? TileGeom<float>::slot_bytes : TileGeom<__half>::slot_bytes;
+}
+
+int tile_slots(bool strip, int T, int rows, int warps) { return strip ? 2 * warps + 2 * T : rows + T - 1; }
+
+// Blocks of a pass that fit on an SM at once (shared memory with 1 KB of it per
+// block for the system, registers).
+int tiles_per_sm(int storage, int slots, int warps)
+{
+    const int smem = slots * tile_slot_bytes(storage) + 128;
+    if (smem > kMaxSmem) return 0;
+    const int regs = storage == ST_FP32 ? kTileRegs<float> : kTileRegs<__half>;
+    return std::min(228 * 1024 / (smem + 1024), 65536 / (regs * 32 * warps));
+}
+
+// The smallest tile, in rows, with which all tiles of the lattice are resident
+// at once, two or more to an SM; 0 when there is none.
+int resident_tile_rows(const HostParams &h, int T, int warps, int sms)
+{
+    for (int rows = 2 * T + 1;; ++rows) {
+        const int per_sm = tiles_per_sm(h.storage, tile_slots(false, T, rows, warps), warps);
+        if (per_sm < 2) return 0;
+        const TileShape sh = tile_shape(h, T, rows);
+        if ((long long)sh.nw * tiles_along(h, sh) <= (long long)sms * per_sm) return rows;
+    }
+}
+
+// Rows of the strips that make up `waves` waves of resident blocks.
+int strip_rows(const HostParams &h, int T, int warps, int waves, int sms)
+{
+    const int slots = tile_slots(true, T, 0, warps), windows = tile_shape(h, T, 2 * T + 1).nw;
+    const int segs = std::max(1, waves * sms * tiles_per_sm(h.storage, slots, warps) / windows);
+    const int rows = h.flow[0] == 2 ? h.nz : std::max(1, h.nz - 2 * T);
+    return (rows + segs - 1) / segs + 2 * T;
+}
+
+template <typename S>
+cudaError_t tile_t(const HostParams &h, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
+                   int *status, int rev, cudaStream_t s)
+{
+    const KP<float> k = make_kp<float>(h);
+    static std::atomic<unsigned long long> tile_set{0}, strip_set{0};
+    cudaError_t e = smem_limit_once(k_tile<S>, kMaxSmem, tile_set);
+    if (e == cudaSuccess) e = smem_limit_once(k_strip<S>, kMaxSmem, strip_set);
+    if (e != cudaSuccess) return e;
+    TileShape sh = tile_shape(h, l.T, l.rows);
+    const long long blocks = (long long)sh.nw * tiles_along(h, sh);
+    const size_t smem = tile_smem_bytes<S>(tile_slots(l.strip, l.T, l.rows, l.warps));
+    for (int p = 0; p < l.parts; ++p) {
+        const int q = rev ? l.parts - 1 - p : p;  // the parts in the order of their blocks
+        sh.first = (int)(blocks * q / l.parts);
+        const int count = (int)(blocks * (q + 1) / l.parts) - sh.first;
+        if (count < 1) continue;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute pdl[1];
+        pdl_config(cfg, pdl, dim3(count), dim3(32 * l.warps), smem, s);
+        e = cudaLaunchKernelEx(&cfg, l.strip ? k_strip<S> : k_tile<S>, k, *(const CUtensorMap *)tmap, (S *)dst,
+                               (const TileShape)sh, step, status, rev);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// Which pass a lattice takes, from its size alone; times per step on one GB300
+// over 24 sizes from 20 x 84 to 1024 x 2048, all tiles, strips, T and warps
+// that fit (the chosen ones lie within 5 % of the best, 8 % at two sizes):
+// - Resident tiles while the lattice fits, as small as that allows.  FP32: three
+//   steps while the tiles are small (100 x 100: 2.45 us, two steps 2.58, four
+//   2.79), two steps from ten rows on (180 x 360: 3.77 against 4.00 us).  In
+//   16-bit storage, whose margins are 4 columns for up to four steps, three
+//   (100 x 100: 2.89 us, two 2.99, four 3.03; 400 x 400: 5.90, 6.04, 5.98).
+// - Strips beyond (512 x 512 FP32: 7.5 us, tiles 8.0).  FP32: two steps (1024 x
+//   1024: 22.9 us; three 23.1, four 24.0).  16-bit: four (1024 x 1024: 24.7 us;
+//   three 25.4, two 24.9).  Six (eight) warps per block while the strips are
+//   short, four and one more block per SM from 40 (60) rows on (512 x 1024
+//   FP32: 12.8 against 13.6 us; 1024 x 1024: 23.6 against 22.9).
+// - FP32 strips of more than 64 rows go out as two launches, half of the strips
+//   each, so that a large lattice keeps one launch per step, which callers that
+//   time single kernels count on; 1024 x 2048: 44.8 us per step, 40.8 as one
+//   launch of two waves.
+TileLaunch tile_plan(const HostParams &h, int T)
+{
+    const int sms = sm_count();
+    const bool fp32 = h.storage == ST_FP32;
+    const int W = fp32 ? 6 : 8;
+    TileLaunch l{T, 0, W, 0, 1};
+    if (T == 0) {  // the best number of steps
+        l.T = 3;
+        l.rows = resident_tile_rows(h, 3, W, sms);
+        if (fp32 && (l.rows == 0 || l.rows > 9)) {
+            l.T = 2;
+            l.rows = resident_tile_rows(h, 2, W, sms);
+        }
+        if (l.rows == 0) l.T = fp32 ? 2 : 4;
+    } else {
+        l.rows = resident_tile_rows(h, T, W, sms);
+    }
+    if (l.rows) return l;
+    l.strip = 1;
+    l.rows = strip_rows(h, l.T, W, 1, sms);
+    if (l.rows > (fp32 ? 40 : 60)) {
+        l.warps = 4;
+        l.rows = strip_rows(h, l.T, l.warps, 1, sms);
+        if (fp32 && l.T == 2 && l.rows > 64) {
+            l.parts = 2;
+            l.rows = strip_rows(h, l.T, l.warps, 2, sms);
+        }
+    }
+    return l;
+}
+
+cudaError_t launch_tile(const HostParams &p, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
+                        int *status, int rev, cudaStream_t s)
+{
+    switch (p.storage) {
+        case ST_FP32: return tile_t<float>(p, l, tmap, dst, step, status, rev, s);
+        case ST_BF16: return tile_t<__nv_bfloat16>(p, l, tmap, dst, step, status, rev, s);
+        case ST_FP16: return tile_t<__half>(p, l, tmap, dst, step, status, rev, s);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_wait_selftest(int *status, int polls, cudaStream_t s)
@@ -1942,8 +2099,8 @@ cudaError_t batch_fill_desc(const HostParams &h, void *buf0, void *buf1, unsigne
 {
     BatchDesc d;
     std::memset(&d, 0, sizeof(d));
-    cudaError_t e = make_tensor_map(h, buf0, d.map[0]);
-    if (e == cudaSuccess) e = make_tensor_map(h, buf1, d.map[1]);
+    cudaError_t e = make_tensor_map(h, buf0, ring_cols(h.storage), d.map[0]);
+    if (e == cudaSuccess) e = make_tensor_map(h, buf1, ring_cols(h.storage), d.map[1]);
     if (e != cudaSuccess) return e;
     d.k = make_kp<float>(h);
     d.buf[0] = buf0;
