@@ -9,7 +9,7 @@
 
 namespace lbk {
 
-enum Mode { MODE_STEP = 0, MODE_FIELDS = 1, MODE_DIAG = 2, MODE_DIAG_STRIP = 3 };
+enum Mode { MODE_FIELDS = 1, MODE_DIAG = 2, MODE_DIAG_STRIP = 3 };
 enum Storage { ST_FP64 = 0, ST_FP32 = 1, ST_BF16 = 2, ST_FP16 = 3 };
 
 constexpr int NQ = 19;        // 9 (f) + 5 (g) + 5 (h) planes

@@ -20,6 +20,7 @@
 // and 19 stores per node update.
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -40,6 +41,7 @@ namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kMaxSmem = 227 * 1024;  // dynamic shared memory of a block
+constexpr int kSmemPerSm = 228 * 1024;  // of an SM, 1 KB of it taken per block by the system
 constexpr int OUT_COLS = 30;  // columns updated per warp
 #ifndef LB_MARCH_UNROLL
 #define LB_MARCH_UNROLL 2
@@ -81,12 +83,12 @@ template <typename S> struct Scaled { static constexpr bool value = std::is_same
 
 // ---- kernel parameters in the compute type --------------------------------
 
-// Parameters of the pair kernels' node update as FP32x2 operands (both halves
-// equal): the packed instructions take them as they lie in the parameters,
-// where a scalar would first be copied into a register pair.
-struct PairConst {
-    float2 rho0, T0, bfx, fb, nu, nuh, alh, k3;              // fb = rho0 g_beta; nu / 2, alpha / 2, rho0 / 3
-    float2 c3, c4, nc4, ch, nch, cg, ct, m9, m6, m5, sg, os; // relaxation and back-transform factors, storage scale
+// Parameters of the node update (update_node2) as its operands: in FP32 as
+// packed pairs with equal halves, which the packed instructions take as they
+// lie in the parameters, where a scalar would first be copied into a pair.
+template <typename E> struct NodeConst {
+    E rho0, T0, bfx, fb, nu, nuh, alh, k3;              // fb = rho0 g_beta; nu / 2, alpha / 2, rho0 / 3
+    E c3, c4, nc4, ch, nch, cg, ct, m9, m6, m5, sg, os; // relaxation and back-transform factors, storage scale
 };
 
 template <typename C> struct KP {
@@ -113,7 +115,7 @@ template <typename C> struct KP {
     // u_theta and T for the central differences.
     C latf[2][3], latgs[2], latgc[2], laths[2], lathc[2], gha[2][4], ghb[2][4];
     const float *ytab;    // y[pitch] then 1/y[pitch] (pair kernels)
-    PairConst pc;
+    NodeConst<typename std::conditional<std::is_same<C, float>::value, float2, C>::type> pc;
     // Nusselt and equivalent-conductivity scales per side (diagnostics)
     double nu_scale[4], keq_scale[4];
 };
@@ -195,17 +197,19 @@ template <typename C> KP<C> make_kp(const HostParams &h)
     }
     k.ytab = h.ytab;
     {
-        const float osc = (float)h.scale, om3 = (float)h.omega3, om4 = (float)omn, omh = (float)h.omega_hi;
-        const float rho0 = (float)h.rho0, nu = (float)h.nu, alpha = (float)h.alpha;
-        auto two = [](float v) { return make_float2(v, v); };
-        PairConst &c = k.pc;
-        c.rho0 = two(rho0), c.T0 = two((float)h.T0), c.bfx = two((float)h.body_fx), c.fb = two(rho0 * (float)h.g_beta);
-        c.nu = two(nu), c.nuh = two(0.5f * nu), c.alh = two(0.5f * alpha), c.k3 = two(rho0 * (1.0f / 3.0f));
-        c.c3 = two(om3 * (1.0f / 12.0f) * osc), c.c4 = two(om4 * 0.25f * osc), c.nc4 = two(om4 * -0.25f * osc);
-        c.ch = two(omh * 0.25f * osc), c.nch = two(omh * -0.25f * osc);
-        c.cg = two(om4 * 0.5f * osc), c.ct = two((float)oma * 0.5f * osc);
-        c.m9 = two((1.0f / 9.0f) * osc), c.m6 = two((1.0f / 6.0f) * osc), c.m5 = two(0.2f * osc);
-        c.sg = two(h.sign_literal ? -1.0f : 1.0f), c.os = two(osc);
+        const C osc = (C)h.scale, om3 = k.om3, om4 = k.om4, omh = k.omhi, third = (C)1 / (C)3, ninth = (C)1 / (C)9;
+        auto e = [](C v) {
+            if constexpr (std::is_same<C, float>::value) return make_float2(v, v);
+            else return v;
+        };
+        auto &c = k.pc;
+        c.rho0 = e(k.rho0), c.T0 = e(k.T0), c.bfx = e(k.bfx), c.fb = e(k.rho0 * k.gbeta);
+        c.nu = e(k.nu), c.nuh = e((C)0.5 * k.nu), c.alh = e((C)0.5 * k.alpha), c.k3 = e(k.rho0 * third);
+        c.c3 = e(om3 * ((C)1 / (C)12) * osc), c.c4 = e(om4 * (C)0.25 * osc), c.nc4 = e(om4 * (C)-0.25 * osc);
+        c.ch = e(omh * (C)0.25 * osc), c.nch = e(omh * (C)-0.25 * osc);
+        c.cg = e(k.omg * (C)0.5 * osc), c.ct = e(k.omh * (C)0.5 * osc);
+        c.m9 = e(ninth * osc), c.m6 = e((C)1 / (C)6 * osc), c.m5 = e((C)0.2 * osc);
+        c.sg = e((C)(h.sign_literal ? -1 : 1)), c.os = e(osc);
     }
     // Nusselt normalisation (Sec. 3.2): lateral walls -R_w / (H dT), end
     // walls -(H / dT) * 2 / (R_o^2 - R_i^2); dT from the Dirichlet values.
@@ -513,6 +517,87 @@ struct DiagAcc {
 
 // ---- the march ---------------------------------------------------------------
 
+// Wall and axis rules (Sec. 3) on the pulled values of node (i, cl), in units
+// of the storage scale sc; the own stored values are read from src.
+template <typename S, typename C>
+__device__ __forceinline__ void wall_rules1(const KP<C> &k, const S *__restrict__ src, int i, int cl, bool at_c0,
+                                            bool at_cN, bool has_m, bool has_p, C y, C sc, C fv[9], C gv[5], C hv[5])
+{
+    const int nr = k.nr, nz = k.nz;
+    // lateral boundaries (Sec. 3): the population entering from r < r0 or
+    // r > r0 + nr is rebuilt from the node's own stored values
+    {
+        if (at_c0) {
+            const int sd = 2;
+            const C rw = k.rho0 * sc;
+            if (k.flow[sd] == 1) {  // axis: mirror images
+                fv[2] = own<S, C>(src, k, 4, i, 0);
+                if (has_m) fv[5] = own<S, C>(src, k, 8, i > 0 ? i - 1 : nz - 1, 0);
+                if (has_p) fv[6] = own<S, C>(src, k, 7, i + 1 < nz ? i + 1 : 0, 0);
+            } else {  // wall: bounce-back + moving-wall term 6 w rho0 (e.u_w)
+                const C ux_w = k.uwx[sd], uy_w = k.uwy[sd];
+                fv[2] = own<S, C>(src, k, 4, i, 0) + rw * (C)(6.0 / 9.0) * uy_w;
+                fv[5] = own<S, C>(src, k, 7, i, 0) + rw * (C)(6.0 / 36.0) * (ux_w + uy_w);
+                fv[6] = own<S, C>(src, k, 8, i, 0) + rw * (C)(6.0 / 36.0) * (-ux_w + uy_w);
+            }
+            gv[2] = scalar_bc<C>(k.swirl[sd], own<S, C>(src, k, G0 + 4, i, 0), wall_psi<C>(k, sd, y) * sc, true);
+            hv[2] = scalar_bc<C>(k.heat[sd], own<S, C>(src, k, H0 + 4, i, 0), (k.Tw[sd] - k.T0) * sc, false);
+        }
+        if (at_cN) {
+            const int sd = 3;
+            const C rw = k.rho0 * sc;
+            const C ux_w = k.uwx[sd], uy_w = k.uwy[sd];
+            fv[4] = own<S, C>(src, k, 2, i, nr - 1) + rw * (C)(6.0 / 9.0) * (-uy_w);
+            fv[7] = own<S, C>(src, k, 5, i, nr - 1) + rw * (C)(6.0 / 36.0) * (-ux_w - uy_w);
+            fv[8] = own<S, C>(src, k, 6, i, nr - 1) + rw * (C)(6.0 / 36.0) * (ux_w - uy_w);
+            gv[4] = scalar_bc<C>(k.swirl[sd], own<S, C>(src, k, G0 + 2, i, nr - 1), wall_psi<C>(k, sd, y) * sc, true);
+            hv[4] = scalar_bc<C>(k.heat[sd], own<S, C>(src, k, H0 + 2, i, nr - 1), (k.Tw[sd] - k.T0) * sc, false);
+        }
+    }
+    // end walls (rows 0 and nz-1 unless periodic); they win in corners.  A
+    // free surface (Sec. 3.6) reflects f specularly: the population that
+    // left the neighbour column towards the wall, e_x reversed; at a corner
+    // column the lateral side's rule for the node itself
+    if (!has_m) {
+        const int sd = end_seg(k, 0, cl);
+        const C rw = k.rho0 * sc, ux_w = k.uwx[sd], uy_w = k.uwy[sd];
+        if (k.flow[sd] == 3) {
+            fv[1] = own<S, C>(src, k, 3, i, cl);
+            fv[5] = at_c0 ? own<S, C>(src, k, 7, i, 0) +
+                                (k.flow[2] == 1 ? (C)0 : rw * (C)(6.0 / 36.0) * (k.uwx[2] + k.uwy[2]))
+                          : own<S, C>(src, k, 6, i, cl > 0 ? cl - 1 : 0);
+            fv[8] = at_cN ? own<S, C>(src, k, 6, i, cl) + rw * (C)(6.0 / 36.0) * (k.uwx[3] - k.uwy[3])
+                          : own<S, C>(src, k, 7, i, cl + 1 < nr ? cl + 1 : cl);
+        } else {
+            fv[1] = own<S, C>(src, k, 3, i, cl) + rw * (C)(6.0 / 9.0) * ux_w;
+            fv[5] = own<S, C>(src, k, 7, i, cl) + rw * (C)(6.0 / 36.0) * (ux_w + uy_w);
+            fv[8] = own<S, C>(src, k, 6, i, cl) + rw * (C)(6.0 / 36.0) * (ux_w - uy_w);
+        }
+        gv[1] = scalar_bc<C>(k.swirl[sd], own<S, C>(src, k, G0 + 3, i, cl), wall_psi<C>(k, sd, y) * sc, true);
+        hv[1] = scalar_bc<C>(heat_rule(k, sd), own<S, C>(src, k, H0 + 3, i, cl), (end_T(k, sd, y) - k.T0) * sc,
+                             false);
+    }
+    if (!has_p) {
+        const int sd = end_seg(k, 1, cl);
+        const C rw = k.rho0 * sc, ux_w = k.uwx[sd], uy_w = k.uwy[sd];
+        if (k.flow[sd] == 3) {
+            fv[3] = own<S, C>(src, k, 1, i, cl);
+            fv[6] = at_c0 ? own<S, C>(src, k, 8, i, 0) +
+                                (k.flow[2] == 1 ? (C)0 : rw * (C)(6.0 / 36.0) * (-k.uwx[2] + k.uwy[2]))
+                          : own<S, C>(src, k, 5, i, cl > 0 ? cl - 1 : 0);
+            fv[7] = at_cN ? own<S, C>(src, k, 5, i, cl) + rw * (C)(6.0 / 36.0) * (-k.uwx[3] - k.uwy[3])
+                          : own<S, C>(src, k, 8, i, cl + 1 < nr ? cl + 1 : cl);
+        } else {
+            fv[3] = own<S, C>(src, k, 1, i, cl) + rw * (C)(6.0 / 9.0) * (-ux_w);
+            fv[6] = own<S, C>(src, k, 8, i, cl) + rw * (C)(6.0 / 36.0) * (-ux_w + uy_w);
+            fv[7] = own<S, C>(src, k, 5, i, cl) + rw * (C)(6.0 / 36.0) * (-ux_w - uy_w);
+        }
+        gv[3] = scalar_bc<C>(k.swirl[sd], own<S, C>(src, k, G0 + 1, i, cl), wall_psi<C>(k, sd, y) * sc, true);
+        hv[3] = scalar_bc<C>(heat_rule(k, sd), own<S, C>(src, k, H0 + 1, i, cl), (end_T(k, sd, y) - k.T0) * sc,
+                             false);
+    }
+}
+
 template <typename S, typename C, int MODE>
 __device__ __forceinline__ void march(const KP<C> &k, const S *__restrict__ src, S *__restrict__ dst,
                                       double *__restrict__ fout, int fout_row0, int fout_rows, int c,
@@ -590,78 +675,7 @@ __device__ __forceinline__ void march(const KP<C> &k, const S *__restrict__ src,
         hv[0] = x0_cur[6]; hv[2] = x0_cur[7]; hv[4] = x0_cur[8];
         fv[3] = xp_n[0]; fv[6] = xp_n[1]; fv[7] = xp_n[2]; gv[3] = xp_n[3]; hv[3] = xp_n[4];
 
-        // lateral boundaries (Sec. 3): the population entering from r < r0 or
-        // r > r0 + nr is rebuilt from the node's own stored values
-        if (edge_warp) {
-            if (at_c0) {
-                const int sd = 2;
-                const C rw = k.rho0 * sc;
-                if (k.flow[sd] == 1) {  // axis: mirror images
-                    fv[2] = own<S, C>(src, k, 4, i, 0);
-                    if (has_m) fv[5] = own<S, C>(src, k, 8, i > 0 ? i - 1 : nz - 1, 0);
-                    if (has_p) fv[6] = own<S, C>(src, k, 7, i + 1 < nz ? i + 1 : 0, 0);
-                } else {  // wall: bounce-back + moving-wall term 6 w rho0 (e.u_w)
-                    const C ux_w = k.uwx[sd], uy_w = k.uwy[sd];
-                    fv[2] = own<S, C>(src, k, 4, i, 0) + rw * (C)(6.0 / 9.0) * uy_w;
-                    fv[5] = own<S, C>(src, k, 7, i, 0) + rw * (C)(6.0 / 36.0) * (ux_w + uy_w);
-                    fv[6] = own<S, C>(src, k, 8, i, 0) + rw * (C)(6.0 / 36.0) * (-ux_w + uy_w);
-                }
-                gv[2] = scalar_bc<C>(k.swirl[sd], own<S, C>(src, k, G0 + 4, i, 0), wall_psi<C>(k, sd, y) * sc, true);
-                hv[2] = scalar_bc<C>(k.heat[sd], own<S, C>(src, k, H0 + 4, i, 0), (k.Tw[sd] - k.T0) * sc, false);
-            }
-            if (at_cN) {
-                const int sd = 3;
-                const C rw = k.rho0 * sc;
-                const C ux_w = k.uwx[sd], uy_w = k.uwy[sd];
-                fv[4] = own<S, C>(src, k, 2, i, nr - 1) + rw * (C)(6.0 / 9.0) * (-uy_w);
-                fv[7] = own<S, C>(src, k, 5, i, nr - 1) + rw * (C)(6.0 / 36.0) * (-ux_w - uy_w);
-                fv[8] = own<S, C>(src, k, 6, i, nr - 1) + rw * (C)(6.0 / 36.0) * (ux_w - uy_w);
-                gv[4] = scalar_bc<C>(k.swirl[sd], own<S, C>(src, k, G0 + 2, i, nr - 1), wall_psi<C>(k, sd, y) * sc, true);
-                hv[4] = scalar_bc<C>(k.heat[sd], own<S, C>(src, k, H0 + 2, i, nr - 1), (k.Tw[sd] - k.T0) * sc, false);
-            }
-        }
-        // end walls (rows 0 and nz-1 unless periodic); they win in corners.  A
-        // free surface (Sec. 3.6) reflects f specularly: the population that
-        // left the neighbour column towards the wall, e_x reversed; at a corner
-        // column the lateral side's rule for the node itself
-        if (!has_m) {
-            const int sd = end_seg(k, 0, cl);
-            const C rw = k.rho0 * sc, ux_w = k.uwx[sd], uy_w = k.uwy[sd];
-            if (k.flow[sd] == 3) {
-                fv[1] = own<S, C>(src, k, 3, i, cl);
-                fv[5] = at_c0 ? own<S, C>(src, k, 7, i, 0) +
-                                    (k.flow[2] == 1 ? (C)0 : rw * (C)(6.0 / 36.0) * (k.uwx[2] + k.uwy[2]))
-                              : own<S, C>(src, k, 6, i, cl > 0 ? cl - 1 : 0);
-                fv[8] = at_cN ? own<S, C>(src, k, 6, i, cl) + rw * (C)(6.0 / 36.0) * (k.uwx[3] - k.uwy[3])
-                              : own<S, C>(src, k, 7, i, cl + 1 < nr ? cl + 1 : cl);
-            } else {
-                fv[1] = own<S, C>(src, k, 3, i, cl) + rw * (C)(6.0 / 9.0) * ux_w;
-                fv[5] = own<S, C>(src, k, 7, i, cl) + rw * (C)(6.0 / 36.0) * (ux_w + uy_w);
-                fv[8] = own<S, C>(src, k, 6, i, cl) + rw * (C)(6.0 / 36.0) * (ux_w - uy_w);
-            }
-            gv[1] = scalar_bc<C>(k.swirl[sd], own<S, C>(src, k, G0 + 3, i, cl), wall_psi<C>(k, sd, y) * sc, true);
-            hv[1] = scalar_bc<C>(heat_rule(k, sd), own<S, C>(src, k, H0 + 3, i, cl), (end_T(k, sd, y) - k.T0) * sc,
-                                 false);
-        }
-        if (!has_p) {
-            const int sd = end_seg(k, 1, cl);
-            const C rw = k.rho0 * sc, ux_w = k.uwx[sd], uy_w = k.uwy[sd];
-            if (k.flow[sd] == 3) {
-                fv[3] = own<S, C>(src, k, 1, i, cl);
-                fv[6] = at_c0 ? own<S, C>(src, k, 8, i, 0) +
-                                    (k.flow[2] == 1 ? (C)0 : rw * (C)(6.0 / 36.0) * (-k.uwx[2] + k.uwy[2]))
-                              : own<S, C>(src, k, 5, i, cl > 0 ? cl - 1 : 0);
-                fv[7] = at_cN ? own<S, C>(src, k, 5, i, cl) + rw * (C)(6.0 / 36.0) * (-k.uwx[3] - k.uwy[3])
-                              : own<S, C>(src, k, 8, i, cl + 1 < nr ? cl + 1 : cl);
-            } else {
-                fv[3] = own<S, C>(src, k, 1, i, cl) + rw * (C)(6.0 / 9.0) * (-ux_w);
-                fv[6] = own<S, C>(src, k, 8, i, cl) + rw * (C)(6.0 / 36.0) * (-ux_w + uy_w);
-                fv[7] = own<S, C>(src, k, 5, i, cl) + rw * (C)(6.0 / 36.0) * (-ux_w - uy_w);
-            }
-            gv[3] = scalar_bc<C>(k.swirl[sd], own<S, C>(src, k, G0 + 1, i, cl), wall_psi<C>(k, sd, y) * sc, true);
-            hv[3] = scalar_bc<C>(heat_rule(k, sd), own<S, C>(src, k, H0 + 1, i, cl), (end_T(k, sd, y) - k.T0) * sc,
-                                 false);
-        }
+        wall_rules1<S, C>(k, src, i, cl, edge_warp && at_c0, edge_warp && at_cN, has_m, has_p, y, sc, fv, gv, hv);
         if (Scaled<S>::value) {
 #pragma unroll
             for (int q = 0; q < 9; ++q) fv[q] *= is;
@@ -711,20 +725,7 @@ __device__ __forceinline__ void march(const KP<C> &k, const S *__restrict__ src,
         NodeOut<C> o;
         update_node<C>(k, y, iy, fv, gv, hv, dxuy, dyux, dyuy, dyut, dyT, o);
 
-        if (MODE == MODE_STEP) {
-            if (out_lane) {
-                S *p = dst + (long long)i * k.pitch + c;
-                const C m = Scaled<S>::value ? sc : (C)1;
-#pragma unroll
-                for (int q = 0; q < 9; ++q) Cvt<S, C>::st(p + q * k.plane, Scaled<S>::value ? o.f[q] * m : o.f[q]);
-#pragma unroll
-                for (int q = 0; q < 5; ++q)
-                    Cvt<S, C>::st(p + (G0 + q) * k.plane, Scaled<S>::value ? o.g[q] * m : o.g[q]);
-#pragma unroll
-                for (int q = 0; q < 5; ++q)
-                    Cvt<S, C>::st(p + (H0 + q) * k.plane, Scaled<S>::value ? o.h[q] * m : o.h[q]);
-            }
-        } else if (MODE == MODE_FIELDS) {
+        if (MODE == MODE_FIELDS) {
             if (out_lane) {
                 const long long n = (long long)fout_rows * nr;  // plane stride of the output chunk
                 double *p = fout + (long long)(i - fout_row0) * nr + c;
@@ -813,25 +814,216 @@ __device__ __forceinline__ void grid_dependency_trigger_and_wait()
 
 #include "lb_tile.cuh"
 
-template <typename S, typename C>
-__device__ __forceinline__ void step_body(const KP<C> &k, const S *__restrict__ src, S *__restrict__ dst,
-                                          int seg_rows, int nwin)
+// FP64 step (the reference path of the other storages).  The FP64 pipe bounds
+// it: an FP64 instruction occupies a scheduler's pipe for 64 cycles whatever
+// the number of active lanes (76 with all four of an SM's busy; measured), so
+// what counts is FP64 instructions per row of 32 columns -- 306 of the node
+// update, 33 of a row's fields -- and schedulers in use.  A block takes `rows`
+// rows of a 32-column window.  First its warps form the fields of the stored
+// state of the rows and their neighbours, once per node, the two halo columns
+// gathered into tasks of 16 rows each; then the warps update the rows.  With
+// split = 2 a row goes to two warps, one storing f and the other g and h, each
+// repeating the source terms (194 and 173 instead of 306 instructions): faster
+// where the lattice has fewer rows of 32 columns than the device schedulers.
+// The distributions are read where they lie (L1 / L2): loads, indices and
+// rules other than arithmetic cost nothing beside the FP64 pipe.
+// 41 x 41: 70.6 us per step before (30-column march, at least four rows per
+// warp, terms not fused), 10.9 us now; 256 x 512: 220 us, 88.5 us.
+constexpr int kFields64Cols = 34;  // 32 columns and the halo columns
+
+// Wall rules of the FP64 step with their constants formed once on the host
+// (entries 0..3 the sides, 4 the outer segment of a split top): the
+// moving-wall terms of the three populations entering from the wall, and sign
+// and constant of the scalar rules x = s x_own + c, the constants of end walls
+// linear in the column radius (psi_w = rho0 omega y; the ramp): c0 + c1 y.
+struct Walls64 {
+    double f[5][3], gs[5], gc0[5], gc1[5], hs[5], hc0[5], hc1[5];
+};
+
+Walls64 make_walls64(const KP<double> &k)
 {
-    const int warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (warp >= nwin) return;  // whole warps only
-    const int c = warp * OUT_COLS - 1 + (threadIdx.x & 31);
-    const int s = blockIdx.y * seg_rows;
-    const int e = min(k.nz, s + seg_rows);
-    grid_dependency_trigger_and_wait();
-    march<S, C, MODE_STEP>(k, src, dst, nullptr, 0, 0, c, s, e, nullptr);
+    Walls64 w;
+    for (int sd = 0; sd < 5; ++sd) {
+        const double a = k.rho0 * (6.0 / 9.0), b = k.rho0 * (6.0 / 36.0), ux = k.uwx[sd], uy = k.uwy[sd];
+        const bool end = sd != 2 && sd != 3, up = sd == 1 || sd == 4;
+        const double f[4][3] = {{a * ux, b * (ux + uy), b * (ux - uy)},      // f1, f5, f8 at the bottom
+                                {-a * ux, b * (-ux + uy), b * (-ux - uy)},   // f3, f6, f7 at the top
+                                {a * uy, b * (ux + uy), b * (-ux + uy)},     // f2, f5, f6 at the inner side
+                                {-a * uy, b * (-ux - uy), b * (ux - uy)}};   // f4, f7, f8 at the outer side
+        for (int q = 0; q < 3; ++q) w.f[sd][q] = f[up ? 1 : sd][q];
+        w.gs[sd] = k.swirl[sd] == 0 || k.swirl[sd] == 2 ? -1.0 : 1.0;
+        const double psi = k.swirl[sd] == 0 ? (2.0 / 6.0) * (k.rho0 * k.omega[sd]) : 0.0;
+        w.gc0[sd] = end ? 0.0 : psi * (sd == 2 ? k.r0c : k.roc);
+        w.gc1[sd] = end ? psi : 0.0;
+        const bool ramp = k.heat[sd] == 4;
+        w.hs[sd] = k.heat[sd] == 0 || ramp ? -1.0 : 1.0;
+        w.hc0[sd] = ramp ? (2.0 / 6.0) * (k.ramp0 - k.T0) : (k.heat[sd] == 0 ? (2.0 / 6.0) * (k.Tw[sd] - k.T0) : 0.0);
+        w.hc1[sd] = ramp ? (2.0 / 6.0) * k.ramp1 : 0.0;
+    }
+    return w;
 }
 
-// FP64 step (the GPU FP64 reference path): the scalar march, 30 columns per warp
-template <typename S, typename C>
-__global__ void __maxnreg__(255) k_step64(KP<C> k, const S *__restrict__ src, S *__restrict__ dst,
-                                          int seg_rows, int nwin)
+__global__ void __launch_bounds__(256) k_step64(const __grid_constant__ KP<double> k, const __grid_constant__ Walls64 w,
+                                                const double *__restrict__ src, double *__restrict__ dst, int rows,
+                                                int nwin, int split)
 {
-    step_body<S, C>(k, src, dst, seg_rows, nwin);
+    extern __shared__ double fields64[];  // [rows + 2][u_x, u_y, u_theta, T][34]
+    const int warp = __shfl_sync(FULL, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31, W = blockDim.x >> 5;
+    const int c0 = (int)(blockIdx.x % nwin) * 32, s = (int)(blockIdx.x / nwin) * rows;
+    const int nr = k.nr, nz = k.nz, n = min(rows, nz - s);
+    const int c = c0 + lane, cl = min(c, nr - 1);
+    const bool at_c0 = c == 0, at_cN = c == nr - 1, inner = c0 == 0, outer = c0 + 32 >= nr;
+    // all of the column's own arithmetic before the wait for the last step
+    const double y = k.r0 + cl + 0.5;
+    const Geo<D1> geo = geo_of(k.pc, D1{k.planar ? 0.0 : rcp1(y)});
+    grid_dependency_trigger_and_wait();
+
+    // Fields of rows s - 1 .. s + n: all four of the block's rows, task by task;
+    // of the halo columns c0 - 1 and c0 + 32, as (row, side) pairs; and u_y of
+    // the rows below and above, one task.
+    const int halo_tasks = (2 * n + 31) / 32;
+    for (int t = warp; t < n + halo_tasks + 1; t += W) {
+        const int h = lane + 32 * (t - n);
+        const bool rim = t == n + halo_tasks, halo = !rim && t >= n;
+        for (int q = 0; q < (rim ? 2 : 1); ++q) {
+            const int r = rim ? q * (n + 1) : (halo ? (h >> 1) + 1 : t + 1);
+            const int cc = halo ? ((h & 1) ? c0 + 32 : c0 - 1) : c;
+            int i = s - 1 + r;
+            if (k.xper) i = i < 0 ? i + nz : (i >= nz ? i - nz : i);
+            if (r > n + 1 || (halo && r > n) || i < 0 || i >= nz || cc < 0 || cc >= nr) continue;
+            double v[NQ];
+            load_row<double, double>(src, k, i, cc, v);
+            const double s13 = v[1] + v[3], s24 = v[2] + v[4], s5678 = (v[5] + v[7]) + (v[6] + v[8]);
+            const double a57 = v[5] - v[7], a86 = v[8] - v[6];
+            const double ir = rcp1(k.rho0 + ((v[0] + s13) + (s24 + s5678)));
+            double *f = fields64 + (r * 4) * kFields64Cols + (cc - c0 + 1);
+            f[kFields64Cols] = ((v[2] - v[4]) + (a57 - a86)) * ir;
+            if (rim) continue;
+            f[0] = ((v[1] - v[3]) + (a57 + a86)) * ir;
+            f[2 * kFields64Cols] = ((v[9] + v[10]) + (v[11] + v[12]) + v[13]) * ir;
+            f[3 * kFields64Cols] = k.T0 + ((v[14] + v[15]) + (v[16] + v[17]) + v[18]);
+        }
+    }
+    __syncthreads();
+
+    for (int t = warp; t < n * split; t += W) {
+        const int r = t / split + 1, i = s + r - 1;
+        const bool has_m = i > 0 || k.xper, has_p = i + 1 < nz || k.xper;
+        // pulled values
+        const int im = i > 0 ? i - 1 : nz - 1, ip = i + 1 < nz ? i + 1 : 0;
+        const int jm = max(cl - 1, 0), jp = min(cl + 1, nr - 1);
+        auto ld = [&](int q, int row, int col) { return src[q * k.plane + (long long)row * k.pitch + col]; };
+        double fv[9] = {ld(0, i, cl),  ld(1, im, cl), ld(2, i, jm),  ld(3, ip, cl), ld(4, i, jp),
+                        ld(5, im, jm), ld(6, ip, jm), ld(7, ip, jp), ld(8, im, jp)};
+        double gv[5] = {ld(9, i, cl), ld(10, im, cl), ld(11, i, jm), ld(12, ip, cl), ld(13, i, jp)};
+        double hv[5] = {ld(14, i, cl), ld(15, im, cl), ld(16, i, jm), ld(17, ip, cl), ld(18, i, jp)};
+        // lateral walls and the axis (Sec. 3)
+        if (inner && at_c0) {
+            if (k.flow[2] == 1) {
+                fv[2] = ld(4, i, 0);
+                if (has_m) fv[5] = ld(8, im, 0);
+                if (has_p) fv[6] = ld(7, ip, 0);
+            } else {
+                fv[2] = ld(4, i, 0) + w.f[2][0];
+                fv[5] = ld(7, i, 0) + w.f[2][1];
+                fv[6] = ld(8, i, 0) + w.f[2][2];
+            }
+            gv[2] = __fma_rn(w.gs[2], ld(13, i, 0), w.gc0[2]);
+            hv[2] = __fma_rn(w.hs[2], ld(18, i, 0), w.hc0[2]);
+        }
+        if (outer && at_cN) {
+            fv[4] = ld(2, i, cl) + w.f[3][0];
+            fv[7] = ld(5, i, cl) + w.f[3][1];
+            fv[8] = ld(6, i, cl) + w.f[3][2];
+            gv[4] = __fma_rn(w.gs[3], ld(11, i, cl), w.gc0[3]);
+            hv[4] = __fma_rn(w.hs[3], ld(16, i, cl), w.hc0[3]);
+        }
+        // end walls; they win in corners.  A free surface reflects f
+        // specularly, at a corner column by the lateral side's rule
+        if (!has_m) {
+            const int sd = 0;
+            if (k.flow[sd] == 3) {
+                fv[1] = ld(3, i, cl);
+                fv[5] = ld(6, i, jm);
+                fv[8] = ld(7, i, jp);
+                if (inner && at_c0) fv[5] = k.flow[2] == 1 ? ld(7, i, 0) : ld(7, i, 0) + w.f[2][1];
+                if (outer && at_cN) fv[8] = ld(6, i, cl) + w.f[3][2];
+            } else {
+                fv[1] = ld(3, i, cl) + w.f[sd][0];
+                fv[5] = ld(7, i, cl) + w.f[sd][1];
+                fv[8] = ld(6, i, cl) + w.f[sd][2];
+            }
+            gv[1] = __fma_rn(w.gs[sd], ld(12, i, cl), w.gc1[sd] * y);
+            hv[1] = __fma_rn(w.hs[sd], ld(17, i, cl), w.hc0[sd]);
+        }
+        if (!has_p) {
+            const int sd = end_seg(k, 1, cl);
+            if (k.flow[sd] == 3) {
+                fv[3] = ld(1, i, cl);
+                fv[6] = ld(5, i, jm);
+                fv[7] = ld(8, i, jp);
+                if (inner && at_c0) fv[6] = k.flow[2] == 1 ? ld(8, i, 0) : ld(8, i, 0) + w.f[2][2];
+                if (outer && at_cN) fv[7] = ld(5, i, cl) + w.f[3][1];
+            } else {
+                fv[3] = ld(1, i, cl) + w.f[sd][0];
+                fv[6] = ld(8, i, cl) + w.f[sd][1];
+                fv[7] = ld(5, i, cl) + w.f[sd][2];
+            }
+            gv[3] = __fma_rn(w.gs[sd], ld(10, i, cl), w.gc1[sd] * y);
+            hv[3] = __fma_rn(w.hs[sd], ld(15, i, cl), __fma_rn(w.hc1[sd], y, w.hc0[sd]));
+        }
+
+        // undivided central differences of the stored-state fields, with ghosts
+        const double *f = fields64 + (r * 4) * kFields64Cols + (cl - c0 + 1);
+        auto at = [&](int q, int dr, int dc) { return f[(dr * 4 + q) * kFields64Cols + dc]; };
+        double l[4], rr[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            l[q] = at(q, 0, -1);
+            rr[q] = at(q, 0, 1);
+        }
+        if (inner && at_c0)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) l[q] = __fma_rn(k.gha[0][q], at(q, 0, 0), k.ghb[0][q]);
+        if (outer && at_cN)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) rr[q] = __fma_rn(k.gha[1][q], at(q, 0, 0), k.ghb[1][q]);
+        double uy_m = at(1, -1, 0), uy_p = at(1, 1, 0);
+        if (!has_m) uy_m = k.flow[0] == 3 ? at(1, 0, 0) : 2.0 * k.uwy[0] - at(1, 0, 0);
+        if (!has_p) {
+            const int st = end_seg(k, 1, cl);
+            uy_p = k.flow[st] == 3 ? at(1, 0, 0) : 2.0 * k.uwy[st] - at(1, 0, 0);
+        }
+
+        D1 f1[9], g1[5], h1[5];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) f1[q] = D1{fv[q]};
+#pragma unroll
+        for (int q = 0; q < 5; ++q) g1[q] = D1{gv[q]}, h1[q] = D1{hv[q]};
+        NodeVals<D1> o;
+        auto update = [&]() {
+            update_node2<false>(k.pc, k.explicit_src, geo, f1, g1, h1, D1{uy_p - uy_m}, D1{rr[0] - l[0]},
+                                D1{rr[1] - l[1]}, D1{rr[2] - l[2]}, D1{rr[3] - l[3]}, o);
+        };
+        double *p = dst + (long long)i * k.pitch + c;
+        // each branch keeps only the arithmetic its planes need
+        if (split == 1) {
+            update();
+            if (c < nr)
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) p[q * k.plane] = o.v[q].v;
+        } else if (t & 1) {
+            update();
+            if (c < nr)
+#pragma unroll
+                for (int q = 9; q < NQ; ++q) p[q * k.plane] = o.v[q].v;
+        } else {
+            update();
+            if (c < nr)
+#pragma unroll
+                for (int q = 0; q < 9; ++q) p[q * k.plane] = o.v[q].v;
+        }
+    }
 }
 
 // Block of a step grid in traversal order: every other step (rev = 1) the
@@ -1701,6 +1893,39 @@ void pdl_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, dim3 grid, d
     cfg.numAttrs = 1;
 }
 
+int nwindows64(int nr) { return (nr + 31) / 32; }
+constexpr int kMaxRows64 = 32;  // rows of a block of the FP64 step (its fields stay within 48 KB of shared memory)
+
+// A row goes to two warps while a block has at most two rows.
+int split64(int rows) { return rows <= 2 ? 2 : 1; }
+
+// Estimated cycles of an FP64 step on blocks of `rows` rows: the FP64
+// instructions of a block's busiest scheduler (tasks and items go round the
+// four), 64 cycles each, 76 with all four busy, or the sum over the blocks of
+// an SM where there are several.  Within 10 % of the measured times, less 2.6
+// us per launch, on nine sizes from 20 x 84 to 1024 x 1024.
+double cycles64(const HostParams &h, int rows, int sms)
+{
+    const int tasks = rows + (2 * rows + 31) / 32 + 1, items = rows * split64(rows);
+    const double node = split64(rows) == 2 ? 194.0 : 306.0;
+    const double alone = 33.0 * ((tasks + 3) / 4) + node * ((items + 3) / 4);
+    const double all = (33.0 * tasks + node * items) / 4.0;
+    const double per_sm = (double)nwindows64(h.nr) * ((h.nz + rows - 1) / rows) / sms;
+    return std::max((items < 4 ? 64.0 : 76.0) * alone, 76.0 * all * (per_sm <= 3.0 ? std::ceil(per_sm) : per_sm + 0.3));
+}
+
+// SMs of the current device (152 on GB300; also the answer without a device)
+int sm_count()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
+                                                  cudaSuccess || sms <= 0) {
+        cudaGetLastError();  // clear the error of a query without a device
+        return 152;
+    }
+    return sms;
+}
+
 template <typename S, typename C>
 cudaError_t step_t(const HostParams &h, const Launch &l, const void *src, void *dst, unsigned long long step,
                    const void *tmap, int *status, cudaStream_t s)
@@ -1709,12 +1934,25 @@ cudaError_t step_t(const HostParams &h, const Launch &l, const void *src, void *
     const int wpb = l.warps_per_block;
     const int seg = l.seg_rows;
     if constexpr (std::is_same<C, double>::value) {
-        const int nwin = nwindows(h.nr);
-        dim3 grid((nwin + wpb - 1) / wpb, (h.nz + seg - 1) / seg);
+        const int nwin = nwindows64(h.nr), rows = std::min(seg, kMaxRows64);
+        const long long blocks = (long long)nwin * ((h.nz + rows - 1) / rows);
+        if (blocks > INT_MAX) return cudaErrorInvalidValue;
+        // A lattice of at most three blocks per SM asks for the shared memory
+        // with which just that many fit: the blocks of the next step, which
+        // come early (programmatic dependent launch), would otherwise gather
+        // on some SMs and leave others idle (70 x 96: 28 us per step, 11.7 us
+        // with the limit; 14.4 us with plain launches)
+        size_t smem = (size_t)(rows + 2) * 4 * kFields64Cols * sizeof(double);
+        const int sms = sm_count(), per_sm = (int)std::min<long long>((blocks + sms - 1) / sms, 4);
+        if (per_sm <= 3) smem = std::max(smem, (size_t)(kSmemPerSm / (per_sm + 1) - 1024 + 256));
+        static std::atomic<unsigned long long> attr_set{0};
+        cudaError_t e = smem_limit_once(k_step64, kMaxSmem, attr_set);
+        if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute pdl[1];
-        pdl_config(cfg, pdl, grid, dim3(32 * wpb), 0, s);
-        cudaError_t e = cudaLaunchKernelEx(&cfg, k_step64<S, C>, k, (const S *)src, (S *)dst, seg, nwin);
+        pdl_config(cfg, pdl, dim3((unsigned)blocks), dim3(32 * wpb), smem, s);
+        e = cudaLaunchKernelEx(&cfg, k_step64, k, make_walls64(k), (const double *)src, (double *)dst,
+                                           rows, nwin, split64(rows));
         if (e != cudaSuccess) return e;
     } else {
         const int nwin2 = nwindows2(h.nr);
@@ -1795,29 +2033,29 @@ size_t storage_bytes(int storage)
     }
 }
 
-// SMs of the current device (152 on GB300; also the answer without a device)
-static int sm_count()
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                  cudaSuccess || sms <= 0) {
-        cudaGetLastError();  // clear the error of a query without a device
-        return 152;
-    }
-    return sms;
-}
-
 Launch default_launch(const HostParams &p)
 {
     Launch l;
-    l.warps_per_block = p.storage == ST_FP64 ? 4 : 1;
-    l.use_tma = p.storage != ST_FP64 ? 2 : 0;
-    // FP64: 32-row segments; pair kernels: 4-row segments in FP32, 6 in
-    // 16-bit storage (measured on the 1024 x 2048 lattice; short segments
-    // balance the last wave, and their halo rows are re-read from L2); fewer
-    // rows when the lattice would otherwise leave SMs idle
-    const int nwin = p.storage == ST_FP64 ? nwindows(p.nr) : nwindows2(p.nr);
-    int seg = p.storage == ST_FP64 ? 32 : (p.storage == ST_FP32 ? 4 : 6);
+    if (p.storage == ST_FP64) {
+        // the rows with the least estimated time (41 x 41: 1, 10.9 us per
+        // step, 2 rows 11.5, 4 rows 15.4; 256 x 512: 4, 88.5 us, 3 rows 97, 8
+        // rows 97.5); eight warps while blocks run one or a few to an SM
+        const int sms = sm_count();
+        l.seg_rows = 1;
+        for (int rows : {2, 3, 4, 6, 8, 12, 16})
+            if (cycles64(p, rows, sms) < cycles64(p, l.seg_rows, sms)) l.seg_rows = rows;
+        l.warps_per_block = (long long)nwindows64(p.nr) * ((p.nz + l.seg_rows - 1) / l.seg_rows) <= 3 * sms ? 8 : 4;
+        l.use_tma = 0;
+        return l;
+    }
+    l.warps_per_block = 1;
+    l.use_tma = 2;
+    // 4-row segments in FP32, 6 in 16-bit storage (measured on the 1024 x 2048
+    // lattice; short segments balance the last wave, and their halo rows are
+    // re-read from L2); fewer rows when the lattice would otherwise leave SMs
+    // idle
+    const int nwin = nwindows2(p.nr);
+    int seg = p.storage == ST_FP32 ? 4 : 6;
     const long long warps = (long long)nwin * ((p.nz + seg - 1) / seg);
     const long long want = 16LL * sm_count();  // about two waves of resident warps
     if (warps < want) {
@@ -1914,7 +2152,7 @@ int tiles_per_sm(int storage, int slots, int warps)
     const int smem = slots * tile_slot_bytes(storage) + 128;
     if (smem > kMaxSmem) return 0;
     const int regs = storage == ST_FP32 ? kTileRegs<float> : kTileRegs<__half>;
-    return std::min(228 * 1024 / (smem + 1024), 65536 / (regs * 32 * warps));
+    return std::min(kSmemPerSm / (smem + 1024), 65536 / (regs * 32 * warps));
 }
 
 // The smallest tile, in rows, with which all tiles of the lattice are resident

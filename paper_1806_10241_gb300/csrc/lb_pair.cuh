@@ -20,6 +20,8 @@
 
 struct F2 {
     float2 v;
+    static __device__ __forceinline__ F2 of(float2 x) { return F2{x}; }
+    static __device__ __forceinline__ F2 lit(double x) { return F2{make_float2((float)x, (float)x)}; }
 };
 __device__ __forceinline__ F2 mk2(float a, float b)
 {
@@ -66,6 +68,28 @@ __device__ __forceinline__ float rcp1(float x)
     return r;
 }
 __device__ __forceinline__ F2 rcp2(F2 a) { return mk2(rcp1(a.v.x), rcp1(a.v.y)); }
+
+// One FP64 value with the same operations, for the FP64 step.  The reciprocal
+// of a density (a normal number) is the hardware's approximation, good to 1e-6,
+// and one cubic iteration, x (1 + e + e^2) with e = 1 - r x: three FP64
+// instructions and a relative error below 2.3e-16 (measured on [0.5, 1.75]).
+struct D1 {
+    double v;
+    static __device__ __forceinline__ D1 of(double x) { return D1{x}; }
+    static __device__ __forceinline__ D1 lit(double x) { return D1{x}; }
+};
+__device__ __forceinline__ D1 operator+(D1 a, D1 b) { return D1{a.v + b.v}; }
+__device__ __forceinline__ D1 operator-(D1 a, D1 b) { return D1{a.v - b.v}; }
+__device__ __forceinline__ D1 operator*(D1 a, D1 b) { return D1{a.v * b.v}; }
+__device__ __forceinline__ D1 fma2(D1 a, D1 b, D1 c) { return D1{__fma_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ double rcp1(double r)
+{
+    double x;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(r));
+    const double e = __fma_rn(-r, x, 1.0);
+    return __fma_rn(x, __fma_rn(e, e, e), x);
+}
+__device__ __forceinline__ D1 rcp2(D1 a) { return D1{rcp1(a.v)}; }
 __device__ __forceinline__ F2 sel2(bool px, bool py, F2 a, F2 b)  // per component: p ? a : b
 {
     return mk2(px ? a.v.x : b.v.x, py ? a.v.y : b.v.y);
@@ -183,13 +207,14 @@ template <> struct LoadScaled<__half> {
 
 // ---- the node update on pairs ------------------------------------------------
 
-struct NodeOut2 {
-    F2 v[NQ];  // f, g, h
+template <class V> struct NodeVals {
+    V v[NQ];  // f, g, h
 };
+using NodeOut2 = NodeVals<F2>;
 
 // The gradient inputs are the undivided central differences (twice the
 // derivatives); the halves are folded into the geometric factors, which is
-// exact.  iy is 1 / y, or 0 in the planar form (no geometric sources).
+// exact.
 // kScale: the post-collision values come out multiplied by osc, a power of two
 // (the FP16 storage scale): osc is folded into the constants of the
 // post-collision moments and into the fused multiply-add that adds them to
@@ -204,52 +229,61 @@ struct NodeOut2 {
 // by term form had 334.  With the bare reciprocal (rcp1) the 1024 x 2048 step
 // executes 809 instead of 883 warp instructions per 64 columns in FP32, 1043
 // instead of 1100 in FP16: 53.4 -> 52.0 us and 49.2 -> 45.7 us.
-template <bool kScale>
-__device__ __forceinline__ void update_node2(const KP<float> &k, F2 iy, const F2 fv[9], const F2 gv[5],
-                                             const F2 hv[5], F2 dxuy, F2 dyux, F2 dyuy, F2 dyut, F2 dyT,
-                                             NodeOut2 &o)
+// The factors of a column's geometric sources, from iy = 1 / y, or 0 in the
+// planar form (no geometric sources).
+template <class V> struct Geo {
+    V gy, ngy, nuiyh, nuiy, alhiy, niy2nu, m2iy2nu;
+};
+template <class V, class NC> __device__ __forceinline__ Geo<V> geo_of(const NC &c, V iy)
 {
-    const PairConst &c = k.pc;
-    auto K = [](const float2 &v) {
-        F2 r;
-        r.v = v;
-        return r;
-    };
-    const F2 m1 = sp(-1.0f);
-    const F2 OS = K(c.os);
-    auto plus = [&](F2 v, F2 m) { return kScale ? fma2(v, OS, m) : v + m; };
+    Geo<V> g;
+    g.gy = iy;
+    g.ngy = iy * V::lit(-1.0);
+    g.nuiyh = iy * V::of(c.nuh);
+    g.nuiy = iy * V::of(c.nu);
+    g.alhiy = iy * V::of(c.alh);
+    g.niy2nu = g.nuiy * g.ngy;
+    g.m2iy2nu = g.niy2nu + g.niy2nu;
+    return g;
+}
+
+template <bool kScale, class V, class NC>
+__device__ __forceinline__ void update_node2(const NC &c, bool explicit_src, const Geo<V> &geo, const V fv[9],
+                                             const V gv[5], const V hv[5], V dxuy, V dyux, V dyuy, V dyut, V dyT,
+                                             NodeVals<V> &o)
+{
+    const V m1 = V::lit(-1.0);
+    const V OS = V::of(c.os);
+    auto plus = [&](V v, V m) { return kScale ? fma2(v, OS, m) : v + m; };
 
     // output moments, Eq. 18, 35, 47 (deviation form)
-    const F2 a57 = fv[5] - fv[7], a86 = fv[8] - fv[6];
-    const F2 s57 = fv[5] + fv[7], s68 = fv[6] + fv[8];
-    const F2 s13 = fv[1] + fv[3], s24 = fv[2] + fv[4];
-    const F2 s5678 = s57 + s68;
-    const F2 rdo = (fv[0] + s13) + (s24 + s5678);
-    const F2 Dxxy = a57 - a86, Dxyy = a57 + a86;
-    const F2 jxo = (fv[1] - fv[3]) + Dxyy;
-    const F2 jyo = (fv[2] - fv[4]) + Dxxy;
-    const F2 pso = (gv[0] + gv[1]) + (gv[2] + gv[3]) + gv[4];
-    const F2 tdo = (hv[0] + hv[1]) + (hv[2] + hv[3]) + hv[4];
+    const V a57 = fv[5] - fv[7], a86 = fv[8] - fv[6];
+    const V s57 = fv[5] + fv[7], s68 = fv[6] + fv[8];
+    const V s13 = fv[1] + fv[3], s24 = fv[2] + fv[4];
+    const V s5678 = s57 + s68;
+    const V rdo = (fv[0] + s13) + (s24 + s5678);
+    const V Dxxy = a57 - a86, Dxyy = a57 + a86;
+    const V jxo = (fv[1] - fv[3]) + Dxyy;
+    const V jyo = (fv[2] - fv[4]) + Dxxy;
+    const V pso = (gv[0] + gv[1]) + (gv[2] + gv[3]) + gv[4];
+    const V tdo = (hv[0] + hv[1]) + (hv[2] + hv[3]) + hv[4];
 
     // sources at the pre-collision state, two sweeps (see update_node)
-    const F2 gy = iy, ngy = gy * m1;
-    const F2 nuiyh = gy * K(c.nuh), nuiy = gy * K(c.nu);
-    const F2 Gx = (dxuy + dyux) * nuiyh;
-    const F2 Gy = dyuy * nuiy;
-    const F2 Gw = dyut * nuiyh;
-    const F2 Gt = dyT * (gy * K(c.alh));
-    const F2 niy2nu = nuiy * ngy;
-    const F2 m2iy2nu = niy2nu + niy2nu;
-    const F2 Fbx = K(c.bfx);
-    const F2 Fb = K(c.fb), rho0 = K(c.rho0), T0 = K(c.T0), half = sp(0.5f);
-    F2 rd = rdo, jx = jxo, jy = jyo, ps = pso, td = tdo;
-    F2 MA, Fx, Fy, Sps, Sph;
+    const V gy = geo.gy, ngy = geo.ngy, niy2nu = geo.niy2nu, m2iy2nu = geo.m2iy2nu;
+    const V Gx = (dxuy + dyux) * geo.nuiyh;
+    const V Gy = dyuy * geo.nuiy;
+    const V Gw = dyut * geo.nuiyh;
+    const V Gt = dyT * geo.alhiy;
+    const V Fbx = V::of(c.bfx);
+    const V Fb = V::of(c.fb), rho0 = V::of(c.rho0), T0 = V::of(c.T0), half = V::lit(0.5);
+    V rd = rdo, jx = jxo, jy = jyo, ps = pso, td = tdo;
+    V MA, Fx, Fy, Sps, Sph;
     auto sweep = [&]() {
-        const F2 r = rho0 + rd, ir = rcp2(r);
-        const F2 uyyn = (jy * ir) * ngy;  // -u_y / y
+        const V r = rho0 + rd, ir = rcp2(r);
+        const V uyyn = (jy * ir) * ngy;  // -u_y / y
         Fx = fma2(Fb, td, fma2(jx, uyyn, fma2(r, Gx, Fbx)));
         Fy = fma2(jy, m2iy2nu, fma2(r, Gy, ((ps - jy) * (ps + jy)) * (ir * gy)));
-        Sps = fma2(ps, fma2(uyyn, sp(2.0f), niy2nu), r * Gw);
+        Sps = fma2(ps, fma2(uyyn, V::lit(2.0), niy2nu), r * Gw);
         Sph = fma2(uyyn, T0 + td, Gt);
         jx = fma2(Fx, half, jxo);
         jy = fma2(Fy, half, jyo);
@@ -259,67 +293,67 @@ __device__ __forceinline__ void update_node2(const KP<float> &k, F2 iy, const F2
         rd = fma2(MA, half, rdo);
     };
     sweep();
-    if (k.explicit_src) {
+    if (explicit_src) {
         MA = jyo * ngy;
         rd = fma2(MA, half, rdo);
     } else {
         sweep();
     }
-    const F2 r = rho0 + rd, ir = rcp2(r);
-    const F2 ux = jx * ir, uy = jy * ir;
-    const F2 phi = T0 + td;
+    const V r = rho0 + rd, ir = rcp2(r);
+    const V ux = jx * ir, uy = jy * ir;
+    const V phi = T0 + td;
 
     // D2Q9 cascaded collision, Eq. 17
-    const F2 Dxx = s13 + s5678, Dyy = s24 + s5678;
-    const F2 Dxy = s57 - s68, Dxxyy = s5678;
-    const F2 k3 = K(c.k3);
-    const F2 Kxx = k3 + Dxx, Kyy = k3 + Dyy;
-    const F2 ux2 = ux * ux, uy2 = uy * uy;
-    const F2 rxx = jx * ux, ryy = jy * uy;  // rho ux^2, rho uy^2
-    const F2 nux = ux * m1, nuy = uy * m1, n2ux = ux * sp(-2.0f), n2uy = uy * sp(-2.0f);
-    const F2 uxy4 = n2ux * n2uy;
-    const F2 p3 = (fma2(rd, sp(2.0f / 3.0f), rxx + ryy) - (Dxx + Dyy)) * K(c.c3);
-    const F2 c4 = K(c.c4), ch = K(c.ch), nch = K(c.nch);
-    const F2 p4 = ((rxx - ryy) - (Dxx - Dyy)) * c4;
-    const F2 x5 = jx * uy - Dxy;
-    const F2 p5 = x5 * c4, np5 = x5 * K(c.nc4);
+    const V Dxx = s13 + s5678, Dyy = s24 + s5678;
+    const V Dxy = s57 - s68, Dxxyy = s5678;
+    const V k3 = V::of(c.k3);
+    const V Kxx = k3 + Dxx, Kyy = k3 + Dyy;
+    const V ux2 = ux * ux, uy2 = uy * uy;
+    const V rxx = jx * ux, ryy = jy * uy;  // rho ux^2, rho uy^2
+    const V nux = ux * m1, nuy = uy * m1, n2ux = ux * V::lit(-2.0), n2uy = uy * V::lit(-2.0);
+    const V uxy4 = n2ux * n2uy;
+    const V p3 = (fma2(rd, V::lit(2.0 / 3.0), rxx + ryy) - (Dxx + Dyy)) * V::of(c.c3);
+    const V c4 = V::of(c.c4), ch = V::of(c.ch), nch = V::of(c.nch);
+    const V p4 = ((rxx - ryy) - (Dxx - Dyy)) * c4;
+    const V x5 = jx * uy - Dxy;
+    const V p5 = x5 * c4, np5 = x5 * V::of(c.nc4);
     // -(3 p3 + p4) / 2 and -(3 p3 - p4) / 2
-    const F2 hp = fma2(p3, sp(-1.5f), p4 * sp(-0.5f)), hm = fma2(p3, sp(-1.5f), p4 * half);
-    const F2 rxx2 = rxx + rxx, ryy2 = ryy + ryy;
+    const V hp = fma2(p3, V::lit(-1.5), p4 * V::lit(-0.5)), hm = fma2(p3, V::lit(-1.5), p4 * half);
+    const V rxx2 = rxx + rxx, ryy2 = ryy + ryy;
     // p6: (2 r ux^2 uy + Dxxy - 2 ux Dxy - uy Kxx) omhi/4 - uy (3 p3 + p4)/2 - 2 ux p5
-    const F2 Z = fma2(nuy, Kxx, fma2(n2ux, Dxy, fma2(rxx2, uy, Dxxy)));
-    const F2 p6 = fma2(Z, ch, fma2(uy, hp, n2ux * p5));
-    const F2 Y = fma2(nux, Kyy, fma2(n2uy, Dxy, fma2(ryy2, ux, Dxyy)));
-    const F2 p7 = fma2(Y, ch, fma2(ux, hm, n2uy * p5));
+    const V Z = fma2(nuy, Kxx, fma2(n2ux, Dxy, fma2(rxx2, uy, Dxxy)));
+    const V p6 = fma2(Z, ch, fma2(uy, hp, n2ux * p5));
+    const V Y = fma2(nux, Kyy, fma2(n2uy, Dxy, fma2(ryy2, ux, Dxyy)));
+    const V p7 = fma2(Y, ch, fma2(ux, hm, n2uy * p5));
     // p8
-    F2 B = fma2(ux2, Kyy, Dxxyy);
+    V B = fma2(ux2, Kyy, Dxxyy);
     B = fma2(uy2, Kxx, B);
     B = fma2(uxy4, Dxy, B);
     B = fma2(n2ux, Dxyy, B);
     B = fma2(n2uy, Dxxy, B);
-    const F2 Wm = fma2(rd, sp(1.0f / 9.0f), (rxx2 * uy2) * sp(1.5f)) - B;
-    F2 p8 = fma2(p3, sp(-2.0f), Wm * ch);
+    const V Wm = fma2(rd, V::lit(1.0 / 9.0), (rxx2 * uy2) * V::lit(1.5)) - B;
+    V p8 = fma2(p3, V::lit(-2.0), Wm * ch);
     p8 = fma2(uy2, hp, p8);
     p8 = fma2(ux2, hm, p8);
     p8 = fma2(uxy4, np5, p8);
     p8 = fma2(n2uy, p6, p8);
     p8 = fma2(n2ux, p7, p8);
     // source moments, Eq. 26
-    const F2 p0 = MA * K(c.m9), p1 = Fx * K(c.m6), p2 = Fy * K(c.m6);
+    const V p0 = MA * V::of(c.m9), p1 = Fx * V::of(c.m6), p2 = Fy * V::of(c.m6);
     // back-transform, Eq. 27, grouped
     {
-        const F2 A0 = p0 - p3;
-        const F2 E = fma2(p8, sp(-2.0f), A0 + p4), Fm = fma2(p8, sp(-2.0f), A0 - p4);
-        const F2 u = fma2(p7, sp(2.0f), p1), w = fma2(p6, sp(2.0f), p2);
-        o.v[0] = fma2(p3 - p8, sp(-4.0f), plus(fv[0], p0));
+        const V A0 = p0 - p3;
+        const V E = fma2(p8, V::lit(-2.0), A0 + p4), Fm = fma2(p8, V::lit(-2.0), A0 - p4);
+        const V u = fma2(p7, V::lit(2.0), p1), w = fma2(p6, V::lit(2.0), p2);
+        o.v[0] = fma2(p3 - p8, V::lit(-4.0), plus(fv[0], p0));
         o.v[1] = plus(fv[1], E) + u;
         o.v[3] = plus(fv[3], E) - u;
         o.v[2] = plus(fv[2], Fm) + w;
         o.v[4] = plus(fv[4], Fm) - w;
-        const F2 B0 = fma2(p3, sp(2.0f), p0 + p8);
-        const F2 C5 = B0 + p5, C6 = B0 + np5;
-        const F2 p17 = p1 - p7, p26 = p2 - p6;
-        const F2 us = p17 + p26, vd = p17 - p26;
+        const V B0 = fma2(p3, V::lit(2.0), p0 + p8);
+        const V C5 = B0 + p5, C6 = B0 + np5;
+        const V p17 = p1 - p7, p26 = p2 - p6;
+        const V us = p17 + p26, vd = p17 - p26;
         o.v[5] = plus(fv[5], C5) + us;
         o.v[7] = plus(fv[7], C5) - us;
         o.v[6] = plus(fv[6], C6) - vd;
@@ -328,41 +362,41 @@ __device__ __forceinline__ void update_node2(const KP<float> &k, F2 iy, const F2
 
     // D2Q5 cascaded collisions, Eq. 34 / 49 (sign reading of the paper: -),
     // the bracket of q3, q4 with its sign turned
-    const F2 uu = ux2 + uy2, ud = ux2 - uy2;
-    const F2 sg = K(c.sg);
-    const F2 ncu = fma2(sg, uu, sp(-2.0f / 3.0f)), ncd = sg * ud;
+    const V uu = ux2 + uy2, ud = ux2 - uy2;
+    const V sg = V::of(c.sg);
+    const V ncu = fma2(sg, uu, V::lit(-2.0 / 3.0)), ncd = sg * ud;
     {
-        const F2 kxn = gv[3] - gv[1], kyn = gv[4] - gv[2];  // -kappa'_x, -kappa'_y
-        const F2 kxx = gv[1] + gv[3], kyy = gv[2] + gv[4];
-        const F2 cg = K(c.cg);
-        const F2 q1 = fma2(ps, ux, kxn) * cg;
-        const F2 q2 = fma2(ps, uy, kyn) * cg;
-        const F2 X3 = fma2(ps, ncu, fma2(fma2(ux, kxn, uy * kyn), sp(2.0f), kxx + kyy));
-        const F2 X4 = fma2(ps, ncd, fma2(fma2(ux, kxn, nuy * kyn), sp(2.0f), kxx - kyy));
-        const F2 q3 = fma2(X3, nch, fma2(ux, q1, uy * q2));
-        const F2 q4 = fma2(X4, nch, fma2(ux, q1, nuy * q2));
-        const F2 q0 = Sps * K(c.m5);
-        const F2 Q = q0 + q3, Qp = Q + q4, Qm = Q - q4;
-        o.v[G0 + 0] = fma2(q3, sp(-4.0f), plus(gv[0], q0));
+        const V kxn = gv[3] - gv[1], kyn = gv[4] - gv[2];  // -kappa'_x, -kappa'_y
+        const V kxx = gv[1] + gv[3], kyy = gv[2] + gv[4];
+        const V cg = V::of(c.cg);
+        const V q1 = fma2(ps, ux, kxn) * cg;
+        const V q2 = fma2(ps, uy, kyn) * cg;
+        const V X3 = fma2(ps, ncu, fma2(fma2(ux, kxn, uy * kyn), V::lit(2.0), kxx + kyy));
+        const V X4 = fma2(ps, ncd, fma2(fma2(ux, kxn, nuy * kyn), V::lit(2.0), kxx - kyy));
+        const V q3 = fma2(X3, nch, fma2(ux, q1, uy * q2));
+        const V q4 = fma2(X4, nch, fma2(ux, q1, nuy * q2));
+        const V q0 = Sps * V::of(c.m5);
+        const V Q = q0 + q3, Qp = Q + q4, Qm = Q - q4;
+        o.v[G0 + 0] = fma2(q3, V::lit(-4.0), plus(gv[0], q0));
         o.v[G0 + 1] = plus(gv[1], Qp) + q1;
         o.v[G0 + 3] = plus(gv[3], Qp) - q1;
         o.v[G0 + 2] = plus(gv[2], Qm) + q2;
         o.v[G0 + 4] = plus(gv[4], Qm) - q2;
     }
     {
-        const F2 kxn = hv[3] - hv[1], kyn = hv[4] - hv[2];
-        const F2 Hxx = hv[1] + hv[3], Hyy = hv[2] + hv[4];
-        const F2 ct = K(c.ct);
-        const F2 r1 = fma2(phi, ux, kxn) * ct;
-        const F2 r2 = fma2(phi, uy, kyn) * ct;
+        const V kxn = hv[3] - hv[1], kyn = hv[4] - hv[2];
+        const V Hxx = hv[1] + hv[3], Hyy = hv[2] + hv[4];
+        const V ct = V::of(c.ct);
+        const V r1 = fma2(phi, ux, kxn) * ct;
+        const V r2 = fma2(phi, uy, kyn) * ct;
         // 2 c^2 phi - (kxx + kyy) with the rest parts written out: 2/3 td - (Hxx + Hyy)
-        const F2 X3 = fma2(sp(-2.0f / 3.0f), td, fma2(phi, sg * uu, fma2(fma2(ux, kxn, uy * kyn), sp(2.0f), Hxx + Hyy)));
-        const F2 X4 = fma2(phi, ncd, fma2(fma2(ux, kxn, nuy * kyn), sp(2.0f), Hxx - Hyy));
-        const F2 r3 = fma2(X3, nch, fma2(ux, r1, uy * r2));
-        const F2 r4 = fma2(X4, nch, fma2(ux, r1, nuy * r2));
-        const F2 r0 = Sph * K(c.m5);
-        const F2 Q = r0 + r3, Qp = Q + r4, Qm = Q - r4;
-        o.v[H0 + 0] = fma2(r3, sp(-4.0f), plus(hv[0], r0));
+        const V X3 = fma2(V::lit(-2.0 / 3.0), td, fma2(phi, sg * uu, fma2(fma2(ux, kxn, uy * kyn), V::lit(2.0), Hxx + Hyy)));
+        const V X4 = fma2(phi, ncd, fma2(fma2(ux, kxn, nuy * kyn), V::lit(2.0), Hxx - Hyy));
+        const V r3 = fma2(X3, nch, fma2(ux, r1, uy * r2));
+        const V r4 = fma2(X4, nch, fma2(ux, r1, nuy * r2));
+        const V r0 = Sph * V::of(c.m5);
+        const V Q = r0 + r3, Qp = Q + r4, Qm = Q - r4;
+        o.v[H0 + 0] = fma2(r3, V::lit(-4.0), plus(hv[0], r0));
         o.v[H0 + 1] = plus(hv[1], Qp) + r1;
         o.v[H0 + 3] = plus(hv[3], Qp) - r1;
         o.v[H0 + 2] = plus(hv[2], Qm) + r2;
@@ -934,7 +968,7 @@ __device__ __forceinline__ void row_tail(const KP<float> &k, const Own &own, S *
 
     // FP16 storage: the update returns the values already times the scale
     NodeOut2 o;
-    update_node2<Scaled<S>::value>(k, L.iy, fv, gv, hv5, uy_xp - uy_xm, across(r.ux, l.ux), across(r.uy, l.uy),
+    update_node2<Scaled<S>::value>(k.pc, k.explicit_src, geo_of(k.pc, L.iy), fv, gv, hv5, uy_xp - uy_xm, across(r.ux, l.ux), across(r.uy, l.uy),
                                    across(r.ut, l.ut), across(r.T, l.T), o);
     if (L.outA) store_row<S>(k, dst, i, L.A, salt, o);
 }

@@ -11,13 +11,12 @@
 // tiles overlap by their margins and recompute them: no block waits for
 // another one.
 //
-// Why tiles: a row update in the marching kernels spends half of its 800
-// instructions on work a tile does once per row and step -- the fields of the
-// stored state are written by the warp that has the new values in registers,
-// and the radial neighbours' fields are plain shared-memory reads instead of
-// shuffles and recomputed halo columns (about 600 instructions with the
-// recomputed margins) -- and one launch boundary and one pass over memory
-// serve T steps.  Measured per step (one step per launch before, tiles now):
+// Why tiles: one launch boundary, one fetch and one pass over memory serve T
+// steps, and a row update needs less: the fields of the stored state are
+// written by the warp that has the new values in registers, and the radial
+// neighbours' fields are plain shared-memory reads instead of shuffles and
+// recomputed halo columns (735 warp instructions per 64 columns of result,
+// recomputed margins included, against 809 of the marching step).  Measured per step (one step per launch before, tiles now):
 // 100 x 100 FP32 7.1 -> 2.3 us, 40 x 400 FP32 7.4 -> 2.7 us, 256 x 512 FP32
 // 11.6 -> 5.0 us, 301 x 257 BF16 12.8 -> 4.9 us.  What bounds a small tile now
 // is the latency of a row update, about 1.3 us, and 2.5 us per launch.
@@ -149,7 +148,7 @@ __device__ __forceinline__ void tile_row(const KP<float> &k, const Lane2 &L, con
              mk2(c.T.v.y, f_0[194 + cA])};
     if (L.edge_warp) lateral_ghosts(k, L, c, l, r);
     auto across = [](F2 right, F2 left) { return mk2(right.v.x - left.v.x, right.v.y - left.v.y); };
-    update_node2<Scaled<S>::value>(k, L.iy, fv, gv, hv5, uy_xp - uy_xm, across(r.ux, l.ux), across(r.uy, l.uy),
+    update_node2<Scaled<S>::value>(k.pc, k.explicit_src, geo_of(k.pc, L.iy), fv, gv, hv5, uy_xp - uy_xm, across(r.ux, l.ux), across(r.uy, l.uy),
                                    across(r.ut, l.ut), across(r.T, l.T), o);
 }
 
@@ -301,9 +300,8 @@ __global__ void __maxnreg__(kTileRegs<S>)
 // are exactly what is live: W rows on their way, W of this tick, and 2 T of
 // the lower neighbours' states).  1024 x 2048: FP32 52.0 us per step with one
 // step per launch, 40.8 us with strips of two steps; what bounds it is the
-// latency of dependent instructions at 12 warps per SM (46 % issue), not
-// memory (3 TB/s).  FP16 45.7 -> 45.6 us at that size, 25.3 -> 23.4 us at
-// 800 x 1283.
+// latency of dependent instructions at 12 warps per SM (47 % issue), not
+// memory.  FP16 45.7 -> 45.6 us at that size, 26.1 -> 20.7 us at 641 x 1283.
 template <typename S>
 __global__ void __maxnreg__(kTileRegs<S>)
     k_strip(const __grid_constant__ KP<float> k, const __grid_constant__ CUtensorMap map, S *__restrict__ dst,
