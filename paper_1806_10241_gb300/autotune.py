@@ -24,6 +24,7 @@ _lock = threading.Lock()
 
 SOLVER_CANDIDATES = [(4, 1, 3), (4, 2, 3), (6, 1, 3), (8, 1, 3), (12, 2, 3), (16, 4, 3),
                      (6, 1, 2), (8, 2, 2), (8, 2, 1), (16, 4, 1)]
+# (4, 1, 3) with one common segment length is the batch's automatic launch (several steps per launch)
 BATCH_CANDIDATES = [(4, 1, 3), (4, 2, 3), (6, 1, 3), (8, 1, 3), (8, 2, 1), (16, 4, 1)]
 
 

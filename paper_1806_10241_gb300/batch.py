@@ -1,8 +1,9 @@
 """Many lattices advanced together through the C ABI batch calls.
 
 All lattices of a batch share the storage type (FP32 or 16-bit); their
-shapes and parameters may differ.  One kernel launch per step covers every
-tile of every lattice, replayed from a CUDA graph.
+shapes and parameters may differ.  Under the settings a batch starts with one
+kernel launch takes every tile of every lattice through several steps; other
+settings take one launch per step, replayed from a CUDA graph.
 """
 from __future__ import annotations
 

@@ -679,6 +679,19 @@ struct lb_batch {
     std::vector<int> hbprefix;
     bool bdiag_uploaded;
     int *d_flags;  // progress counters of the persistent step (row fetch 5)
+    // the automatic launch: tiles of several steps
+    lbk::TileLaunch tiles;
+    int *d_tprefix;
+    std::vector<int> htprefix;
+
+    // the launch settings a batch starts with select the automatic launch
+    bool automatic() const
+    {
+        if (seg_rows != 4 || wpb != 1 || row_fetch != 3) return false;
+        for (int s : seg_of)
+            if (s) return false;
+        return true;
+    }
 };
 
 // Work queued on the lattices' own streams (initialisation, state uploads,
@@ -698,13 +711,15 @@ static cudaError_t batch_streams_wait(lb_batch *b, bool batch_waits)
 constexpr size_t kDiagSlot = 256;  // per lattice: its NSUM sums and status word, gathered on the device
 
 // Batch buffer: descriptors, item prefix sums, step counter, gathered
-// diagnostics, diagnostics descriptors, diagnostics block prefix sums.
+// diagnostics, diagnostics descriptors, diagnostics block prefix sums,
+// progress counters, tile prefix sums.
 // Work items the persistent batched step (row fetch 5) can track: one
 // progress counter each.
 constexpr int kMaxPersistItems = 16384;
 
 static size_t batch_layout(int32_t n, size_t *desc_off, size_t *prefix_off, size_t *ctl_off, size_t *diag_off,
-                           size_t *bdiag_off = nullptr, size_t *bprefix_off = nullptr, size_t *flags_off = nullptr)
+                           size_t *bdiag_off = nullptr, size_t *bprefix_off = nullptr, size_t *flags_off = nullptr,
+                           size_t *tprefix_off = nullptr)
 {
     const size_t d = align256((size_t)n * lbk::batch_desc_bytes());
     const size_t p = align256((size_t)(n + 1) * sizeof(int));
@@ -719,7 +734,8 @@ static size_t batch_layout(int32_t n, size_t *desc_off, size_t *prefix_off, size
     if (bdiag_off) *bdiag_off = d + p + t + g;
     if (bprefix_off) *bprefix_off = d + p + t + g + bd;
     if (flags_off) *flags_off = d + p + t + g + bd + bp;
-    return d + p + t + g + bd + bp + (size_t)kMaxPersistItems * sizeof(int);
+    if (tprefix_off) *tprefix_off = d + p + t + g + bd + bp + (size_t)kMaxPersistItems * sizeof(int);
+    return d + p + t + g + bd + bp + (size_t)kMaxPersistItems * sizeof(int) + p;
 }
 
 static lb_status batch_upload(lb_batch *b)
@@ -728,20 +744,27 @@ static lb_status batch_upload(lb_batch *b)
     const size_t db = lbk::batch_desc_bytes();
     b->hdesc.assign((size_t)n * db, 0);
     b->hprefix.assign((size_t)n + 1, 0);
+    b->htprefix.assign((size_t)n + 1, 0);
     for (int m = 0; m < n; ++m) {
         lb_ctx *c = b->ctxs[m];
         const int seg = b->seg_of[m] ? b->seg_of[m] : b->seg_rows;
         cudaError_t e = lbk::batch_fill_desc(c->hp, c->dist[0], c->dist[1], b->step0[m], b->parity0[m], seg,
-                                             c->status, b->hdesc.data() + (size_t)m * db);
+                                             b->tiles, c->status, b->hdesc.data() + (size_t)m * db);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch descriptor (tensor map)");
         const long long items = (long long)b->hprefix[m] + lbk::batch_items(c->hp, seg);
         if (items > (1LL << 30)) return fail(nullptr, LB_ERR_ARG, "too many work items in the batch");
         b->hprefix[m + 1] = (int)items;
+        const long long tiles = (long long)b->htprefix[m] + lbk::batch_tile_count(c->hp, b->tiles);
+        if (tiles > (1LL << 30)) return fail(nullptr, LB_ERR_ARG, "too many work items in the batch");
+        b->htprefix[m + 1] = (int)tiles;
     }
     b->total = b->hprefix[n];
     cudaError_t e = cudaMemcpyAsync(b->d_desc, b->hdesc.data(), b->hdesc.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->d_prefix, b->hprefix.data(), b->hprefix.size() * sizeof(int), cudaMemcpyHostToDevice,
+                            b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->d_tprefix, b->htprefix.data(), b->htprefix.size() * sizeof(int), cudaMemcpyHostToDevice,
                             b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch upload");
@@ -765,8 +788,8 @@ lb_status lb_batch_create(lb_ctx *const *ctxs, int32_t n, void *dev_buf, size_t 
 {
     if (!out || !ctxs || n < 1 || !dev_buf) return fail(nullptr, LB_ERR_ARG, "NULL argument or n < 1");
     *out = nullptr;
-    size_t doff, poff, coff, goff, bdoff, bpoff, foff;
-    const size_t need = batch_layout(n, &doff, &poff, &coff, &goff, &bdoff, &bpoff, &foff);
+    size_t doff, poff, coff, goff, bdoff, bpoff, foff, toff;
+    const size_t need = batch_layout(n, &doff, &poff, &coff, &goff, &bdoff, &bpoff, &foff, &toff);
     if (bytes < need) return fail(nullptr, LB_ERR_NOMEM, "batch buffer holds %zu bytes, %zu needed", bytes, need);
     if (((uintptr_t)dev_buf & 255) != 0) return fail(nullptr, LB_ERR_ARG, "dev_buf must be 256-byte aligned");
     const int storage = ctxs[0] ? ctxs[0]->hp.storage : -1;
@@ -795,6 +818,10 @@ lb_status lb_batch_create(lb_ctx *const *ctxs, int32_t n, void *dev_buf, size_t 
     b->d_bdiag = b->buf + bdoff;
     b->d_bprefix = (int *)(b->buf + bpoff);
     b->d_flags = (int *)(b->buf + foff);
+    b->d_tprefix = (int *)(b->buf + toff);
+    std::vector<const HostParams *> hps;
+    for (int m = 0; m < n; ++m) hps.push_back(&ctxs[m]->hp);
+    b->tiles = lbk::tile_plan_batch(hps.data(), n);
     b->bdiag_uploaded = false;
     b->stream = (cudaStream_t)cuda_stream;
     b->seg_rows = 4;
@@ -903,7 +930,26 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
     }
     int32_t left = nsteps;
     unsigned long long t = b->counter;  // batch step of the next launch
-    const bool use_graph = b->graph_steps > 1 && b->stream != nullptr && left >= b->graph_steps;
+    if (b->automatic() && nsteps > 0) {
+        // passes of several steps, as many as make the buffers alternate with the step count (lb_step)
+        int32_t m = (nsteps + b->tiles.T - 1) / b->tiles.T;
+        if ((nsteps - m) & 1) ++m;
+        for (int32_t p = 0; p < m; ++p) {
+            const int32_t T = nsteps / m + (p < nsteps % m ? 1 : 0);
+            const unsigned long long flip = (b->counter + (unsigned long long)p) & 1ULL;
+            cudaError_t e;
+            if (T == 1 && b->tiles.strip && flip == (t & 1ULL))  // large lattices' single step: one warp per work item
+                e = lbk::launch_batch(b->storage, 3, b->d_desc, b->d_prefix, (int)b->ctxs.size(), b->total, b->d_ctl,
+                                      b->wpb, b->blocks, t, 0, b->stream);
+            else
+                e = lbk::launch_batch_tiles(b->storage, b->tiles, T, b->d_desc, b->d_tprefix, (int)b->ctxs.size(),
+                                            b->htprefix.back(), t, (int)flip, b->stream);
+            if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch launch");
+            t += (unsigned long long)T;
+            left -= T;
+        }
+    }
+    const bool use_graph = left > 0 && b->graph_steps > 1 && b->stream != nullptr && left >= b->graph_steps;
     if (use_graph && !b->graph_valid) {
         // launches j = 0 .. K - 1 take steps counter + j; the last node adds K
         cudaGraph_t g;

@@ -116,7 +116,15 @@ int batch_items(const HostParams &h, int seg_rows);
 // maps, the step count and current buffer when the batch was made, and the
 // lattice's device status word (bounded-wait timeouts).
 cudaError_t batch_fill_desc(const HostParams &h, void *buf0, void *buf1, unsigned long long step0, int parity0,
-                            int seg_rows, int *status, void *out);
+                            int seg_rows, const TileLaunch &l, int *status, void *out);
+// The automatic pass of a batch, a lattice's tiles under it, and one pass of T
+// <= l.T steps from batch step t on (total: the tiles of all lattices, prefix
+// their prefix sums; flip: 0 when the state of step t lies in the buffers that
+// were current when the batch was made).
+TileLaunch tile_plan_batch(const HostParams *const *h, int n);
+int batch_tile_count(const HostParams &h, const TileLaunch &l);
+cudaError_t launch_batch_tiles(int storage, const TileLaunch &l, int T, const void *desc, const int *prefix, int n,
+                               int total, unsigned long long t, int flip, cudaStream_t s);
 int batch_grid(int storage, int wpb);
 // Warps of the batched step (row_fetch 1 or 3, wpb warps per block) that can
 // be resident on the device at once.

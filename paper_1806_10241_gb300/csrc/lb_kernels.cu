@@ -1498,6 +1498,8 @@ int nwindows(int nr) { return (nr + OUT_COLS - 1) / OUT_COLS; }
 
 struct alignas(128) BatchDesc {
     unsigned char map[2][128];  // CUtensorMap of buf[0], buf[1] (64-byte aligned in the device array)
+    unsigned char map64[2][128];  // the same with 64-column boxes (tiles)
+    TileShape tiles;            // the lattice's tiles (automatic launch)
     KP<float> k;
     void *buf[2];
     int *status;               // the lattice's device status word
@@ -1834,6 +1836,47 @@ __global__ void __launch_bounds__(256) k_batch_wall(const BatchDesc *__restrict_
     wall_block<float>(bd.k, (const double *)bd.buf[cur ^ 1], out + (size_t)m * slot_doubles);
 }
 
+// T steps of every lattice of a batch on tiles or strips (lb_tile.cuh): the
+// tiles of all lattices numbered by a prefix sum, one block each.  The pass
+// takes the batch from step t on; `flip` says which buffer holds that state.
+// Shared memory: the block's slots, then the lattice's parameters.  The plan is
+// tile_plan's for the tiles of all lattices together.  40 lattices of 64 to 128
+// columns in FP32: 19.0 us per step with the best one-step launch (segment plan
+// of one wave), 14.8 us on strips of two steps; 64 annuli of 32 to 512 rows and
+// columns in FP16: 146 us with 4-row segments, 107 us on strips of four steps.
+// Bound as the single lattice's strips, and by the columns that a window of a
+// narrow lattice leaves empty (a fifth of them in the first batch).
+template <typename S, bool kStrip>
+__global__ void __maxnreg__(kTileRegs<S>)
+    k_batch_tiles(const BatchDesc *__restrict__ d, const int *__restrict__ prefix, int n, int total, int T,
+                  unsigned long long t, int flip, int kp_off, int rev)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    grid_dependency_trigger();
+    const int lane = threadIdx.x & 31;
+    const int item = rev ? total - 1 - (int)blockIdx.x : (int)blockIdx.x;
+    const int lo = batch_instance(prefix, n, item, lane);
+    const BatchDesc *bd = d + lo;
+    {
+        const uint32_t *s = reinterpret_cast<const uint32_t *>(&bd->k);
+        uint32_t *o = reinterpret_cast<uint32_t *>(smem + kp_off);
+        for (int w = threadIdx.x; w < (int)(sizeof(KP<float>) / 4); w += blockDim.x) o[w] = s[w];
+    }
+    if (threadIdx.x < 2)
+        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
+                         (unsigned long long)bd->map64[threadIdx.x])
+                     : "memory");
+    __syncthreads();
+    const KP<float> &k = *reinterpret_cast<const KP<float> *>(smem + kp_off);
+    const TileShape sh = bd->tiles;
+    const int local = item - prefix[lo], cur = (bd->parity0 + flip) & 1;
+    const CUtensorMap *map = reinterpret_cast<const CUtensorMap *>(bd->map64[cur]);
+    S *dst = (S *)bd->buf[cur ^ 1];
+    if constexpr (kStrip)
+        strip_steps<S>(k, map, dst, sh, T, local % sh.nw, local / sh.nw, bd->step0 + t, bd->status, smem);
+    else tile_steps<S>(k, map, dst, sh, T, local % sh.nw, local / sh.nw, bd->step0 + t, bd->status, smem);
+}
+
 // Self-test of the bounded waits: one warp waits on an mbarrier that nothing
 // arrives at, for `polls` polls of the same bounded wait the TMA rings use;
 // the timeout must reach the status word as it does for a row that never
@@ -2115,27 +2158,31 @@ cudaError_t make_tensor_map(const HostParams &p, void *buf, int box_cols, void *
 
 namespace {
 
-// The geometry of a pass of T steps: windows of 64 columns whose starts lie on
-// 16-byte boundaries (TMA), so the margin is T rounded up to 2 columns in
-// FP32, 4 in 16-bit storage.
+// The tiles of a lattice for passes of up to T steps: windows of 64 columns
+// whose starts lie on 16-byte boundaries (TMA), so the column margin is T
+// rounded up to 2 columns in FP32, 4 in 16-bit storage.
 TileShape tile_shape(const HostParams &h, int T, int rows)
 {
     TileShape sh;
-    sh.T = T;
-    sh.cm = h.storage == ST_FP32 ? (T + 1) / 2 * 2 : (T + 3) / 4 * 4;
-    sh.cs = 64 - 2 * sh.cm;
     sh.rows = rows;
+    sh.rm = T;
+    sh.cm = h.storage == ST_FP32 ? (T + 1) / 2 * 2 : (T + 3) / 4 * 4;
     sh.rs = rows - 2 * T;
+    sh.cs = 64 - 2 * sh.cm;
     sh.nw = h.nr <= 64 ? 1 : (h.nr - 64 + sh.cs - 1) / sh.cs + 1;
-    sh.first = 0;
     return sh;
 }
 
-// Tiles along z.
+// Tiles along z, and in all.
 int tiles_along(const HostParams &h, const TileShape &sh)
 {
     if (h.flow[0] == 2) return (h.nz + sh.rs - 1) / sh.rs;
     return h.nz <= sh.rows ? 1 : (h.nz - sh.rows + sh.rs - 1) / sh.rs + 1;
+}
+long long tile_count(const HostParams &h, int T, int rows)
+{
+    const TileShape sh = tile_shape(h, T, rows);
+    return (long long)sh.nw * tiles_along(h, sh);
 }
 
 int tile_slot_bytes(int storage)
@@ -2145,35 +2192,59 @@ int tile_slot_bytes(int storage)
 
 int tile_slots(bool strip, int T, int rows, int warps) { return strip ? 2 * warps + 2 * T : rows + T - 1; }
 
+constexpr int kBatchKpBytes = (int)((sizeof(KP<float>) + 127) / 128 * 128);
+
 // Blocks of a pass that fit on an SM at once (shared memory with 1 KB of it per
 // block for the system, registers).
-int tiles_per_sm(int storage, int slots, int warps)
+int tiles_per_sm(int storage, int slots, int warps, bool batch)
 {
-    const int smem = slots * tile_slot_bytes(storage) + 128;
+    const int smem = slots * tile_slot_bytes(storage) + 128 + (batch ? kBatchKpBytes : 0);
     if (smem > kMaxSmem) return 0;
     const int regs = storage == ST_FP32 ? kTileRegs<float> : kTileRegs<__half>;
     return std::min(kSmemPerSm / (smem + 1024), 65536 / (regs * 32 * warps));
 }
 
-// The smallest tile, in rows, with which all tiles of the lattice are resident
-// at once, two or more to an SM; 0 when there is none.
-int resident_tile_rows(const HostParams &h, int T, int warps, int sms)
+// The lattices that share a pass, and their tiles at a common tile height.
+struct Lattices {
+    const HostParams *const *h;
+    int n, storage;
+    long long tiles(int T, int rows) const
+    {
+        long long sum = 0;
+        for (int m = 0; m < n; ++m) sum += tile_count(*h[m], T, rows);
+        return sum;
+    }
+    int max_rows() const
+    {
+        int r = 0;
+        for (int m = 0; m < n; ++m) r = std::max(r, h[m]->nz);
+        return r;
+    }
+};
+
+// The smallest tile, in rows, with which all tiles are resident at once, two
+// or more to an SM; 0 when there is none.
+int resident_tile_rows(const Lattices &ls, int T, int warps, int sms)
 {
     for (int rows = 2 * T + 1;; ++rows) {
-        const int per_sm = tiles_per_sm(h.storage, tile_slots(false, T, rows, warps), warps);
+        const int per_sm = tiles_per_sm(ls.storage, tile_slots(false, T, rows, warps), warps, ls.n > 1);
         if (per_sm < 2) return 0;
-        const TileShape sh = tile_shape(h, T, rows);
-        if ((long long)sh.nw * tiles_along(h, sh) <= (long long)sms * per_sm) return rows;
+        if (ls.tiles(T, rows) <= (long long)sms * per_sm) return rows;
     }
 }
 
-// Rows of the strips that make up `waves` waves of resident blocks.
-int strip_rows(const HostParams &h, int T, int warps, int waves, int sms)
+// The shortest strips, in rows, that make up at most `waves` waves of resident
+// blocks; whole lattices where even those are more.
+int strip_rows(const Lattices &ls, int T, int warps, int waves, int sms)
 {
-    const int slots = tile_slots(true, T, 0, warps), windows = tile_shape(h, T, 2 * T + 1).nw;
-    const int segs = std::max(1, waves * sms * tiles_per_sm(h.storage, slots, warps) / windows);
-    const int rows = h.flow[0] == 2 ? h.nz : std::max(1, h.nz - 2 * T);
-    return (rows + segs - 1) / segs + 2 * T;
+    const long long most = (long long)waves * sms * tiles_per_sm(ls.storage, tile_slots(true, T, 0, warps), warps, ls.n > 1);
+    int lo = 2 * T + 1, hi = ls.max_rows() + 2 * T;
+    while (lo < hi) {
+        const int mid = lo + (hi - lo) / 2;
+        if (ls.tiles(T, mid) <= most) hi = mid;
+        else lo = mid + 1;
+    }
+    return lo;
 }
 
 template <typename S>
@@ -2182,25 +2253,51 @@ cudaError_t tile_t(const HostParams &h, const TileLaunch &l, const void *tmap, v
 {
     const KP<float> k = make_kp<float>(h);
     static std::atomic<unsigned long long> tile_set{0}, strip_set{0};
-    cudaError_t e = smem_limit_once(k_tile<S>, kMaxSmem, tile_set);
-    if (e == cudaSuccess) e = smem_limit_once(k_strip<S>, kMaxSmem, strip_set);
+    cudaError_t e = smem_limit_once(k_tiles<S, false>, kMaxSmem, tile_set);
+    if (e == cudaSuccess) e = smem_limit_once(k_tiles<S, true>, kMaxSmem, strip_set);
     if (e != cudaSuccess) return e;
-    TileShape sh = tile_shape(h, l.T, l.rows);
+    const TileShape sh = tile_shape(h, l.T, l.rows);
     const long long blocks = (long long)sh.nw * tiles_along(h, sh);
     const size_t smem = tile_smem_bytes<S>(tile_slots(l.strip, l.T, l.rows, l.warps));
     for (int p = 0; p < l.parts; ++p) {
         const int q = rev ? l.parts - 1 - p : p;  // the parts in the order of their blocks
-        sh.first = (int)(blocks * q / l.parts);
-        const int count = (int)(blocks * (q + 1) / l.parts) - sh.first;
+        const int first = (int)(blocks * q / l.parts), count = (int)(blocks * (q + 1) / l.parts) - first;
         if (count < 1) continue;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute pdl[1];
         pdl_config(cfg, pdl, dim3(count), dim3(32 * l.warps), smem, s);
-        e = cudaLaunchKernelEx(&cfg, l.strip ? k_strip<S> : k_tile<S>, k, *(const CUtensorMap *)tmap, (S *)dst,
-                               (const TileShape)sh, step, status, rev);
+        e = cudaLaunchKernelEx(&cfg, l.strip ? k_tiles<S, true> : k_tiles<S, false>, k, *(const CUtensorMap *)tmap,
+                               (S *)dst, sh, l.T, first, step, status, rev);
         if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
+}
+
+TileLaunch plan_tiles(const Lattices &ls, int T)
+{
+    const int sms = sm_count();
+    const bool fp32 = ls.storage == ST_FP32;
+    const int W = fp32 ? 6 : 8;
+    TileLaunch l{T, 0, W, 0, 1};
+    if (T == 0) {  // the best number of steps
+        l.T = 3;
+        l.rows = resident_tile_rows(ls, 3, W, sms);
+        if (fp32 && (l.rows == 0 || l.rows > 9)) {
+            l.T = 2;
+            l.rows = resident_tile_rows(ls, 2, W, sms);
+        }
+        if (l.rows == 0) l.T = fp32 ? 2 : 4;
+    } else {
+        l.rows = resident_tile_rows(ls, T, W, sms);
+    }
+    if (l.rows) return l;
+    l.strip = 1;
+    l.rows = strip_rows(ls, l.T, W, 1, sms);
+    if (l.rows > (fp32 ? 40 : 60)) {
+        l.warps = 4;
+        l.rows = strip_rows(ls, l.T, l.warps, 1, sms);
+    }
+    return l;
 }
 
 }  // namespace
@@ -2224,34 +2321,17 @@ cudaError_t tile_t(const HostParams &h, const TileLaunch &l, const void *tmap, v
 //   launch of two waves.
 TileLaunch tile_plan(const HostParams &h, int T)
 {
-    const int sms = sm_count();
-    const bool fp32 = h.storage == ST_FP32;
-    const int W = fp32 ? 6 : 8;
-    TileLaunch l{T, 0, W, 0, 1};
-    if (T == 0) {  // the best number of steps
-        l.T = 3;
-        l.rows = resident_tile_rows(h, 3, W, sms);
-        if (fp32 && (l.rows == 0 || l.rows > 9)) {
-            l.T = 2;
-            l.rows = resident_tile_rows(h, 2, W, sms);
-        }
-        if (l.rows == 0) l.T = fp32 ? 2 : 4;
-    } else {
-        l.rows = resident_tile_rows(h, T, W, sms);
-    }
-    if (l.rows) return l;
-    l.strip = 1;
-    l.rows = strip_rows(h, l.T, W, 1, sms);
-    if (l.rows > (fp32 ? 40 : 60)) {
-        l.warps = 4;
-        l.rows = strip_rows(h, l.T, l.warps, 1, sms);
-        if (fp32 && l.T == 2 && l.rows > 64) {
-            l.parts = 2;
-            l.rows = strip_rows(h, l.T, l.warps, 2, sms);
-        }
+    const HostParams *one = &h;
+    const Lattices ls{&one, 1, h.storage};
+    TileLaunch l = plan_tiles(ls, T);
+    if (l.strip && h.storage == ST_FP32 && l.T == 2 && l.rows > 64) {
+        l.parts = 2;
+        l.rows = strip_rows(ls, l.T, l.warps, 2, sm_count());
     }
     return l;
 }
+
+TileLaunch tile_plan_batch(const HostParams *const *h, int n) { return plan_tiles(Lattices{h, n, h[0]->storage}, 0); }
 
 cudaError_t launch_tile(const HostParams &p, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
                         int *status, int rev, cudaStream_t s)
@@ -2327,18 +2407,35 @@ namespace lbk {
 size_t batch_desc_bytes() { return sizeof(BatchDesc); }
 size_t batch_ctl_bytes() { return sizeof(BatchCtl); }
 
+// The lattice's tiles under a pass made for the whole batch: strips of equal
+// length, no longer than the pass's.
+static TileShape batch_tiles(const HostParams &h, const TileLaunch &l)
+{
+    TileShape sh = tile_shape(h, l.T, l.rows);
+    const int nt = tiles_along(h, sh), rows = h.flow[0] == 2 ? h.nz : std::max(1, h.nz - 2 * l.T);
+    return nt > 1 || h.flow[0] == 2 ? tile_shape(h, l.T, (rows + nt - 1) / nt + 2 * l.T) : sh;
+}
+
+int batch_tile_count(const HostParams &h, const TileLaunch &l)
+{
+    const TileShape sh = batch_tiles(h, l);
+    return sh.nw * tiles_along(h, sh);
+}
+
 int batch_items(const HostParams &h, int seg_rows)
 {
     return nwindows2(h.nr) * ((h.nz + seg_rows - 1) / seg_rows);
 }
 
 cudaError_t batch_fill_desc(const HostParams &h, void *buf0, void *buf1, unsigned long long step0, int parity0,
-                            int seg_rows, int *status, void *out)
+                            int seg_rows, const TileLaunch &l, int *status, void *out)
 {
     BatchDesc d;
     std::memset(&d, 0, sizeof(d));
     cudaError_t e = make_tensor_map(h, buf0, ring_cols(h.storage), d.map[0]);
     if (e == cudaSuccess) e = make_tensor_map(h, buf1, ring_cols(h.storage), d.map[1]);
+    if (e == cudaSuccess) e = make_tensor_map(h, buf0, 64, d.map64[0]);
+    if (e == cudaSuccess) e = make_tensor_map(h, buf1, 64, d.map64[1]);
     if (e != cudaSuccess) return e;
     d.k = make_kp<float>(h);
     d.buf[0] = buf0;
@@ -2348,6 +2445,7 @@ cudaError_t batch_fill_desc(const HostParams &h, void *buf0, void *buf1, unsigne
     d.parity0 = parity0;
     d.nwin2 = nwindows2(h.nr);
     d.seg_rows = seg_rows;
+    d.tiles = batch_tiles(h, l);
     std::memcpy(out, &d, sizeof(d));
     return cudaSuccess;
 }
@@ -2472,6 +2570,34 @@ cudaError_t launch_batch_persist(int storage, const void *desc, const int *prefi
         case ST_BF16:
             return cudaLaunchCooperativeKernel((const void *)k_batch3p<__nv_bfloat16, 4>, grid, block, args,
                                                batch3_smem_bytes<__nv_bfloat16>(wpb), s);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+template <typename S>
+static cudaError_t batch_tiles_t(const TileLaunch &l, int T, const BatchDesc *d, const int *prefix, int n, int total,
+                                 unsigned long long t, int flip, cudaStream_t s)
+{
+    static std::atomic<unsigned long long> tile_set{0}, strip_set{0};
+    cudaError_t e = smem_limit_once(k_batch_tiles<S, false>, kMaxSmem, tile_set);
+    if (e == cudaSuccess) e = smem_limit_once(k_batch_tiles<S, true>, kMaxSmem, strip_set);
+    if (e != cudaSuccess) return e;
+    const int kp_off = (int)tile_smem_bytes<S>(tile_slots(l.strip, T, l.rows, l.warps));
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute pdl[1];
+    pdl_config(cfg, pdl, dim3(total), dim3(32 * l.warps), kp_off + sizeof(KP<float>), s);
+    return cudaLaunchKernelEx(&cfg, l.strip ? k_batch_tiles<S, true> : k_batch_tiles<S, false>, d, prefix, n, total, T,
+                              t, flip, kp_off, flip);
+}
+
+cudaError_t launch_batch_tiles(int storage, const TileLaunch &l, int T, const void *desc, const int *prefix, int n,
+                               int total, unsigned long long t, int flip, cudaStream_t s)
+{
+    const BatchDesc *d = (const BatchDesc *)desc;
+    switch (storage) {
+        case ST_FP32: return batch_tiles_t<float>(l, T, d, prefix, n, total, t, flip, s);
+        case ST_FP16: return batch_tiles_t<__half>(l, T, d, prefix, n, total, t, flip, s);
+        case ST_BF16: return batch_tiles_t<__nv_bfloat16>(l, T, d, prefix, n, total, t, flip, s);
         default: return cudaErrorInvalidValue;
     }
 }

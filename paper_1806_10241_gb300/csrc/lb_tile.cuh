@@ -29,16 +29,15 @@ template <typename S> struct TileGeom {
     static_assert(row_bytes % 128 == 0, "TMA destinations stay 128-byte aligned");
 };
 
-// A launch of tiles.  Tile j of window w holds the columns [w * cs, w * cs +
-// 64) and, on a lattice with end walls, the rows [j * rs, j * rs + rows); on a
-// periodic one the rows [j * rs - T, (j + 1) * rs + T), modulo nz.
+// The tiles of a lattice.  Tile j of window w holds the columns [w * cs, w * cs
+// + 64) and, on a lattice with end walls, the rows [j * rs, j * rs + rows); on a
+// periodic one the rows [j * rs - rm, (j + 1) * rs + rm), modulo nz.  Made for
+// passes of rm steps, they serve shorter ones as well.
 struct TileShape {
-    int T;          // time steps
     int rows;       // rows loaded by a full tile
-    int rs, cs;     // distance of consecutive tiles in rows and columns
-    int cm;         // column margin, >= T
+    int rm, cm;     // margins in rows and columns
+    int rs, cs;     // distance of consecutive tiles: rows - 2 rm, 64 - 2 cm
     int nw;         // windows across
-    int first;      // the launch's first block in the numbering of all tiles
 };
 
 // Rows of a tile as they lie in shared memory.  The state after step t of
@@ -212,26 +211,22 @@ __device__ __forceinline__ int wrap_row(int row, int nz)
     return row < 0 ? row + nz : row;
 }
 
+// T steps on one tile by a block.  smem: (sh.rows + T - 1) slots and 128 bytes.
 template <typename S>
-__global__ void __maxnreg__(kTileRegs<S>)
-    k_tile(const __grid_constant__ KP<float> k, const __grid_constant__ CUtensorMap map, S *__restrict__ dst,
-           const TileShape sh, unsigned long long step, int *status, int rev)
+__device__ __forceinline__ void tile_steps(const KP<float> &k, const CUtensorMap *map, S *__restrict__ dst,
+                                           const TileShape &sh, int T, int win, int tile, unsigned long long step,
+                                           int *status, unsigned char *smem)
 {
-    extern __shared__ __align__(128) unsigned char smem[];
     constexpr int SB = TileGeom<S>::slot_bytes / (int)sizeof(S);
     const int warp = __shfl_sync(FULL, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31, W = blockDim.x >> 5;
-    const int b = sh.first + (rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x);
-    const int win = b % sh.nw, tile = b / sh.nw;
-    const int T = sh.T, nz = k.nz;
-    const int c0 = win * sh.cs;
+    const int nz = k.nz, c0 = win * sh.cs;
     // rows of this tile: local row 0 is lattice row r0
-    const int r0 = k.xper ? tile * sh.rs - T : tile * sh.rs;
-    const int n = k.xper ? min(sh.rs, nz - tile * sh.rs) + 2 * T : min(sh.rows, nz - r0);
+    const int r0 = k.xper ? tile * sh.rs - sh.rm : tile * sh.rs;
+    const int n = k.xper ? min(sh.rs, nz - tile * sh.rs) + 2 * sh.rm : min(sh.rows, nz - r0);
     const bool bottom = !k.xper && r0 == 0, top = !k.xper && r0 + n == nz;
 
     S *slots = reinterpret_cast<S *>(smem);
     const uint32_t bar = smem_u32(smem + (size_t)(sh.rows + T - 1) * TileGeom<S>::slot_bytes);
-    grid_dependency_trigger();
     const int groups = (n + W - 1) / W;
     if (threadIdx.x == 0) {
         for (int g = 0; g < groups && g < 8; ++g)
@@ -250,7 +245,7 @@ __global__ void __maxnreg__(kTileRegs<S>)
         __syncwarp();
         const uint32_t base = smem_u32(smem) + (uint32_t)(T - 1) * TileGeom<S>::slot_bytes;
         for (int r = lane; r < n; r += 32)
-            tile_fetch<S>(&map, base + (uint32_t)r * TileGeom<S>::slot_bytes, c0, k.xper ? wrap_row(r0 + r, nz) : r0 + r,
+            tile_fetch<S>(map, base + (uint32_t)r * TileGeom<S>::slot_bytes, c0, k.xper ? wrap_row(r0 + r, nz) : r0 + r,
                           bar + 8u * min(r / W, 7));
     }
 
@@ -268,9 +263,10 @@ __global__ void __maxnreg__(kTileRegs<S>)
 
     const int vlo = win == 0 ? 0 : c0 + sh.cm, vhi = win == sh.nw - 1 ? k.nr : c0 + TileGeom<S>::cols - sh.cm;
     const bool out_cols = L.A >= vlo && L.A < vhi;
+    const int out_lo = bottom ? 0 : sh.rm, out_hi = top ? n : n - sh.rm;  // T < rm: rows of the margin are not stored
     for (int t = 0; t < T; ++t) {
-        const int lo = bottom ? 0 : t + 1, hi = top ? n : n - (t + 1);
         const bool last = t == T - 1;
+        const int lo = bottom ? 0 : t + 1, hi = top ? n : n - (t + 1);
         const uint32_t salt = PairIO<S>::rounds ? salt_of(step + (unsigned long long)t) : 0u;
         for (int g = lo; g < hi; g += W) {
             const int r = g + warp;
@@ -280,7 +276,7 @@ __global__ void __maxnreg__(kTileRegs<S>)
             S *b_0 = slots + (r + T - 1 - t) * SB;
             if (active) tile_row<S>(k, L, b_0 - SB, b_0, b_0 + SB, !bottom || r > 0, !top || r < n - 1, o);
             if (last) {
-                if (active && out_cols) store_row<S>(k, dst, row, L.A, salt, o);
+                if (active && out_cols && r >= out_lo && r < out_hi) store_row<S>(k, dst, row, L.A, salt, o);
                 continue;
             }
             __syncthreads();  // the group's reads are done: its slots may be written
@@ -303,24 +299,19 @@ __global__ void __maxnreg__(kTileRegs<S>)
 // latency of dependent instructions at 12 warps per SM (47 % issue), not
 // memory.  FP16 45.7 -> 45.6 us at that size, 26.1 -> 20.7 us at 641 x 1283.
 template <typename S>
-__global__ void __maxnreg__(kTileRegs<S>)
-    k_strip(const __grid_constant__ KP<float> k, const __grid_constant__ CUtensorMap map, S *__restrict__ dst,
-            const TileShape sh, unsigned long long step, int *status, int rev)
+__device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMap *map, S *__restrict__ dst,
+                                            const TileShape &sh, int T, int win, int tile, unsigned long long step,
+                                            int *status, unsigned char *smem)
 {
-    extern __shared__ __align__(128) unsigned char smem[];
     constexpr int SB = TileGeom<S>::slot_bytes / (int)sizeof(S);
     const int warp = __shfl_sync(FULL, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31, W = blockDim.x >> 5;
-    const int b = sh.first + (rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x);
-    const int win = b % sh.nw, tile = b / sh.nw;
-    const int T = sh.T, nz = k.nz, R = 2 * W + 2 * T;
-    const int c0 = win * sh.cs;
-    const int r0 = k.xper ? tile * sh.rs - T : tile * sh.rs;
-    const int n = k.xper ? min(sh.rs, nz - tile * sh.rs) + 2 * T : min(sh.rows, nz - r0);
+    const int nz = k.nz, R = 2 * W + 2 * T, c0 = win * sh.cs;
+    const int r0 = k.xper ? tile * sh.rs - sh.rm : tile * sh.rs;
+    const int n = k.xper ? min(sh.rs, nz - tile * sh.rs) + 2 * sh.rm : min(sh.rows, nz - r0);
     const bool bottom = !k.xper && r0 == 0, top = !k.xper && r0 + n == nz;
 
     S *slots = reinterpret_cast<S *>(smem);
     const uint32_t ring = smem_u32(smem), bar = ring + (uint32_t)(R * TileGeom<S>::slot_bytes);
-    grid_dependency_trigger();
     if (threadIdx.x == 0) {
         for (int g = 0; g < 2; ++g)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8u * g) : "memory");
@@ -337,7 +328,7 @@ __global__ void __maxnreg__(kTileRegs<S>)
         if (lane < cnt) {
             int slot = slot0 + lane;
             slot -= slot >= R ? R : 0;
-            tile_fetch<S>(&map, ring + (uint32_t)(slot * TileGeom<S>::slot_bytes), c0,
+            tile_fetch<S>(map, ring + (uint32_t)(slot * TileGeom<S>::slot_bytes), c0,
                           k.xper ? wrap_row(r0 + first + lane, nz) : r0 + first + lane, bar + 8u * (m & 1));
         }
     };
@@ -348,6 +339,7 @@ __global__ void __maxnreg__(kTileRegs<S>)
 
     const int vlo = win == 0 ? 0 : c0 + sh.cm, vhi = win == sh.nw - 1 ? k.nr : c0 + TileGeom<S>::cols - sh.cm;
     const bool out_cols = L.A >= vlo && L.A < vhi;
+    const int out_lo = bottom ? 0 : sh.rm, out_hi = top ? n : n - sh.rm;  // T < rm: rows of the margin are not stored
     const int cA = 2 * lane;
     const int ticks = ((top ? n + T : n) + W - 1) / W;
     int s0 = 0;  // slot of row m W, state 0
@@ -372,8 +364,9 @@ __global__ void __maxnreg__(kTileRegs<S>)
         }
         for (int t = 0; t < T; ++t) {
             const int r = m * W - 1 - t + warp;
+            const bool last = t == T - 1;
             const int lo = bottom ? 0 : t + 1, hi = top ? n : n - (t + 1);
-            const bool active = r >= lo && r < hi, last = t == T - 1;
+            const bool active = r >= lo && r < hi;
             const int row = k.xper ? wrap_row(r0 + r, nz) : r0 + r;
             const uint32_t salt = PairIO<S>::rounds ? salt_of(step + (unsigned long long)t) : 0u;
             int s = s0 + warp - 1 - 2 * t;  // slot of row r, state t
@@ -384,7 +377,7 @@ __global__ void __maxnreg__(kTileRegs<S>)
             NodeOut2 o;
             if (active) tile_row<S>(k, L, b_m, b_0, b_p, !bottom || r > 0, !top || r < n - 1, o);
             if (last) {
-                if (active && out_cols) store_row<S>(k, dst, row, L.A, salt, o);
+                if (active && out_cols && r >= out_lo && r < out_hi) store_row<S>(k, dst, row, L.A, salt, o);
             } else {
                 __syncthreads();  // the reads of step t are done: its slots may be written
                 if (active) tile_store<S>(k, b_m, cA, row, L.A, salt, o);
@@ -394,4 +387,18 @@ __global__ void __maxnreg__(kTileRegs<S>)
         s0 += W;
         s0 -= s0 >= R ? R : 0;
     }
+}
+
+// One lattice: block b of the launch takes tile `first + b` (rev: from the last
+// one back), windows running fastest.
+template <typename S, bool kStrip>
+__global__ void __maxnreg__(kTileRegs<S>)
+    k_tiles(const __grid_constant__ KP<float> k, const __grid_constant__ CUtensorMap map, S *__restrict__ dst,
+            const TileShape sh, int T, int first, unsigned long long step, int *status, int rev)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    grid_dependency_trigger();
+    const int b = first + (rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x);
+    if constexpr (kStrip) strip_steps<S>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem);
+    else tile_steps<S>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem);
 }

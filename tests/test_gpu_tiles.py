@@ -54,3 +54,30 @@ def test_tiles_equal_one_launch_per_step(name, nr, nz, storage):
                                         ("periodic_annulus", 66, 9001), ("free_ends_annulus", 1283, 517)])
 def test_strips_equal_one_launch_per_step(name, nr, nz, storage):
     _agree(BUILDERS[name](nr, nz), storage, (1, 5, 8))
+
+
+# a batch on resident tiles, and one too large for them, uneven lattices with a periodic and a split-top one among them
+@pytest.mark.parametrize("storage", ["fp32", "fp16", "bf16"])
+@pytest.mark.parametrize("shapes", [[("cylinder_axis", 33, 17), ("periodic_annulus", 66, 12), ("czochralski", 125, 31),
+                                     ("planar_box", 2, 2)],
+                                    [("cylinder_axis", 513, 301), ("periodic_annulus", 70, 1500), ("czochralski", 640, 333),
+                                     ("annulus_walls", 65, 4000), ("free_ends_annulus", 20, 9), ("sliding_annulus", 700, 411)]])
+def test_batched_tiles_equal_one_launch_per_step(shapes, storage):
+    from paper_1806_10241_gb300.batch import Batch
+    from paper_1806_10241_gb300.solver import Solver
+    stream = torch.cuda.Stream()
+    params = [BUILDERS[name](nr, nz) for name, nr, nz in shapes]
+    plain, tiled = ([Solver(p, storage=storage, stream=stream) for p in params] for _ in range(2))
+    for seed, (a, b, p) in enumerate(zip(plain, tiled, params)):
+        a.set_launch(4, 1, 1)
+        state = random_state(p, seed)
+        a.set_dist(state)
+        b.set_dist(state)
+    batch = Batch(tiled, stream=stream, graph_steps=4)
+    for n in (1, 2, 5, 7, 8):
+        batch.step(n)
+        for (name, nr, nz), a, b in zip(shapes, plain, tiled):
+            a.step(n)
+            assert b.step_count == a.step_count
+            assert np.array_equal(a.get_dist(), b.get_dist()), (name, nr, nz, n)
+    batch.close()
