@@ -21,7 +21,10 @@
  * Memory ownership: the caller allocates one device buffer of
  * lb_required_bytes() bytes (256-byte aligned) and one CUDA stream and hands
  * both to lb_create(); the library never allocates device memory and never
- * frees the caller's buffer.  All kernels and copies run on that stream.
+ * frees the caller's buffer.  All kernels and copies run on that stream,
+ * but for large lb_init_fields and lb_get_fields calls: these put their copies
+ * on a stream of the context's own, ordered after the work queued before and
+ * finished before the call returns.
  *
  * Errors: every call returns an lb_status and never aborts, traps or exits;
  * lb_last_error() gives a one-line description of the last failure of a
@@ -264,9 +267,9 @@ LB_EXPORT lb_status lb_get_launch(const lb_ctx *ctx, int32_t *seg_rows, int32_t 
  * bytes of an lb_get_state blob after its 16-byte header, 256-byte aligned);
  * desc and params describe it and pass the checks of lb_create and
  * lb_set_params; step is copied to out->step.  The reductions use the
- * default launch of the lattice: the result is bitwise that of
- * lb_diagnostics on the same state under the default launch, and equal to
- * reduction round-off under another launch (lb_set_launch, autotuning).
+ * grid of lb_diagnostics, which depends on the lattice alone: the result is
+ * bitwise that of lb_diagnostics on the same state (to reduction round-off
+ * for lattices of more than 2048 blocks of 128 columns and 32 rows).
  *
  * Scratch: a 1 MiB array (2^17 doubles) in the library's static device
  * memory, which every GPU that loads the library holds until the process
@@ -330,7 +333,7 @@ LB_EXPORT lb_status lb_batch_set_segments(lb_batch *b, const int32_t *seg_rows);
 LB_EXPORT lb_status lb_batch_get_occupancy(const lb_batch *b, int32_t *resident_warps, int32_t *items);
 LB_EXPORT lb_status lb_batch_step(lb_batch *b, int32_t nsteps);
 /* lb_diagnostics of every lattice of the batch (out[n], in the order of
- * lb_batch_create), bitwise equal to lb_diagnostics of each lattice: three
+ * lb_batch_create), bitwise equal to lb_diagnostics of each lattice: two
  * launches on the batch stream for all lattices (each lattice's reduction
  * grid and order as lb_diagnostics uses them), one copy back; synchronises
  * the batch stream. */

@@ -6,9 +6,11 @@
 // entries each), computed in FP64 and rounded once to FP32.
 // A and B alternate as source and destination of the time steps; the one
 // that is not current doubles as staging space for host exchanges and for
-// the temperature field of the diagnostics.
+// the wall temperatures of the diagnostics.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -40,6 +42,8 @@ struct lb_ctx {
     alignas(64) unsigned char tmap[2][128];  // TMA tensor maps of dist[0], dist[1]
     alignas(64) unsigned char tmap64[2][128];  // the same with 64-column boxes, for the tiles
     bool tmap_ready;
+    cudaStream_t copy_stream;         // copies of an exchange beside its kernels (made at the first large one)
+    cudaEvent_t ev_copy[4], ev_kernel[4];
     unsigned passes;  // launches of several steps so far (their block order alternates)
     int *status;  // device status word (bounded-wait timeouts of the step kernel)
     char err[256];
@@ -256,21 +260,6 @@ lb_status need_params(lb_ctx *ctx)
     return LB_OK;
 }
 
-Launch diag_launch(const lb_ctx *ctx)
-{
-    Launch l = ctx->launch;
-    if (l.seg_rows < 32) l.seg_rows = 32;  // the diagnostics march: longer segments, fewer partial sums
-    const long long nwin = (ctx->hp.nr + 29) / 30;
-    const long long bx = (nwin + 3) / 4;
-    long long segs = (ctx->hp.nz + l.seg_rows - 1) / l.seg_rows;
-    if (bx * segs > lbk::MAX_DIAG_BLOCKS) {
-        segs = lbk::MAX_DIAG_BLOCKS / bx;
-        if (segs < 1) segs = 1;
-        l.seg_rows = (int)((ctx->hp.nz + segs - 1) / segs);
-    }
-    return l;
-}
-
 }  // namespace
 
 extern "C" {
@@ -318,6 +307,8 @@ lb_status lb_create(const lb_grid_desc *desc, void *dev_buf, size_t bytes, void 
     c->launch = lbk::default_launch(h);
     c->launch_auto = true;
     c->passes = 0;
+    c->copy_stream = nullptr;
+    for (int q = 0; q < 4; ++q) c->ev_copy[q] = c->ev_kernel[q] = nullptr;
     c->err[0] = 0;
     *out = c;
     return LB_OK;
@@ -350,31 +341,115 @@ lb_status lb_set_params(lb_ctx *ctx, const lb_params *p)
     return LB_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+constexpr size_t kOverlapBytes = (size_t)4 << 20;  // exchanges below this are copied in one piece
+
+cudaError_t copy_stream(lb_ctx *ctx)
+{
+    if (ctx->copy_stream) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    for (int q = 0; q < 4 && e == cudaSuccess; ++q) {
+        if (!ctx->ev_copy[q]) e = cudaEventCreateWithFlags(&ctx->ev_copy[q], cudaEventDisableTiming);
+        if (e == cudaSuccess && !ctx->ev_kernel[q]) e = cudaEventCreateWithFlags(&ctx->ev_kernel[q], cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking);
+    return e;
+}
+
+// n values of each of the five planes, N values apart on the host
+cudaError_t copy_planes(double *stage, double *host, size_t n, size_t N, bool to_device, cudaStream_t s)
+{
+    const size_t w = n * sizeof(double), p = N * sizeof(double);
+    if (p <= (size_t)INT_MAX)
+        return to_device ? cudaMemcpy2DAsync(stage, w, host, p, w, 5, cudaMemcpyHostToDevice, s)
+                         : cudaMemcpy2DAsync(host, p, stage, w, w, 5, cudaMemcpyDeviceToHost, s);
+    for (int q = 0; q < 5; ++q) {
+        const cudaError_t e = to_device
+            ? cudaMemcpyAsync(stage + q * n, host + q * N, w, cudaMemcpyHostToDevice, s)
+            : cudaMemcpyAsync(host + q * N, stage + q * n, w, cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// Fields between the host ([5][nz][nr] doubles) and the device, in chunks of
+// rows through the staging area.  A large exchange overlaps the copies of a
+// chunk with the kernels of its neighbours: the copies go to a second stream,
+// ordered against the context's stream by events, in up to four parts of the
+// staging area (512 x 1024 FP32: fields in and out 480 us before, 300 us
+// now; the copies alone take 233 us).  kernel(stage, r0, r1) queues the work of
+// a chunk on the context's stream.
+template <typename Kernel>
+lb_status exchange(lb_ctx *ctx, double *host, bool to_device, const char *what, Kernel kernel)
+{
+    double *stage;
+    int rows;
+    const lb_status st = staging(ctx, 5, &stage, &rows);
+    if (st != LB_OK) return st;
+    const int nr = ctx->hp.nr, nz = ctx->hp.nz;
+    const size_t N = (size_t)nr * nz, total = 5 * N * sizeof(double);
+    int chunk = rows, parts = 1;
+    const bool large = total >= kOverlapBytes && rows >= 2, overlap = large && copy_stream(ctx) == cudaSuccess;
+    if (large && !overlap) cudaGetLastError();  // without a copy stream the chunks follow each other
+    if (overlap) {
+        // chunks of about 2.5 MB, at most 32
+        const int count = (int)std::min<size_t>(32, std::max<size_t>(2, total / (5 << 19)));
+        chunk = std::min((nz + count - 1) / count, rows / 2);
+        parts = std::min(4, rows / chunk);
+    }
+    const cudaStream_t s = ctx->stream, c = parts > 1 ? ctx->copy_stream : s;
+    const size_t part = (size_t)chunk * 5 * nr;
+    cudaError_t e = cudaSuccess;
+    if (parts > 1) {  // the staging area is free once the work queued so far is done
+        e = cudaEventRecord(ctx->ev_kernel[0], s);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(c, ctx->ev_kernel[0], 0);
+    }
+    auto then = [&](cudaEvent_t ev, cudaStream_t from, cudaStream_t to) {  // `to` continues after `from`
+        if (parts == 1 || e != cudaSuccess) return;
+        e = cudaEventRecord(ev, from);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(to, ev, 0);
+    };
+    for (int r0 = 0, i = 0; r0 < nz && e == cudaSuccess; r0 += chunk, ++i) {
+        const int r1 = std::min(nz, r0 + chunk), q = i % parts;
+        const size_t n = (size_t)(r1 - r0) * nr;
+        double *at = stage + q * part;
+        if (to_device) {
+            if (i >= parts && parts > 1) e = cudaStreamWaitEvent(c, ctx->ev_kernel[q], 0);
+            if (e == cudaSuccess) e = copy_planes(at, host + (size_t)r0 * nr, n, N, true, c);
+            then(ctx->ev_copy[q], c, s);
+            if (e == cudaSuccess) e = kernel(at, r0, r1);
+            if (e == cudaSuccess && parts > 1) e = cudaEventRecord(ctx->ev_kernel[q], s);
+        } else {
+            if (i >= parts && parts > 1) e = cudaStreamWaitEvent(s, ctx->ev_copy[q], 0);
+            if (e == cudaSuccess) e = kernel(at, r0, r1);
+            then(ctx->ev_kernel[q], s, c);
+            if (e == cudaSuccess) e = copy_planes(at, host + (size_t)r0 * nr, n, N, false, c);
+            if (e == cudaSuccess && parts > 1) e = cudaEventRecord(ctx->ev_copy[q], c);
+        }
+    }
+    // both streams are done with the host array and the staging area
+    const cudaError_t e1 = cudaStreamSynchronize(s), e2 = parts > 1 ? cudaStreamSynchronize(c) : cudaSuccess;
+    if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
+    return e == cudaSuccess ? LB_OK : cuda_fail(ctx, e, what);
+}
+
+}  // namespace
+
+extern "C" {
+
 lb_status lb_init_fields(lb_ctx *ctx, const double *host_fields)
 {
     lb_status st = need_params(ctx);
     if (st != LB_OK) return st;
     if (!host_fields) return fail(ctx, LB_ERR_ARG, "host_fields is NULL");
-    double *stage;
-    int rows;
-    if ((st = staging(ctx, 5, &stage, &rows)) != LB_OK) return st;
-    const int nr = ctx->hp.nr, nz = ctx->hp.nz;
-    const size_t N = (size_t)nr * nz;
-    for (int r0 = 0; r0 < nz; r0 += rows) {
-        const int r1 = r0 + rows < nz ? r0 + rows : nz;
-        const size_t n = (size_t)(r1 - r0) * nr;
-        for (int q = 0; q < 5; ++q) {
-            cudaError_t e = cudaMemcpyAsync(stage + q * n, host_fields + q * N + (size_t)r0 * nr, n * sizeof(double),
-                                            cudaMemcpyHostToDevice, ctx->stream);
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "init upload");
-        }
-        cudaError_t e = lbk::launch_init_fields(ctx->hp, stage, ctx->dist[ctx->cur], r0, r1, ctx->stream);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "init kernel");
-    }
-    cudaError_t e = cudaStreamSynchronize(ctx->stream);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "init sync");
-    ctx->step = 0;
-    return LB_OK;
+    st = exchange(ctx, const_cast<double *>(host_fields), true, "init", [&](const double *stage, int r0, int r1) {
+        return lbk::launch_init_fields(ctx->hp, stage, ctx->dist[ctx->cur], r0, r1, ctx->stream);
+    });
+    if (st == LB_OK) ctx->step = 0;
+    return st;
 }
 
 lb_status lb_step(lb_ctx *ctx, int32_t nsteps)
@@ -390,7 +465,8 @@ lb_status lb_step(lb_ctx *ctx, int32_t nsteps)
         }
         ctx->tmap_ready = true;
     }
-    const int32_t fused = ctx->hp.storage != LB_FP64 && ctx->launch_auto ? nsteps : 0;
+    const int32_t fused =
+        ctx->hp.storage != LB_FP64 && ctx->launch_auto ? nsteps : 0;
     if (fused > 0) {
         // Passes of up to T steps.  Their number is made even or odd as the
         // number of steps is, so that the current buffer alternates with the
@@ -428,28 +504,12 @@ lb_status lb_step(lb_ctx *ctx, int32_t nsteps)
 
 lb_status lb_get_fields(lb_ctx *ctx, double *host_fields)
 {
-    lb_status st = need_params(ctx);
+    const lb_status st = need_params(ctx);
     if (st != LB_OK) return st;
     if (!host_fields) return fail(ctx, LB_ERR_ARG, "host_fields is NULL");
-    double *stage;
-    int rows;
-    if ((st = staging(ctx, 5, &stage, &rows)) != LB_OK) return st;
-    const int nr = ctx->hp.nr, nz = ctx->hp.nz;
-    const size_t N = (size_t)nr * nz;
-    for (int r0 = 0; r0 < nz; r0 += rows) {
-        const int r1 = r0 + rows < nz ? r0 + rows : nz;
-        const size_t n = (size_t)(r1 - r0) * nr;
-        cudaError_t e = lbk::launch_fields(ctx->hp, ctx->launch, ctx->dist[ctx->cur], stage, r0, r1, ctx->stream);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "fields kernel");
-        for (int q = 0; q < 5; ++q) {
-            e = cudaMemcpyAsync(host_fields + q * N + (size_t)r0 * nr, stage + q * n, n * sizeof(double),
-                                cudaMemcpyDeviceToHost, ctx->stream);
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "fields download");
-        }
-        e = cudaStreamSynchronize(ctx->stream);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "fields sync");
-    }
-    return LB_OK;
+    return exchange(ctx, host_fields, false, "fields", [&](double *stage, int r0, int r1) {
+        return lbk::launch_fields(ctx->hp, ctx->dist[ctx->cur], stage, r0, r1, ctx->stream);
+    });
 }
 
 lb_status lb_selftest_timeout(lb_ctx *ctx, int32_t polls)
@@ -477,7 +537,7 @@ lb_status lb_stream_function(lb_ctx *ctx, double *host_psi, double *psi_max)
         const int r1 = r0 + rows < nz ? r0 + rows : nz;
         const size_t n = (size_t)(r1 - r0) * nr;
         // fields into planes 0..4 of the stage; Psi over plane 0, row maxima over plane 2
-        cudaError_t e = lbk::launch_fields(ctx->hp, ctx->launch, ctx->dist[ctx->cur], stage, r0, r1, ctx->stream);
+        cudaError_t e = lbk::launch_fields(ctx->hp, ctx->dist[ctx->cur], stage, r0, r1, ctx->stream);
         if (e == cudaSuccess)
             e = lbk::launch_psi(stage + n, stage, stage + 2 * n, r1 - r0, nr, ctx->hp.r0, ctx->stream);
         if (e == cudaSuccess && host_psi)
@@ -507,15 +567,17 @@ lb_status lb_diagnostics(lb_ctx *ctx, lb_diag *out)
     if (st != LB_OK) return st;
     if (!out) return fail(ctx, LB_ERR_ARG, "out is NULL");
     const HostParams &h = ctx->hp;
-    double res[lbk::NSUM];
-    int kstatus = 0;
-    cudaError_t e = lbk::launch_diag(h, diag_launch(ctx), ctx->dist[ctx->cur], ctx->partial,
-                                     (double *)ctx->dist[1 - ctx->cur], ctx->result, ctx->stream);
+    // the sums and, 128 bytes on, the status word
+    double res[17];
+    static_assert(lbk::NSUM <= 16, "the status word follows the sums");
+    cudaError_t e = lbk::launch_diag(h, ctx->dist[ctx->cur], ctx->partial, (double *)ctx->dist[1 - ctx->cur],
+                                     ctx->result, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "diagnostics kernel");
-    e = cudaMemcpyAsync(&kstatus, ctx->status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(res, ctx->result, sizeof(res), cudaMemcpyDeviceToHost, ctx->stream);
+    e = cudaMemcpyAsync(res, ctx->result, 128 + sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "diagnostics download");
+    int kstatus;
+    std::memcpy(&kstatus, &res[16], sizeof(int));
     fill_diag(ctx, res, kstatus, out);
     return LB_OK;
 }
@@ -642,6 +704,13 @@ lb_status lb_get_launch(const lb_ctx *ctx, int32_t *seg_rows, int32_t *warps_per
 
 lb_status lb_destroy(lb_ctx *ctx)
 {
+    if (ctx) {
+        for (int q = 0; q < 4; ++q) {
+            if (ctx->ev_copy[q]) cudaEventDestroy(ctx->ev_copy[q]);
+            if (ctx->ev_kernel[q]) cudaEventDestroy(ctx->ev_kernel[q]);
+        }
+        if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
+    }
     delete ctx;
     return LB_OK;
 }
@@ -930,6 +999,11 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
     }
     int32_t left = nsteps;
     unsigned long long t = b->counter;  // batch step of the next launch
+    const int n = (int)b->ctxs.size();
+    auto step_once = [&](unsigned long long at, int from_counter) {
+        return lbk::launch_batch(b->storage, b->row_fetch, b->d_desc, b->d_prefix, n, b->total, b->d_ctl, b->wpb,
+                                 b->blocks, at, from_counter, b->stream);
+    };
     if (b->automatic() && nsteps > 0) {
         // passes of several steps, as many as make the buffers alternate with the step count (lb_step)
         int32_t m = (nsteps + b->tiles.T - 1) / b->tiles.T;
@@ -939,11 +1013,10 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
             const unsigned long long flip = (b->counter + (unsigned long long)p) & 1ULL;
             cudaError_t e;
             if (T == 1 && b->tiles.strip && flip == (t & 1ULL))  // large lattices' single step: one warp per work item
-                e = lbk::launch_batch(b->storage, 3, b->d_desc, b->d_prefix, (int)b->ctxs.size(), b->total, b->d_ctl,
-                                      b->wpb, b->blocks, t, 0, b->stream);
+                e = step_once(t, 0);
             else
-                e = lbk::launch_batch_tiles(b->storage, b->tiles, T, b->d_desc, b->d_tprefix, (int)b->ctxs.size(),
-                                            b->htprefix.back(), t, (int)flip, b->stream);
+                e = lbk::launch_batch_tiles(b->storage, b->tiles, T, b->d_desc, b->d_tprefix, n, b->htprefix.back(), t,
+                                            (int)flip, b->stream);
             if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch launch");
             t += (unsigned long long)T;
             left -= T;
@@ -955,8 +1028,7 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
         cudaGraph_t g;
         cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
         for (int j = 0; e == cudaSuccess && j < b->graph_steps; ++j)
-            e = lbk::launch_batch(b->storage, b->row_fetch, b->d_desc, b->d_prefix, (int)b->ctxs.size(), b->total,
-                                  b->d_ctl, b->wpb, b->blocks, (unsigned long long)j, 1, b->stream);
+            e = step_once((unsigned long long)j, 1);
         if (e == cudaSuccess)
             e = lbk::launch_batch_counter(b->d_ctl, (unsigned long long)b->graph_steps, 1, b->stream);
         cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
@@ -977,8 +1049,7 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
         }
     }
     for (; left > 0; --left, ++t) {
-        cudaError_t e = lbk::launch_batch(b->storage, b->row_fetch, b->d_desc, b->d_prefix, (int)b->ctxs.size(), b->total,
-                                          b->d_ctl, b->wpb, b->blocks, t, 0, b->stream);
+        cudaError_t e = step_once(t, 0);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch launch");
     }
     b->counter += (unsigned long long)nsteps;
@@ -996,15 +1067,14 @@ lb_status lb_batch_diagnostics(lb_batch *b, lb_diag *out)
 {
     if (!b || !out) return fail(nullptr, LB_ERR_ARG, "batch or out is NULL");
     cudaError_t e = batch_streams_wait(b, true);
-    // each lattice's diagnostics grid as lb_diagnostics would launch it (its
-    // launch settings may have changed since the last call)
+    // each lattice's diagnostics grid as lb_diagnostics launches it
     const int n = (int)b->ctxs.size();
     const size_t gb = lbk::batch_diag_bytes();
     std::vector<unsigned char> hd((size_t)n * gb);
     std::vector<int> hp((size_t)n + 1, 0);
     for (int m = 0; m < n; ++m) {
         lb_ctx *c = b->ctxs[m];
-        const int nb = lbk::batch_fill_diag(c->hp, diag_launch(c), c->partial, hd.data() + (size_t)m * gb);
+        const int nb = lbk::batch_fill_diag(c->hp, c->partial, hd.data() + (size_t)m * gb);
         if (nb < 1) return fail(nullptr, LB_ERR_ARG, "lattice %d: diagnostics grid too large", m);
         hp[m + 1] = hp[m] + nb;
     }

@@ -9,7 +9,6 @@
 
 namespace lbk {
 
-enum Mode { MODE_FIELDS = 1, MODE_DIAG = 2, MODE_DIAG_STRIP = 3 };
 enum Storage { ST_FP64 = 0, ST_FP32 = 1, ST_BF16 = 2, ST_FP16 = 3 };
 
 constexpr int NQ = 19;        // 9 (f) + 5 (g) + 5 (h) planes
@@ -81,8 +80,7 @@ TileLaunch tile_plan(const HostParams &p, int T);
 cudaError_t launch_tile(const HostParams &p, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
                         int *status, int rev, cudaStream_t s);
 // Pre-collision fields of rows [row0, row1) into out[5][row1-row0][nr] (double).
-cudaError_t launch_fields(const HostParams &p, const Launch &l, const void *src, double *out,
-                          int row0, int row1, cudaStream_t s);
+cudaError_t launch_fields(const HostParams &p, const void *src, double *out, int row0, int row1, cudaStream_t s);
 // Bounded-wait self-test: a warp polls an mbarrier nothing arrives at,
 // `polls` times, and sets *status to LB_ERR_TIMEOUT.
 cudaError_t launch_wait_selftest(int *status, int polls, cudaStream_t s);
@@ -90,13 +88,18 @@ cudaError_t launch_wait_selftest(int *status, int polls, cudaStream_t s);
 // (pre-collision fields): psi[nrows][nr] on the cell faces y = r0 + j + 1
 // (psi may be null) and rowmax[nrows] = max |Psi| per row.
 cudaError_t launch_psi(const double *ux, double *psi, double *rowmax, int nrows, int nr, double r0, cudaStream_t s);
+// Grid of a lattice's diagnostics: gx x gy blocks of 128 columns and seg rows.
+struct DiagGrid {
+    int gx, gy, seg;
+};
+DiagGrid diag_grid(const HostParams &p, int max_blocks);
 // Diagnostics of the stored state src: block partial sums (partial), the
-// pre-collision T field (tfield, nz * nr doubles of scratch) and the final
-// values in result[NSUM]: 0 sum(rho - rho0), 1 sum((rho - rho0) y), 2 sum T,
-// 3 max |u|, 4..7 Nusselt number per side, 8 divergence flag, 9 / 10 the
+// pre-collision T next to the walls (strips, 4 (nr + nz) doubles of scratch) and
+// the final values in result[NSUM]: 0 sum(rho - rho0), 1 sum((rho - rho0) y), 2
+// sum T, 3 max |u|, 4..7 Nusselt number per side, 8 divergence flag, 9 / 10 the
 // equivalent conductivity k_eq of the inner / outer wall of an annulus.
-cudaError_t launch_diag(const HostParams &p, const Launch &l, const void *src, double *partial,
-                        double *tfield, double *result, cudaStream_t s);
+cudaError_t launch_diag(const HostParams &p, const void *src, double *partial, double *strips, double *result,
+                        cudaStream_t s);
 // Equilibria of host-format fields [5][rows][nr] (double) into rows [row0,row1) of dst.
 cudaError_t launch_init_fields(const HostParams &p, const double *fields, void *dst, int row0,
                                int row1, cudaStream_t s);
@@ -145,12 +148,12 @@ cudaError_t launch_batch_persist(int storage, const void *desc, const int *prefi
 // The device counter of a batch: set to value, or advanced by it (add != 0).
 cudaError_t launch_batch_counter(void *ctl, unsigned long long value, int add, cudaStream_t s);
 // Batched diagnostics: one descriptor per lattice (its partial-sum buffer and
-// the grid of its own diagnostics under launch l; returns the number of
-// blocks, -1 above MAX_DIAG_BLOCKS), block prefix sums over the lattices, and
-// the three launches that write each lattice's sums and status word into
+// the grid of its own diagnostics; returns the number of blocks, -1 above
+// MAX_DIAG_BLOCKS), block prefix sums over the lattices, and the two launches
+// that write each lattice's sums and status word into
 // out + m * slot_doubles after t batch steps.
 size_t batch_diag_bytes();
-int batch_fill_diag(const HostParams &h, const Launch &l, double *partial, void *out);
+int batch_fill_diag(const HostParams &h, double *partial, void *out);
 cudaError_t launch_batch_diag(int storage, const void *desc, const void *bdiag, const int *bprefix, int n, int total,
                               unsigned long long t, double *out, int slot_doubles, cudaStream_t s);
 // Message for lb_last_error(NULL) on this thread.

@@ -7,17 +7,10 @@
 // Eq. 28.  f and h are stored as deviations from the rest state (w_a rho0,
 // w_a T0), g as is, all multiplied by `scale` (1 except for FP16).
 //
-// Work decomposition: one thread owns one radial column c and marches along
-// z over a segment of rows.  Each plane row is loaded once, at the thread's
-// own column (aligned, coalesced 128-byte rows per warp).  Pull streaming
-// (Eq. 16b, 33b, 46b) shifts in r by warp shuffles and in z by carrying the
-// row groups in registers: populations with e_x = +1 come from the previous
-// row, e_x = 0 from the current row and e_x = -1 from the next row.  The
-// macroscopic fields of the stored (previous time level) state -- the
-// moments of the same loaded values -- give the central differences of the
-// geometric sources.  A warp covers 32 columns and updates the 30 inner
-// ones; lanes 0 and 31 are halo columns.  HBM traffic is therefore 19 loads
-// and 19 stores per node update.
+// Kernels: the FP32 / 16-bit step on column pairs (lb_pair.cuh: one launch per
+// step, rows marched by a warp; lb_tile.cuh: several steps per launch on tiles
+// in shared memory), the FP64 step (k_step64), the pre-collision fields and the
+// diagnostics (block_fields), and the exchange with the host.
 #include <algorithm>
 #include <atomic>
 #include <climits>
@@ -42,11 +35,6 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kMaxSmem = 227 * 1024;  // dynamic shared memory of a block
 constexpr int kSmemPerSm = 228 * 1024;  // of an SM, 1 KB of it taken per block by the system
-constexpr int OUT_COLS = 30;  // columns updated per warp
-#ifndef LB_MARCH_UNROLL
-#define LB_MARCH_UNROLL 2
-#endif
-constexpr int kMarchUnroll = LB_MARCH_UNROLL;  // rows per unrolled march iteration
 
 // ---- storage conversions ------------------------------------------------
 
@@ -270,37 +258,6 @@ template <typename S, typename C> __device__ __forceinline__ PM<C> moments(const
     return m;
 }
 
-template <typename C> __device__ __forceinline__ C shup(C v) { return __shfl_up_sync(FULL, v, 1); }
-template <typename C> __device__ __forceinline__ C shdn(C v) { return __shfl_down_sync(FULL, v, 1); }
-
-// Row groups (already shifted in r):
-//   XM (from row i-1): f1, f5, f8, g1, h1
-//   X0 (from row i)  : f0, f2, f4, g0, g2, g4, h0, h2, h4
-//   XP (from row i+1): f3, f6, f7, g3, h3
-template <typename C>
-__device__ __forceinline__ void groups(const C v[NQ], C xm[5], C x0[9], C xp[5])
-{
-    xm[0] = v[1];
-    xm[1] = shup(v[5]);
-    xm[2] = shdn(v[8]);
-    xm[3] = v[G0 + 1];
-    xm[4] = v[H0 + 1];
-    x0[0] = v[0];
-    x0[1] = shup(v[2]);
-    x0[2] = shdn(v[4]);
-    x0[3] = v[G0 + 0];
-    x0[4] = shup(v[G0 + 2]);
-    x0[5] = shdn(v[G0 + 4]);
-    x0[6] = v[H0 + 0];
-    x0[7] = shup(v[H0 + 2]);
-    x0[8] = shdn(v[H0 + 4]);
-    xp[0] = v[3];
-    xp[1] = shup(v[6]);
-    xp[2] = shdn(v[7]);
-    xp[3] = v[G0 + 3];
-    xp[4] = v[H0 + 3];
-}
-
 template <typename S, typename C>
 __device__ __forceinline__ void load_row(const S *__restrict__ src, const KP<C> &k, int row, int col,
                                          C v[NQ])
@@ -308,15 +265,6 @@ __device__ __forceinline__ void load_row(const S *__restrict__ src, const KP<C> 
     const S *p = src + (long long)row * k.pitch + col;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) v[q] = Cvt<S, C>::ld(p + q * k.plane);
-}
-
-// raw (unconverted) loads of one row, issued ahead of their use
-template <typename S, typename C>
-__device__ __forceinline__ void load_raw(const S *__restrict__ src, const KP<C> &k, int row, int col, S r[NQ])
-{
-    const S *p = src + (long long)row * k.pitch + col;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) r[q] = p[q * k.plane];
 }
 
 template <typename S, typename C>
@@ -509,13 +457,7 @@ __device__ __forceinline__ void update_node(const KP<C> &k, C y, C iy, C fv[9], 
     }
 }
 
-// ---- diagnostics accumulator ------------------------------------------------
-
-struct DiagAcc {
-    double mass_dev, mass_r_dev, tsum, umax, bad;
-};
-
-// ---- the march ---------------------------------------------------------------
+// ---- scalar wall rules ----------------------------------------------------------
 
 // Wall and axis rules (Sec. 3) on the pulled values of node (i, cl), in units
 // of the storage scale sc; the own stored values are read from src.
@@ -595,188 +537,6 @@ __device__ __forceinline__ void wall_rules1(const KP<C> &k, const S *__restrict_
         gv[3] = scalar_bc<C>(k.swirl[sd], own<S, C>(src, k, G0 + 1, i, cl), wall_psi<C>(k, sd, y) * sc, true);
         hv[3] = scalar_bc<C>(heat_rule(k, sd), own<S, C>(src, k, H0 + 1, i, cl), (end_T(k, sd, y) - k.T0) * sc,
                              false);
-    }
-}
-
-template <typename S, typename C, int MODE>
-__device__ __forceinline__ void march(const KP<C> &k, const S *__restrict__ src, S *__restrict__ dst,
-                                      double *__restrict__ fout, int fout_row0, int fout_rows, int c,
-                                      int row_s, int row_e, DiagAcc *acc)
-{
-    const int lane = threadIdx.x & 31;
-    const int nr = k.nr, nz = k.nz;
-    const int cl = c < 0 ? 0 : (c >= nr ? nr - 1 : c);
-    const bool out_lane = lane >= 1 && lane <= OUT_COLS && c < nr;
-    const bool at_c0 = c == 0, at_cN = c == nr - 1;
-    const bool edge_warp = __any_sync(FULL, at_c0 || at_cN);
-    // radius of the column, its inverse computed in FP64 and rounded once
-    const double yd = k.r0 + cl + 0.5;
-    const C y = (C)yd, iy = (C)(1.0 / yd);
-    const C is = k.inv_scale, sc = k.scale;
-
-    C v[NQ];
-    C xm_prev[5], xm_cur[5], x0_cur[9];
-    PM<C> pm_cur;
-    C uy_prev = 0;
-    bool has_m;
-
-    // prologue: rows s-1 and s
-    if (row_s > 0 || k.xper) {
-        const int rm = row_s > 0 ? row_s - 1 : nz - 1;
-        load_row<S, C>(src, k, rm, cl, v);
-        C x0t[9], xpt[5];
-        groups<C>(v, xm_prev, x0t, xpt);
-        uy_prev = moments<S, C>(v, k).uy;
-        has_m = true;
-    } else {
-        has_m = false;
-#pragma unroll
-        for (int q = 0; q < 5; ++q) xm_prev[q] = 0;
-    }
-    // software pipeline: the raw values of row i+1 are loaded during the
-    // iteration for row i-1, so a row's DRAM latency overlaps the previous
-    // row's arithmetic
-    S nb[NQ];
-    if ((row_s + 1 < nz) || k.xper) load_raw<S, C>(src, k, row_s + 1 < nz ? row_s + 1 : 0, cl, nb);
-    {
-        load_row<S, C>(src, k, row_s, cl, v);
-        C xpt[5];
-        groups<C>(v, xm_cur, x0_cur, xpt);
-        pm_cur = moments<S, C>(v, k);
-    }
-
-#pragma unroll kMarchUnroll
-    for (int i = row_s; i < row_e; ++i) {
-        const bool has_p = (i + 1 < nz) || k.xper;
-        C xp_n[5], x0_n[9], xm_n[5];
-        PM<C> pm_n;
-        if (has_p) {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) v[q] = Cvt<S, C>::cv(nb[q]);
-        }
-        if (i + 1 < row_e && ((i + 2 < nz) || k.xper))
-            load_raw<S, C>(src, k, i + 2 < nz ? i + 2 : i + 2 - nz, cl, nb);
-        if (has_p) {
-            groups<C>(v, xm_n, x0_n, xp_n);
-            pm_n = moments<S, C>(v, k);
-        } else {
-#pragma unroll
-            for (int q = 0; q < 5; ++q) xp_n[q] = xm_n[q] = 0;
-#pragma unroll
-            for (int q = 0; q < 9; ++q) x0_n[q] = 0;
-            pm_n = pm_cur;
-        }
-
-        // pulled values (scaled storage units)
-        C fv[9], gv[5], hv[5];
-        fv[1] = xm_prev[0]; fv[5] = xm_prev[1]; fv[8] = xm_prev[2]; gv[1] = xm_prev[3]; hv[1] = xm_prev[4];
-        fv[0] = x0_cur[0]; fv[2] = x0_cur[1]; fv[4] = x0_cur[2];
-        gv[0] = x0_cur[3]; gv[2] = x0_cur[4]; gv[4] = x0_cur[5];
-        hv[0] = x0_cur[6]; hv[2] = x0_cur[7]; hv[4] = x0_cur[8];
-        fv[3] = xp_n[0]; fv[6] = xp_n[1]; fv[7] = xp_n[2]; gv[3] = xp_n[3]; hv[3] = xp_n[4];
-
-        wall_rules1<S, C>(k, src, i, cl, edge_warp && at_c0, edge_warp && at_cN, has_m, has_p, y, sc, fv, gv, hv);
-        if (Scaled<S>::value) {
-#pragma unroll
-            for (int q = 0; q < 9; ++q) fv[q] *= is;
-#pragma unroll
-            for (int q = 0; q < 5; ++q) {
-                gv[q] *= is;
-                hv[q] *= is;
-            }
-        }
-
-        // central differences of the stored-state fields, with ghosts
-        // (a free surface: no shear, u_y even across it)
-        const int sb = end_seg(k, 0, cl), st = end_seg(k, 1, cl);
-        const C uy_xm = has_m ? uy_prev : (k.flow[sb] == 3 ? pm_cur.uy : (C)2 * k.uwy[sb] - pm_cur.uy);
-        const C uy_xp = has_p ? pm_n.uy : (k.flow[st] == 3 ? pm_cur.uy : (C)2 * k.uwy[st] - pm_cur.uy);
-        C ux_l = shup(pm_cur.ux), uy_l = shup(pm_cur.uy), ut_l = shup(pm_cur.ut), T_l = shup(pm_cur.T);
-        C ux_r = shdn(pm_cur.ux), uy_r = shdn(pm_cur.uy), ut_r = shdn(pm_cur.ut), T_r = shdn(pm_cur.T);
-        if (edge_warp) {
-            if (at_c0) {
-                const int sd = 2;
-                if (k.flow[sd] == 1) {
-                    ux_l = pm_cur.ux;
-                    uy_l = -pm_cur.uy;
-                } else {
-                    ux_l = (C)2 * k.uwx[sd] - pm_cur.ux;
-                    uy_l = (C)2 * k.uwy[sd] - pm_cur.uy;
-                }
-                const int sw = k.swirl[sd], ht = k.heat[sd];
-                ut_l = sw == 2 ? -pm_cur.ut : (sw == 0 ? (C)2 * k.omega[sd] * (C)k.r0 - pm_cur.ut : pm_cur.ut);
-                T_l = ht == 0 ? (C)2 * k.Tw[sd] - pm_cur.T : pm_cur.T;
-            }
-            if (at_cN) {
-                const int sd = 3;
-                ux_r = (C)2 * k.uwx[sd] - pm_cur.ux;
-                uy_r = (C)2 * k.uwy[sd] - pm_cur.uy;
-                const int sw = k.swirl[sd], ht = k.heat[sd];
-                ut_r = sw == 0 ? (C)2 * k.omega[sd] * (C)(k.r0 + k.nr) - pm_cur.ut : pm_cur.ut;
-                T_r = ht == 0 ? (C)2 * k.Tw[sd] - pm_cur.T : pm_cur.T;
-            }
-        }
-        const C dxuy = (C)0.5 * (uy_xp - uy_xm);
-        const C dyux = (C)0.5 * (ux_r - ux_l);
-        const C dyuy = (C)0.5 * (uy_r - uy_l);
-        const C dyut = (C)0.5 * (ut_r - ut_l);
-        const C dyT = (C)0.5 * (T_r - T_l);
-
-        NodeOut<C> o;
-        update_node<C>(k, y, iy, fv, gv, hv, dxuy, dyux, dyuy, dyut, dyT, o);
-
-        if (MODE == MODE_FIELDS) {
-            if (out_lane) {
-                const long long n = (long long)fout_rows * nr;  // plane stride of the output chunk
-                double *p = fout + (long long)(i - fout_row0) * nr + c;
-                p[0] = (double)o.rho;
-                p[n] = (double)o.ux;
-                p[2 * n] = (double)o.uy;
-                p[3 * n] = (double)o.ut;
-                p[4 * n] = (double)o.T;
-            }
-        } else {  // MODE_DIAG
-            if (out_lane) {
-                const double rdp = (double)pm_cur.rd;
-                acc->mass_dev += rdp;
-                acc->mass_r_dev += rdp * yd;
-                acc->tsum += (double)o.T;
-                const double um = sqrt((double)o.ux * (double)o.ux + (double)o.uy * (double)o.uy);
-                acc->umax = fmax(acc->umax, um);
-                const bool finite = isfinite((double)o.rho) && isfinite((double)o.ux) &&
-                                    isfinite((double)o.uy) && isfinite((double)o.ut) &&
-                                    isfinite((double)o.T);
-                if (!finite || o.rho < (C)0.5 || o.rho > (C)1.5) acc->bad = 1.0;
-                if (MODE == MODE_DIAG) {
-                    fout[(long long)i * nr + c] = (double)o.T;  // for the wall fluxes
-                } else {
-                    // wall-adjacent temperatures only: rows 0, 1, nz-2, nz-1
-                    // (4 x nr values), then columns 0, 1, nr-2, nr-1 (4 x nz)
-                    const double T = (double)o.T;
-                    if (i == 0) fout[c] = T;
-                    if (i == 1) fout[nr + c] = T;
-                    if (i == nz - 2) fout[2 * nr + c] = T;
-                    if (i == nz - 1) fout[3 * nr + c] = T;
-                    double *cs = fout + 4LL * nr;
-                    if (c == 0) cs[i] = T;
-                    if (c == 1) cs[nz + i] = T;
-                    if (c == nr - 2) cs[2LL * nz + i] = T;
-                    if (c == nr - 1) cs[3LL * nz + i] = T;
-                }
-            }
-        }
-
-        // rotate the row window
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-            xm_prev[q] = xm_cur[q];
-            xm_cur[q] = xm_n[q];
-        }
-#pragma unroll
-        for (int q = 0; q < 9; ++q) x0_cur[q] = x0_n[q];
-        uy_prev = pm_cur.uy;
-        pm_cur = pm_n;
-        has_m = true;
     }
 }
 
@@ -1190,17 +950,132 @@ __global__ void __launch_bounds__(128) k_psi(const double *__restrict__ ux, doub
     if (lane == 0) rowmax[row] = m;
 }
 
-constexpr int kFieldRows = 32;  // rows per z-segment of the field export
+// Pre-collision fields of the nodes of a block: 128 columns from c0, rows s ..
+// s + n - 1, by 256 threads, a thread's nodes all in one column.  Eight rows at
+// a time the block forms the macroscopic fields of the stored state of the rows
+// and their neighbours in shared memory (F: ten rows, two of which stay for
+// the next eight), then each thread its nodes.  stored(i, c, fields) sees every
+// node's stored state once, node(i, c, out) its pre-collision state.  (A warp
+// marching 32 rows of 30 columns on its own, as before, is a serial chain of
+// 32 row updates; these are four nodes per thread and round, all independent: the
+// diagnostics of 1024 x 2048 FP32 took 220 us and take 124.)
+constexpr int kBlockCols = 128, kBlockChunk = 8, kBlockThreads = 256, kBlockPitch = kBlockCols + 2;
+template <typename C> constexpr size_t kBlockSmem = (size_t)(kBlockChunk + 2) * 4 * kBlockPitch * sizeof(C);
 
-template <typename S, typename C>
-__global__ void __launch_bounds__(256) k_fields(KP<C> k, const S *__restrict__ src, double *__restrict__ out,
-                                                int row0, int row1, int nwin)
+template <typename S, typename C, typename Stored, typename Node>
+__device__ __forceinline__ void block_fields(const KP<C> &k, const S *__restrict__ src, int c0, int s, int n, C *F,
+                                             Stored stored, Node node)
 {
-    const int warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (warp >= nwin) return;
-    const int c = warp * OUT_COLS - 1 + (threadIdx.x & 31);
-    const int s = row0 + blockIdx.y * kFieldRows, e = min(row1, s + kFieldRows);
-    march<S, C, MODE_FIELDS>(k, src, nullptr, out, row0, row1 - row0, c, s, e, nullptr);
+    const int nr = k.nr, nz = k.nz;
+    const int c = c0 + (int)(threadIdx.x % kBlockCols), half = threadIdx.x / kBlockCols;
+    const bool at_c0 = c == 0, at_cN = c == nr - 1;
+    const double yd = k.r0 + c + 0.5;
+    const C y = (C)yd, iy = (C)(1.0 / yd);
+    auto slot = [&](int rel) { return F + ((rel + 1) % (kBlockChunk + 2)) * 4 * kBlockPitch; };
+    // the fields of row s + rel, column cc; rows and columns outside the lattice have none
+    auto form = [&](int rel, int cc, bool own_node) {
+        int i = s + rel;
+        if (k.xper) i = i < 0 ? i + nz : (i >= nz ? i - nz : i);
+        if (i < 0 || i >= nz || cc < 0 || cc >= nr) return;
+        C v[NQ];
+        load_row<S, C>(src, k, i, cc, v);
+        const PM<C> m = moments<S, C>(v, k);
+        C *f = slot(rel) + (cc - c0 + 1);
+        f[0] = m.ux;
+        f[kBlockPitch] = m.uy;
+        f[2 * kBlockPitch] = m.ut;
+        f[3 * kBlockPitch] = m.T;
+        if (own_node) stored(i, cc, m);
+    };
+    for (int r0 = 0; r0 < n; r0 += kBlockChunk) {
+        const int m = min(kBlockChunk, n - r0), first = r0 == 0 ? -1 : r0 + 1;
+#pragma unroll 2
+        for (int rel = first + half; rel <= r0 + m; rel += 2) form(rel, c, rel >= 0 && rel < n);
+        if ((int)threadIdx.x < 2 * (r0 + m - first + 1))
+            form(first + (int)(threadIdx.x >> 1), (threadIdx.x & 1) ? c0 + kBlockCols : c0 - 1, false);
+        __syncthreads();
+        if (c < nr)
+            for (int rel = r0 + half; rel < r0 + m; rel += 2) {
+                const int i = s + rel;
+                const bool has_m = i > 0 || k.xper, has_p = i + 1 < nz || k.xper;
+                const int im = i > 0 ? i - 1 : nz - 1, ip = i + 1 < nz ? i + 1 : 0;
+                const int jm = max(c - 1, 0), jp = min(c + 1, nr - 1);
+                auto ld = [&](int q, int row, int col) { return own<S, C>(src, k, q, row, col); };
+                // pulled values (scaled storage units)
+                C fv[9] = {ld(0, i, c),   ld(1, im, c),  ld(2, i, jm),  ld(3, ip, c), ld(4, i, jp),
+                           ld(5, im, jm), ld(6, ip, jm), ld(7, ip, jp), ld(8, im, jp)};
+                C gv[5] = {ld(9, i, c), ld(10, im, c), ld(11, i, jm), ld(12, ip, c), ld(13, i, jp)};
+                C hv[5] = {ld(14, i, c), ld(15, im, c), ld(16, i, jm), ld(17, ip, c), ld(18, i, jp)};
+                wall_rules1<S, C>(k, src, i, c, at_c0, at_cN, has_m, has_p, y, k.scale, fv, gv, hv);
+                if (Scaled<S>::value) {
+#pragma unroll
+                    for (int q = 0; q < 9; ++q) fv[q] *= k.inv_scale;
+#pragma unroll
+                    for (int q = 0; q < 5; ++q) {
+                        gv[q] *= k.inv_scale;
+                        hv[q] *= k.inv_scale;
+                    }
+                }
+                // central differences of the stored-state fields, with ghosts
+                // (a free surface: no shear, u_y even across it)
+                const C *f = slot(rel) + (c - c0 + 1), *fm = slot(rel - 1) + (c - c0 + 1), *fp = slot(rel + 1) + (c - c0 + 1);
+                constexpr int P = kBlockPitch;
+                const C uy = f[P];
+                C uy_m = uy, uy_p = uy;
+                if (has_m) uy_m = fm[P];
+                else if (k.flow[end_seg(k, 0, c)] != 3) uy_m = (C)2 * k.uwy[end_seg(k, 0, c)] - uy;
+                if (has_p) uy_p = fp[P];
+                else if (k.flow[end_seg(k, 1, c)] != 3) uy_p = (C)2 * k.uwy[end_seg(k, 1, c)] - uy;
+                C l[4], r[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    l[q] = f[q * P - 1];
+                    r[q] = f[q * P + 1];
+                }
+                if (at_c0) {
+                    const bool axis = k.flow[2] == 1;
+                    l[0] = axis ? f[0] : (C)2 * k.uwx[2] - f[0];
+                    l[1] = axis ? -uy : (C)2 * k.uwy[2] - uy;
+                    const C ut = f[2 * P], T = f[3 * P];
+                    l[2] = k.swirl[2] == 2 ? -ut : (k.swirl[2] == 0 ? (C)2 * k.omega[2] * (C)k.r0 - ut : ut);
+                    l[3] = k.heat[2] == 0 ? (C)2 * k.Tw[2] - T : T;
+                }
+                if (at_cN) {
+                    r[0] = (C)2 * k.uwx[3] - f[0];
+                    r[1] = (C)2 * k.uwy[3] - uy;
+                    const C ut = f[2 * P], T = f[3 * P];
+                    r[2] = k.swirl[3] == 0 ? (C)2 * k.omega[3] * (C)(k.r0 + k.nr) - ut : ut;
+                    r[3] = k.heat[3] == 0 ? (C)2 * k.Tw[3] - T : T;
+                }
+                NodeOut<C> o;
+                update_node<C>(k, y, iy, fv, gv, hv, (C)0.5 * (uy_p - uy_m), (C)0.5 * (r[0] - l[0]),
+                               (C)0.5 * (r[1] - l[1]), (C)0.5 * (r[2] - l[2]), (C)0.5 * (r[3] - l[3]), o);
+                node(i, c, o);
+            }
+        __syncthreads();
+    }
+}
+
+// Pre-collision fields of rows [row0, row1) as doubles, out[5][row1 - row0][nr]:
+// a block per kBlockChunk rows.
+template <typename S, typename C>
+__global__ void __launch_bounds__(kBlockThreads) k_fields(const __grid_constant__ KP<C> k, const S *__restrict__ src,
+                                                          double *__restrict__ out, int row0, int row1, int nbx)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int s = row0 + (int)(blockIdx.x / nbx) * kBlockChunk;
+    const long long n = (long long)(row1 - row0) * k.nr;  // plane stride of the output chunk
+    block_fields<S, C>(
+        k, src, (int)(blockIdx.x % nbx) * kBlockCols, s, min(row1, s + kBlockChunk) - s, reinterpret_cast<C *>(smem),
+        [](int, int, const PM<C> &) {},
+        [&](int i, int c, const NodeOut<C> &o) {
+            double *p = out + (long long)(i - row0) * k.nr + c;
+            p[0] = (double)o.rho;
+            p[n] = (double)o.ux;
+            p[2 * n] = (double)o.uy;
+            p[3 * n] = (double)o.ut;
+            p[4 * n] = (double)o.T;
+        });
 }
 
 __device__ __forceinline__ double warp_sum(double v)
@@ -1216,249 +1091,221 @@ __device__ __forceinline__ double warp_max(double v)
     return v;
 }
 
-// One warp per 30-column window, whole height (the end-wall fluxes need rows
-// 0, 1 and nz-2, nz-1 in the same march).  Block partial sums in a fixed
-// order, then a single-block final reduction: deterministic.
-// Block (bx, by) of a diagnostics grid gx blocks wide; 128 threads.
+// Sums over a thread's nodes.  FP64 instructions are what a diagnostic of an
+// FP32 lattice would spend its time on (the pipe takes one per SM every 19
+// cycles, conversions to and from FP64 included), so an FP32 thread keeps its
+// few sums as a value and the exact rounding error of each addition (Knuth's
+// two-sum), and turns them into FP64 once, at its end: an error of 2^-47 of a
+// sum over at most some dozens of nodes.
+template <typename C> struct NodeSum {
+    C hi = 0, lo = 0;
+    __device__ __forceinline__ void add(C x)
+    {
+        if constexpr (std::is_same<C, double>::value) {
+            hi += x;
+        } else {
+            const C t = hi + x, b = t - hi;
+            lo += (hi - (t - b)) + (x - b);
+            hi = t;
+        }
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+// The largest u_x^2 + u_y^2, FP32 squares as unevaluated sums of two FP32
+// values (exact products by FMA, two-sum), scaled away from the subnormal range.
+template <typename C> struct NodeMax {
+    C hi = 0, lo = 0;
+    __device__ __forceinline__ void add(C ux, C uy)
+    {
+        if constexpr (std::is_same<C, double>::value) {
+            hi = fmax(hi, ux * ux + uy * uy);
+        } else {
+            const float x = ux * 0x1p32f, y = uy * 0x1p32f;
+            const float p = x * x, q = y * y, t = p + q, b = t - p;
+            const float e = ((p - (t - b)) + (q - b)) + (__fmaf_rn(x, x, -p) + __fmaf_rn(y, y, -q));
+            const float h = t + e, l = e - (h - t);
+            if (h > hi || (h == hi && l > lo)) {
+                hi = h;
+                lo = l;
+            }
+            if (t == INFINITY) {  // (the error terms are not numbers)
+                hi = t;
+                lo = 0.0f;
+            }
+        }
+    }
+    __device__ __forceinline__ double value() const
+    {
+        if constexpr (std::is_same<C, double>::value) return sqrt(hi);
+        else return sqrt((double)hi + (double)lo) * 0x1p-32;
+    }
+};
+
+// Diagnostics of block (bx, by) of a grid gx blocks wide, seg_rows rows each:
+// partial sums in a fixed order, and the temperatures next to the walls in
+// strips: rows 0, 1, nz - 2, nz - 1 (4 x nr values), then columns 0, 1, nr - 2,
+// nr - 1 (4 x nz).
 template <typename S, typename C>
 __device__ __forceinline__ void diag_block(const KP<C> &k, const S *__restrict__ src, double *__restrict__ partial,
-                                           double *__restrict__ tfield, int seg_rows, int nwin, int bx, int by,
-                                           int gx)
+                                           double *__restrict__ strips, int seg_rows, int bx, int by, int gx, C *F)
 {
-    __shared__ double sh[4][NSUM];
-    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int warp = bx * (blockDim.x >> 5) + wib;
-    DiagAcc a = {0, 0, 0, 0, 0};
-    if (warp < nwin) {
-        const int c = warp * OUT_COLS - 1 + lane;
-        const int s = by * seg_rows, e = min(k.nz, s + seg_rows);
-        march<S, C, MODE_DIAG>(k, src, nullptr, tfield, 0, 0, c, s, e, &a);
-    }
-    double vals[NSUM] = {a.mass_dev, a.mass_r_dev, a.tsum, a.umax, 0, 0, 0, 0, a.bad, 0, 0, 0};
+    constexpr int warps = kBlockThreads / 32;
+    __shared__ double sh[warps][5];
+    const int nr = k.nr, nz = k.nz, s = by * seg_rows;
+    NodeSum<C> rd, T;
+    NodeMax<C> u;
+    bool bad = false;
+    block_fields<S, C>(
+        k, src, bx * kBlockCols, s, min(nz, s + seg_rows) - s, F, [&](int, int, const PM<C> &m) { rd.add(m.rd); },
+        [&](int i, int c, const NodeOut<C> &o) {
+            T.add(o.T);
+            u.add(o.ux, o.uy);
+            bad |= !(isfinite(o.rho) && isfinite(o.ux) && isfinite(o.uy) && isfinite(o.ut) && isfinite(o.T)) ||
+                   o.rho < (C)0.5 || o.rho > (C)1.5;
+            double *cs = strips + 4LL * nr;
+            if (i <= 1) strips[(long long)i * nr + c] = (double)o.T;
+            if (i >= nz - 2) strips[(long long)(i - nz + 4) * nr + c] = (double)o.T;
+            if (c <= 1) cs[(long long)c * nz + i] = (double)o.T;
+            if (c >= nr - 2) cs[(long long)(c - nr + 4) * nz + i] = (double)o.T;
+        });
+    const double m = rd.value();
+    const double y = k.r0 + (bx * kBlockCols + (int)(threadIdx.x % kBlockCols)) + 0.5;
+    double vals[5] = {m, m * y, T.value(), u.value(), bad ? 1.0 : 0.0};
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
 #pragma unroll
-    for (int q = 0; q < NSUM; ++q) vals[q] = (q == 3 || q == 8) ? warp_max(vals[q]) : warp_sum(vals[q]);
+    for (int q = 0; q < 5; ++q) vals[q] = q >= 3 ? warp_max(vals[q]) : warp_sum(vals[q]);
     if (lane == 0)
-        for (int q = 0; q < NSUM; ++q) sh[wib][q] = vals[q];
+        for (int q = 0; q < 5; ++q) sh[wib][q] = vals[q];
     __syncthreads();
-    if (threadIdx.x < NSUM) {
+    if (threadIdx.x < 5) {
         const int q = threadIdx.x;
         double r = sh[0][q];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = (q == 3 || q == 8) ? fmax(r, sh[w][q]) : r + sh[w][q];
-        partial[(by * gx + bx) * NSUM + q] = r;
+        for (int w = 1; w < warps; ++w) r = q >= 3 ? fmax(r, sh[w][q]) : r + sh[w][q];
+        partial[(by * gx + bx) * NSUM + (q == 4 ? 8 : q)] = r;
     }
 }
 
 template <typename S, typename C>
-__global__ void __launch_bounds__(128) k_diag(KP<C> k, const S *__restrict__ src, double *__restrict__ partial,
-                                              double *__restrict__ tfield, int seg_rows, int nwin)
+__global__ void __launch_bounds__(kBlockThreads) k_diag(const __grid_constant__ KP<C> k, const S *__restrict__ src,
+                                                        double *__restrict__ partial, double *__restrict__ strips,
+                                                        int seg_rows, int gx)
 {
-    diag_block<S, C>(k, src, partial, tfield, seg_rows, nwin, blockIdx.x, blockIdx.y, gridDim.x);
+    extern __shared__ __align__(128) unsigned char smem[];
+    diag_block<S, C>(k, src, partial, strips, seg_rows, blockIdx.x % gx, blockIdx.x / gx, gx, reinterpret_cast<C *>(smem));
 }
 
-// Wall heat-flux sums (Sec. 3.2) from the pre-collision T field: one-sided
-// second-order derivative through the wall value, wall half a cell away,
-// (-8 T_w + 9 T_1 - T_2) / 3 along the inward direction; end walls weighted
-// by the radius.  One block, fixed-order tree reduction (deterministic).
-template <typename C>
-__device__ __forceinline__ void wall_block(const KP<C> &k, const double *__restrict__ T, double *__restrict__ result)
+// A block's sum (or largest) of 256 values, a fixed tree (deterministic).
+__device__ __forceinline__ double tree256(double v, bool mx)
 {
     __shared__ double sh[256];
-    const int nr = k.nr, nz = k.nz;
-    for (int sd = 0; sd < 4; ++sd) {
-        double acc = 0;
-        if (wall_heated(k, sd)) {
-            const double Tw = (double)k.Tw[sd];
-            if (sd == 2)
-                for (int i = threadIdx.x; i < nz; i += blockDim.x)
-                    acc += (-8.0 * Tw + 9.0 * T[(long long)i * nr] - T[(long long)i * nr + 1]) / 3.0;
-            else if (sd == 3)
-                for (int i = threadIdx.x; i < nz; i += blockDim.x)
-                    acc += (8.0 * Tw - 9.0 * T[(long long)i * nr + nr - 1] + T[(long long)i * nr + nr - 2]) / 3.0;
-            else if (sd == 0)
-                for (int j = threadIdx.x; j < nr; j += blockDim.x)
-                    acc += (k.r0 + j + 0.5) * (-8.0 * Tw + 9.0 * T[j] - T[nr + j]) / 3.0;
-            else  // the top: the columns whose segment holds a wall temperature, each with its own value
-                for (int j = threadIdx.x; j < nr; j += blockDim.x) {
-                    const int sg = end_seg(k, 1, j);
-                    if (k.heat[sg] != 0 && k.heat[sg] != 4) continue;
-                    const double Tj = (double)end_T(k, sg, (C)(k.r0 + j + 0.5));
-                    acc += (k.r0 + j + 0.5) *
-                           (8.0 * Tj - 9.0 * T[(long long)(nz - 1) * nr + j] + T[(long long)(nz - 2) * nr + j]) / 3.0;
-                }
-        }
-        sh[threadIdx.x] = acc;
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            result[4 + sd] = wall_heated(k, sd) ? sh[0] * k.nu_scale[sd] : 0.0;
-            if (sd >= 2) result[7 + sd] = k.heat[sd] == 0 ? sh[0] * k.keq_scale[sd] : 0.0;  // 9, 10: k_eq
-        }
-        __syncthreads();
-    }
-}
-
-template <typename C>
-__global__ void __launch_bounds__(256) k_wall(KP<C> k, const double *__restrict__ T, double *__restrict__ result)
-{
-    wall_block<C>(k, T, result);
-}
-
-// Variant of k_diag whose temperature output is the wall-adjacent strips
-// only (4 (nr + nz) doubles), for the scratch-free diagnostics entry point.
-template <typename S, typename C>
-__global__ void __launch_bounds__(128) k_diag_strip(KP<C> k, const S *__restrict__ src,
-                                                    double *__restrict__ partial, double *__restrict__ strips,
-                                                    int seg_rows, int nwin)
-{
-    __shared__ double sh[4][NSUM];
-    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int warp = blockIdx.x * (blockDim.x >> 5) + wib;
-    DiagAcc a = {0, 0, 0, 0, 0};
-    if (warp < nwin) {
-        const int c = warp * OUT_COLS - 1 + lane;
-        const int s = blockIdx.y * seg_rows, e = min(k.nz, s + seg_rows);
-        march<S, C, MODE_DIAG_STRIP>(k, src, nullptr, strips, 0, 0, c, s, e, &a);
-    }
-    double vals[NSUM] = {a.mass_dev, a.mass_r_dev, a.tsum, a.umax, 0, 0, 0, 0, a.bad, 0, 0, 0};
-#pragma unroll
-    for (int q = 0; q < NSUM; ++q) vals[q] = (q == 3 || q == 8) ? warp_max(vals[q]) : warp_sum(vals[q]);
-    if (lane == 0)
-        for (int q = 0; q < NSUM; ++q) sh[wib][q] = vals[q];
+    sh[threadIdx.x] = v;
     __syncthreads();
-    if (threadIdx.x < NSUM) {
-        const int q = threadIdx.x;
-        double r = sh[0][q];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = (q == 3 || q == 8) ? fmax(r, sh[w][q]) : r + sh[w][q];
-        partial[(blockIdx.y * gridDim.x + blockIdx.x) * NSUM + q] = r;
+    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+        if ((int)threadIdx.x < w) {
+            const double a = sh[threadIdx.x], b = sh[threadIdx.x + w];
+            sh[threadIdx.x] = mx ? fmax(a, b) : a + b;
+        }
+        __syncthreads();
     }
+    return sh[0];
 }
 
-// k_wall on the strips written by k_diag_strip (same summation order).
+// The last reductions of a diagnostics, one block of 256 threads each: tasks 0
+// .. 3 the wall heat-flux sums of the sides, 4 .. 8 the sums over the blocks.
+//
+// Wall heat fluxes (Sec. 3.2) from the pre-collision T next to the walls
+// (strips of diag_block): one-sided second-order derivative through the wall
+// value, wall half a cell away, (-8 T_w + 9 T_1 - T_2) / 3 along the inward
+// direction; end walls weighted by the radius.
+constexpr int kDiagTasks = 9;
 template <typename C>
-__global__ void __launch_bounds__(256) k_wall_strip(KP<C> k, const double *__restrict__ strips,
-                                                    double *__restrict__ result)
+__device__ __forceinline__ void diag_task(const KP<C> &k, int task, const double *__restrict__ partial, int nblocks,
+                                          const double *__restrict__ strips, double *__restrict__ result)
 {
-    __shared__ double sh[256];
-    const int nr = k.nr, nz = k.nz;
-    const double *r0 = strips, *r1 = strips + nr, *r2 = strips + 2 * nr, *r3 = strips + 3 * nr;
-    const double *c0 = strips + 4 * nr, *c1 = c0 + nz, *c2 = c0 + 2 * nz, *c3 = c0 + 3 * nz;
-    for (int sd = 0; sd < 4; ++sd) {
-        double acc = 0;
-        if (wall_heated(k, sd)) {
-            const double Tw = (double)k.Tw[sd];
-            if (sd == 2)
-                for (int i = threadIdx.x; i < nz; i += blockDim.x) acc += (-8.0 * Tw + 9.0 * c0[i] - c1[i]) / 3.0;
-            else if (sd == 3)
-                for (int i = threadIdx.x; i < nz; i += blockDim.x) acc += (8.0 * Tw - 9.0 * c3[i] + c2[i]) / 3.0;
-            else if (sd == 0)
-                for (int j = threadIdx.x; j < nr; j += blockDim.x)
-                    acc += (k.r0 + j + 0.5) * (-8.0 * Tw + 9.0 * r0[j] - r1[j]) / 3.0;
-            else
-                for (int j = threadIdx.x; j < nr; j += blockDim.x) {
-                    const int sg = end_seg(k, 1, j);
-                    if (k.heat[sg] != 0 && k.heat[sg] != 4) continue;
-                    const double Tj = (double)end_T(k, sg, (C)(k.r0 + j + 0.5));
-                    acc += (k.r0 + j + 0.5) * (8.0 * Tj - 9.0 * r3[j] + r2[j]) / 3.0;
-                }
-        }
-        sh[threadIdx.x] = acc;
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            result[4 + sd] = wall_heated(k, sd) ? sh[0] * k.nu_scale[sd] : 0.0;
-            if (sd >= 2) result[7 + sd] = k.heat[sd] == 0 ? sh[0] * k.keq_scale[sd] : 0.0;  // 9, 10: k_eq
-        }
-        __syncthreads();
-    }
-}
-
-// One block of 256 threads: per sum, strided partial sums in a fixed order,
-// then a fixed tree (deterministic for a given number of blocks).
-__device__ __forceinline__ void diag_final_block(const double *__restrict__ partial, int nblocks,
-                                                 double *__restrict__ result)
-{
-    __shared__ double sh[256];
-    for (int q = 0; q < NSUM; ++q) {
-        if ((q >= 4 && q < 8) || q == 9 || q == 10) continue;  // 4..7, 9, 10: wall sums (k_wall)
+    if (task >= 4) {
+        const int q = task == 8 ? 8 : task - 4;
         const bool mx = q == 3 || q == 8;
         double r = 0.0;
         for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
             const double v = partial[b * NSUM + q];
             r = mx ? fmax(r, v) : r + v;
         }
-        sh[threadIdx.x] = r;
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if ((int)threadIdx.x < w) sh[threadIdx.x] = mx ? fmax(sh[threadIdx.x], sh[threadIdx.x + w])
-                                                            : sh[threadIdx.x] + sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) result[q] = sh[0];
-        __syncthreads();
+        r = tree256(r, mx);
+        if (threadIdx.x == 0) result[q] = r;
+        return;
+    }
+    const int sd = task, nr = k.nr, nz = k.nz;
+    const double *r0 = strips, *r1 = strips + nr, *r2 = strips + 2 * nr, *r3 = strips + 3 * nr;
+    const double *c0 = strips + 4 * nr, *c1 = c0 + nz, *c2 = c0 + 2 * nz, *c3 = c0 + 3 * nz;
+    double acc = 0;
+    if (wall_heated(k, sd)) {
+        const double Tw = (double)k.Tw[sd];
+        if (sd == 2)
+            for (int i = threadIdx.x; i < nz; i += blockDim.x) acc += (-8.0 * Tw + 9.0 * c0[i] - c1[i]) / 3.0;
+        else if (sd == 3)
+            for (int i = threadIdx.x; i < nz; i += blockDim.x) acc += (8.0 * Tw - 9.0 * c3[i] + c2[i]) / 3.0;
+        else if (sd == 0)
+            for (int j = threadIdx.x; j < nr; j += blockDim.x)
+                acc += (k.r0 + j + 0.5) * (-8.0 * Tw + 9.0 * r0[j] - r1[j]) / 3.0;
+        else  // the top: the columns whose segment holds a wall temperature, each with its own value
+            for (int j = threadIdx.x; j < nr; j += blockDim.x) {
+                const int sg = end_seg(k, 1, j);
+                if (k.heat[sg] != 0 && k.heat[sg] != 4) continue;
+                const double Tj = (double)end_T(k, sg, (C)(k.r0 + j + 0.5));
+                acc += (k.r0 + j + 0.5) * (8.0 * Tj - 9.0 * r3[j] + r2[j]) / 3.0;
+            }
+    }
+    acc = tree256(acc, false);
+    if (threadIdx.x == 0) {
+        result[4 + sd] = wall_heated(k, sd) ? acc * k.nu_scale[sd] : 0.0;
+        if (sd >= 2) result[7 + sd] = k.heat[sd] == 0 ? acc * k.keq_scale[sd] : 0.0;  // 9, 10: k_eq
     }
 }
 
-__global__ void __launch_bounds__(256) k_diag_final(const double *__restrict__ partial, int nblocks,
+template <typename C>
+__global__ void __launch_bounds__(256) k_diag_final(const __grid_constant__ KP<C> k, const double *__restrict__ partial,
+                                                    int nblocks, const double *__restrict__ strips,
                                                     double *__restrict__ result)
 {
-    diag_final_block(partial, nblocks, result);
+    diag_task<C>(k, blockIdx.x, partial, nblocks, strips, result);
 }
 
 // ---- initialisation and exchange ---------------------------------------------
 
-// D2Q9 equilibrium with Maxwellian raw moments, factorised per axis
-__device__ __forceinline__ double axis_factor(int e, double u)
-{
-    const double c2 = 1.0 / 3.0;
-    return e == 0 ? 1.0 - c2 - u * u : 0.5 * (c2 + u * u + e * u);
-}
-
-__constant__ int c_ex9[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
-__constant__ int c_ey9[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
 __constant__ double c_w9[9] = {4.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 36, 1.0 / 36, 1.0 / 36, 1.0 / 36};
 __constant__ double c_w5[5] = {1.0 / 3, 1.0 / 6, 1.0 / 6, 1.0 / 6, 1.0 / 6};
 
-__device__ __forceinline__ void eq_d2q5(double s, double ux, double uy, double o[5])
-{
-    const double c2 = 1.0 / 3.0;
-    o[0] = s * (1.0 - 2.0 * c2 - ux * ux - uy * uy);
-    o[1] = 0.5 * s * (c2 + ux * ux + ux);
-    o[3] = 0.5 * s * (c2 + ux * ux - ux);
-    o[2] = 0.5 * s * (c2 + uy * uy + uy);
-    o[4] = 0.5 * s * (c2 + uy * uy - uy);
-}
-
+// Equilibria of given fields: the D2Q9 one with Maxwellian raw moments is a
+// product of a factor per axis, 2/3 - u^2 for e = 0 and (1/3 + u^2 +- u) / 2 for
+// e = +-1; the D2Q5 ones use the same factors.  Bound by the FP64 pipe (35
+// instructions and 19 conversions per node; the term by term form had over
+// 100), behind the copy of its fields from the host.
 template <typename S>
 __global__ void k_init_fields(HostParams h, const double *__restrict__ fields, S *__restrict__ dst, int row0,
                               int row1)
 {
+    using C = typename std::conditional<std::is_same<S, double>::value, double, float>::type;
+    const C scale = (C)h.scale;
+    const double w0 = -4.0 / 9 * h.rho0, w1 = -1.0 / 9 * h.rho0, w5 = -1.0 / 36 * h.rho0, t0 = -1.0 / 3 * h.T0,
+                 t1 = -1.0 / 6 * h.T0;
     const long long nrow = row1 - row0;
     const long long n = nrow * h.nr;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
         const int i = row0 + (int)(t / h.nr), j = (int)(t % h.nr);
         const double rho = fields[t], ux = fields[n + t], uy = fields[2 * n + t];
         const double ut = fields[3 * n + t], T = fields[4 * n + t];
+        const double hx = 0.5 * ux, hy = 0.5 * uy;
+        const double x0 = __fma_rn(-ux, ux, 2.0 / 3), mx = __fma_rn(hx, ux, 1.0 / 6), xp = mx + hx, xm = mx - hx;
+        const double y0 = __fma_rn(-uy, uy, 2.0 / 3), my = __fma_rn(hy, uy, 1.0 / 6), yp = my + hy, ym = my - hy;
+        const double r0 = rho * x0, rp = rho * xp, rm = rho * xm, c0 = __fma_rn(-uy, uy, x0 - 1.0 / 3), ps = rho * ut;
+        const double v[NQ] = {__fma_rn(r0, y0, w0), __fma_rn(rp, y0, w1), __fma_rn(r0, yp, w1), __fma_rn(rm, y0, w1),
+                              __fma_rn(r0, ym, w1), __fma_rn(rp, yp, w5), __fma_rn(rm, yp, w5), __fma_rn(rm, ym, w5),
+                              __fma_rn(rp, ym, w5), ps * c0, ps * xp, ps * yp, ps * xm, ps * ym,
+                              __fma_rn(T, c0, t0), __fma_rn(T, xp, t1), __fma_rn(T, yp, t1), __fma_rn(T, xm, t1),
+                              __fma_rn(T, ym, t1)};
         S *p = dst + (long long)i * h.pitch + j;
-        for (int a = 0; a < 9; ++a) {
-            const double fe = rho * axis_factor(c_ex9[a], ux) * axis_factor(c_ey9[a], uy);
-            Cvt<S, typename std::conditional<std::is_same<S, double>::value, double, float>::type>::st(
-                p + a * h.plane, (fe - c_w9[a] * h.rho0) * h.scale);
-        }
-        double ge[5], he[5];
-        eq_d2q5(rho * ut, ux, uy, ge);
-        eq_d2q5(T, ux, uy, he);
-        for (int a = 0; a < 5; ++a) {
-            Cvt<S, typename std::conditional<std::is_same<S, double>::value, double, float>::type>::st(
-                p + (G0 + a) * h.plane, ge[a] * h.scale);
-            Cvt<S, typename std::conditional<std::is_same<S, double>::value, double, float>::type>::st(
-                p + (H0 + a) * h.plane, (he[a] - c_w5[a] * h.T0) * h.scale);
-        }
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) Cvt<S, C>::st(p + q * h.plane, Scaled<S>::value ? (C)v[q] * scale : (C)v[q]);
     }
 }
 
@@ -1491,8 +1338,6 @@ __global__ void k_import(HostParams h, const double *__restrict__ in, S *__restr
         }
     }
 }
-
-int nwindows(int nr) { return (nr + OUT_COLS - 1) / OUT_COLS; }
 
 // ---- batched step: many lattices, one launch per step ----------------------------
 
@@ -1665,7 +1510,7 @@ __global__ void __maxnreg__(LB_STEP3_MAXREG) k_batch3(const BatchDesc *__restric
         rs.status = bd->status;
         rs.start();
         march3<S, R, false, true>(k, (const S *)bd->buf[cur], (S *)bd->buf[cur ^ 1], w * 64, s, e,
-                                               salt_of(bd->step0 + t), rs);
+                                           salt_of(bd->step0 + t), rs);
     }
 }
 
@@ -1784,21 +1629,21 @@ __global__ void __maxnreg__(LB_STEP3_MAXREG) k_batch3p(const BatchDesc *__restri
     }
 }
 
-// Diagnostics of every lattice of a batch in three launches instead of three
-// per lattice: the blocks of all the lattices' diagnostics grids in one grid,
-// then one final-reduction block and one wall-flux block per lattice.  Each
-// lattice keeps the grid and summation order of its own diagnostics, so the
-// results are bitwise those of lb_diagnostics.
+// Diagnostics of every lattice of a batch in two launches: the blocks of all the
+// lattices' diagnostics grids in one grid, then the last reductions of every
+// lattice.  Each lattice keeps the grid and summation order of its own
+// diagnostics, so the results are bitwise those of lb_diagnostics.
 struct BatchDiag {
     double *partial;         // the lattice's block partial sums
-    int gx, gy, seg, nwin;   // its diagnostics grid (diag_t)
+    int gx, gy, seg, pad;    // its diagnostics grid (diag_grid)
 };
 
 template <typename S>
-__global__ void __launch_bounds__(128) k_batch_diag(const BatchDesc *__restrict__ d,
+__global__ void __launch_bounds__(kBlockThreads) k_batch_diag(const BatchDesc *__restrict__ d,
                                                     const BatchDiag *__restrict__ dd, const int *__restrict__ prefix,
                                                     int n, unsigned long long t)
 {
+    extern __shared__ __align__(128) unsigned char smem[];
     // the lattice of this block: the last m with prefix[m] <= blockIdx.x
     const int blk = blockIdx.x;
     int lo = 0, hi = n;
@@ -1811,29 +1656,22 @@ __global__ void __launch_bounds__(128) k_batch_diag(const BatchDesc *__restrict_
     const BatchDiag &g = dd[lo];
     const int local = blk - prefix[lo];
     const int cur = (bd.parity0 + (int)(t & 1ULL)) & 1;  // the lattice's current buffer after t batch steps
-    diag_block<S, float>(bd.k, (const S *)bd.buf[cur], g.partial, (double *)bd.buf[cur ^ 1], g.seg, g.nwin,
-                         local % g.gx, local / g.gx, g.gx);
+    diag_block<S, float>(bd.k, (const S *)bd.buf[cur], g.partial, (double *)bd.buf[cur ^ 1], g.seg, local % g.gx,
+                         local / g.gx, g.gx, reinterpret_cast<float *>(smem));
 }
 
 // out: one slot of slot_doubles per lattice, its NSUM sums and, 128 bytes in,
 // the lattice's status word
 __global__ void __launch_bounds__(256) k_batch_diag_final(const BatchDesc *__restrict__ d,
                                                           const BatchDiag *__restrict__ dd, double *__restrict__ out,
-                                                          int slot_doubles)
+                                                          int slot_doubles, unsigned long long t)
 {
-    const int m = blockIdx.x;
-    double *res = out + (size_t)m * slot_doubles;
-    diag_final_block(dd[m].partial, dd[m].gx * dd[m].gy, res);
-    if (threadIdx.x == 0) *reinterpret_cast<int *>(res + 16) = *d[m].status;
-}
-
-__global__ void __launch_bounds__(256) k_batch_wall(const BatchDesc *__restrict__ d, double *__restrict__ out,
-                                                    int slot_doubles, unsigned long long t)
-{
-    const int m = blockIdx.x;
+    const int m = blockIdx.x / kDiagTasks, task = blockIdx.x % kDiagTasks;
     const BatchDesc &bd = d[m];
     const int cur = (bd.parity0 + (int)(t & 1ULL)) & 1;
-    wall_block<float>(bd.k, (const double *)bd.buf[cur ^ 1], out + (size_t)m * slot_doubles);
+    double *res = out + (size_t)m * slot_doubles;
+    diag_task<float>(bd.k, task, dd[m].partial, dd[m].gx * dd[m].gy, (const double *)bd.buf[cur ^ 1], res);
+    if (task == 0 && threadIdx.x == 0) *reinterpret_cast<int *>(res + 16) = *bd.status;
 }
 
 // T steps of every lattice of a batch on tiles or strips (lb_tile.cuh): the
@@ -2000,7 +1838,7 @@ cudaError_t step_t(const HostParams &h, const Launch &l, const void *src, void *
     } else {
         const int nwin2 = nwindows2(h.nr);
         dim3 grid((nwin2 + wpb - 1) / wpb, (h.nz + seg - 1) / seg);
-        if (tmap && l.use_tma == 2) {
+        if (tmap && (l.use_tma == 2)) {
             const size_t sm = ring_smem_bytes<S>(wpb);
             static std::atomic<unsigned long long> attr_set{0};
             cudaError_t e = smem_limit_once(k_step3_tma<S>, (int)ring_smem_bytes<S>(8), attr_set);
@@ -2008,8 +1846,9 @@ cudaError_t step_t(const HostParams &h, const Launch &l, const void *src, void *
             cudaLaunchConfig_t cfg = {};
             cudaLaunchAttribute pdl[1];
             pdl_config(cfg, pdl, grid, dim3(32 * wpb), sm, s);
-            e = cudaLaunchKernelEx(&cfg, k_step3_tma<S>, k, *(const CUtensorMap *)tmap, (const S *)src, (S *)dst,
-                                   seg, nwin2, step_salt(step), status, (int)(step & 1ULL));
+            e = cudaLaunchKernelEx(&cfg, k_step3_tma<S>, k,
+                                   *(const CUtensorMap *)tmap, (const S *)src, (S *)dst, seg, nwin2, step_salt(step),
+                                   status, (int)(step & 1ULL));
             if (e != cudaSuccess) return e;
         } else if (tmap && l.use_tma) {
             const size_t sm = tma_smem_bytes<S>(wpb);
@@ -2035,31 +1874,23 @@ cudaError_t step_t(const HostParams &h, const Launch &l, const void *src, void *
 }
 
 template <typename S, typename C>
-cudaError_t fields_t(const HostParams &h, const Launch &l, const void *src, double *out, int row0, int row1,
-                     cudaStream_t s)
+cudaError_t fields_t(const HostParams &h, const void *src, double *out, int row0, int row1, cudaStream_t s)
 {
-    const KP<C> k = make_kp<C>(h);
-    const int nwin = nwindows(h.nr);
-    const int wpb = l.warps_per_block;
-    dim3 grid((nwin + wpb - 1) / wpb, (row1 - row0 + kFieldRows - 1) / kFieldRows);
-    k_fields<S, C><<<grid, 32 * wpb, 0, s>>>(k, (const S *)src, out, row0, row1, nwin);
+    const int nbx = (h.nr + kBlockCols - 1) / kBlockCols;
+    const long long blocks = (long long)nbx * ((row1 - row0 + kBlockChunk - 1) / kBlockChunk);
+    if (blocks > INT_MAX) return cudaErrorInvalidValue;
+    k_fields<S, C><<<(unsigned)blocks, kBlockThreads, kBlockSmem<C>, s>>>(make_kp<C>(h), (const S *)src, out, row0, row1, nbx);
     return cudaGetLastError();
 }
 
+// The two launches of a diagnostics: strips holds 4 (nr + nz) doubles.
 template <typename S, typename C>
-cudaError_t diag_t(const HostParams &h, const Launch &l, const void *src, double *partial, double *tfield,
+cudaError_t diag_t(const HostParams &h, const DiagGrid &g, const void *src, double *partial, double *strips,
                    double *result, cudaStream_t s)
 {
     const KP<C> k = make_kp<C>(h);
-    const int nwin = nwindows(h.nr);
-    const int wpb = 4;
-    const int seg = l.seg_rows;
-    dim3 grid((nwin + wpb - 1) / wpb, (h.nz + seg - 1) / seg);
-    const int nb = grid.x * grid.y;
-    if (nb > MAX_DIAG_BLOCKS) return cudaErrorInvalidValue;
-    k_diag<S, C><<<grid, 32 * wpb, 0, s>>>(k, (const S *)src, partial, tfield, seg, nwin);
-    k_diag_final<<<1, 256, 0, s>>>(partial, nb, result);
-    k_wall<C><<<1, 256, 0, s>>>(k, tfield, result);
+    k_diag<S, C><<<g.gx * g.gy, kBlockThreads, kBlockSmem<C>, s>>>(k, (const S *)src, partial, strips, g.seg, g.gx);
+    k_diag_final<C><<<kDiagTasks, 256, 0, s>>>(k, partial, g.gx * g.gy, strips, result);
     return cudaGetLastError();
 }
 
@@ -2125,6 +1956,7 @@ cudaError_t launch_step(const HostParams &p, const Launch &l, const void *src, v
 {
     DISPATCH(p, (step_t<S, C>(p, l, src, dst, step, tmap, status, s)));
 }
+
 
 int ring_cols(int storage) { return 64 + 2 * (16 / (int)storage_bytes(storage)); }
 
@@ -2357,16 +2189,35 @@ cudaError_t launch_psi(const double *ux, double *psi, double *rowmax, int nrows,
     return cudaGetLastError();
 }
 
-cudaError_t launch_fields(const HostParams &p, const Launch &l, const void *src, double *out, int row0, int row1,
-                          cudaStream_t s)
+cudaError_t launch_fields(const HostParams &p, const void *src, double *out, int row0, int row1, cudaStream_t s)
 {
-    DISPATCH(p, (fields_t<S, C>(p, l, src, out, row0, row1, s)));
+    DISPATCH(p, (fields_t<S, C>(p, src, out, row0, row1, s)));
 }
 
-cudaError_t launch_diag(const HostParams &p, const Launch &l, const void *src, double *partial, double *tfield,
-                        double *result, cudaStream_t s)
+// Blocks of 32 rows, fewer while there would be less than two blocks per SM,
+// more where there would be more than max_blocks.
+DiagGrid diag_grid(const HostParams &p, int max_blocks)
 {
-    DISPATCH(p, (diag_t<S, C>(p, l, src, partial, tfield, result, s)));
+    DiagGrid g;
+    g.gx = (p.nr + kBlockCols - 1) / kBlockCols;
+    // 32 rows, fewer on a lattice that would leave SMs idle; not on the longest,
+    // whose sums have to fit beside their strips (lb_diagnostics_static)
+    g.seg = 32;
+    while (g.seg > 4 && p.nr + p.nz <= 16384 && (long long)g.gx * ((p.nz + g.seg - 1) / g.seg) < 304) g.seg /= 2;
+    if ((long long)g.gx * ((p.nz + g.seg - 1) / g.seg) > max_blocks) {
+        const int segs = std::max(1, max_blocks / g.gx);
+        g.seg = (p.nz + segs - 1) / segs;
+    }
+    g.gy = (p.nz + g.seg - 1) / g.seg;
+    return g;
+}
+
+cudaError_t launch_diag(const HostParams &p, const void *src, double *partial, double *strips, double *result,
+                        cudaStream_t s)
+{
+    const DiagGrid g = diag_grid(p, MAX_DIAG_BLOCKS);
+    if ((long long)g.gx * g.gy > MAX_DIAG_BLOCKS) return cudaErrorInvalidValue;
+    DISPATCH(p, (diag_t<S, C>(p, g, src, partial, strips, result, s)));
 }
 
 #define DISPATCH_S(p, CALL)                                         \
@@ -2654,17 +2505,18 @@ cudaError_t launch_batch(int storage, int row_fetch, const void *desc, const int
 
 size_t batch_diag_bytes() { return sizeof(BatchDiag); }
 
-int batch_fill_diag(const HostParams &h, const Launch &l, double *partial, void *out)
+int batch_fill_diag(const HostParams &h, double *partial, void *out)
 {
+    const DiagGrid grid = diag_grid(h, MAX_DIAG_BLOCKS);
     BatchDiag g;
+    std::memset(&g, 0, sizeof g);
     g.partial = partial;
-    g.nwin = nwindows(h.nr);
-    g.seg = l.seg_rows;
-    g.gx = (g.nwin + 3) / 4;
-    g.gy = (h.nz + g.seg - 1) / g.seg;
+    g.seg = grid.seg;
+    g.gx = grid.gx;
+    g.gy = grid.gy;
     std::memcpy(out, &g, sizeof g);
-    const int nb = g.gx * g.gy;
-    return nb <= MAX_DIAG_BLOCKS ? nb : -1;
+    const long long nb = (long long)g.gx * g.gy;
+    return nb <= MAX_DIAG_BLOCKS ? (int)nb : -1;
 }
 
 cudaError_t launch_batch_diag(int storage, const void *desc, const void *bdiag, const int *bprefix, int n, int total,
@@ -2673,13 +2525,12 @@ cudaError_t launch_batch_diag(int storage, const void *desc, const void *bdiag, 
     const BatchDesc *d = (const BatchDesc *)desc;
     const BatchDiag *dd = (const BatchDiag *)bdiag;
     switch (storage) {
-        case ST_FP32: k_batch_diag<float><<<total, 128, 0, s>>>(d, dd, bprefix, n, t); break;
-        case ST_FP16: k_batch_diag<__half><<<total, 128, 0, s>>>(d, dd, bprefix, n, t); break;
-        case ST_BF16: k_batch_diag<__nv_bfloat16><<<total, 128, 0, s>>>(d, dd, bprefix, n, t); break;
+        case ST_FP32: k_batch_diag<float><<<total, kBlockThreads, kBlockSmem<float>, s>>>(d, dd, bprefix, n, t); break;
+        case ST_FP16: k_batch_diag<__half><<<total, kBlockThreads, kBlockSmem<float>, s>>>(d, dd, bprefix, n, t); break;
+        case ST_BF16: k_batch_diag<__nv_bfloat16><<<total, kBlockThreads, kBlockSmem<float>, s>>>(d, dd, bprefix, n, t); break;
         default: return cudaErrorInvalidValue;
     }
-    k_batch_diag_final<<<n, 256, 0, s>>>(d, dd, out, slot_doubles);
-    k_batch_wall<<<n, 256, 0, s>>>(d, out, slot_doubles, t);
+    k_batch_diag_final<<<n * kDiagTasks, 256, 0, s>>>(d, dd, out, slot_doubles, t);
     return cudaGetLastError();
 }
 
@@ -2716,20 +2567,6 @@ cudaError_t scratch_address(double **out)
     return cudaSuccess;
 }
 
-template <typename S, typename C>
-cudaError_t diag_static_t(const HostParams &h, const Launch &l, const void *src, double *scratch, int nb,
-                          cudaStream_t s)
-{
-    const KP<C> k = make_kp<C>(h);
-    const int nwin = nwindows(h.nr);
-    dim3 grid((nwin + 3) / 4, (h.nz + l.seg_rows - 1) / l.seg_rows);
-    double *result = scratch, *partial = scratch + 16, *strips = scratch + 16 + (size_t)nb * NSUM;
-    k_diag_strip<S, C><<<grid, 128, 0, s>>>(k, (const S *)src, partial, strips, l.seg_rows, nwin);
-    k_diag_final<<<1, 256, 0, s>>>(partial, nb, result);
-    k_wall_strip<C><<<1, 256, 0, s>>>(k, strips, result);
-    return cudaGetLastError();
-}
-
 }  // namespace
 }  // namespace lbk
 
@@ -2754,20 +2591,16 @@ extern "C" lb_status lb_diagnostics_static(const lb_grid_desc *desc, const lb_pa
         set_global_error("lb_diagnostics_static: dev_state must be 256-byte aligned");
         return LB_ERR_ARG;
     }
-    // launch shape within the static scratch: at most kScratchMaxBlocks blocks
-    Launch l = default_launch(h);
-    if (l.seg_rows < 32) l.seg_rows = 32;  // as lb_diagnostics
-    const long long bx = (nwindows(h.nr) + 3) / 4;
-    long long segs = (h.nz + l.seg_rows - 1) / l.seg_rows;
-    if (bx * segs > kScratchMaxBlocks) {
-        segs = kScratchMaxBlocks / bx;
-        if (segs < 1) segs = 1;
-        l.seg_rows = (int)((h.nz + segs - 1) / segs);
-        segs = (h.nz + l.seg_rows - 1) / l.seg_rows;
-    }
-    const long long nb = bx * segs;
-    const size_t need = 16 + (size_t)nb * NSUM + 4 * ((size_t)h.nr + (size_t)h.nz);
-    if (nb > kScratchMaxBlocks || need > kScratchDoubles) {
+    // The size is limited by blocks of 120 columns and 32 rows, taller ones
+    // where these were more than kScratchMaxBlocks; the diagnostics grid then
+    // has no more blocks than that.
+    const long long bx = (h.nr + 119) / 120, by = (h.nz + 31) / 32;
+    const long long cap = std::max(1LL, std::min(by, kScratchMaxBlocks / bx)), seg = (h.nz + cap - 1) / cap;
+    const long long most = bx * ((h.nz + seg - 1) / seg);
+    const size_t need = 16 + (size_t)most * NSUM + 4 * ((size_t)h.nr + (size_t)h.nz);
+    const DiagGrid g = diag_grid(h, bx * by > kScratchMaxBlocks ? (int)most : kScratchMaxBlocks);
+    const long long nb = (long long)g.gx * g.gy;
+    if (most > kScratchMaxBlocks || need > kScratchDoubles) {
         char msg[200];
         snprintf(msg, sizeof(msg),
                  "lb_diagnostics_static: a %d x %d lattice needs %zu scratch doubles, the static array holds %zu "
@@ -2779,13 +2612,15 @@ extern "C" lb_status lb_diagnostics_static(const lb_grid_desc *desc, const lb_pa
     double *scratch = nullptr;
     cudaError_t e = scratch_address(&scratch);
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, need * sizeof(double), st);
+    const size_t used = 16 + (size_t)nb * NSUM + 4 * ((size_t)h.nr + (size_t)h.nz);
+    if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, used * sizeof(double), st);
     if (e == cudaSuccess) {
+        double *partial = scratch + 16, *strips = partial + (size_t)nb * NSUM;
         switch (h.storage) {
-            case ST_FP64: e = diag_static_t<double, double>(h, l, dev_state, scratch, (int)nb, st); break;
-            case ST_FP32: e = diag_static_t<float, float>(h, l, dev_state, scratch, (int)nb, st); break;
-            case ST_BF16: e = diag_static_t<__nv_bfloat16, float>(h, l, dev_state, scratch, (int)nb, st); break;
-            default: e = diag_static_t<__half, float>(h, l, dev_state, scratch, (int)nb, st); break;
+            case ST_FP64: e = diag_t<double, double>(h, g, dev_state, partial, strips, scratch, st); break;
+            case ST_FP32: e = diag_t<float, float>(h, g, dev_state, partial, strips, scratch, st); break;
+            case ST_BF16: e = diag_t<__nv_bfloat16, float>(h, g, dev_state, partial, strips, scratch, st); break;
+            default: e = diag_t<__half, float>(h, g, dev_state, partial, strips, scratch, st); break;
         }
     }
     double res[NSUM];
