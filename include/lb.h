@@ -192,8 +192,10 @@ LB_EXPORT lb_status lb_init_fields(lb_ctx *ctx, const double *host_fields);
 
 /* Advance nsteps >= 0 time steps, asynchronously on the context's stream.
  * Under the automatic launch (lb_set_launch) FP32 and 16-bit lattices take up
- * to four steps per kernel launch; the results are bitwise those of nsteps
- * calls of one step. */
+ * to four steps per kernel launch (one where max(nu, alpha) > 3 (r_inner +
+ * 1/2) in axisymmetric geometry: their explicit geometric sources let
+ * round-off grow for some steps, and their arithmetic keeps one fixed order);
+ * the results are bitwise those of nsteps calls of one step. */
 LB_EXPORT lb_status lb_step(lb_ctx *ctx, int32_t nsteps);
 
 /* Pre-collision fields of the current state (the rho, u, u_theta, T the

@@ -466,7 +466,7 @@ lb_status lb_step(lb_ctx *ctx, int32_t nsteps)
         ctx->tmap_ready = true;
     }
     const int32_t fused =
-        ctx->hp.storage != LB_FP64 && ctx->launch_auto ? nsteps : 0;
+        ctx->hp.storage != LB_FP64 && ctx->launch_auto && !lbk::step_is_pinned(ctx->hp) ? nsteps : 0;
     if (fused > 0) {
         // Passes of up to T steps.  Their number is made even or odd as the
         // number of steps is, so that the current buffer alternates with the
@@ -752,11 +752,12 @@ struct lb_batch {
     lbk::TileLaunch tiles;
     int *d_tprefix;
     std::vector<int> htprefix;
+    int pinned;  // lattices with a pinned order of operations (one launch per step)
 
     // the launch settings a batch starts with select the automatic launch
     bool automatic() const
     {
-        if (seg_rows != 4 || wpb != 1 || row_fetch != 3) return false;
+        if (pinned == (int)ctxs.size() || seg_rows != 4 || wpb != 1 || row_fetch != 3) return false;
         for (int s : seg_of)
             if (s) return false;
         return true;
@@ -814,8 +815,10 @@ static lb_status batch_upload(lb_batch *b)
     b->hdesc.assign((size_t)n * db, 0);
     b->hprefix.assign((size_t)n + 1, 0);
     b->htprefix.assign((size_t)n + 1, 0);
+    b->pinned = 0;
     for (int m = 0; m < n; ++m) {
         lb_ctx *c = b->ctxs[m];
+        b->pinned += lbk::step_is_pinned(c->hp);
         const int seg = b->seg_of[m] ? b->seg_of[m] : b->seg_rows;
         cudaError_t e = lbk::batch_fill_desc(c->hp, c->dist[0], c->dist[1], b->step0[m], b->parity0[m], seg,
                                              b->tiles, c->status, b->hdesc.data() + (size_t)m * db);
@@ -986,6 +989,9 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
                         b->total, resident, kMaxPersistItems);
         e = lbk::launch_batch_persist(b->storage, b->d_desc, b->d_prefix, (int)b->ctxs.size(), b->total, b->wpb,
                                       b->counter, nsteps, b->d_flags, b->stream);
+        for (int32_t j = 0; j < nsteps && b->pinned && e == cudaSuccess; ++j)
+            e = lbk::launch_batch_pinned(b->storage, b->d_desc, b->d_prefix, (int)b->ctxs.size(), b->total, b->d_ctl,
+                                         b->wpb, b->counter + (unsigned long long)j, 0, b->stream);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "persistent batch launch");
         b->counter += (unsigned long long)nsteps;
         for (size_t m = 0; m < b->ctxs.size(); ++m) {
@@ -1000,9 +1006,18 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
     int32_t left = nsteps;
     unsigned long long t = b->counter;  // batch step of the next launch
     const int n = (int)b->ctxs.size();
-    auto step_once = [&](unsigned long long at, int from_counter) {
+    auto step_others = [&](unsigned long long at, int from_counter) {
         return lbk::launch_batch(b->storage, b->row_fetch, b->d_desc, b->d_prefix, n, b->total, b->d_ctl, b->wpb,
                                  b->blocks, at, from_counter, b->stream);
+    };
+    auto step_pinned = [&](unsigned long long at, int from_counter) {
+        return lbk::launch_batch_pinned(b->storage, b->d_desc, b->d_prefix, n, b->total, b->d_ctl, b->wpb, at,
+                                        from_counter, b->stream);
+    };
+    auto step_once = [&](unsigned long long at, int from_counter) {
+        cudaError_t e = b->pinned < n ? step_others(at, from_counter) : cudaSuccess;
+        if (e == cudaSuccess && b->pinned) e = step_pinned(at, from_counter);
+        return e;
     };
     if (b->automatic() && nsteps > 0) {
         // passes of several steps, as many as make the buffers alternate with the step count (lb_step)
@@ -1013,13 +1028,17 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
             const unsigned long long flip = (b->counter + (unsigned long long)p) & 1ULL;
             cudaError_t e;
             if (T == 1 && b->tiles.strip && flip == (t & 1ULL))  // large lattices' single step: one warp per work item
-                e = step_once(t, 0);
+                e = step_others(t, 0);
             else
                 e = lbk::launch_batch_tiles(b->storage, b->tiles, T, b->d_desc, b->d_tprefix, n, b->htprefix.back(), t,
                                             (int)flip, b->stream);
             if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch launch");
             t += (unsigned long long)T;
             left -= T;
+        }
+        for (int32_t j = 0; j < nsteps && b->pinned; ++j) {
+            cudaError_t e = step_pinned(b->counter + (unsigned long long)j, 0);
+            if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch launch");
         }
     }
     const bool use_graph = left > 0 && b->graph_steps > 1 && b->stream != nullptr && left >= b->graph_steps;

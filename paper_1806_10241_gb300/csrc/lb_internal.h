@@ -68,6 +68,9 @@ cudaError_t launch_step(const HostParams &p, const Launch &l, const void *src, v
 // for the row rings, 64 for the tiles.
 int ring_cols(int storage);
 cudaError_t make_tensor_map(const HostParams &p, void *buf, int box_cols, void *map_out);
+// Whether the lattice's node update keeps its pinned order of operations (then
+// it takes one launch per step).
+bool step_is_pinned(const HostParams &h);
 // T time steps on tiles in shared memory (FP32 / 16-bit storage), from the
 // buffer of tmap (64-column boxes) to dst.
 struct TileLaunch {
@@ -120,7 +123,8 @@ int batch_items(const HostParams &h, int seg_rows);
 // lattice's device status word (bounded-wait timeouts).
 cudaError_t batch_fill_desc(const HostParams &h, void *buf0, void *buf1, unsigned long long step0, int parity0,
                             int seg_rows, const TileLaunch &l, int *status, void *out);
-// The automatic pass of a batch, a lattice's tiles under it, and one pass of T
+// The automatic pass of a batch, a lattice's tiles under it (none for a pinned
+// one), and one pass of T
 // <= l.T steps from batch step t on (total: the tiles of all lattices, prefix
 // their prefix sums; flip: 0 when the state of step t lies in the buffers that
 // were current when the batch was made).
@@ -140,6 +144,10 @@ cudaError_t batch_prepare(int storage);
 cudaError_t launch_batch(int storage, int row_fetch, const void *desc, const int *prefix, int n, int total,
                          void *ctl, int wpb, int blocks, unsigned long long t0, int from_counter,
                          cudaStream_t s);
+// The same step of the batch's pinned lattices (step_is_pinned), which
+// launch_batch and launch_batch_persist leave out.
+cudaError_t launch_batch_pinned(int storage, const void *desc, const int *prefix, int n, int total, void *ctl, int wpb,
+                                unsigned long long t0, int from_counter, cudaStream_t s);
 // nsteps batch steps t0 .. t0 + nsteps - 1 in one cooperative launch (every
 // work item resident; items wait only for their neighbours' progress in
 // done[total], cleared here first).

@@ -18,6 +18,7 @@
 #include <cstdio>
 #include <cstring>
 #include <type_traits>
+#include <vector>
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -106,7 +107,15 @@ template <typename C> struct KP {
     NodeConst<typename std::conditional<std::is_same<C, float>::value, float2, C>::type> pc;
     // Nusselt and equivalent-conductivity scales per side (diagnostics)
     double nu_scale[4], keq_scale[4];
+    int pinned;           // pinned_order
 };
+
+// A lattice whose geometric sources amplify disturbances (see update_pinned):
+// a diffusivity above 3 radii of its innermost node.
+bool pinned_order(const HostParams &h)
+{
+    return h.storage != ST_FP64 && !h.planar && std::max(h.nu, h.alpha) > 3.0 * (h.r0 + 0.5);
+}
 
 template <typename C> KP<C> make_kp(const HostParams &h)
 {
@@ -132,6 +141,7 @@ template <typename C> KP<C> make_kp(const HostParams &h)
     k.planar = h.planar;
     k.sign_lit = h.sign_literal;
     k.explicit_src = h.explicit_sources;
+    k.pinned = pinned_order(h);
     for (int s = 0; s < 5; ++s) {
         k.flow[s] = h.flow[s];
         k.swirl[s] = h.swirl[s];
@@ -883,7 +893,7 @@ __host__ __device__ size_t ring_smem_bytes(int wpb)
     return (size_t)wpb * (kRingStages<S> * TmaGeom<S>::stage_bytes + 128);
 }
 
-template <typename S>
+template <typename S, bool kPinned>
 __global__ void __maxnreg__(LB_STEP3_MAXREG)
     k_step3_tma(KP<float> k, const __grid_constant__ CUtensorMap map, const S *__restrict__ src,
                 S *__restrict__ dst, int seg_rows, int nwin2, uint32_t salt, int *status, int rev)
@@ -916,7 +926,7 @@ __global__ void __maxnreg__(LB_STEP3_MAXREG)
     // resident now, and touch no distribution before the previous step is done
     grid_dependency_trigger_and_wait();
     rs.start();
-    march3<S, R, kStepSplit<S>, true>(k, src, dst, warp * 64, s, e, salt, rs);
+    march3<S, R, kStepSplit<S>, true, kPinned>(k, src, dst, warp * 64, s, e, salt, rs);
 }
 
 // Stream function of the meridian flow (Sec. 3.6): dPsi/dy = -y u_x with
@@ -1405,6 +1415,7 @@ __global__ void __maxnreg__(LB_STEP2_MAXREG) k_batch(const BatchDesc *__restrict
     for (int item = blockIdx.x * wpb + wib; item < total; item += gridDim.x * wpb) {
         const int lo = batch_instance(prefix, n, item, lane);
         const BatchDesc *bd = d + lo;
+        if (bd->k.pinned) continue;  // a launch of its own takes the pinned lattices
         __syncwarp();
         {
             const uint32_t *s = reinterpret_cast<const uint32_t *>(&bd->k);
@@ -1453,7 +1464,7 @@ __host__ __device__ size_t batch3_smem_bytes(int wpb)
     return (size_t)wpb * (batch3_ring_bytes<S, R>() + sizeof(KP<float>));
 }
 
-template <typename S, int R>
+template <typename S, int R, bool kPinned = false>
 __global__ void __maxnreg__(LB_STEP3_MAXREG) k_batch3(const BatchDesc *__restrict__ d, const int *__restrict__ prefix,
                                                       int n, int total, const BatchCtl *ctl, unsigned long long t0,
                                                       int from_counter, int rev)
@@ -1474,6 +1485,7 @@ __global__ void __maxnreg__(LB_STEP3_MAXREG) k_batch3(const BatchDesc *__restric
     if (item0 < total) {
         const int lo = batch_instance(prefix, n, item, lane);
         const BatchDesc *bd = d + lo;
+        if ((bd->k.pinned != 0) != kPinned) return;  // a launch of its own takes the pinned lattices
         {
             const uint32_t *s = reinterpret_cast<const uint32_t *>(&bd->k);
             uint32_t *o = reinterpret_cast<uint32_t *>(&skp[wib]);
@@ -1509,7 +1521,7 @@ __global__ void __maxnreg__(LB_STEP3_MAXREG) k_batch3(const BatchDesc *__restric
         rs.lane = lane;
         rs.status = bd->status;
         rs.start();
-        march3<S, R, false, true>(k, (const S *)bd->buf[cur], (S *)bd->buf[cur ^ 1], w * 64, s, e,
+        march3<S, R, false, true, kPinned>(k, (const S *)bd->buf[cur], (S *)bd->buf[cur ^ 1], w * 64, s, e,
                                            salt_of(bd->step0 + t), rs);
     }
 }
@@ -1552,6 +1564,7 @@ __global__ void __maxnreg__(LB_STEP3_MAXREG) k_batch3p(const BatchDesc *__restri
     if (item >= total) return;
     const int lo = batch_instance(prefix, n, item, lane);
     const BatchDesc *bd = d + lo;
+    if (bd->k.pinned) return;  // launches of their own take the pinned lattices
     {
         const uint32_t *src = reinterpret_cast<const uint32_t *>(&bd->k);
         uint32_t *o = reinterpret_cast<uint32_t *>(&skp[wib]);
@@ -1838,15 +1851,16 @@ cudaError_t step_t(const HostParams &h, const Launch &l, const void *src, void *
     } else {
         const int nwin2 = nwindows2(h.nr);
         dim3 grid((nwin2 + wpb - 1) / wpb, (h.nz + seg - 1) / seg);
-        if (tmap && (l.use_tma == 2)) {
+        if (tmap && (l.use_tma == 2 || k.pinned)) {
             const size_t sm = ring_smem_bytes<S>(wpb);
-            static std::atomic<unsigned long long> attr_set{0};
-            cudaError_t e = smem_limit_once(k_step3_tma<S>, (int)ring_smem_bytes<S>(8), attr_set);
+            static std::atomic<unsigned long long> attr_set{0}, pinned_set{0};
+            cudaError_t e = smem_limit_once(k_step3_tma<S, false>, (int)ring_smem_bytes<S>(8), attr_set);
+            if (e == cudaSuccess) e = smem_limit_once(k_step3_tma<S, true>, (int)ring_smem_bytes<S>(8), pinned_set);
             if (e != cudaSuccess) return e;
             cudaLaunchConfig_t cfg = {};
             cudaLaunchAttribute pdl[1];
             pdl_config(cfg, pdl, grid, dim3(32 * wpb), sm, s);
-            e = cudaLaunchKernelEx(&cfg, k_step3_tma<S>, k,
+            e = cudaLaunchKernelEx(&cfg, k.pinned ? k_step3_tma<S, true> : k_step3_tma<S, false>, k,
                                    *(const CUtensorMap *)tmap, (const S *)src, (S *)dst, seg, nwin2, step_salt(step),
                                    status, (int)(step & 1ULL));
             if (e != cudaSuccess) return e;
@@ -1957,6 +1971,7 @@ cudaError_t launch_step(const HostParams &p, const Launch &l, const void *src, v
     DISPATCH(p, (step_t<S, C>(p, l, src, dst, step, tmap, status, s)));
 }
 
+bool step_is_pinned(const HostParams &h) { return pinned_order(h); }
 
 int ring_cols(int storage) { return 64 + 2 * (16 / (int)storage_bytes(storage)); }
 
@@ -2163,7 +2178,14 @@ TileLaunch tile_plan(const HostParams &h, int T)
     return l;
 }
 
-TileLaunch tile_plan_batch(const HostParams *const *h, int n) { return plan_tiles(Lattices{h, n, h[0]->storage}, 0); }
+TileLaunch tile_plan_batch(const HostParams *const *h, int n)
+{
+    std::vector<const HostParams *> tiled;  // pinned lattices take launches of their own
+    for (int m = 0; m < n; ++m)
+        if (!pinned_order(*h[m])) tiled.push_back(h[m]);
+    if (tiled.empty()) tiled.assign(h, h + n);
+    return plan_tiles(Lattices{tiled.data(), (int)tiled.size(), h[0]->storage}, 0);
+}
 
 cudaError_t launch_tile(const HostParams &p, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
                         int *status, int rev, cudaStream_t s)
@@ -2269,6 +2291,7 @@ static TileShape batch_tiles(const HostParams &h, const TileLaunch &l)
 
 int batch_tile_count(const HostParams &h, const TileLaunch &l)
 {
+    if (pinned_order(h)) return 0;
     const TileShape sh = batch_tiles(h, l);
     return sh.nw * tiles_along(h, sh);
 }
@@ -2399,6 +2422,33 @@ cudaError_t batch_resident_warps(int storage, int row_fetch, int wpb, int *out)
     }
     *out = sms * per * wpb;
     return e;
+}
+
+// One step of the pinned lattices of a batch, whatever its row fetch.
+template <typename S>
+static cudaError_t batch_pinned_t(const BatchDesc *d, const int *prefix, int n, int total, const BatchCtl *ctl, int wpb,
+                                  unsigned long long t0, int from_counter, cudaStream_t s)
+{
+    static std::atomic<unsigned long long> attr_set{0};
+    cudaError_t e = smem_limit_once(k_batch3<S, 4, true>, (int)batch3_smem_bytes<S, 4>(8), attr_set);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute pdl[1];
+    pdl_config(cfg, pdl, dim3((total + wpb - 1) / wpb), dim3(32 * wpb), batch3_smem_bytes<S, 4>(wpb), s);
+    return cudaLaunchKernelEx(&cfg, k_batch3<S, 4, true>, d, prefix, n, total, ctl, t0, from_counter, (int)(t0 & 1ULL));
+}
+
+cudaError_t launch_batch_pinned(int storage, const void *desc, const int *prefix, int n, int total, void *ctl, int wpb,
+                                unsigned long long t0, int from_counter, cudaStream_t s)
+{
+    const BatchDesc *d = (const BatchDesc *)desc;
+    const BatchCtl *c = (const BatchCtl *)ctl;
+    switch (storage) {
+        case ST_FP32: return batch_pinned_t<float>(d, prefix, n, total, c, wpb, t0, from_counter, s);
+        case ST_FP16: return batch_pinned_t<__half>(d, prefix, n, total, c, wpb, t0, from_counter, s);
+        case ST_BF16: return batch_pinned_t<__nv_bfloat16>(d, prefix, n, total, c, wpb, t0, from_counter, s);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_batch_persist(int storage, const void *desc, const int *prefix, int n, int total, int wpb,

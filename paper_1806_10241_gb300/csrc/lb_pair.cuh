@@ -49,6 +49,10 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
     r.v = __ffma2_rn(a.v, b.v, c.v);
     return r;
 }
+// a - b, with the packed subtraction written out: as fma2(b, -1, a) the tiles
+// took 2-3 % longer per step (100 x 100 FP32 2.51 against 2.46 us, 256 x 512
+// 5.25 against 5.13 us).  The assembler may fuse a product b into it, which
+// saves that product's rounding.
 __device__ __forceinline__ F2 operator-(F2 a, F2 b)
 {
     F2 r;
@@ -404,6 +408,193 @@ __device__ __forceinline__ void update_node2(const NC &c, bool explicit_src, con
     }
 }
 
+// The update with its terms and their order as they were before update_node2
+// took its present form, for the lattices that KP::pinned marks.  The geometric
+// source of T near the axis, alpha d_y T / y with an explicit central
+// difference, lets a disturbance grow for some tens of steps before it decays
+// once alpha / y is above about 4 at the innermost node (10^2-fold at alpha =
+// 4): there another order of rounding shows in the results (10^-4 in FP32, all
+// digits in 16 bits), so these lattices keep the bits that they always had, and
+// one launch per step.
+// P2 are pairs whose difference is fma2(b, -1, a), which fuses no product.
+struct P2 {
+    F2 f;
+    __device__ __forceinline__ operator F2() const { return f; }
+};
+__device__ __forceinline__ P2 fma2(P2 a, P2 b, P2 c) { return P2{fma2(a.f, b.f, c.f)}; }
+__device__ __forceinline__ P2 operator+(P2 a, P2 b) { return P2{a.f + b.f}; }
+__device__ __forceinline__ P2 operator*(P2 a, P2 b) { return P2{a.f * b.f}; }
+__device__ __forceinline__ P2 operator-(P2 a, P2 b) { return P2{fma2(b.f, sp(-1.0f), a.f)}; }
+
+__device__ __forceinline__ void update_pinned(const KP<float> &k, F2 iy_, const F2 f_[9], const F2 g_[5],
+                                              const F2 h_[5], F2 dxuy_, F2 dyux_, F2 dyuy_, F2 dyut_, F2 dyT_,
+                                              float osc, NodeOut2 &o)
+{
+    const P2 iy{iy_}, dxuy{dxuy_}, dyux{dyux_}, dyuy{dyuy_}, dyut{dyut_}, dyT{dyT_};
+    P2 fv[9], gv[5], hv[5];
+    for (int q = 0; q < 9; ++q) fv[q] = P2{f_[q]};
+    for (int q = 0; q < 5; ++q) {
+        gv[q] = P2{g_[q]};
+        hv[q] = P2{h_[q]};
+    }
+    const auto sp = [](float x) { return P2{mk2(x, x)}; };
+    const P2 OS = sp(osc);
+    // output moments, Eq. 18, 35, 47 (deviation form)
+    const P2 a57 = fv[5] - fv[7], a86 = fv[8] - fv[6];
+    const P2 s57 = fv[5] + fv[7], s68 = fv[6] + fv[8];
+    const P2 s13 = fv[1] + fv[3], s24 = fv[2] + fv[4];
+    const P2 s5678 = s57 + s68;
+    const P2 rdo = (fv[0] + s13) + (s24 + s5678);
+    const P2 jxo = (fv[1] - fv[3]) + (a57 + a86);
+    const P2 jyo = (fv[2] - fv[4]) + (a57 - a86);
+    const P2 pso = (gv[0] + gv[1]) + (gv[2] + gv[3]) + gv[4];
+    const P2 tdo = (hv[0] + hv[1]) + (hv[2] + hv[3]) + hv[4];
+
+    // sources at the pre-collision state, two sweeps (see update_node)
+    const bool geo = !k.planar;
+    const P2 gy = geo ? iy : sp(0.0f);
+    const P2 ngy = gy * sp(-1.0f);
+    const P2 nuiy = gy * sp(k.nu);
+    const P2 Gx = (dxuy + dyux) * nuiy;
+    const P2 Gy = dyuy * (nuiy + nuiy);
+    const P2 Gw = dyut * nuiy;
+    const P2 Gt = dyT * (gy * sp(k.alpha));
+    const P2 iy2nu = nuiy * gy;
+    const P2 m2iy2nu = iy2nu * sp(-2.0f);
+    const P2 Fbx = sp(k.bfx);
+    const P2 Fb = sp(k.rho0 * k.gbeta), rho0 = sp(k.rho0), T0 = sp(k.T0), half = sp(0.5f);
+    P2 rd = rdo, jx = jxo, jy = jyo, ps = pso, td = tdo;
+    P2 MA = sp(0.0f), Fx = sp(0.0f), Fy = sp(0.0f), Sps = sp(0.0f), Sph = sp(0.0f);
+    const int sweeps = k.explicit_src ? 1 : 2;
+    for (int sw = 0; sw < sweeps; ++sw) {
+        const P2 r = rho0 + rd, ir = P2{rcp2(r)};
+        const P2 uyyn = (jy * ir) * ngy;  // -u_y / y
+        const P2 igy = ir * gy;
+        const P2 FAx = fma2(jx, uyyn, r * Gx);
+        const P2 FAy = fma2(jy, m2iy2nu, fma2(r, Gy, ((ps - jy) * (ps + jy)) * igy));
+        Sps = fma2(ps, fma2(uyyn, sp(2.0f), iy2nu * sp(-1.0f)), r * Gw);
+        Sph = fma2(uyyn, T0 + td, Gt);
+        Fx = fma2(Fb, td, FAx + Fbx);
+        Fy = FAy;
+        jx = fma2(Fx, half, jxo);
+        jy = fma2(Fy, half, jyo);
+        ps = fma2(Sps, half, pso);
+        td = fma2(Sph, half, tdo);
+        MA = (k.explicit_src ? jyo : jy) * ngy;
+        rd = fma2(MA, half, rdo);
+    }
+    const P2 r = rho0 + rd, ir = P2{rcp2(r)};
+    const P2 ux = jx * ir, uy = jy * ir;
+    const P2 phi = T0 + td;
+
+    // D2Q9 cascaded collision, Eq. 17
+    const P2 Dxx = s13 + s5678, Dyy = s24 + s5678;
+    const P2 Dxy = s57 - s68, Dxxy = a57 - a86, Dxyy = a57 + a86, Dxxyy = s5678;
+    const P2 k3 = sp(k.rho0 * (1.0f / 3.0f));
+    const P2 Kxx = k3 + Dxx, Kyy = k3 + Dyy;
+    const P2 ux2 = ux * ux, uy2 = uy * uy, uxy = ux * uy;
+    const P2 uu = ux2 + uy2, ud = ux2 - uy2;
+    const P2 p3 = (fma2(rd, sp(2.0f / 3.0f), r * uu) - (Dxx + Dyy)) * sp(k.om3 * (1.0f / 12.0f) * osc);
+    const P2 c4 = sp(k.om4 * 0.25f * osc);
+    const P2 p4 = ((r * ud) - (Dxx - Dyy)) * c4;
+    const P2 p5 = ((r * uxy) - Dxy) * c4;
+    const P2 q34p = fma2(p3, sp(3.0f), p4), q34m = fma2(p3, sp(3.0f), p4 * sp(-1.0f));
+    const P2 ch = sp(k.omhi * 0.25f * osc);
+    const P2 m2p5 = p5 * sp(-2.0f);
+    const P2 m2Dxy = Dxy * sp(-2.0f);
+    const P2 r2 = r + r;
+    // p6: (2 r ux^2 uy + Dxxy - 2 ux Dxy - uy Kxx) omhi/4 - uy (3 p3 + p4)/2 - 2 ux p5
+    P2 Z = fma2(r2 * ux2, uy, Dxxy);
+    Z = fma2(ux, m2Dxy, Z);
+    Z = fma2(uy, Kxx * sp(-1.0f), Z);
+    const P2 p6 = fma2(Z, ch, fma2(uy, q34p * sp(-0.5f), ux * m2p5));
+    P2 Y = fma2(r2 * ux, uy2, Dxyy);
+    Y = fma2(uy, m2Dxy, Y);
+    Y = fma2(ux, Kyy * sp(-1.0f), Y);
+    const P2 p7 = fma2(Y, ch, fma2(ux, q34m * sp(-0.5f), uy * m2p5));
+    // p8
+    P2 B = fma2(ux2, Kyy, Dxxyy);
+    B = fma2(uy2, Kxx, B);
+    B = fma2(uxy, Dxy * sp(4.0f), B);
+    B = fma2(ux, Dxyy * sp(-2.0f), B);
+    B = fma2(uy, Dxxy * sp(-2.0f), B);
+    const P2 W = fma2(rd, sp(1.0f / 9.0f), (r * sp(3.0f)) * (ux2 * uy2)) - B;
+    P2 p8 = W * ch;
+    p8 = fma2(p3, sp(-2.0f), p8);
+    p8 = fma2(uy2, q34p * sp(-0.5f), p8);
+    p8 = fma2(ux2, q34m * sp(-0.5f), p8);
+    p8 = fma2(uxy, p5 * sp(-4.0f), p8);
+    p8 = fma2(uy, p6 * sp(-2.0f), p8);
+    p8 = fma2(ux, p7 * sp(-2.0f), p8);
+    // source moments, Eq. 26
+    const P2 p0 = MA * sp((1.0f / 9.0f) * osc), p1 = Fx * sp((1.0f / 6.0f) * osc), p2 = Fy * sp((1.0f / 6.0f) * osc);
+    // back-transform, Eq. 27, grouped
+    {
+        const P2 A0 = p0 - p3;
+        const P2 E = A0 + p4, Fm = A0 - p4;
+        const P2 t78m = p7 - p8, t78p = p7 + p8, t68m = p6 - p8, t68p = p6 + p8;
+        o.v[0] = fma2(p3 - p8, sp(-4.0f), fma2(fv[0], OS, p0));
+        o.v[1] = fma2(fv[1], OS, E) + fma2(t78m, sp(2.0f), p1);
+        o.v[3] = fma2(fv[3], OS, E) - fma2(t78p, sp(2.0f), p1);
+        o.v[2] = fma2(fv[2], OS, Fm) + fma2(t68m, sp(2.0f), p2);
+        o.v[4] = fma2(fv[4], OS, Fm) - fma2(t68p, sp(2.0f), p2);
+        const P2 B0 = fma2(p3, sp(2.0f), p0 + p8);
+        const P2 u12 = p1 + p2, v12 = p1 - p2, s67 = p6 + p7, d67 = p6 - p7;
+        const P2 C5 = B0 + p5, C6 = B0 - p5;
+        const P2 us = u12 - s67, vd = v12 + d67;
+        o.v[5] = fma2(fv[5], OS, C5) + us;
+        o.v[7] = fma2(fv[7], OS, C5) - us;
+        o.v[6] = fma2(fv[6], OS, C6) - vd;
+        o.v[8] = fma2(fv[8], OS, C6) + vd;
+    }
+
+    // D2Q5 cascaded collisions, Eq. 34 / 49 (sign reading of the paper: -)
+    const P2 coefu = fma2(sp(k.sign_lit ? 1.0f : -1.0f), uu, sp(2.0f / 3.0f));
+    const P2 coefd = sp(k.sign_lit ? 1.0f : -1.0f) * ud;
+    {
+        const P2 kxn = gv[3] - gv[1], kyn = gv[4] - gv[2];  // -kappa'_x, -kappa'_y
+        const P2 kxx = gv[1] + gv[3], kyy = gv[2] + gv[4];
+        const P2 cg = sp(k.omg * 0.5f * osc);
+        const P2 q1 = fma2(ps, ux, kxn) * cg;
+        const P2 q2 = fma2(ps, uy, kyn) * cg;
+        const P2 m = fma2(ux, kxn, uy * kyn);  // -(ux kx + uy ky)
+        const P2 mm = fma2(ux, kxn, uy * (gv[2] - gv[4]));  // -(ux kx - uy ky)
+        const P2 X3 = fma2(ps, coefu, fma2(m, sp(-2.0f), (kxx + kyy) * sp(-1.0f)));
+        const P2 X4 = fma2(ps, coefd, fma2(mm, sp(-2.0f), (kxx - kyy) * sp(-1.0f)));
+        const P2 q3 = fma2(X3, ch, fma2(ux, q1, uy * q2));
+        const P2 q4 = fma2(X4, ch, fma2(ux, q1, uy * q2 * sp(-1.0f)));
+        const P2 q0 = Sps * sp(0.2f * osc);
+        const P2 Q = q0 + q3, Qp = Q + q4, Qm = Q - q4;
+        o.v[G0 + 0] = fma2(q3, sp(-4.0f), fma2(gv[0], OS, q0));
+        o.v[G0 + 1] = fma2(gv[1], OS, Qp) + q1;
+        o.v[G0 + 3] = fma2(gv[3], OS, Qp) - q1;
+        o.v[G0 + 2] = fma2(gv[2], OS, Qm) + q2;
+        o.v[G0 + 4] = fma2(gv[4], OS, Qm) - q2;
+    }
+    {
+        const P2 kxn = hv[3] - hv[1], kyn = hv[4] - hv[2];
+        const P2 Hxx = hv[1] + hv[3], Hyy = hv[2] + hv[4];
+        const P2 ct = sp(k.omh * 0.5f * osc);
+        const P2 r1 = fma2(phi, ux, kxn) * ct;
+        const P2 r2t = fma2(phi, uy, kyn) * ct;
+        const P2 m = fma2(ux, kxn, uy * kyn);
+        const P2 mm = fma2(ux, kxn, uy * (hv[2] - hv[4]));
+        // 2 c^2 phi - (kxx + kyy) with the rest parts written out: 2/3 td - (Hxx + Hyy)
+        const P2 X3 = fma2(sp(2.0f / 3.0f), td, fma2(phi, coefu - sp(2.0f / 3.0f), fma2(m, sp(-2.0f),
+                                                                                    (Hxx + Hyy) * sp(-1.0f))));
+        const P2 X4 = fma2(phi, coefd, fma2(mm, sp(-2.0f), (Hxx - Hyy) * sp(-1.0f)));
+        const P2 r3 = fma2(X3, ch, fma2(ux, r1, uy * r2t));
+        const P2 r4 = fma2(X4, ch, fma2(ux, r1, uy * r2t * sp(-1.0f)));
+        const P2 r0 = Sph * sp(0.2f * osc);
+        const P2 Q = r0 + r3, Qp = Q + r4, Qm = Q - r4;
+        o.v[H0 + 0] = fma2(r3, sp(-4.0f), fma2(hv[0], OS, r0));
+        o.v[H0 + 1] = fma2(hv[1], OS, Qp) + r1;
+        o.v[H0 + 3] = fma2(hv[3], OS, Qp) - r1;
+        o.v[H0 + 2] = fma2(hv[2], OS, Qm) + r2t;
+        o.v[H0 + 4] = fma2(hv[4], OS, Qm) - r2t;
+    }
+}
+
 // ---- the march on pairs ---------------------------------------------------------
 
 struct PM2 {
@@ -675,6 +866,18 @@ __device__ __forceinline__ void halo_fields(const KP<float> &k, const float h[NQ
     T = k.T0 + ((h[14] + h[15]) + (h[16] + h[17]) + h[18]);
 }
 
+// The same in the order of a pinned lattice (update_pinned).
+__device__ __forceinline__ void halo_fields_pinned(const KP<float> &k, const float h[NQ], float &ux, float &uy, float &ut,
+                                            float &T)
+{
+    const float rd = h[0] + h[1] + h[2] + h[3] + h[4] + h[5] + h[6] + h[7] + h[8];
+    const float ir = rcp1(k.rho0 + rd);
+    ux = (h[1] - h[3] + h[5] - h[6] - h[7] + h[8]) * ir;
+    uy = (h[2] - h[4] + h[5] + h[6] - h[7] - h[8]) * ir;
+    ut = (h[9] + h[10] + h[11] + h[12] + h[13]) * ir;
+    T = k.T0 + (h[14] + h[15] + h[16] + h[17] + h[18]);
+}
+
 // Own post-collision values that the wall and axis rules need (own(q): the
 // lane's pair on row i; own0(q): column 0 on row i; m8 / p7: f8 on row i - 1
 // and f7 on row i + 1 at column 0, for the axis mirror).  OwnGlobal reads them
@@ -931,7 +1134,7 @@ __device__ __forceinline__ void store_row(const KP<float> &k, S *__restrict__ ds
 // form, for a warp with no wall or axis column on a row with both neighbour
 // rows: the rules are left out at compile time instead of being branched or
 // predicated around.
-template <typename S, bool kBc, typename Own>
+template <typename S, bool kBc, bool kPinned = false, typename Own>
 __device__ __forceinline__ void row_tail(const KP<float> &k, const Own &own, S *__restrict__ dst,
                                          const Lane2 &L, int i, bool has_m_, bool has_p_, uint32_t salt, F2 fv[9],
                                          F2 gv[5], F2 hv5[5], const PM2 &pm_cur, const PM2 &pm_n, F2 uy_prev,
@@ -968,8 +1171,16 @@ __device__ __forceinline__ void row_tail(const KP<float> &k, const Own &own, S *
 
     // FP16 storage: the update returns the values already times the scale
     NodeOut2 o;
-    update_node2<Scaled<S>::value>(k.pc, k.explicit_src, geo_of(k.pc, L.iy), fv, gv, hv5, uy_xp - uy_xm, across(r.ux, l.ux), across(r.uy, l.uy),
-                                   across(r.ut, l.ut), across(r.T, l.T), o);
+    const F2 dxuy = uy_xp - uy_xm, dyux = across(r.ux, l.ux), dyuy = across(r.uy, l.uy), dyut = across(r.ut, l.ut),
+             dyT = across(r.T, l.T);
+    if constexpr (kPinned) {
+        const F2 hf = sp(0.5f);
+        update_pinned(k, L.iy, fv, gv, hv5, dxuy * hf, dyux * hf, dyuy * hf, dyut * hf, dyT * hf,
+                      Scaled<S>::value ? k.scale : 1.0f, o);
+    } else {
+        update_node2<Scaled<S>::value>(k.pc, k.explicit_src, geo_of(k.pc, L.iy), fv, gv, hv5, dxuy, dyux, dyuy, dyut,
+                                       dyT, o);
+    }
     if (L.outA) store_row<S>(k, dst, i, L.A, salt, o);
 }
 
@@ -1195,7 +1406,7 @@ template <typename S, int C> struct StageRd {
 // kSplit: interior rows of warps without wall or axis columns take the
 // interior form of row_tail.  kOwnStage: the wall and axis rules read the own
 // values from the ring (else from src).
-template <typename S, int R, bool kSplit, bool kOwnStage>
+template <typename S, int R, bool kSplit, bool kOwnStage, bool kPinned = false>
 __device__ __forceinline__ void march3(const KP<float> &k, const S *__restrict__ src, S *__restrict__ dst, int c0,
                                        int row_s, int row_e, uint32_t salt, RowRing<S, R> &rs)
 {
@@ -1227,7 +1438,8 @@ __device__ __forceinline__ void march3(const KP<float> &k, const S *__restrict__
             hv[q] = rd.col(q, hc);
         }
         pm_cur = moments2(v, k);
-        halo_fields(k, hv, pmh_ux, pmh_uy, pmh_ut, pmh_T);
+        if constexpr (kPinned) halo_fields_pinned(k, hv, pmh_ux, pmh_uy, pmh_ut, pmh_T);
+        else halo_fields(k, hv, pmh_ux, pmh_uy, pmh_ut, pmh_T);
     }
 
     for (int i = row_s; i < row_e; ++i) {
@@ -1275,7 +1487,8 @@ __device__ __forceinline__ void march3(const KP<float> &k, const S *__restrict__
                 hv[q] = rd.col(q, hc);
             }
             pm_n = moments2(v, k);
-            halo_fields(k, hv, nh_ux, nh_uy, nh_ut, nh_T);
+            if constexpr (kPinned) halo_fields_pinned(k, hv, nh_ux, nh_uy, nh_ut, nh_T);
+            else halo_fields(k, hv, nh_ux, nh_uy, nh_ut, nh_T);
             fv[3] = v[3];
             fv[6] = rd.left(6);
             fv[7] = rd.right(7);
@@ -1288,13 +1501,13 @@ __device__ __forceinline__ void march3(const KP<float> &k, const S *__restrict__
         }
 
         if (kSplit && has_m && has_p && !L.edge_warp)
-            row_tail<S, false>(k, own, dst, L, i, has_m, has_p, salt, fv, gv, hv5, pm_cur, pm_n, uy_prev, pmh_ux,
+            row_tail<S, false, kPinned>(k, own, dst, L, i, has_m, has_p, salt, fv, gv, hv5, pm_cur, pm_n, uy_prev, pmh_ux,
                                pmh_uy, pmh_ut, pmh_T);
         else if (kOwnStage)
-            row_tail<S, true>(k, own, dst, L, i, has_m, has_p, salt, fv, gv, hv5, pm_cur, pm_n, uy_prev, pmh_ux,
+            row_tail<S, true, kPinned>(k, own, dst, L, i, has_m, has_p, salt, fv, gv, hv5, pm_cur, pm_n, uy_prev, pmh_ux,
                               pmh_uy, pmh_ut, pmh_T);
         else
-            row_tail<S, true>(k, OwnGlobal<S>{src, &k, i, L.Ac}, dst, L, i, has_m, has_p, salt, fv, gv, hv5, pm_cur,
+            row_tail<S, true, kPinned>(k, OwnGlobal<S>{src, &k, i, L.Ac}, dst, L, i, has_m, has_p, salt, fv, gv, hv5, pm_cur,
                               pm_n, uy_prev, pmh_ux, pmh_uy, pmh_ut, pmh_T);
 
         uy_prev = pm_cur.uy;
