@@ -2106,6 +2106,7 @@ cudaError_t tile_t(const HostParams &h, const TileLaunch &l, const void *tmap, v
     const TileShape sh = tile_shape(h, l.T, l.rows);
     const long long blocks = (long long)sh.nw * tiles_along(h, sh);
     const size_t smem = tile_smem_bytes<S>(tile_slots(l.strip, l.T, l.rows, l.warps));
+    const bool two = l.strip && l.parts == 2 && blocks >= 2;
     for (int p = 0; p < l.parts; ++p) {
         const int q = rev ? l.parts - 1 - p : p;  // the parts in the order of their blocks
         const int first = (int)(blocks * q / l.parts), count = (int)(blocks * (q + 1) / l.parts) - first;
@@ -2114,7 +2115,7 @@ cudaError_t tile_t(const HostParams &h, const TileLaunch &l, const void *tmap, v
         cudaLaunchAttribute pdl[1];
         pdl_config(cfg, pdl, dim3(count), dim3(32 * l.warps), smem, s);
         e = cudaLaunchKernelEx(&cfg, l.strip ? k_tiles<S, true> : k_tiles<S, false>, k, *(const CUtensorMap *)tmap,
-                               (S *)dst, sh, l.T, first, step, status, rev);
+                               (S *)dst, sh, l.T, first, step, status, rev, two ? 1 + p : 0);
         if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
@@ -2164,7 +2165,7 @@ TileLaunch plan_tiles(const Lattices &ls, int T)
 //   FP32: 12.8 against 13.6 us; 1024 x 1024: 23.6 against 22.9).
 // - FP32 strips of more than 64 rows go out as two launches, half of the strips
 //   each, so that a large lattice keeps one launch per step, which callers that
-//   time single kernels count on; 1024 x 2048: 44.8 us per step, 40.8 as one
+//   time single kernels count on; 1024 x 2048: 41.6 us per step, 40.8 as one
 //   launch of two waves.
 TileLaunch tile_plan(const HostParams &h, int T)
 {

@@ -301,7 +301,7 @@ __device__ __forceinline__ void tile_steps(const KP<float> &k, const CUtensorMap
 template <typename S>
 __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMap *map, S *__restrict__ dst,
                                             const TileShape &sh, int T, int win, int tile, unsigned long long step,
-                                            int *status, unsigned char *smem)
+                                            int *status, unsigned char *smem, int part = 0)
 {
     constexpr int SB = TileGeom<S>::slot_bytes / (int)sizeof(S);
     const int warp = __shfl_sync(FULL, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31, W = blockDim.x >> 5;
@@ -319,7 +319,11 @@ __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMa
     }
     const Lane2 L = lane2(k, c0);
     __syncthreads();
-    grid_dependency_wait();
+    if (part != 2) grid_dependency_wait();
+    if (part == 1) {  // the second part relies on this wait (k_tiles)
+        __threadfence();
+        grid_dependency_trigger();
+    }
     auto fetch = [&](int m, int slot0) {  // the rows of tick m (warp 0)
         const int first = m * W, cnt = min(W, n - first);
         if (cnt <= 0) return;
@@ -391,14 +395,24 @@ __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMa
 
 // One lattice: block b of the launch takes tile `first + b` (rev: from the last
 // one back), windows running fastest.
+// A pass cut into two launches (part 1 and 2; 0: the only one) runs them side
+// by side, the second filling the SMs as the blocks of the first finish: it
+// reads the state of the pass before and writes other rows, so it does not
+// wait for the first at its start.  What it needs is that the pass before is
+// complete.  A block of part 1 allows the dependent launch only after it has
+// waited for that pass, and part 2 starts when every block of part 1 has done
+// so.  A block of part 2 waits for part 1 before it ends: a launch that waits
+// for part 2 then finds both complete.  (1024 x 2048 FP32: 45.4 us per step
+// with part 2 waiting at its start, 41.6 so.)
 template <typename S, bool kStrip>
 __global__ void __maxnreg__(kTileRegs<S>)
     k_tiles(const __grid_constant__ KP<float> k, const __grid_constant__ CUtensorMap map, S *__restrict__ dst,
-            const TileShape sh, int T, int first, unsigned long long step, int *status, int rev)
+            const TileShape sh, int T, int first, unsigned long long step, int *status, int rev, int part)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    grid_dependency_trigger();
+    if (sizeof(S) != 4 || part != 1) grid_dependency_trigger();
     const int b = first + (rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x);
-    if constexpr (kStrip) strip_steps<S>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem);
+    if constexpr (kStrip) strip_steps<S>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem, sizeof(S) == 4 ? part : 0);
     else tile_steps<S>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem);
+    if (sizeof(S) == 4 && part == 2) grid_dependency_wait();
 }
