@@ -97,6 +97,11 @@ template <typename S>
 __device__ __forceinline__ void tile_row(const KP<float> &k, const Lane2 &L, const S *b_m, const S *b_0, const S *b_p,
                                          bool has_m, bool has_p, NodeOut2 &o)
 {
+    // without a neighbour row the wall rules replace what it would have given:
+    // the row itself is read in its place, and no load is conditional (1024 x
+    // 2048 FP16: 46.2 -> 44.6 us per step)
+    b_m = has_m ? b_m : b_0;
+    b_p = has_p ? b_p : b_0;
     const float *f_m = fields_of(b_m), *f_0 = fields_of(b_0), *f_p = fields_of(b_p);
     constexpr int C = TileGeom<S>::cols;
     const int cA = 2 * L.lane;
@@ -104,16 +109,11 @@ __device__ __forceinline__ void tile_row(const KP<float> &k, const Lane2 &L, con
     F2 fv[9], gv[5], hv5[5];
     OwnStage<S, C> own{b_0, cA, is, 0.0f, 0.0f};
     StageRd<S, C> rd{b_m, cA, is};
-    if (has_m) {
-        fv[1] = rd.pair(1);
-        fv[5] = rd.left(5);
-        fv[8] = rd.right(8);
-        gv[1] = rd.pair(G0 + 1);
-        hv5[1] = rd.pair(H0 + 1);
-        if (L.edge_warp) own.m8v = rd.pair(8).v.x;
-    } else {
-        fv[1] = fv[5] = fv[8] = gv[1] = hv5[1] = sp(0.0f);
-    }
+    fv[1] = rd.pair(1);
+    fv[5] = rd.left(5);
+    fv[8] = rd.right(8);
+    gv[1] = rd.pair(G0 + 1);
+    hv5[1] = rd.pair(H0 + 1);
     rd.b = b_0;
     fv[0] = rd.pair(0);
     fv[2] = rd.left(2);
@@ -125,22 +125,21 @@ __device__ __forceinline__ void tile_row(const KP<float> &k, const Lane2 &L, con
     hv5[2] = rd.left(H0 + 2);
     hv5[4] = rd.right(H0 + 4);
     rd.b = b_p;
-    if (has_p) {
-        fv[3] = rd.pair(3);
-        fv[6] = rd.left(6);
-        fv[7] = rd.right(7);
-        gv[3] = rd.pair(G0 + 3);
-        hv5[3] = rd.pair(H0 + 3);
-        if (L.edge_warp) own.p7v = rd.pair(7).v.x;
-    } else {
-        fv[3] = fv[6] = fv[7] = gv[3] = hv5[3] = sp(0.0f);
+    fv[3] = rd.pair(3);
+    fv[6] = rd.left(6);
+    fv[7] = rd.right(7);
+    gv[3] = rd.pair(G0 + 3);
+    hv5[3] = rd.pair(H0 + 3);
+    if (L.edge_warp) {
+        own.m8v = StageRd<S, C>{b_m, cA, is}.pair(8).v.x;
+        own.p7v = rd.pair(7).v.x;
     }
     wall_rules(k, own, L, L.edge_warp, has_m, has_p, fv, gv, hv5);
-
     // central differences of the stored-state fields
     const Sides2 c{fpair(f_0, cA), fpair(f_0 + 64, cA), fpair(f_0 + 128, cA), fpair(f_0 + 192, cA)};
-    const F2 uy_xm = has_m ? fpair(f_m + 64, cA) : end_ghost_uy(k, L, 0, c.uy);
-    const F2 uy_xp = has_p ? fpair(f_p + 64, cA) : end_ghost_uy(k, L, 1, c.uy);
+    F2 uy_xm = fpair(f_m + 64, cA), uy_xp = fpair(f_p + 64, cA);
+    if (!has_m) uy_xm = end_ghost_uy(k, L, 0, c.uy);
+    if (!has_p) uy_xp = end_ghost_uy(k, L, 1, c.uy);
     Sides2 l{mk2(f_0[cA - 1], c.ux.v.x), mk2(f_0[63 + cA], c.uy.v.x), mk2(f_0[127 + cA], c.ut.v.x),
              mk2(f_0[191 + cA], c.T.v.x)};
     Sides2 r{mk2(c.ux.v.y, f_0[cA + 2]), mk2(c.uy.v.y, f_0[66 + cA]), mk2(c.ut.v.y, f_0[130 + cA]),
@@ -211,6 +210,16 @@ __device__ __forceinline__ int wrap_row(int row, int nz)
     return row < 0 ? row + nz : row;
 }
 
+// The rounding salts of the steps of a pass, behind the barriers (visible after
+// the next barrier of the block).
+template <typename S>
+__device__ __forceinline__ uint32_t *tile_salts(unsigned char *smem, int slots, int T, unsigned long long step)
+{
+    uint32_t *salts = reinterpret_cast<uint32_t *>(smem + (size_t)slots * TileGeom<S>::slot_bytes + 64);
+    if (PairIO<S>::rounds && (int)threadIdx.x < T) salts[threadIdx.x] = salt_of(step + threadIdx.x);
+    return salts;
+}
+
 // T steps on one tile by a block.  smem: (sh.rows + T - 1) slots and 128 bytes.
 template <typename S>
 __device__ __forceinline__ void tile_steps(const KP<float> &k, const CUtensorMap *map, S *__restrict__ dst,
@@ -228,6 +237,7 @@ __device__ __forceinline__ void tile_steps(const KP<float> &k, const CUtensorMap
     S *slots = reinterpret_cast<S *>(smem);
     const uint32_t bar = smem_u32(smem + (size_t)(sh.rows + T - 1) * TileGeom<S>::slot_bytes);
     const int groups = (n + W - 1) / W;
+    uint32_t *salts = tile_salts<S>(smem, sh.rows + T - 1, T, step);
     if (threadIdx.x == 0) {
         for (int g = 0; g < groups && g < 8; ++g)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8u * g) : "memory");
@@ -267,7 +277,7 @@ __device__ __forceinline__ void tile_steps(const KP<float> &k, const CUtensorMap
     for (int t = 0; t < T; ++t) {
         const bool last = t == T - 1;
         const int lo = bottom ? 0 : t + 1, hi = top ? n : n - (t + 1);
-        const uint32_t salt = PairIO<S>::rounds ? salt_of(step + (unsigned long long)t) : 0u;
+        const uint32_t salt = PairIO<S>::rounds ? salts[t] : 0u;
         for (int g = lo; g < hi; g += W) {
             const int r = g + warp;
             const bool active = r < hi;
@@ -295,9 +305,12 @@ __device__ __forceinline__ void tile_steps(const KP<float> &k, const CUtensorMap
 // the ring.  A slot is refilled one tick after its last read (2 W + 2 T slots
 // are exactly what is live: W rows on their way, W of this tick, and 2 T of
 // the lower neighbours' states).  1024 x 2048: FP32 52.0 us per step with one
-// step per launch, 40.8 us with strips of two steps; what bounds it is the
+// step per launch, 39.8 us with strips of two steps; what bounds it is the
 // latency of dependent instructions at 12 warps per SM (47 % issue), not
-// memory.  FP16 45.7 -> 45.6 us at that size, 26.1 -> 20.7 us at 641 x 1283.
+// memory.  FP16 45.7 -> 44.4 us at that size.
+// The position in the ring, the lattice row and the limits of the active rows
+// run along with t instead of being formed from it (10 % fewer instructions in
+// 16-bit storage, 2 % in FP32: 41.3 -> 39.8 us).
 template <typename S>
 __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMap *map, S *__restrict__ dst,
                                             const TileShape &sh, int T, int win, int tile, unsigned long long step,
@@ -312,6 +325,7 @@ __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMa
 
     S *slots = reinterpret_cast<S *>(smem);
     const uint32_t ring = smem_u32(smem), bar = ring + (uint32_t)(R * TileGeom<S>::slot_bytes);
+    uint32_t *salts = tile_salts<S>(smem, R, T, step);
     if (threadIdx.x == 0) {
         for (int g = 0; g < 2; ++g)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8u * g) : "memory");
@@ -346,7 +360,10 @@ __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMa
     const int out_lo = bottom ? 0 : sh.rm, out_hi = top ? n : n - sh.rm;  // T < rm: rows of the margin are not stored
     const int cA = 2 * lane;
     const int ticks = ((top ? n + T : n) + W - 1) / W;
+    // rows r of step t that the strip advances: from lo + t dlo on, below hi + t dhi, with r + t for r
+    const int lo = bottom ? 0 : 1, dlo = bottom ? 1 : 2, hi = top ? n : n - 1, dhi = top ? 1 : 0;
     int s0 = 0;  // slot of row m W, state 0
+    int row0 = wrap_row(r0 - 1 + warp, nz);  // lattice row of step 0 in this tick
     for (int m = 0; m < ticks; ++m) {
         bool ok = true;
         const int rf = m * W + warp;
@@ -366,18 +383,14 @@ __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMa
             s1 -= s1 >= R ? R : 0;
             fetch(m + 1, s1);
         }
-        for (int t = 0; t < T; ++t) {
-            const int r = m * W - 1 - t + warp;
-            const bool last = t == T - 1;
-            const int lo = bottom ? 0 : t + 1, hi = top ? n : n - (t + 1);
-            const bool active = r >= lo && r < hi;
-            const int row = k.xper ? wrap_row(r0 + r, nz) : r0 + r;
-            const uint32_t salt = PairIO<S>::rounds ? salt_of(step + (unsigned long long)t) : 0u;
-            int s = s0 + warp - 1 - 2 * t;  // slot of row r, state t
-            s += s < 0 ? R : 0;
-            s -= s >= R ? R : 0;
-            S *b_0 = slots + s * SB, *b_m = slots + (s == 0 ? R - 1 : s - 1) * SB,
-              *b_p = slots + (s == R - 1 ? 0 : s + 1) * SB;
+        int sl = sf == 0 ? R - 1 : sf - 1;  // slot of the warp's row in step t, state t
+        int row = row0;
+        for (int t = 0, lo_t = lo, hi_t = hi; t < T; ++t, lo_t += dlo, hi_t += dhi) {
+            const bool last = t == T - 1, active = rf - 1 >= lo_t && rf - 1 < hi_t;
+            const int r = rf - 1 - t;
+            S *b_0 = slots + sl * SB, *b_m = sl == 0 ? slots + (R - 1) * SB : b_0 - SB,
+              *b_p = sl == R - 1 ? slots : b_0 + SB;
+            const uint32_t salt = PairIO<S>::rounds ? salts[t] : 0u;
             NodeOut2 o;
             if (active) tile_row<S>(k, L, b_m, b_0, b_p, !bottom || r > 0, !top || r < n - 1, o);
             if (last) {
@@ -387,9 +400,14 @@ __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMa
                 if (active) tile_store<S>(k, b_m, cA, row, L.A, salt, o);
                 __syncthreads();
             }
+            row = row == 0 ? nz - 1 : row - 1;
+            sl -= 2;
+            sl += sl < 0 ? R : 0;
         }
         s0 += W;
         s0 -= s0 >= R ? R : 0;
+        row0 += W;
+        if (row0 >= nz) row0 = wrap_row(row0, nz);
     }
 }
 
