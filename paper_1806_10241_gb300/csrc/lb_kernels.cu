@@ -1724,7 +1724,7 @@ __global__ void __maxnreg__(kTileRegs<S>)
     const CUtensorMap *map = reinterpret_cast<const CUtensorMap *>(bd->map64[cur]);
     S *dst = (S *)bd->buf[cur ^ 1];
     if constexpr (kStrip)
-        strip_steps<S>(k, map, dst, sh, T, local % sh.nw, local / sh.nw, bd->step0 + t, bd->status, smem);
+        strip_steps<S, sizeof(S) != 4>(k, map, dst, sh, T, local % sh.nw, local / sh.nw, bd->step0 + t, bd->status, smem);
     else tile_steps<S>(k, map, dst, sh, T, local % sh.nw, local / sh.nw, bd->step0 + t, bd->status, smem);
 }
 

@@ -308,10 +308,12 @@ __device__ __forceinline__ void tile_steps(const KP<float> &k, const CUtensorMap
 // step per launch, 39.8 us with strips of two steps; what bounds it is the
 // latency of dependent instructions at 12 warps per SM (47 % issue), not
 // memory.  FP16 45.7 -> 44.4 us at that size.
-// The position in the ring, the lattice row and the limits of the active rows
-// run along with t instead of being formed from it (10 % fewer instructions in
-// 16-bit storage, 2 % in FP32: 41.3 -> 39.8 us).
-template <typename S>
+// kRunning: the position in the ring, the lattice row and the limits of the
+// active rows run along with t instead of being formed from it (10 % fewer
+// instructions in 16-bit storage, 2 % in FP32: 41.3 -> 39.8 us).  FP32 batches,
+// whose parameters are in shared memory, have no registers left for that (40
+// lattices of 64 to 128 columns: 18.7 us formed, 19.9 running).
+template <typename S, bool kRunning>
 __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMap *map, S *__restrict__ dst,
                                             const TileShape &sh, int T, int win, int tile, unsigned long long step,
                                             int *status, unsigned char *smem, int part = 0)
@@ -386,8 +388,16 @@ __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMa
         int sl = sf == 0 ? R - 1 : sf - 1;  // slot of the warp's row in step t, state t
         int row = row0;
         for (int t = 0, lo_t = lo, hi_t = hi; t < T; ++t, lo_t += dlo, hi_t += dhi) {
-            const bool last = t == T - 1, active = rf - 1 >= lo_t && rf - 1 < hi_t;
             const int r = rf - 1 - t;
+            if constexpr (!kRunning) {
+                lo_t = t + (bottom ? 0 : t + 1);
+                hi_t = t + (top ? n : n - (t + 1));
+                row = k.xper ? wrap_row(r0 + r, nz) : r0 + r;
+                sl = s0 + warp - 1 - 2 * t;
+                sl += sl < 0 ? R : 0;
+                sl -= sl >= R ? R : 0;
+            }
+            const bool last = t == T - 1, active = rf - 1 >= lo_t && rf - 1 < hi_t;
             S *b_0 = slots + sl * SB, *b_m = sl == 0 ? slots + (R - 1) * SB : b_0 - SB,
               *b_p = sl == R - 1 ? slots : b_0 + SB;
             const uint32_t salt = PairIO<S>::rounds ? salts[t] : 0u;
@@ -430,7 +440,7 @@ __global__ void __maxnreg__(kTileRegs<S>)
     extern __shared__ __align__(128) unsigned char smem[];
     if (sizeof(S) != 4 || part != 1) grid_dependency_trigger();
     const int b = first + (rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x);
-    if constexpr (kStrip) strip_steps<S>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem, sizeof(S) == 4 ? part : 0);
+    if constexpr (kStrip) strip_steps<S, true>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem, sizeof(S) == 4 ? part : 0);
     else tile_steps<S>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem);
     if (sizeof(S) == 4 && part == 2) grid_dependency_wait();
 }
