@@ -177,14 +177,12 @@ template <typename S>
 __device__ __forceinline__ void tile_store(const KP<float> &k, S *slot, int cA, int row, int A, uint32_t salt,
                                            const NodeOut2 &o)
 {
-    uint32_t w = 0;
-    if (PairIO<S>::rounds) w = pcg_hash(((uint32_t)row * (uint32_t)k.pitch + (uint32_t)A) ^ salt) | 1u;
+    RoundWords<S> w((uint32_t)row * (uint32_t)k.pitch + (uint32_t)A, salt);
     F2 v[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         v[q] = o.v[q];
-        if (PairIO<S>::rounds) w = xorshift32(w);
-        tile_put<S>(slot + q * TileGeom<S>::cols + cA, v[q], w, k.inv_scale);
+        tile_put<S>(slot + q * TileGeom<S>::cols + cA, v[q], PairIO<S>::rounds ? w.next() : 0u, k.inv_scale);
     }
     put_fields<S>(slot, cA, moments2(v, k));
 }
