@@ -1691,12 +1691,14 @@ __global__ void __launch_bounds__(256) k_batch_diag_final(const BatchDesc *__res
 // tiles of all lattices numbered by a prefix sum, one block each.  The pass
 // takes the batch from step t on; `flip` says which buffer holds that state.
 // Shared memory: the block's slots, then the lattice's parameters.  The plan is
-// tile_plan's for the tiles of all lattices together.  40 lattices of 64 to 128
-// columns in FP32: 19.0 us per step with the best one-step launch (segment plan
-// of one wave), 14.8 us on strips of two steps; 64 annuli of 32 to 512 rows and
-// columns in FP16: 146 us with 4-row segments, 107 us on strips of four steps.
-// Bound as the single lattice's strips, and by the columns that a window of a
-// narrow lattice leaves empty (a fifth of them in the first batch).
+// tile_plan's for the tiles of all lattices together.  With three
+// batches on streams of their own, per step: 40 lattices of 64 to 128 columns
+// in FP32 19.0 us with the best one-step launch (segment plan of one wave),
+// 15.0 us on strips of two steps; 64 annuli of 32 to 512 rows and columns in
+// FP16 156 us with 4-row segments, 94 us on strips of four steps (18.8 and 131
+// us for one batch alone, whose last wave nothing fills).  Bound as the single
+// lattice's strips, and by the columns that a window of a narrow lattice leaves
+// empty (a fifth of them in the first batch).
 template <typename S, bool kStrip>
 __global__ void __maxnreg__(kTileRegs<S>)
     k_batch_tiles(const BatchDesc *__restrict__ d, const int *__restrict__ prefix, int n, int total, int T,
@@ -2159,13 +2161,15 @@ TileLaunch plan_tiles(const Lattices &ls, int T)
 //   16-bit storage, whose margins are 4 columns for up to four steps, three
 //   (100 x 100: 2.89 us, two 2.99, four 3.03; 400 x 400: 5.90, 6.04, 5.98).
 // - Strips beyond (512 x 512 FP32: 7.5 us, tiles 8.0).  FP32: two steps (1024 x
-//   1024: 22.9 us; three 23.1, four 24.0).  16-bit: four (1024 x 1024: 24.7 us;
-//   three 25.4, two 24.9).  Six (eight) warps per block while the strips are
+//   2048: 39.4 us as one launch; three 45.2, four 42.5; 512 x 1024: 12.5, 12.7,
+//   12.8).  16-bit: four (1024 x 2048 FP16: 41.5 us; three 43.0, two 43.1; 512 x
+//   1024: 12.2, 12.8, 12.8).  Six (eight) warps per block while the strips are
 //   short, four and one more block per SM from 40 (60) rows on (512 x 1024
-//   FP32: 12.8 against 13.6 us; 1024 x 1024: 23.6 against 22.9).
+//   FP32: 12.5 against 13.1 us; 1024 x 2048: 42.4 against 39.4; two, three or
+//   five warps: 8-20 % slower).
 // - FP32 strips of more than 64 rows go out as two launches, half of the strips
 //   each, so that a large lattice keeps one launch per step, which callers that
-//   time single kernels count on; 1024 x 2048: 41.6 us per step, 40.8 as one
+//   time single kernels count on; 1024 x 2048: 39.9 us per step, 39.4 as one
 //   launch of two waves.
 TileLaunch tile_plan(const HostParams &h, int T)
 {

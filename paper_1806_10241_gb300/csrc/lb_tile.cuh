@@ -15,11 +15,12 @@
 // steps, and a row update needs less: the fields of the stored state are
 // written by the warp that has the new values in registers, and the radial
 // neighbours' fields are plain shared-memory reads instead of shuffles and
-// recomputed halo columns (735 warp instructions per 64 columns of result,
-// recomputed margins included, against 809 of the marching step).  Measured per step (one step per launch before, tiles now):
-// 100 x 100 FP32 7.1 -> 2.3 us, 40 x 400 FP32 7.4 -> 2.7 us, 256 x 512 FP32
-// 11.6 -> 5.0 us, 301 x 257 BF16 12.8 -> 4.9 us.  What bounds a small tile now
-// is the latency of a row update, about 1.3 us, and 2.5 us per launch.
+// recomputed halo columns (640 warp instructions per 64 columns of result in
+// FP32, recomputed margins included, against 809 of the marching step).
+// Measured per step (one step per launch before, tiles now): 100 x 100 FP32 7.1
+// -> 2.4 us, 40 x 400 FP32 7.4 -> 2.8 us, 256 x 512 FP32 11.6 -> 5.0 us, 301 x
+// 257 BF16 12.8 -> 4.7 us.  What bounds a small tile now is the latency of a
+// row update, about 1.3 us, and 2.5 us per launch.
 
 template <typename S> struct TileGeom {
     static constexpr int cols = 64;
