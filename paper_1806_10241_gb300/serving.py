@@ -2,7 +2,7 @@
 
 Requests (workloads.Request: arrival time + lattice) arrive as a stream.  The
 server keeps every admitted lattice resident on the device and advances all
-of them together with the batched step (one persistent launch per step,
+of them together with the batched step (all lattices in each launch,
 replayed from a CUDA graph).  Between rounds it
   * admits the requests that have arrived while their bytes fit the device
     memory budget (lb_required_bytes against free HBM less a reserve) and,
