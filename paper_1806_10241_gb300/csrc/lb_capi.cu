@@ -379,7 +379,7 @@ cudaError_t copy_planes(double *stage, double *host, size_t n, size_t N, bool to
 // rows through the staging area.  A large exchange overlaps the copies of a
 // chunk with the kernels of its neighbours: the copies go to a second stream,
 // ordered against the context's stream by events, in up to four parts of the
-// staging area (512 x 1024 FP32: fields in and out 480 us before, 300 us
+// staging area (512 x 1024 FP32: fields in and out 480 us before, 285 us
 // now; the copies alone take 233 us).  kernel(stage, r0, r1) queues the work of
 // a chunk on the context's stream.
 template <typename Kernel>
@@ -395,8 +395,10 @@ lb_status exchange(lb_ctx *ctx, double *host, bool to_device, const char *what, 
     const bool large = total >= kOverlapBytes && rows >= 2, overlap = large && copy_stream(ctx) == cudaSuccess;
     if (large && !overlap) cudaGetLastError();  // without a copy stream the chunks follow each other
     if (overlap) {
-        // chunks of about 2.5 MB, at most 32
-        const int count = (int)std::min<size_t>(32, std::max<size_t>(2, total / (5 << 19)));
+        // chunks of about 5 MB, at most 32: smaller ones leave the FP64 kernels'
+        // blocks too few for the SMs (512 x 1024 FP64 out: 570 us at 2.5 MB, 315 at
+        // 5, 335 at 10; FP32 in and out: 297, 282, 292)
+        const int count = (int)std::min<size_t>(32, std::max<size_t>(2, total / (5 << 20)));
         chunk = std::min((nz + count - 1) / count, rows / 2);
         parts = std::min(4, rows / chunk);
     }
