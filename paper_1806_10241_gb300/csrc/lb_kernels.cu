@@ -2227,10 +2227,14 @@ DiagGrid diag_grid(const HostParams &p, int max_blocks)
 {
     DiagGrid g;
     g.gx = (p.nr + kBlockCols - 1) / kBlockCols;
-    // 32 rows, fewer on a lattice that would leave SMs idle; not on the longest,
-    // whose sums have to fit beside their strips (lb_diagnostics_static)
+    // 32 rows, down to 8 on a lattice of less than two blocks per SM, 4 where
+    // even those are less than a quarter of the SMs (512 x 512 FP32: 8 rows 41 us,
+    // 4 rows 54, 16 rows 43; 41 x 41 FP64: 65, 48, 97; 64 annuli in one batch: 8
+    // rows 508 us, 4 rows 743, whose blocks form 6 rows of fields each); not on the
+    // longest, whose sums have to fit beside their strips (lb_diagnostics_static)
     g.seg = 32;
-    while (g.seg > 4 && p.nr + p.nz <= 16384 && (long long)g.gx * ((p.nz + g.seg - 1) / g.seg) < 304) g.seg /= 2;
+    auto blocks = [&]() { return (long long)g.gx * ((p.nz + g.seg - 1) / g.seg); };
+    while (p.nr + p.nz <= 16384 && ((g.seg > 8 && blocks() < 304) || (g.seg == 8 && blocks() < 38))) g.seg /= 2;
     if ((long long)g.gx * ((p.nz + g.seg - 1) / g.seg) > max_blocks) {
         const int segs = std::max(1, max_blocks / g.gx);
         g.seg = (p.nz + segs - 1) / segs;
