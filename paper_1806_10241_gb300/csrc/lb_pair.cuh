@@ -102,40 +102,27 @@ __device__ __forceinline__ F2 sel2(bool px, bool py, F2 a, F2 b)  // per compone
 // ---- pair loads / stores ------------------------------------------------------
 
 // Counter-based random words for stochastic rounding, one per pair store: the
-// PCG hash of Jarzynski & Olano (2020) of (node, step salt) seeds a sequence.
-// In FP16 storage it is linear congruential, with the 32-bit multiplier of
-// Steele & Vigna (2021): one operation a word, where xorshift32 (Marsaglia
-// 2003) takes six in a serial chain.  The conversion takes bits 0-12 and 16-28
-// of a word; over the 19 words of a node these are uniform, correlated in pairs
-// by at most 1.1 %, and sums over the planes have the variance of independent
-// draws to 0.5 %.  The errors are those of xorshift32: over 48 draws of a
-// cylinder, a crucible and an annulus, 1500 to 2000 steps against FP64, the RMS
-// error of Nu is 8.5e-4, 1.6e-3, 5.7e-4 (xorshift32 8.7e-4, 1.6e-3, 6.9e-4),
-// that of every field equal to 3 %.  1024 x 2048: 44.4 -> 41.4 us per step.
-// BF16 storage and the pinned lattices (update_pinned) keep xorshift32: there
-// two sequences differ by more than 1 % in the distributions of one step.
+// PCG hash of Jarzynski & Olano (2020) of (node, step salt) seeds a xorshift32
+// sequence (Marsaglia 2003).  The conversion takes bits 0-12 and 16-28 of a
+// word for the two FP16 elements, 0-15 and 16-31 for BF16.  A linear
+// congruential sequence from the same seed takes one operation a word instead
+// of six (1024 x 2048 FP16: 41.4 us per step, 44.4 with these), but its bits
+// 0-12 are a function of the low 13 bits of the seed alone, correlated over the
+// planes of a node, and results were further from FP64 by some per cent.
 __device__ __forceinline__ uint32_t pcg_hash(uint32_t v)
 {
     const uint32_t s = v * 747796405u + 2891336453u;
     const uint32_t w = ((s >> ((s >> 28u) + 4u)) ^ s) * 277803737u;
     return (w >> 22u) ^ w;
 }
-template <typename S, bool kPinned = false> struct RoundWords {
-    static constexpr bool congruential = std::is_same<S, __half>::value && !kPinned;
+struct RoundWords {
     uint32_t w;
-    __device__ __forceinline__ RoundWords(uint32_t node, uint32_t salt)
-        : w(pcg_hash(node ^ salt) | (congruential ? 0u : 1u))
-    {
-    }
+    __device__ __forceinline__ RoundWords(uint32_t node, uint32_t salt) : w(pcg_hash(node ^ salt) | 1u) {}
     __device__ __forceinline__ uint32_t next()
     {
-        if constexpr (congruential) {
-            w = w * 0x93D765DDu + 0x9E3779B9u;
-        } else {
-            w ^= w << 13;
-            w ^= w >> 17;
-            w ^= w << 5;
-        }
+        w ^= w << 13;
+        w ^= w >> 17;
+        w ^= w << 5;
         return w;
     }
 };
@@ -1137,12 +1124,12 @@ __device__ __forceinline__ void lateral_ghosts(const KP<float> &k, const Lane2 &
 }
 
 // The pair's post-collision values to row i of dst (whole rows of planes).
-template <typename S, bool kPinned = false>
+template <typename S>
 __device__ __forceinline__ void store_row(const KP<float> &k, S *__restrict__ dst, int i, int A, uint32_t salt,
                                           const NodeOut2 &o)
 {
     S *p = dst + (long long)i * k.pitch + A;
-    RoundWords<S, kPinned> w((uint32_t)i * (uint32_t)k.pitch + (uint32_t)A, salt);
+    RoundWords w((uint32_t)i * (uint32_t)k.pitch + (uint32_t)A, salt);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) PairIO<S>::st(p + q * k.plane, o.v[q], PairIO<S>::rounds ? w.next() : 0u);
 }
@@ -1200,7 +1187,7 @@ __device__ __forceinline__ void row_tail(const KP<float> &k, const Own &own, S *
         update_node2<Scaled<S>::value>(k.pc, k.explicit_src, geo_of(k.pc, L.iy), fv, gv, hv5, dxuy, dyux, dyuy, dyut,
                                        dyT, o);
     }
-    if (L.outA) store_row<S, kPinned>(k, dst, i, L.A, salt, o);
+    if (L.outA) store_row<S>(k, dst, i, L.A, salt, o);
 }
 
 template <typename S, typename RS>

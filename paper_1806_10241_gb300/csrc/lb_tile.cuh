@@ -178,7 +178,7 @@ template <typename S>
 __device__ __forceinline__ void tile_store(const KP<float> &k, S *slot, int cA, int row, int A, uint32_t salt,
                                            const NodeOut2 &o)
 {
-    RoundWords<S> w((uint32_t)row * (uint32_t)k.pitch + (uint32_t)A, salt);
+    RoundWords w((uint32_t)row * (uint32_t)k.pitch + (uint32_t)A, salt);
     F2 v[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
