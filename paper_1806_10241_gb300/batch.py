@@ -27,6 +27,9 @@ class Batch:
         nb = C.c_size_t()
         _abi.check(self.L.lb_batch_required_bytes(n, C.byref(nb)))
         self.buffer = torch.empty(int(nb.value), dtype=torch.uint8, device=self.solvers[0].device)
+        # the batch's launches read its descriptors and the lattices, also after the caller has let go of them
+        for t in [self.buffer] + [s.buffer for s in self.solvers]:
+            t.record_stream(self.stream)
         arr = (C.c_void_p * n)(*[s.ctx.value for s in self.solvers])
         h = C.c_void_p()
         _abi.check(self.L.lb_batch_create(arr, n, C.c_void_p(self.buffer.data_ptr()), self.buffer.numel(),

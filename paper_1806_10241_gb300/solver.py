@@ -56,6 +56,8 @@ class Solver:
             buffer = torch.empty(self.nbytes, dtype=torch.uint8, device=self.device)
         if buffer.numel() < self.nbytes:
             raise ValueError("buffer too small")
+        # work may still be queued when the caller lets go of the lattice: its memory is not reused before that is done
+        buffer.record_stream(self.stream)
         self.buffer = buffer
         desc = _abi.make_desc(params, storage)
         ctx = C.c_void_p()
