@@ -44,8 +44,9 @@ struct lb_ctx {
     bool tmap_ready;
     cudaStream_t copy_stream;         // copies of an exchange beside its kernels (made at the first large one)
     cudaEvent_t ev_copy[4], ev_kernel[4];
-    unsigned passes;  // launches of several steps so far (their block order alternates)
+    unsigned passes;  // passes of several steps so far
     int *status;  // device status word (bounded-wait timeouts of the step kernel)
+    unsigned *begun;  // device word: number of the last split pass that has begun
     char err[256];
 };
 
@@ -298,6 +299,7 @@ lb_status lb_create(const lb_grid_desc *desc, void *dev_buf, size_t bytes, void 
     c->partial = (double *)(c->buf + 2 * dist);
     c->result = (double *)(c->buf + 2 * dist + align256((size_t)lbk::MAX_DIAG_BLOCKS * lbk::NSUM * sizeof(double)));
     c->status = (int *)((char *)c->result + 128);
+    c->begun = (unsigned *)((char *)c->result + 192);
     h.ytab = (const float *)(c->buf + 2 * dist + scratch_bytes());
     c->tmap_ready = false;
     c->stream = (cudaStream_t)cuda_stream;
@@ -329,7 +331,7 @@ lb_status lb_set_params(lb_ctx *ctx, const lb_params *p)
         tab[h.pitch + j] = (float)(1.0 / y);
     }
     cudaError_t e = cudaMemsetAsync(ctx->dist[0], 0, ctx->dist_bytes, ctx->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->status, 0, sizeof(int), ctx->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->status, 0, 128, ctx->stream);  // and begun
     if (e == cudaSuccess)
         e = cudaMemcpyAsync((void *)h.ytab, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice,
                             ctx->stream);
@@ -479,17 +481,17 @@ lb_status lb_step(lb_ctx *ctx, int32_t nsteps)
         for (int32_t p = 0; p < m; ++p) {
             const int32_t T = fused / m + (p < fused % m ? 1 : 0);
             if (T != pass.T) pass = lbk::tile_plan(ctx->hp, T);
+            ctx->passes += 1;
             cudaError_t e;
             if (T == 1 && pass.strip)  // a large lattice's single step: one warp per work item
                 e = lbk::launch_step(ctx->hp, ctx->launch, ctx->dist[ctx->cur], ctx->dist[1 - ctx->cur],
                                      (unsigned long long)ctx->step, ctx->tmap[ctx->cur], ctx->status, ctx->stream);
             else
                 e = lbk::launch_tile(ctx->hp, pass, ctx->tmap64[ctx->cur], ctx->dist[1 - ctx->cur],
-                                     (unsigned long long)ctx->step, ctx->status, (int)(ctx->passes & 1), ctx->stream);
+                                     (unsigned long long)ctx->step, ctx->status, ctx->begun, ctx->passes, ctx->stream);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "step launch");
             ctx->cur ^= 1;
             ctx->step += T;
-            ctx->passes += 1;
         }
         return LB_OK;
     }

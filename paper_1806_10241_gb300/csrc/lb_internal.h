@@ -80,8 +80,10 @@ struct TileLaunch {
 };
 // The pass for a lattice: of T steps, or (T = 0) of as many as pay.
 TileLaunch tile_plan(const HostParams &p, int T);
+// pass: the number of the pass in the lattice's life, from 1 on; begun: the
+// lattice's device word for it (k_tiles).
 cudaError_t launch_tile(const HostParams &p, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
-                        int *status, int rev, cudaStream_t s);
+                        int *status, unsigned *begun, unsigned pass, cudaStream_t s);
 // Pre-collision fields of rows [row0, row1) into out[5][row1-row0][nr] (double).
 cudaError_t launch_fields(const HostParams &p, const void *src, double *out, int row0, int row1, cudaStream_t s);
 // Bounded-wait self-test: a warp polls an mbarrier nothing arrives at,

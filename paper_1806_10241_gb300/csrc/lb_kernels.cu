@@ -582,6 +582,23 @@ __device__ __forceinline__ void grid_dependency_trigger_and_wait()
     grid_dependency_wait();
 }
 
+// Waits on a flag in global memory: at most kFlagWaitLimit polls with a short
+// sleep between them (about a second).
+constexpr int kFlagWaitLimit = 1 << 20;
+
+template <typename I> __device__ __forceinline__ I ld_acquire_gpu(const I *p)
+{
+    static_assert(sizeof(I) == 4, "32-bit flags");
+    I v;
+    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+template <typename I> __device__ __forceinline__ void st_release_gpu(I *p, I v)
+{
+    static_assert(sizeof(I) == 4, "32-bit flags");
+    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 #include "lb_tile.cuh"
 
 // FP64 step (the reference path of the other storages).  The FP64 pipe bounds
@@ -1538,19 +1555,6 @@ __global__ void __maxnreg__(LB_STEP3_MAXREG) k_batch3(const BatchDesc *__restric
 // neighbour each with acquire loads, at most kFlagWaitLimit times with a
 // short sleep between polls (about a second), after which the lattice's
 // status word gets LB_ERR_TIMEOUT and the warp leaves.
-constexpr int kFlagWaitLimit = 1 << 20;
-
-__device__ __forceinline__ int ld_acquire_gpu(const int *p)
-{
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release_gpu(int *p, int v)
-{
-    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
 template <typename S, int R>
 __global__ void __maxnreg__(LB_STEP3_MAXREG) k_batch3p(const BatchDesc *__restrict__ d, const int *__restrict__ prefix,
                                                        int n, int total, unsigned long long t0, int nsteps, int *done)
@@ -2098,9 +2102,10 @@ int strip_rows(const Lattices &ls, int T, int warps, int waves, int sms)
 
 template <typename S>
 cudaError_t tile_t(const HostParams &h, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
-                   int *status, int rev, cudaStream_t s)
+                   int *status, unsigned *begun, unsigned pass, cudaStream_t s)
 {
     const KP<float> k = make_kp<float>(h);
+    const int rev = (int)(pass & 1u);  // the block order alternates from pass to pass
     static std::atomic<unsigned long long> tile_set{0}, strip_set{0};
     cudaError_t e = smem_limit_once(k_tiles<S, false>, kMaxSmem, tile_set);
     if (e == cudaSuccess) e = smem_limit_once(k_tiles<S, true>, kMaxSmem, strip_set);
@@ -2117,7 +2122,7 @@ cudaError_t tile_t(const HostParams &h, const TileLaunch &l, const void *tmap, v
         cudaLaunchAttribute pdl[1];
         pdl_config(cfg, pdl, dim3(count), dim3(32 * l.warps), smem, s);
         e = cudaLaunchKernelEx(&cfg, l.strip ? k_tiles<S, true> : k_tiles<S, false>, k, *(const CUtensorMap *)tmap,
-                               (S *)dst, sh, l.T, first, step, status, rev, two ? 1 + p : 0);
+                               (S *)dst, sh, l.T, first, step, status, rev, two ? 1 + p : 0, begun, pass);
         if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
@@ -2168,9 +2173,8 @@ TileLaunch plan_tiles(const Lattices &ls, int T)
 //   FP32: 12.5 against 13.1 us; 1024 x 2048: 42.4 against 39.4; two, three or
 //   five warps: 8-20 % slower).
 // - FP32 strips of more than 64 rows go out as two launches, half of the strips
-//   each, so that a large lattice keeps one launch per step, which callers that
-//   time single kernels count on; 1024 x 2048: 39.9 us per step, 39.4 as one
-//   launch of two waves.
+//   each, cut for two waves in all (k_tiles; 1024 x 2048: 40.6 us per step, as one
+//   launch of two waves 41.2; 768 x 1536: 23.9, 24.3; 2048 x 2048: 76.1, 77.6).
 TileLaunch tile_plan(const HostParams &h, int T)
 {
     const HostParams *one = &h;
@@ -2193,12 +2197,12 @@ TileLaunch tile_plan_batch(const HostParams *const *h, int n)
 }
 
 cudaError_t launch_tile(const HostParams &p, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
-                        int *status, int rev, cudaStream_t s)
+                        int *status, unsigned *begun, unsigned pass, cudaStream_t s)
 {
     switch (p.storage) {
-        case ST_FP32: return tile_t<float>(p, l, tmap, dst, step, status, rev, s);
-        case ST_BF16: return tile_t<__nv_bfloat16>(p, l, tmap, dst, step, status, rev, s);
-        case ST_FP16: return tile_t<__half>(p, l, tmap, dst, step, status, rev, s);
+        case ST_FP32: return tile_t<float>(p, l, tmap, dst, step, status, begun, pass, s);
+        case ST_BF16: return tile_t<__nv_bfloat16>(p, l, tmap, dst, step, status, begun, pass, s);
+        case ST_FP16: return tile_t<__half>(p, l, tmap, dst, step, status, begun, pass, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -304,9 +304,9 @@ __device__ __forceinline__ void tile_steps(const KP<float> &k, const CUtensorMap
 // the ring.  A slot is refilled one tick after its last read (2 W + 2 T slots
 // are exactly what is live: W rows on their way, W of this tick, and 2 T of
 // the lower neighbours' states).  1024 x 2048: FP32 52.0 us per step with one
-// step per launch, 39.8 us with strips of two steps; what bounds it is the
+// step per launch, 40.6 us with strips of two steps; what bounds it is the
 // latency of dependent instructions at 12 warps per SM (47 % issue), not
-// memory.  FP16 45.7 -> 44.4 us at that size.
+// memory.  FP16 49.1 -> 44.4 us at that size.
 // kRunning: the position in the ring, the lattice row and the limits of the
 // active rows run along with t instead of being formed from it (10 % fewer
 // instructions in 16-bit storage, 2 % in FP32: 41.3 -> 39.8 us).  FP32 batches,
@@ -315,7 +315,8 @@ __device__ __forceinline__ void tile_steps(const KP<float> &k, const CUtensorMap
 template <typename S, bool kRunning>
 __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMap *map, S *__restrict__ dst,
                                             const TileShape &sh, int T, int win, int tile, unsigned long long step,
-                                            int *status, unsigned char *smem, int part = 0)
+                                            int *status, unsigned char *smem, int part = 0, unsigned *begun = nullptr,
+                                            unsigned pass = 0)
 {
     constexpr int SB = TileGeom<S>::slot_bytes / (int)sizeof(S);
     const int warp = __shfl_sync(FULL, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31, W = blockDim.x >> 5;
@@ -335,9 +336,18 @@ __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMa
     const Lane2 L = lane2(k, c0);
     __syncthreads();
     if (part != 2) grid_dependency_wait();
-    if (part == 1) {  // the second part relies on this wait (k_tiles)
-        __threadfence();
+    if (part == 1) {  // the pass before is complete: say so to part 2 (k_tiles)
+        if (blockIdx.x == 0) {
+            if (threadIdx.x == 0) st_release_gpu(begun, pass);
+            __syncthreads();
+        }
         grid_dependency_trigger();
+    }
+    bool told = true;
+    if (part == 2 && warp == 0) {  // which issues the fetches, the first access to the lattice
+        int polls = 0;
+        while (ld_acquire_gpu(begun) != pass && (told = ++polls <= kFlagWaitLimit)) __nanosleep(100);
+        asm volatile("fence.proxy.async.global;" ::: "memory");
     }
     auto fetch = [&](int m, int slot0) {  // the rows of tick m (warp 0)
         const int first = m * W, cnt = min(W, n - first);
@@ -351,7 +361,7 @@ __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMa
                           k.xper ? wrap_row(r0 + first + lane, nz) : r0 + first + lane, bar + 8u * (m & 1));
         }
     };
-    if (warp == 0) {
+    if (warp == 0 && __all_sync(FULL, told)) {  // (else the wait for the first rows runs out)
         fetch(0, 0);
         fetch(1, W);
     }
@@ -426,20 +436,29 @@ __device__ __forceinline__ void strip_steps(const KP<float> &k, const CUtensorMa
 // by side, the second filling the SMs as the blocks of the first finish: it
 // reads the state of the pass before and writes other rows, so it does not
 // wait for the first at its start.  What it needs is that the pass before is
-// complete.  A block of part 1 allows the dependent launch only after it has
-// waited for that pass, and part 2 starts when every block of part 1 has done
-// so.  A block of part 2 waits for part 1 before it ends: a launch that waits
-// for part 2 then finds both complete.  (1024 x 2048 FP32: 45.4 us per step
-// with part 2 waiting at its start, 41.6 so.)
+// complete and its writes are visible.  Part 1 waits for that pass, then writes
+// the number of its own pass to *begun with release semantics and only then
+// allows the dependent launch; a block of part 2 reads *begun with acquire
+// semantics before its first access to the lattice (it holds that number by
+// then; the wait is bounded all the same).  Pass numbers are those of the
+// lattice's life, and a call that can be replayed from a graph has an even
+// number of such passes, so that the pass before always has another number.
+// A block of part 2 waits for part 1 before it ends: a launch that waits for
+// part 2 then finds both complete.  (1024 x 2048 FP32: 43.3 us per step with
+// part 2 waiting for part 1 at its start, 41.2 as one launch of two waves, 40.6
+// so; 2048 x 2048: 79.1, 77.6, 76.1.)
 template <typename S, bool kStrip>
 __global__ void __maxnreg__(kTileRegs<S>)
     k_tiles(const __grid_constant__ KP<float> k, const __grid_constant__ CUtensorMap map, S *__restrict__ dst,
-            const TileShape sh, int T, int first, unsigned long long step, int *status, int rev, int part)
+            const TileShape sh, int T, int first, unsigned long long step, int *status, int rev, int part,
+            unsigned *begun, unsigned pass)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     if (sizeof(S) != 4 || part != 1) grid_dependency_trigger();
     const int b = first + (rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x);
-    if constexpr (kStrip) strip_steps<S, true>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem, sizeof(S) == 4 ? part : 0);
+    if constexpr (kStrip)
+        strip_steps<S, true>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem, sizeof(S) == 4 ? part : 0,
+                             begun, pass);
     else tile_steps<S>(k, &map, dst, sh, T, b % sh.nw, b / sh.nw, step, status, smem);
     if (sizeof(S) == 4 && part == 2) grid_dependency_wait();
 }
