@@ -472,14 +472,10 @@ lb_status lb_step(lb_ctx *ctx, int32_t nsteps)
     const int32_t fused =
         ctx->hp.storage != LB_FP64 && ctx->launch_auto && !lbk::step_is_pinned(ctx->hp) ? nsteps : 0;
     if (fused > 0) {
-        // Passes of up to T steps.  Their number is made even or odd as the
-        // number of steps is, so that the current buffer alternates with the
-        // step count as it does with one launch per step.
         lbk::TileLaunch pass = lbk::tile_plan(ctx->hp, 0);
-        int32_t m = (fused + pass.T - 1) / pass.T;
-        if ((fused - m) & 1) ++m;
-        for (int32_t p = 0; p < m; ++p) {
-            const int32_t T = fused / m + (p < fused % m ? 1 : 0);
+        const int64_t m = lbk::pass_count(fused, pass.T);
+        for (int64_t p = 0; p < m; ++p) {
+            const int T = (int)(fused / m + (p < fused % m ? 1 : 0));
             if (T != pass.T) pass = lbk::tile_plan(ctx->hp, T);
             ctx->passes += 1;
             cudaError_t e;
@@ -1024,11 +1020,9 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
         return e;
     };
     if (b->automatic() && nsteps > 0) {
-        // passes of several steps, as many as make the buffers alternate with the step count (lb_step)
-        int32_t m = (nsteps + b->tiles.T - 1) / b->tiles.T;
-        if ((nsteps - m) & 1) ++m;
-        for (int32_t p = 0; p < m; ++p) {
-            const int32_t T = nsteps / m + (p < nsteps % m ? 1 : 0);
+        const int64_t m = lbk::pass_count(nsteps, b->tiles.T);
+        for (int64_t p = 0; p < m; ++p) {
+            const int T = (int)(nsteps / m + (p < nsteps % m ? 1 : 0));
             const unsigned long long flip = (b->counter + (unsigned long long)p) & 1ULL;
             cudaError_t e;
             if (T == 1 && b->tiles.strip && flip == (t & 1ULL))  // large lattices' single step: one warp per work item

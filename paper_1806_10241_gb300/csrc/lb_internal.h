@@ -80,6 +80,15 @@ struct TileLaunch {
 };
 // The pass for a lattice: of T steps, or (T = 0) of as many as pay.
 TileLaunch tile_plan(const HostParams &p, int T);
+// Passes of a call of n steps, up to T in each: as few as that takes, their
+// number odd or even as n is, so that the current buffer alternates with the
+// step count as it does with one launch per step.  Pass p takes
+// n / m + (p < n % m) steps.
+inline int64_t pass_count(int64_t n, int T)
+{
+    const int64_t m = (n + T - 1) / T;
+    return m + ((n - m) & 1);
+}
 // pass: the number of the pass in the lattice's life, from 1 on; begun: the
 // lattice's device word for it (k_tiles).
 cudaError_t launch_tile(const HostParams &p, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
