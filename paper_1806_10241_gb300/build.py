@@ -22,8 +22,8 @@ NVCC = os.environ.get("NVCC", "nvcc")
 # fields) is contracted into an FMA behind the source's back.  Whether the
 # compiler contracts depends on the inlining context, so the same rule could
 # round differently in the single-lattice and the batched kernels, or with
-# plain loads and the TMA ring.  The node update spells its FMAs out
-# (packed FP32x2 intrinsics) and is unaffected.
+# plain loads and the TMA ring.  Packed FP32x2 operations are fused all the
+# same; the node update leaves nothing to fuse (lb_node.cuh).
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-fmad=false", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "--expt-relaxed-constexpr"]
 

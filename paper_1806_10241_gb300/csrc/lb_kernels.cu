@@ -72,13 +72,7 @@ template <typename S> struct Scaled { static constexpr bool value = std::is_same
 
 // ---- kernel parameters in the compute type --------------------------------
 
-// Parameters of the node update (update_node2) as its operands: in FP32 as
-// packed pairs with equal halves, which the packed instructions take as they
-// lie in the parameters, where a scalar would first be copied into a pair.
-template <typename E> struct NodeConst {
-    E rho0, T0, bfx, fb, nu, nuh, alh, k3;              // fb = rho0 g_beta; nu / 2, alpha / 2, rho0 / 3
-    E c3, c4, nc4, ch, nch, cg, ct, m9, m6, m5, sg, os; // relaxation and back-transform factors, storage scale
-};
+#include "lb_node.cuh"
 
 template <typename C> struct KP {
     int nr, nz, pitch, xper;
@@ -207,7 +201,7 @@ template <typename C> KP<C> make_kp(const HostParams &h)
         c.ch = e(omh * (C)0.25 * osc), c.nch = e(omh * (C)-0.25 * osc);
         c.cg = e(k.omg * (C)0.5 * osc), c.ct = e(k.omh * (C)0.5 * osc);
         c.m9 = e(ninth * osc), c.m6 = e((C)1 / (C)6 * osc), c.m5 = e((C)0.2 * osc);
-        c.sg = e((C)(h.sign_literal ? -1 : 1)), c.os = e(osc);
+        c.sg = e((C)(h.sign_literal ? -1 : 1)), c.os = e(osc), c.one = e((C)1), c.mone = e((C)-1);
     }
     // Nusselt normalisation (Sec. 3.2): lateral walls -R_w / (H dT), end
     // walls -(H / dT) * 2 / (R_o^2 - R_i^2); dT from the Dirichlet values.
@@ -234,9 +228,6 @@ template <typename C> KP<C> make_kp(const HostParams &h)
 }
 
 // ---- per-row helpers -------------------------------------------------------
-
-// Plane indices
-enum { F0 = 0, G0 = 9, H0 = 14 };
 
 template <typename C> struct PM {  // macroscopic fields of the stored state
     C rd, ux, uy, ut, T;
