@@ -28,6 +28,7 @@
 
 #include "../../include/lb.h"
 #include "lb_internal.h"
+#include "lb_rcp.cuh"
 
 namespace lbk {
 
@@ -606,7 +607,7 @@ template <typename I> __device__ __forceinline__ void st_release_gpu(I *p, I v)
 // The distributions are read where they lie (L1 / L2): loads, indices and
 // rules other than arithmetic cost nothing beside the FP64 pipe.
 // 41 x 41: 70.6 us per step before (30-column march, at least four rows per
-// warp, terms not fused), 10.9 us now; 256 x 512: 220 us, 88.5 us.
+// warp, terms not fused), 10.6 us now; 256 x 512: 220 us, 89.3 us.
 constexpr int kFields64Cols = 34;  // 32 columns and the halo columns
 
 // Wall rules of the FP64 step with their constants formed once on the host

@@ -64,21 +64,9 @@ __device__ __forceinline__ F2 operator-(F2 a, F2 b)
         : "f"(a.v.x), "f"(a.v.y), "f"(b.v.x), "f"(b.v.y));
     return r;
 }
-// 1 / x of a density: the hardware reciprocal alone.  __fdividef(1, x) has the
-// same bits for every normal x whose reciprocal is normal, but wraps the
-// reciprocal in a rescaling for the others (five more instructions each).
-__device__ __forceinline__ float rcp1(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 __device__ __forceinline__ F2 rcp2(F2 a) { return mk2(rcp1(a.v.x), rcp1(a.v.y)); }
 
-// One FP64 value with the same operations, for the FP64 step.  The reciprocal
-// of a density (a normal number) is the hardware's approximation, good to 1e-6,
-// and one cubic iteration, x (1 + e + e^2) with e = 1 - r x: three FP64
-// instructions and a relative error below 2.3e-16 (measured on [0.5, 1.75]).
+// One FP64 value with the same operations, for the FP64 step.
 struct D1 {
     double v;
     static __device__ __forceinline__ D1 of(double x) { return D1{x}; }
@@ -89,13 +77,6 @@ __device__ __forceinline__ D1 operator+(D1 a, D1 b) { return D1{a.v + b.v}; }
 __device__ __forceinline__ D1 operator-(D1 a, D1 b) { return D1{a.v - b.v}; }
 __device__ __forceinline__ D1 operator*(D1 a, D1 b) { return D1{a.v * b.v}; }
 __device__ __forceinline__ D1 fma2(D1 a, D1 b, D1 c) { return D1{__fma_rn(a.v, b.v, c.v)}; }
-__device__ __forceinline__ double rcp1(double r)
-{
-    double x;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(r));
-    const double e = __fma_rn(-r, x, 1.0);
-    return __fma_rn(x, __fma_rn(e, e, e), x);
-}
 __device__ __forceinline__ D1 rcp2(D1 a) { return D1{rcp1(a.v)}; }
 __device__ __forceinline__ F2 sel2(bool px, bool py, F2 a, F2 b)  // per component: p ? a : b
 {
