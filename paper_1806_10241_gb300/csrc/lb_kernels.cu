@@ -977,7 +977,7 @@ __global__ void __launch_bounds__(128) k_psi(const double *__restrict__ ux, doub
 // node's stored state once, node(i, c, out) its pre-collision state.  (A warp
 // marching 32 rows of 30 columns on its own, as before, is a serial chain of
 // 32 row updates; these are four nodes per thread and round, all independent: the
-// diagnostics of 1024 x 2048 FP32 took 220 us and take 124.)
+// diagnostics of 1024 x 2048 FP32 took 220 us and take 122.)
 constexpr int kBlockCols = 128, kBlockChunk = 8, kBlockThreads = 256, kBlockPitch = kBlockCols + 2;
 template <typename C> constexpr size_t kBlockSmem = (size_t)(kBlockChunk + 2) * 4 * kBlockPitch * sizeof(C);
 
@@ -1110,55 +1110,40 @@ __device__ __forceinline__ double warp_max(double v)
     return v;
 }
 
-// Sums over a thread's nodes.  FP64 instructions are what a diagnostic of an
-// FP32 lattice would spend its time on (the pipe takes one per SM every 19
-// cycles, conversions to and from FP64 included), so an FP32 thread keeps its
-// few sums as a value and the exact rounding error of each addition (Knuth's
-// two-sum), and turns them into FP64 once, at its end: an error of 2^-47 of a
-// sum over at most some dozens of nodes.
-template <typename C> struct NodeSum {
-    C hi = 0, lo = 0;
-    __device__ __forceinline__ void add(C x)
-    {
-        if constexpr (std::is_same<C, double>::value) {
-            hi += x;
-        } else {
-            const C t = hi + x, b = t - hi;
-            lo += (hi - (t - b)) + (x - b);
-            hi = t;
-        }
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-// The largest u_x^2 + u_y^2, FP32 squares as unevaluated sums of two FP32
-// values (exact products by FMA, two-sum), scaled away from the subnormal range.
+// The largest |u|, of FP64 squares.  FP64 instructions are scarce (the pipe takes
+// one per SM every 19 cycles, conversions included), so an FP32 thread keeps the
+// velocity whose FP32 square is the largest and squares it in FP64 (where FP32
+// squares are exact) at its end: 1024 x 2048 FP32 128 us, 140 with every node's
+// square in FP64.  Two nodes whose FP32 squares do not tell which is larger, as
+// these are within 2^-22 of the exact ones, or which lie near the ends of the
+// range, are compared in FP64.
 template <typename C> struct NodeMax {
-    C hi = 0, lo = 0;
+    C x = 0, y = 0, top = 0;
+    static __device__ __forceinline__ double square(C x, C y) { return (double)x * (double)x + (double)y * (double)y; }
     __device__ __forceinline__ void add(C ux, C uy)
     {
         if constexpr (std::is_same<C, double>::value) {
-            hi = fmax(hi, ux * ux + uy * uy);
+            top = fmax(top, square(ux, uy));
         } else {
-            const float x = ux * 0x1p32f, y = uy * 0x1p32f;
-            const float p = x * x, q = y * y, t = p + q, b = t - p;
-            const float e = ((p - (t - b)) + (q - b)) + (__fmaf_rn(x, x, -p) + __fmaf_rn(y, y, -q));
-            const float h = t + e, l = e - (h - t);
-            if (h > hi || (h == hi && l > lo)) {
-                hi = h;
-                lo = l;
-            }
-            if (t == INFINITY) {  // (the error terms are not numbers)
-                hi = t;
-                lo = 0.0f;
-            }
+            const C t = ux * ux + uy * uy;
+            if ((t < 0.999999f * top && top > 1e-30f) || (ux == 0 && uy == 0)) return;
+            if (!(t > 1.000001f * top && t > 1e-30f && t < 3e38f) && !(square(ux, uy) > square(x, y))) return;
+            x = ux;
+            y = uy;
+            top = fminf(t, 3.4e38f);
         }
     }
     __device__ __forceinline__ double value() const
     {
-        if constexpr (std::is_same<C, double>::value) return sqrt(hi);
-        else return sqrt((double)hi + (double)lo) * 0x1p-32;
+        if constexpr (std::is_same<C, double>::value) return sqrt(top);
+        else return sqrt(square(x, y));
     }
 };
+
+// Registers for three blocks on an SM, where FP32 has two by itself: 1024 x 2048
+// 128 -> 122 us; 64 annuli in one batch, whose kernel also takes the lattice's
+// parameters from shared memory, 538 -> 464 us (before the blocks 498 us).
+template <typename C> constexpr int kDiagBlocks = std::is_same<C, float>::value ? 3 : 1;
 
 // Diagnostics of block (bx, by) of a grid gx blocks wide, seg_rows rows each:
 // partial sums in a fixed order, and the temperatures next to the walls in
@@ -1171,13 +1156,13 @@ __device__ __forceinline__ void diag_block(const KP<C> &k, const S *__restrict__
     constexpr int warps = kBlockThreads / 32;
     __shared__ double sh[warps][5];
     const int nr = k.nr, nz = k.nz, s = by * seg_rows;
-    NodeSum<C> rd, T;
+    double rd = 0.0, T = 0.0;
     NodeMax<C> u;
     bool bad = false;
     block_fields<S, C>(
-        k, src, bx * kBlockCols, s, min(nz, s + seg_rows) - s, F, [&](int, int, const PM<C> &m) { rd.add(m.rd); },
+        k, src, bx * kBlockCols, s, min(nz, s + seg_rows) - s, F, [&](int, int, const PM<C> &m) { rd += (double)m.rd; },
         [&](int i, int c, const NodeOut<C> &o) {
-            T.add(o.T);
+            T += (double)o.T;
             u.add(o.ux, o.uy);
             bad |= !(isfinite(o.rho) && isfinite(o.ux) && isfinite(o.uy) && isfinite(o.ut) && isfinite(o.T)) ||
                    o.rho < (C)0.5 || o.rho > (C)1.5;
@@ -1187,9 +1172,8 @@ __device__ __forceinline__ void diag_block(const KP<C> &k, const S *__restrict__
             if (c <= 1) cs[(long long)c * nz + i] = (double)o.T;
             if (c >= nr - 2) cs[(long long)(c - nr + 4) * nz + i] = (double)o.T;
         });
-    const double m = rd.value();
     const double y = k.r0 + (bx * kBlockCols + (int)(threadIdx.x % kBlockCols)) + 0.5;
-    double vals[5] = {m, m * y, T.value(), u.value(), bad ? 1.0 : 0.0};
+    double vals[5] = {rd, rd * y, T, u.value(), bad ? 1.0 : 0.0};
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < 5; ++q) vals[q] = q >= 3 ? warp_max(vals[q]) : warp_sum(vals[q]);
@@ -1205,7 +1189,7 @@ __device__ __forceinline__ void diag_block(const KP<C> &k, const S *__restrict__
 }
 
 template <typename S, typename C>
-__global__ void __launch_bounds__(kBlockThreads) k_diag(const __grid_constant__ KP<C> k, const S *__restrict__ src,
+__global__ void __launch_bounds__(kBlockThreads, kDiagBlocks<C>) k_diag(const __grid_constant__ KP<C> k, const S *__restrict__ src,
                                                         double *__restrict__ partial, double *__restrict__ strips,
                                                         int seg_rows, int gx)
 {
@@ -1648,7 +1632,7 @@ struct BatchDiag {
 };
 
 template <typename S>
-__global__ void __launch_bounds__(kBlockThreads) k_batch_diag(const BatchDesc *__restrict__ d,
+__global__ void __launch_bounds__(kBlockThreads, kDiagBlocks<float>) k_batch_diag(const BatchDesc *__restrict__ d,
                                                     const BatchDiag *__restrict__ dd, const int *__restrict__ prefix,
                                                     int n, unsigned long long t)
 {
@@ -1663,9 +1647,13 @@ __global__ void __launch_bounds__(kBlockThreads) k_batch_diag(const BatchDesc *_
     }
     const BatchDesc &bd = d[lo];
     const BatchDiag &g = dd[lo];
+    __shared__ KP<float> sk;  // the lattice's parameters
+    for (int w = threadIdx.x; w < (int)(sizeof(KP<float>) / 4); w += blockDim.x)
+        reinterpret_cast<uint32_t *>(&sk)[w] = reinterpret_cast<const uint32_t *>(&bd.k)[w];
+    __syncthreads();
     const int local = blk - prefix[lo];
     const int cur = (bd.parity0 + (int)(t & 1ULL)) & 1;  // the lattice's current buffer after t batch steps
-    diag_block<S, float>(bd.k, (const S *)bd.buf[cur], g.partial, (double *)bd.buf[cur ^ 1], g.seg, local % g.gx,
+    diag_block<S, float>(sk, (const S *)bd.buf[cur], g.partial, (double *)bd.buf[cur ^ 1], g.seg, local % g.gx,
                          local / g.gx, g.gx, reinterpret_cast<float *>(smem));
 }
 
