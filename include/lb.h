@@ -270,13 +270,15 @@ LB_EXPORT lb_status lb_get_launch(const lb_ctx *ctx, int32_t *seg_rows, int32_t 
  * desc and params describe it and pass the checks of lb_create and
  * lb_set_params; step is copied to out->step.  The reductions use the
  * grid of lb_diagnostics, which depends on the lattice alone: the result is
- * bitwise that of lb_diagnostics on the same state (to reduction round-off
- * for lattices of more than 2048 blocks of 128 columns and 32 rows).
+ * bitwise that of lb_diagnostics on the same state, for every lattice with nr
+ * + nz <= 20000 and every one whose grid fits the scratch (12 doubles a block
+ * of 128 columns and up to 32 rows, at most 4096 blocks); to reduction
+ * round-off beyond.
  *
  * Scratch: a 1 MiB array (2^17 doubles) in the library's static device
  * memory, which every GPU that loads the library holds until the process
- * exits.  A lattice needs 16 + 12 x (blocks <= 2048) + 4 (nr + nz) doubles;
- * larger lattices (nr + nz above about 26600) are rejected with LB_ERR_ARG.
+ * exits.  A lattice needs 16 + 12 x blocks + 4 (nr + nz) doubles, with 2048
+ * blocks at most where the array has no room for more; larger lattices (nr + nz above about 26600) are rejected with LB_ERR_ARG.
  * No call allocates or frees memory.  Every call looks up the array's device
  * address in the current context (cudaGetSymbolAddress); the first call on a
  * device may load the library's device code there, so make it before any

@@ -2635,13 +2635,16 @@ extern "C" lb_status lb_diagnostics_static(const lb_grid_desc *desc, const lb_pa
         return LB_ERR_ARG;
     }
     // The size is limited by blocks of 120 columns and 32 rows, taller ones
-    // where these were more than kScratchMaxBlocks; the diagnostics grid then
-    // has no more blocks than that.
+    // where these were more than kScratchMaxBlocks.  The grid is lb_diagnostics's
+    // where its partial sums fit beside the strips, else one with no more blocks
+    // than counted here.
     const long long bx = (h.nr + 119) / 120, by = (h.nz + 31) / 32;
     const long long cap = std::max(1LL, std::min(by, kScratchMaxBlocks / bx)), seg = (h.nz + cap - 1) / cap;
     const long long most = bx * ((h.nz + seg - 1) / seg);
     const size_t need = 16 + (size_t)most * NSUM + 4 * ((size_t)h.nr + (size_t)h.nz);
-    const DiagGrid g = diag_grid(h, bx * by > kScratchMaxBlocks ? (int)most : kScratchMaxBlocks);
+    auto doubles = [&](const DiagGrid &g) { return 16 + (size_t)g.gx * g.gy * NSUM + 4 * ((size_t)h.nr + (size_t)h.nz); };
+    DiagGrid g = diag_grid(h, MAX_DIAG_BLOCKS);
+    if (doubles(g) > kScratchDoubles) g = diag_grid(h, (int)most);
     const long long nb = (long long)g.gx * g.gy;
     if (most > kScratchMaxBlocks || need > kScratchDoubles) {
         char msg[200];
@@ -2655,8 +2658,7 @@ extern "C" lb_status lb_diagnostics_static(const lb_grid_desc *desc, const lb_pa
     double *scratch = nullptr;
     cudaError_t e = scratch_address(&scratch);
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const size_t used = 16 + (size_t)nb * NSUM + 4 * ((size_t)h.nr + (size_t)h.nz);
-    if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, used * sizeof(double), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, doubles(g) * sizeof(double), st);
     if (e == cudaSuccess) {
         double *partial = scratch + 16, *strips = partial + (size_t)nb * NSUM;
         switch (h.storage) {
