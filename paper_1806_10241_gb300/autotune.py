@@ -28,6 +28,19 @@ SOLVER_CANDIDATES = [(4, 1, 3), (4, 2, 3), (6, 1, 3), (8, 1, 3), (12, 2, 3), (16
 BATCH_CANDIDATES = [(4, 1, 3), (4, 2, 3), (6, 1, 3), (8, 1, 3), (8, 2, 1), (16, 4, 1)]
 
 
+# Steps of a timed call: a multiple of this is whole passes of two, three and
+# four steps, and an even number of them.  (A call of three steps takes three
+# passes of one where passes hold two, and would time the automatic launch as
+# the one-step launch that it then is.)
+WHOLE_PASSES = 24
+# Steps of a warm-up call: passes of two, the kernel that the timed call runs.
+WARM = 4
+
+
+def _whole_passes(steps: int) -> int:
+    return max(1, -(-steps // WHOLE_PASSES)) * WHOLE_PASSES
+
+
 def _size_class(n: int) -> int:
     return max(0, int(n - 1).bit_length())
 
@@ -60,8 +73,10 @@ def _time(stream, fn, steps: int) -> float:
 def tune_solver(solver, steps: int = 20, use_cache: bool = True) -> tuple:
     """Pick the launch for this solver's shape: one of SOLVER_CANDIDATES, or the
     automatic one (several steps per launch; reported as lb_get_launch does).
-    Returns (seg_rows, warps_per_block, row_fetch)."""
+    Returns (seg_rows, warps_per_block, row_fetch).  Each candidate is timed
+    over `steps` steps, rounded up to whole passes."""
     key = f"solver/{solver.storage}/{_size_class(solver.nr)}/{_size_class(solver.nz)}"
+    steps = _whole_passes(steps)
     with _lock:
         cache = _load() if use_cache else {}
     if key in cache:
@@ -74,7 +89,7 @@ def tune_solver(solver, steps: int = 20, use_cache: bool = True) -> tuple:
     # the automatic launch first: of equal times it wins, as it takes several steps per launch
     for c in [(0, 0, 0)] + list(cands):
         solver.set_launch(*c)
-        solver.step(2)  # warm
+        solver.step(WARM)
         results.append((_time(solver.stream, solver.step, steps), c))
     ms, best = min(results, key=lambda r: r[0])
     solver.set_launch(*best)
@@ -138,8 +153,10 @@ def tune_batch(batch, steps: int = 30, graph_steps: int = 50, use_cache: bool = 
     every lattice, or a per-lattice segment plan (segment_plan) for a number
     of waves, with the TMA-ring step; keyed by storage, node count and
     lattice count.  Returns (seg_rows, warps_per_block, row_fetch, waves),
-    waves = 0 for a common segment length."""
+    waves = 0 for a common segment length.  Each candidate is timed over
+    `steps` steps, rounded up to whole passes."""
     key = _batch_key(batch)
+    steps = _whole_passes(steps)
     with _lock:
         cache = _load() if use_cache else {}
     if key in cache and len(cache[key].get("launch", [])) == 3 and "waves" in cache[key]:
@@ -163,7 +180,7 @@ def tune_batch(batch, steps: int = 30, graph_steps: int = 50, use_cache: bool = 
             resident, items = batch.occupancy()
             if items > resident:
                 continue
-        batch.step(2)
+        batch.step(WARM)
         results.append((_time(batch.stream, batch.step, steps), launch, waves))
     results.sort(key=lambda r: r[0])
     _, launch, waves = results[0]

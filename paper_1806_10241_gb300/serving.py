@@ -31,7 +31,7 @@ from dataclasses import dataclass, field
 import numpy as np
 import torch
 
-from .autotune import has_cached_batch_launch, tune_batch
+from .autotune import WHOLE_PASSES, has_cached_batch_launch, tune_batch
 from .batch import Batch
 from .solver import Solver, required_bytes
 from .workloads import Request
@@ -155,11 +155,11 @@ class Server:
                 scratch.append(s)
             sb = Batch(scratch, stream=self.stream, seg_rows=self.seg_rows, warps_per_block=self.warps_per_block,
                        graph_steps=self.graph_steps)
-            tune_batch(sb, steps=3, graph_steps=self.graph_steps)
+            tune_batch(sb, steps=WHOLE_PASSES, graph_steps=self.graph_steps)
             sb.close()
             for s in scratch:
                 s.close()
-        tune_batch(batch, steps=3, graph_steps=self.graph_steps)
+        tune_batch(batch, steps=WHOLE_PASSES, graph_steps=self.graph_steps)
 
     def _check(self, a: _Active, d: dict | None = None) -> bool:
         """Diagnostics of an active lattice (given, or computed here); True

@@ -1,0 +1,59 @@
+"""What the autotuner times: candidates in calls of whole passes."""
+import pytest
+
+from paper_1806_10241_gb300 import autotune, serving
+from test_autotune_cpu import FakeBatch, FakeSolver
+
+
+class Solver(FakeSolver):
+    def __init__(self, storage="fp32", alpha=0.05, nr=64, nz=64, **more):
+        super().__init__(storage, nr, nz)
+        self.params = {"nr": nr, "nz": nz, "nu": 0.05, "alpha": alpha, **more}
+        self.stream, self.calls = None, []
+
+    def step(self, n=1):
+        self.calls.append(n)
+
+    def get_launch(self):
+        return (4, 1, 3)
+
+
+class Batch(FakeBatch):
+    def __init__(self, solvers):
+        super().__init__(resident=1000, items=50)
+        self.solvers, self.calls = solvers, []
+
+    def step(self, n=1):
+        self.calls.append(n)
+
+
+@pytest.fixture
+def cache(tmp_path, monkeypatch):
+    path = tmp_path / "autotune.json"
+    monkeypatch.setattr(autotune, "_CACHE", str(path))
+    monkeypatch.setattr(autotune, "_time", lambda stream, fn, steps: fn(steps) or 1.0)
+    return path
+
+
+def passes(n, T):
+    """The passes of a call, as lb_step cuts it."""
+    m = -(-n // T)
+    m += (n - m) & 1
+    return [n // m + (p < n % m) for p in range(m)]
+
+
+@pytest.mark.parametrize("steps", [1, 3, 20, 24, 30])
+def test_candidates_are_timed_over_whole_passes(cache, steps):
+    solver, batch = Solver(), Batch([Solver()])
+    autotune.tune_solver(solver, steps=steps)
+    autotune.tune_batch(batch, steps=steps)
+    for calls, candidates in ((solver.calls, 1 + len(autotune.SOLVER_CANDIDATES)), (batch.calls, len(batch.calls) // 2)):
+        assert len(calls) == 2 * candidates > 2  # a warm-up and a timed call each
+        for warm, timed in zip(calls[::2], calls[1::2]):
+            for T in (2, 3, 4):
+                assert timed >= steps and set(passes(timed, T)) == {T}
+                assert min(passes(warm, T)) >= 2  # not the kernel of single steps
+
+
+def test_server_asks_for_whole_passes():
+    assert serving.WHOLE_PASSES == autotune.WHOLE_PASSES
