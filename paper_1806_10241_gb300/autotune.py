@@ -3,8 +3,9 @@
 Candidates (rows per z-segment, warps per block, row fetch) are timed with
 CUDA events on the solver's own stream for a few steps each; the steps taken
 while tuning are real time steps (results do not depend on the launch shape).
-The best shape is applied and remembered in a JSON cache keyed by storage and
-lattice size class.
+The best shape is applied and remembered in a JSON cache keyed by storage,
+lattice size class and how many lattices are pinned (lb.h: those take one launch
+per step whatever the launch, so that their best launch is nobody else's).
 
 For a batch of uneven lattices the candidates also include per-lattice
 segment plans: every lattice's z-segments sized so that all work items hold
@@ -39,6 +40,14 @@ WARM = 4
 
 def _whole_passes(steps: int) -> int:
     return max(1, -(-steps // WHOLE_PASSES)) * WHOLE_PASSES
+
+
+def _pinned(solver) -> bool:
+    """Whether the lattice takes one launch per step whatever the launch (lb.h, lb_step)."""
+    p = getattr(solver, "params", None)
+    if p is None or solver.storage == "fp64" or p.get("planar", 0):
+        return False
+    return max(float(p["nu"]), float(p["alpha"])) > 3.0 * (float(p.get("r0", 0.0)) + 0.5)
 
 
 def _size_class(n: int) -> int:
@@ -76,6 +85,7 @@ def tune_solver(solver, steps: int = 20, use_cache: bool = True) -> tuple:
     Returns (seg_rows, warps_per_block, row_fetch).  Each candidate is timed
     over `steps` steps, rounded up to whole passes."""
     key = f"solver/{solver.storage}/{_size_class(solver.nr)}/{_size_class(solver.nz)}"
+    key += "/pinned" if _pinned(solver) else ""
     steps = _whole_passes(steps)
     with _lock:
         cache = _load() if use_cache else {}
@@ -133,7 +143,9 @@ def _apply(batch, launch, waves, graph_steps):
 
 
 def _batch_key(batch) -> str:
-    return f"batch/{batch.solvers[0].storage}/{_size_class(batch.nodes)}/{_size_class(len(batch.solvers))}"
+    pinned = sum(_pinned(s) for s in batch.solvers)
+    return f"batch/{batch.solvers[0].storage}/{_size_class(batch.nodes)}/{_size_class(len(batch.solvers))}" + \
+        (f"/pinned{_size_class(pinned)}" if pinned else "")
 
 
 def has_cached_batch_launch(batch, graph_steps: int = 50) -> bool:

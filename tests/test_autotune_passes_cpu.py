@@ -1,4 +1,7 @@
-"""What the autotuner times: candidates in calls of whole passes."""
+"""What the autotuner times and how it keeps it: candidates in calls of whole
+passes, and launches of pinned lattices apart from the others'."""
+import json
+
 import pytest
 
 from paper_1806_10241_gb300 import autotune, serving
@@ -57,3 +60,17 @@ def test_candidates_are_timed_over_whole_passes(cache, steps):
 
 def test_server_asks_for_whole_passes():
     assert serving.WHOLE_PASSES == autotune.WHOLE_PASSES
+
+
+def test_pinned_lattices_have_entries_of_their_own(cache):
+    plain, pinned = Solver(), Solver(alpha=4.0)
+    assert not autotune._pinned(plain) and autotune._pinned(pinned)
+    assert not autotune._pinned(Solver("fp64", alpha=4.0)) and not autotune._pinned(Solver(alpha=4.0, planar=1))
+    assert not autotune._pinned(Solver(alpha=1.5)) and autotune._pinned(Solver(alpha=1.500001))  # 3 (r0 + 1/2)
+    assert not autotune._pinned(Solver(alpha=4.0, r0=10.0))
+    autotune.tune_solver(pinned)
+    autotune.tune_solver(plain)
+    assert plain.calls  # not taken from the pinned one's entry
+    keys = {autotune._batch_key(Batch([Solver(alpha=a) for a in alphas])) for alphas in
+            ((0.1, 0.1, 0.1, 0.1), (4.0, 0.1, 0.1, 0.1), (4.0, 4.0, 4.0, 4.0))}
+    assert len(keys) == 3 and len(json.loads(cache.read_text())) == 2
