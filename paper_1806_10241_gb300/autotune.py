@@ -3,9 +3,10 @@
 Candidates (rows per z-segment, warps per block, row fetch) are timed with
 CUDA events on the solver's own stream for a few steps each; the steps taken
 while tuning are real time steps (results do not depend on the launch shape).
-The best shape is applied and remembered in a JSON cache keyed by storage,
-lattice size class and how many lattices are pinned (lb.h: those take one launch
-per step whatever the launch, so that their best launch is nobody else's).
+The best shape is applied and remembered in a JSON cache, one file per version
+of the kernels, keyed by storage, lattice size class and how many lattices are
+pinned (lb.h: those take one launch per step whatever the launch, so that their
+best launch is nobody else's).
 
 For a batch of uneven lattices the candidates also include per-lattice
 segment plans: every lattice's z-segments sized so that all work items hold
@@ -20,7 +21,9 @@ import threading
 
 import torch
 
-_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "autotune.json")
+from . import build
+
+_CACHE = os.path.join(build.BUILD, f"autotune-{build.source_hash()}.json")
 _lock = threading.Lock()
 
 SOLVER_CANDIDATES = [(4, 1, 3), (4, 2, 3), (6, 1, 3), (8, 1, 3), (12, 2, 3), (16, 4, 3),

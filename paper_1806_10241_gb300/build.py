@@ -7,6 +7,7 @@ header is newer.
 from __future__ import annotations
 
 import glob
+import hashlib
 import os
 import subprocess
 import sys
@@ -35,6 +36,15 @@ def _sources():
 def _deps():
     return _sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         [os.path.join(ROOT, "include", "lb.h"), os.path.abspath(__file__)]
+
+
+def source_hash() -> str:
+    """Hash of the library's sources and build flags: launches tuned on other kernels do not carry over."""
+    h = hashlib.sha256(" ".join(ARCH + FLAGS).encode())
+    for path in sorted(p for p in _deps() if not p.endswith(".py")):
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def up_to_date() -> bool:

@@ -1,10 +1,12 @@
 """What the autotuner times and how it keeps it: candidates in calls of whole
-passes, and launches of pinned lattices apart from the others'."""
+passes, launches of pinned lattices apart from the others', and none from other
+kernels."""
 import json
+import os
 
 import pytest
 
-from paper_1806_10241_gb300 import autotune, serving
+from paper_1806_10241_gb300 import autotune, build, serving
 from test_autotune_cpu import FakeBatch, FakeSolver
 
 
@@ -74,3 +76,10 @@ def test_pinned_lattices_have_entries_of_their_own(cache):
     keys = {autotune._batch_key(Batch([Solver(alpha=a) for a in alphas])) for alphas in
             ((0.1, 0.1, 0.1, 0.1), (4.0, 0.1, 0.1, 0.1), (4.0, 4.0, 4.0, 4.0))}
     assert len(keys) == 3 and len(json.loads(cache.read_text())) == 2
+
+
+def test_cache_is_one_file_per_version_of_the_kernels(monkeypatch):
+    assert build.source_hash() in os.path.basename(autotune._CACHE)
+    before = build.source_hash()
+    monkeypatch.setattr(build, "FLAGS", build.FLAGS + ["-DOTHER"])
+    assert build.source_hash() != before
