@@ -294,7 +294,8 @@ LB_EXPORT lb_status lb_diagnostics_static(const lb_grid_desc *desc, const lb_par
  * parameters) together.  Under the settings it starts with (4 rows per
  * z-segment, 1 warp per block, row fetch 3, no per-lattice segments) that is
  * the automatic launch: all lattices' tiles in one launch of several steps, as
- * lb_step takes them.  Any other setting takes one kernel launch per step over
+ * lb_step takes them, and for single steps that are left over work items of
+ * equal length over all lattices.  Any other setting takes one kernel launch per step over
  * all their 64-column x z-segment tiles (work items numbered by a prefix sum
  * over the lattices), replayed from a CUDA graph of graph_steps launches when
  * the stream is not the legacy default stream.  Each lattice's
@@ -332,7 +333,7 @@ LB_EXPORT lb_status lb_batch_set_launch(lb_batch *b, int32_t seg_rows, int32_t w
 LB_EXPORT lb_status lb_batch_set_segments(lb_batch *b, const int32_t *seg_rows);
 /* Warps of the batched step that can be resident on the device at once
  * under the current settings with one launch per step, and the number of work
- * items (64-column window x z-segment) of one step.  NULL outputs are
+ * items (64-column window x z-segment) of such a step.  NULL outputs are
  * skipped. */
 LB_EXPORT lb_status lb_batch_get_occupancy(const lb_batch *b, int32_t *resident_warps, int32_t *items);
 LB_EXPORT lb_status lb_batch_step(lb_batch *b, int32_t nsteps);

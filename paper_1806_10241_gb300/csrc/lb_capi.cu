@@ -808,6 +808,26 @@ static size_t batch_layout(int32_t n, size_t *desc_off, size_t *prefix_off, size
     return d + p + t + g + bd + bp + (size_t)kMaxPersistItems * sizeof(int) + p;
 }
 
+// Single steps that a call has left over under the automatic launch, where the
+// lattices are cut into strips: one launch, one warp per work item.  Items of
+// about the same length over all lattices, in whole waves of the warps resident
+// at once, about 17 rows each, or one wave where that makes them shorter.  Per
+// step: 40 lattices of 64 to 128 columns FP32 21.9 us (one wave of 6.6 rows;
+// 4-row items 29.5, two waves 26.6), 64 annuli FP32 147 us (three waves of 17
+// rows; 188, one wave 184), 256 annuli FP16 506 us (twelve; 624; six 502).
+static int one_step_fetch(const lb_batch *b) { return b->storage == LB_FP32 ? 4 : 3; }
+static cudaError_t one_step_rows(const lb_batch *b, double *rows)
+{
+    int resident = 0;
+    const cudaError_t e = lbk::batch_resident_warps(b->storage, one_step_fetch(b), 1, &resident);
+    if (e != cudaSuccess) return e;
+    double all = 0.0;  // rows of 64 columns of all lattices
+    for (const lb_ctx *c : b->ctxs) all += lbk::batch_items(c->hp, 1);
+    const double per_wave = all / std::max(1, resident);
+    *rows = std::max(1.0, per_wave / std::max(1.0, std::round(per_wave / 17.0)));
+    return cudaSuccess;
+}
+
 static lb_status batch_upload(lb_batch *b)
 {
     const int n = (int)b->ctxs.size();
@@ -816,10 +836,19 @@ static lb_status batch_upload(lb_batch *b)
     b->hprefix.assign((size_t)n + 1, 0);
     b->htprefix.assign((size_t)n + 1, 0);
     b->pinned = 0;
+    for (const lb_ctx *c : b->ctxs) b->pinned += lbk::step_is_pinned(c->hp);
+    double plan_rows = 0.0;  // rows per work item of single steps under the automatic launch
+    if (b->automatic()) {
+        const cudaError_t e = one_step_rows(b, &plan_rows);
+        if (e != cudaSuccess) return cuda_fail(nullptr, e, "occupancy");
+    }
     for (int m = 0; m < n; ++m) {
         lb_ctx *c = b->ctxs[m];
-        b->pinned += lbk::step_is_pinned(c->hp);
-        const int seg = b->seg_of[m] ? b->seg_of[m] : b->seg_rows;
+        int seg = b->seg_of[m] ? b->seg_of[m] : b->seg_rows;
+        if (plan_rows > 0.0) {
+            const int nseg = std::max(1, (int)std::lround(c->hp.nz / plan_rows));
+            seg = (c->hp.nz + nseg - 1) / nseg;
+        }
         cudaError_t e = lbk::batch_fill_desc(c->hp, c->dist[0], c->dist[1], b->step0[m], b->parity0[m], seg,
                                              b->tiles, c->status, b->hdesc.data() + (size_t)m * db);
         if (e != cudaSuccess) return cuda_fail(nullptr, e, "batch descriptor (tensor map)");
@@ -1007,7 +1036,7 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
     unsigned long long t = b->counter;  // batch step of the next launch
     const int n = (int)b->ctxs.size();
     auto step_others = [&](unsigned long long at, int from_counter) {
-        return lbk::launch_batch(b->storage, b->row_fetch, b->d_desc, b->d_prefix, n, b->total, b->d_ctl, b->wpb,
+        return lbk::launch_batch(b->storage, b->automatic() ? one_step_fetch(b) : b->row_fetch, b->d_desc, b->d_prefix, n, b->total, b->d_ctl, b->wpb,
                                  b->blocks, at, from_counter, b->stream);
     };
     auto step_pinned = [&](unsigned long long at, int from_counter) {
@@ -1025,7 +1054,7 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
             const int T = (int)(nsteps / m + (p < nsteps % m ? 1 : 0));
             const unsigned long long flip = (b->counter + (unsigned long long)p) & 1ULL;
             cudaError_t e;
-            if (T == 1 && b->tiles.strip && flip == (t & 1ULL))  // large lattices' single step: one warp per work item
+            if (T == 1 && b->tiles.strip && flip == (t & 1ULL))  // single step (one_step_rows)
                 e = step_others(t, 0);
             else
                 e = lbk::launch_batch_tiles(b->storage, b->tiles, T, b->d_desc, b->d_tprefix, n, b->htprefix.back(), t,
