@@ -17,6 +17,8 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <functional>
+#include <queue>
 #include <type_traits>
 #include <vector>
 
@@ -2167,13 +2169,61 @@ TileLaunch tile_plan(const HostParams &h, int T)
     return l;
 }
 
+// The lattice's tiles under a pass made for the whole batch: strips of equal
+// length, no longer than the pass's.
+static TileShape batch_tiles(const HostParams &h, const TileLaunch &l)
+{
+    TileShape sh = tile_shape(h, l.T, l.rows);
+    const int nt = tiles_along(h, sh), rows = h.flow[0] == 2 ? h.nz : std::max(1, h.nz - 2 * l.T);
+    return nt > 1 || h.flow[0] == 2 ? tile_shape(h, l.T, (rows + nt - 1) / nt + 2 * l.T) : sh;
+}
+
+// How much of the time of a pass on strips its resident blocks are busy, with
+// the strips started in order as blocks end; a strip takes its rows and the
+// filling of its ring.
+static double strips_busy(const std::vector<const HostParams *> &hs, const TileLaunch &l, int sms)
+{
+    const long long resident =
+        (long long)sms * tiles_per_sm(hs[0]->storage, tile_slots(true, l.T, 0, l.warps), l.warps, hs.size() > 1);
+    std::priority_queue<double, std::vector<double>, std::greater<double>> ends;
+    double work = 0.0, end = 0.0;
+    for (const HostParams *h : hs) {
+        const TileShape sh = batch_tiles(*h, l);
+        const bool per = h->flow[0] == 2;
+        for (int t = 0, nt = tiles_along(*h, sh); t < nt; ++t) {
+            const int rows = per ? std::min(sh.rs, h->nz - t * sh.rs) + 2 * sh.rm : std::min(sh.rows, h->nz - t * sh.rs);
+            for (int w = 0; w < sh.nw; ++w) {
+                double at = rows + l.warps;
+                work += at;
+                if ((long long)ends.size() >= resident) {
+                    at += ends.top();
+                    ends.pop();
+                }
+                ends.push(at);
+                end = std::max(end, at);
+            }
+        }
+    }
+    return work / (end * resident);
+}
+
+// The pass of a batch: tile_plan's for the tiles of all lattices together, but
+// single steps (T = 1, work items of equal length) where a few tall lattices
+// would keep the blocks waiting.  Per step, annuli of 32 to 512 columns and rows,
+// one batch alone and one of three side by side, which fill each other's gaps:
+// FP16, 128 of them (0.58 busy) 329 and 209 us on strips, 261 and 242 in single
+// steps, 64 (0.73) 148 and 105, 135 and 120; FP32, 96 (0.53) 265 and 158, 228 and
+// 215.  (One launch per step of 4-row items, before the strips: 324 and 316, 163
+// and 156, 284 and 277.)
 TileLaunch tile_plan_batch(const HostParams *const *h, int n)
 {
     std::vector<const HostParams *> tiled;  // pinned lattices take launches of their own
     for (int m = 0; m < n; ++m)
         if (!pinned_order(*h[m])) tiled.push_back(h[m]);
     if (tiled.empty()) tiled.assign(h, h + n);
-    return plan_tiles(Lattices{tiled.data(), (int)tiled.size(), h[0]->storage}, 0);
+    TileLaunch l = plan_tiles(Lattices{tiled.data(), (int)tiled.size(), h[0]->storage}, 0);
+    if (l.strip && strips_busy(tiled, l, sm_count()) < (h[0]->storage == ST_FP32 ? 0.5 : 0.6)) l.T = 1;
+    return l;
 }
 
 cudaError_t launch_tile(const HostParams &p, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
@@ -2272,15 +2322,6 @@ namespace lbk {
 
 size_t batch_desc_bytes() { return sizeof(BatchDesc); }
 size_t batch_ctl_bytes() { return sizeof(BatchCtl); }
-
-// The lattice's tiles under a pass made for the whole batch: strips of equal
-// length, no longer than the pass's.
-static TileShape batch_tiles(const HostParams &h, const TileLaunch &l)
-{
-    TileShape sh = tile_shape(h, l.T, l.rows);
-    const int nt = tiles_along(h, sh), rows = h.flow[0] == 2 ? h.nz : std::max(1, h.nz - 2 * l.T);
-    return nt > 1 || h.flow[0] == 2 ? tile_shape(h, l.T, (rows + nt - 1) / nt + 2 * l.T) : sh;
-}
 
 int batch_tile_count(const HostParams &h, const TileLaunch &l)
 {
