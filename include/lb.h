@@ -247,13 +247,16 @@ LB_EXPORT lb_status lb_get_step(const lb_ctx *ctx, int64_t *step);
  * a shared-memory ring, 3 = the same ring holding rows i - 1, i, i + 1 of
  * the step, read in place).  With all three 0 (the state after lb_create)
  * FP32 and 16-bit lattices are stepped on tiles held in shared memory, several
- * steps per launch; any other setting takes one launch per step.  Results do
- * not depend on the launch shape.  LB_ERR_ARG for values out of range. */
+ * steps per launch; any other setting takes one launch per step.  A lattice
+ * that keeps one fixed order of operations (lb_step) is fetched as with 3,
+ * whatever row_fetch, one launch per step.  Results do not depend on the launch
+ * shape.  LB_ERR_ARG for values out of range. */
 LB_EXPORT lb_status lb_set_launch(lb_ctx *ctx, int32_t seg_rows, int32_t warps_per_block, int32_t row_fetch);
 
 /* The launch the next single step uses, with the automatic choices resolved:
  * rows per z-segment, warps per block and row fetch (1, 2 or 3 as for
- * lb_set_launch; FP64 storage always 1).  NULL outputs are skipped. */
+ * lb_set_launch; FP64 storage always 1, a lattice with a fixed order of
+ * operations always 3).  NULL outputs are skipped. */
 LB_EXPORT lb_status lb_get_launch(const lb_ctx *ctx, int32_t *seg_rows, int32_t *warps_per_block,
                                   int32_t *row_fetch);
 

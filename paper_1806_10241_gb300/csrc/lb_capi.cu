@@ -698,7 +698,7 @@ lb_status lb_get_launch(const lb_ctx *ctx, int32_t *seg_rows, int32_t *warps_per
     if (!ctx) return fail(nullptr, LB_ERR_ARG, "ctx is NULL");
     if (seg_rows) *seg_rows = ctx->launch.seg_rows;
     if (warps_per_block) *warps_per_block = ctx->launch.warps_per_block;
-    if (row_fetch) *row_fetch = ctx->launch.use_tma + 1;
+    if (row_fetch) *row_fetch = lbk::step_is_pinned(ctx->hp) ? 3 : ctx->launch.use_tma + 1;
     return LB_OK;
 }
 
