@@ -361,11 +361,23 @@ cudaError_t copy_stream(lb_ctx *ctx)
     return e;
 }
 
-// n values of each of the five planes, N values apart on the host
-cudaError_t copy_planes(double *stage, double *host, size_t n, size_t N, bool to_device, cudaStream_t s)
+// Whether the driver knows the host array as page-locked.
+bool page_locked(const double *host)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type != cudaMemoryTypeUnregistered;
+}
+
+// n values of each of the five planes, N values apart on the host: one strided
+// copy (rows) or a copy per plane
+cudaError_t copy_planes(double *stage, double *host, size_t n, size_t N, bool to_device, bool strided, cudaStream_t s)
 {
     const size_t w = n * sizeof(double), p = N * sizeof(double);
-    if (p <= (size_t)INT_MAX)
+    if (strided && p <= (size_t)INT_MAX)
         return to_device ? cudaMemcpy2DAsync(stage, w, host, p, w, 5, cudaMemcpyHostToDevice, s)
                          : cudaMemcpy2DAsync(host, p, stage, w, w, 5, cudaMemcpyDeviceToHost, s);
     for (int q = 0; q < 5; ++q) {
@@ -382,8 +394,12 @@ cudaError_t copy_planes(double *stage, double *host, size_t n, size_t N, bool to
 // chunk with the kernels of its neighbours: the copies go to a second stream,
 // ordered against the context's stream by events, in up to four parts of the
 // staging area (512 x 1024 FP32: fields in and out 480 us before, 285 us
-// now; the copies alone take 233 us).  kernel(stage, r0, r1) queues the work of
-// a chunk on the context's stream.
+// now; the copies alone take 233 us).  A large array that is not page-locked is
+// filled with one copy per plane instead, as many rows at a time as the staging
+// area holds: strided copies into it are slow in chunks (1024 x 2048 FP32: 827
+// us into memory used before, 577 so) and where its pages are new (72 ms, mostly
+// 8 ms so).  kernel(stage, r0, r1) queues the work of a chunk on the context's
+// stream.
 template <typename Kernel>
 lb_status exchange(lb_ctx *ctx, double *host, bool to_device, const char *what, Kernel kernel)
 {
@@ -394,7 +410,8 @@ lb_status exchange(lb_ctx *ctx, double *host, bool to_device, const char *what, 
     const int nr = ctx->hp.nr, nz = ctx->hp.nz;
     const size_t N = (size_t)nr * nz, total = 5 * N * sizeof(double);
     int chunk = rows, parts = 1;
-    const bool large = total >= kOverlapBytes && rows >= 2, overlap = large && copy_stream(ctx) == cudaSuccess;
+    const bool paged = !to_device && total >= kOverlapBytes && !page_locked(host);
+    const bool large = total >= kOverlapBytes && rows >= 2 && !paged, overlap = large && copy_stream(ctx) == cudaSuccess;
     if (large && !overlap) cudaGetLastError();  // without a copy stream the chunks follow each other
     if (overlap) {
         // chunks of about 5 MB, at most 32: smaller ones leave the FP64 kernels'
@@ -422,7 +439,7 @@ lb_status exchange(lb_ctx *ctx, double *host, bool to_device, const char *what, 
         double *at = stage + q * part;
         if (to_device) {
             if (i >= parts && parts > 1) e = cudaStreamWaitEvent(c, ctx->ev_kernel[q], 0);
-            if (e == cudaSuccess) e = copy_planes(at, host + (size_t)r0 * nr, n, N, true, c);
+            if (e == cudaSuccess) e = copy_planes(at, host + (size_t)r0 * nr, n, N, true, true, c);
             then(ctx->ev_copy[q], c, s);
             if (e == cudaSuccess) e = kernel(at, r0, r1);
             if (e == cudaSuccess && parts > 1) e = cudaEventRecord(ctx->ev_kernel[q], s);
@@ -430,7 +447,7 @@ lb_status exchange(lb_ctx *ctx, double *host, bool to_device, const char *what, 
             if (i >= parts && parts > 1) e = cudaStreamWaitEvent(s, ctx->ev_copy[q], 0);
             if (e == cudaSuccess) e = kernel(at, r0, r1);
             then(ctx->ev_kernel[q], s, c);
-            if (e == cudaSuccess) e = copy_planes(at, host + (size_t)r0 * nr, n, N, false, c);
+            if (e == cudaSuccess) e = copy_planes(at, host + (size_t)r0 * nr, n, N, false, !paged, c);
             if (e == cudaSuccess && parts > 1) e = cudaEventRecord(ctx->ev_copy[q], c);
         }
     }

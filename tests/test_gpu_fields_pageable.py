@@ -1,0 +1,45 @@
+"""Fields into host memory that is not page-locked: the values that page-locked
+memory gets, and not much later."""
+import time
+
+import numpy as np
+import pytest
+
+from paper_1806_10241_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1806_10241_gb300 import build
+    build.build()
+
+
+def _best(fn):
+    times = []
+    for _ in range(12):
+        t = time.perf_counter()
+        fn()
+        times.append(time.perf_counter() - t)
+    return min(times[2:])
+
+
+@pytest.mark.parametrize("nr,nz,storage", [(1024, 2048, "fp32"), (1023, 2047, "fp16"), (700, 1501, "fp64")])
+def test_pageable_fields(nr, nz, storage):
+    from paper_1806_10241_gb300.solver import Solver
+    c = W.swirling_cylinder(nr=nr, nz=nz, Re=200.0, Ra=1e4, amp=1e-3, seed=1)
+    s = Solver(c.params, storage=storage)
+    s.init_fields(c.fields)
+    s.step(4)
+    pinned = torch.empty(5, nz, nr, dtype=torch.float64, pin_memory=True).numpy()
+    plain = np.zeros((5, nz, nr))
+    s.fields(out=pinned)
+    s.fields(out=plain)
+    assert np.array_equal(pinned, plain) and np.array_equal(s.fields(), plain)
+    # one kernel and then the copies, where page-locked memory has them overlap: 1.2 times as long; 1.7 with strided
+    # copies of chunks
+    assert _best(lambda: s.fields(out=plain)) < 1.45 * _best(lambda: s.fields(out=pinned))
