@@ -979,7 +979,7 @@ __global__ void __launch_bounds__(128) k_psi(const double *__restrict__ ux, doub
 // node's stored state once, node(i, c, out) its pre-collision state.  (A warp
 // marching 32 rows of 30 columns on its own, as before, is a serial chain of
 // 32 row updates; these are four nodes per thread and round, all independent: the
-// diagnostics of 1024 x 2048 FP32 took 220 us and take 122.)
+// diagnostics of 1024 x 2048 FP32 took 220 us and take 110.)
 constexpr int kBlockCols = 128, kBlockChunk = 8, kBlockThreads = 256, kBlockPitch = kBlockCols + 2;
 template <typename C> constexpr size_t kBlockSmem = (size_t)(kBlockChunk + 2) * 4 * kBlockPitch * sizeof(C);
 
@@ -1077,17 +1077,24 @@ __device__ __forceinline__ void block_fields(const KP<C> &k, const S *__restrict
     }
 }
 
+// Registers for four of these blocks on an SM, where an FP32 kernel has two by
+// itself, as they wait for their loads: fields of 2048 x 2048 FP32 290 us in all
+// as lb_stream_function takes them, 267 with three, 251 so; diagnostics of 1024 x
+// 2048 FP32 128, 122 and 110 us, of 64 annuli in one FP16 batch, whose kernel also
+// takes the lattice's parameters from shared memory, 538, 464 and 445 us.
+template <typename C> constexpr int kBlocksPerSm = std::is_same<C, float>::value ? 4 : 1;
+
 // Pre-collision fields of rows [row0, row1) as doubles, out[5][row1 - row0][nr]:
-// a block per kBlockChunk rows.
+// a block per `rows` rows.
 template <typename S, typename C>
-__global__ void __launch_bounds__(kBlockThreads) k_fields(const __grid_constant__ KP<C> k, const S *__restrict__ src,
-                                                          double *__restrict__ out, int row0, int row1, int nbx)
+__global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<C>) k_fields(const __grid_constant__ KP<C> k, const S *__restrict__ src,
+                                                          double *__restrict__ out, int row0, int row1, int nbx, int rows)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    const int s = row0 + (int)(blockIdx.x / nbx) * kBlockChunk;
+    const int s = row0 + (int)(blockIdx.x / nbx) * rows;
     const long long n = (long long)(row1 - row0) * k.nr;  // plane stride of the output chunk
     block_fields<S, C>(
-        k, src, (int)(blockIdx.x % nbx) * kBlockCols, s, min(row1, s + kBlockChunk) - s, reinterpret_cast<C *>(smem),
+        k, src, (int)(blockIdx.x % nbx) * kBlockCols, s, min(row1, s + rows) - s, reinterpret_cast<C *>(smem),
         [](int, int, const PM<C> &) {},
         [&](int i, int c, const NodeOut<C> &o) {
             double *p = out + (long long)(i - row0) * k.nr + c;
@@ -1142,11 +1149,6 @@ template <typename C> struct NodeMax {
     }
 };
 
-// Registers for three blocks on an SM, where FP32 has two by itself: 1024 x 2048
-// 128 -> 122 us; 64 annuli in one batch, whose kernel also takes the lattice's
-// parameters from shared memory, 538 -> 464 us (before the blocks 498 us).
-template <typename C> constexpr int kDiagBlocks = std::is_same<C, float>::value ? 3 : 1;
-
 // Diagnostics of block (bx, by) of a grid gx blocks wide, seg_rows rows each:
 // partial sums in a fixed order, and the temperatures next to the walls in
 // strips: rows 0, 1, nz - 2, nz - 1 (4 x nr values), then columns 0, 1, nr - 2,
@@ -1191,7 +1193,7 @@ __device__ __forceinline__ void diag_block(const KP<C> &k, const S *__restrict__
 }
 
 template <typename S, typename C>
-__global__ void __launch_bounds__(kBlockThreads, kDiagBlocks<C>) k_diag(const __grid_constant__ KP<C> k, const S *__restrict__ src,
+__global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<C>) k_diag(const __grid_constant__ KP<C> k, const S *__restrict__ src,
                                                         double *__restrict__ partial, double *__restrict__ strips,
                                                         int seg_rows, int gx)
 {
@@ -1634,7 +1636,7 @@ struct BatchDiag {
 };
 
 template <typename S>
-__global__ void __launch_bounds__(kBlockThreads, kDiagBlocks<float>) k_batch_diag(const BatchDesc *__restrict__ d,
+__global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<float>) k_batch_diag(const BatchDesc *__restrict__ d,
                                                     const BatchDiag *__restrict__ dd, const int *__restrict__ prefix,
                                                     int n, unsigned long long t)
 {
@@ -1879,9 +1881,14 @@ template <typename S, typename C>
 cudaError_t fields_t(const HostParams &h, const void *src, double *out, int row0, int row1, cudaStream_t s)
 {
     const int nbx = (h.nr + kBlockCols - 1) / kBlockCols;
-    const long long blocks = (long long)nbx * ((row1 - row0 + kBlockChunk - 1) / kBlockChunk);
-    if (blocks > INT_MAX) return cudaErrorInvalidValue;
-    k_fields<S, C><<<(unsigned)blocks, kBlockThreads, kBlockSmem<C>, s>>>(make_kp<C>(h), (const S *)src, out, row0, row1, nbx);
+    // 16 rows, 8 on few blocks (1024 x 2048 FP64: 941 us as lb_stream_function takes
+    // them, 977 with 8 throughout)
+    int rows = 2 * kBlockChunk;
+    auto blocks = [&]() { return (long long)nbx * ((row1 - row0 + rows - 1) / rows); };
+    while (rows > kBlockChunk && blocks() < 4 * sm_count()) rows /= 2;
+    if (blocks() > INT_MAX) return cudaErrorInvalidValue;
+    k_fields<S, C><<<(unsigned)blocks(), kBlockThreads, kBlockSmem<C>, s>>>(make_kp<C>(h), (const S *)src, out, row0, row1,
+                                                                            nbx, rows);
     return cudaGetLastError();
 }
 
