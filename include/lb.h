@@ -297,11 +297,13 @@ LB_EXPORT lb_status lb_diagnostics_static(const lb_grid_desc *desc, const lb_par
  * parameters) together.  Under the settings it starts with (4 rows per
  * z-segment, 1 warp per block, row fetch 3, no per-lattice segments) that is
  * the automatic launch: all lattices' tiles in one launch of several steps, as
- * lb_step takes them, and for single steps that are left over work items of
- * equal length over all lattices.  Any other setting takes one kernel launch per step over
- * all their 64-column x z-segment tiles (work items numbered by a prefix sum
- * over the lattices), replayed from a CUDA graph of graph_steps launches when
- * the stream is not the legacy default stream.  Each lattice's
+ * lb_step takes them, and for single steps that are left over, or where the
+ * lattices are too uneven for common tiles, work items of equal length over all
+ * lattices.  Any other setting takes one kernel launch per step over all their
+ * 64-column x z-segment tiles (work items numbered by a prefix sum over the
+ * lattices), replayed from a CUDA graph of graph_steps launches when the stream
+ * is not the legacy default stream; so do 4 rows, 1 warp and row fetch 3 with
+ * lb_batch_set_segments giving 4 for every lattice.  Each lattice's
  * update is the one lb_step performs (same arithmetic, same rounding bits).
  * While a batch exists its lattices are stepped through it only; their step
  * counters and current buffers follow the batch, so lb_diagnostics and the

@@ -9,8 +9,9 @@
 //
 // Kernels: the FP32 / 16-bit step on column pairs (lb_pair.cuh: one launch per
 // step, rows marched by a warp; lb_tile.cuh: several steps per launch on tiles
-// in shared memory), the FP64 step (k_step64), the pre-collision fields and the
-// diagnostics (block_fields), and the exchange with the host.
+// in shared memory) and the FP64 step (k_step64), which share the node update of
+// lb_node.cuh, the pre-collision fields and the diagnostics (block_fields), and
+// the exchange with the host.
 #include <algorithm>
 #include <atomic>
 #include <climits>
@@ -1681,10 +1682,10 @@ __global__ void __launch_bounds__(256) k_batch_diag_final(const BatchDesc *__res
 // Shared memory: the block's slots, then the lattice's parameters.  The plan is
 // tile_plan's for the tiles of all lattices together.  With three
 // batches on streams of their own, per step: 40 lattices of 64 to 128 columns
-// in FP32 19.0 us with the best one-step launch (segment plan of one wave),
-// 15.0 us on strips of two steps; 64 annuli of 32 to 512 rows and columns in
-// FP16 156 us with 4-row segments, 94 us on strips of four steps (18.8 and 131
-// us for one batch alone, whose last wave nothing fills).  Bound as the single
+// in FP32 19.6 us in single steps, 15.2 us on strips of two steps; 64 annuli of
+// 32 to 512 rows and columns in FP16 156 us with 4-row segments, 120 us in single
+// steps, 105 us on strips of four (19.1 and 148 us for one batch alone, whose
+// last wave nothing fills).  Bound as the single
 // lattice's strips, and by the columns that a window of a narrow lattice leaves
 // empty (a fifth of them in the first batch).
 template <typename S, bool kStrip>
@@ -2157,7 +2158,7 @@ TileLaunch plan_tiles(const Lattices &ls, int T)
 // - Strips beyond (512 x 512 FP32: 7.5 us, tiles 8.0).  FP32: two steps (1024 x
 //   2048: 39.4 us as one launch; three 45.2, four 42.5; 512 x 1024: 12.5, 12.7,
 //   12.8).  16-bit: four (1024 x 2048 FP16: 41.5 us; three 43.0, two 43.1; 512 x
-//   1024: 12.2, 12.8, 12.8).  Six (eight) warps per block while the strips are
+//   1024: 12.2, 12.8, 12.8; with cheaper rounding words, 44.6 and 13.4 now).  Six (eight) warps per block while the strips are
 //   short, four and one more block per SM from 40 (60) rows on (512 x 1024
 //   FP32: 12.5 against 13.1 us; 1024 x 2048: 42.4 against 39.4; two, three or
 //   five warps: 8-20 % slower).

@@ -90,7 +90,7 @@ __device__ __forceinline__ F2 sel2(bool px, bool py, F2 a, F2 b)  // per compone
 // sequence (Marsaglia 2003).  The conversion takes bits 0-12 and 16-28 of a
 // word for the two FP16 elements, 0-15 and 16-31 for BF16.  A linear
 // congruential sequence from the same seed takes one operation a word instead
-// of six (1024 x 2048 FP16: 41.4 us per step, 44.4 with these), but its bits
+// of six (1024 x 2048 FP16: 41.4 us per step, 44.6 with these), but its bits
 // 0-12 are a function of the low 13 bits of the seed alone, correlated over the
 // planes of a node, and results were further from FP64 by some per cent.
 __device__ __forceinline__ uint32_t pcg_hash(uint32_t v)

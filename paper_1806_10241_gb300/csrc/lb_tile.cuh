@@ -306,7 +306,7 @@ __device__ __forceinline__ void tile_steps(const KP<float> &k, const CUtensorMap
 // the lower neighbours' states).  1024 x 2048: FP32 52.0 us per step with one
 // step per launch, 40.6 us with strips of two steps; what bounds it is the
 // latency of dependent instructions at 12 warps per SM (47 % issue), not
-// memory.  FP16 49.1 -> 44.4 us at that size.
+// memory.  FP16 49.1 -> 44.6 us at that size.
 // kRunning: the position in the ring, the lattice row and the limits of the
 // active rows run along with t instead of being formed from it (10 % fewer
 // instructions in 16-bit storage, 2 % in FP32: 41.3 -> 39.8 us).  FP32 batches,
