@@ -366,7 +366,8 @@ def batch_measure(instances, lo, hi, storage, steps, warmup, graph_steps, oracle
     med = sorted(ms)[len(ms) // 2]
     peaks, peak_kind = measured_peaks()
     bpn = BYTES_PER_NODE[storage]
-    achieved = bpn * nodes * steps / (med * 1e-3) / 1e9
+    passes = launches if kernel.startswith("k_batch_tiles") else steps  # over memory
+    achieved = bpn * nodes * passes / (med * 1e-3) / 1e9
     order = sorted(range(len(cases)), key=lambda m: cases[m].nr * cases[m].nz)
     pick = [m for m in order if cases[m].nr <= 64 and cases[m].nz <= 64] or order[:oracle_instances]
     nu = []
@@ -395,7 +396,7 @@ def batch_measure(instances, lo, hi, storage, steps, warmup, graph_steps, oracle
                               "working set %.0f MB fits in the L2: an L2-resident rate" % (bpn * nodes / 1e6))},
             "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": float(peaks["hbm_gbs"]),
                          "unit": "GB/s", "frac": round(achieved / float(peaks["hbm_gbs"]), 4), "traffic": None,
-                         "peak_kind": peak_kind, "algorithmic_bytes_per_node": bpn,
+                         "peak_kind": peak_kind, "algorithmic_bytes_per_node": round(bpn * passes / steps, 1),
                          "kernel": kernel},
             "gpu_launches": launches * repeats, "clocks": clocks.summary(t0, t1) if clocks is not None else None,
             "nu_vs_oracle": nu, "dtype": DTYPE[storage]}
@@ -554,8 +555,8 @@ def storage_forms(case, steps, warmup, repeats, sm_mhz=None):
         bpn = BYTES_PER_NODE[storage]
         out[storage] = {"value": round(nodes * steps / (med * 1e3), 1), "unit": "MLUPS",
                         "ms_per_step": round(med / steps, 5), "launch": list(g.get_launch()),
-                        "roofline_frac": round(bpn * nodes / (med / steps * 1e-3) / 1e9 / peak, 4),
-                        "algorithmic_bytes_per_node": bpn, "nu_avg": d["nu_avg"],
+                        "roofline_frac": round(bpn / STEPS_PER_PASS[storage] * nodes / (med / steps * 1e-3) / 1e9 / peak, 4),
+                        "algorithmic_bytes_per_node": bpn / STEPS_PER_PASS[storage], "nu_avg": d["nu_avg"],
                         "steps_total": warmup + steps * repeats, "status": d["status"]}
         kname = kernel_name(storage)
         iss = issue_roofline(f"{kname}_{storage}_{case.nr}x{case.nz}", med / steps, sm_mhz)
@@ -744,7 +745,8 @@ def main():
 
     peaks, peak_kind = measured_peaks()
     bpn = BYTES_PER_NODE[args.storage]
-    achieved = bpn * nodes / (ms_per_step * 1e-3) / 1e9  # GB/s of one launch
+    per_step = bpn / STEPS_PER_PASS[args.storage]  # the state read and written once per pass
+    achieved = per_step * nodes / (ms_per_step * 1e-3) / 1e9
     peak = float(peaks["hbm_gbs"])
     seg, wpb, fetch = g.get_launch()
     kname = kernel_name(args.storage)
@@ -755,9 +757,9 @@ def main():
                 "frac_of_nominal_7900_GBs": round(achieved / 7900.0, 4),
                 "peak_kind": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured"
                 else "fallback 6.8 TB/s",
-                "algorithmic_bytes_per_node": bpn,
+                "algorithmic_bytes_per_node": per_step,
                 "kernel": f"{kname} (fused stream + sources + collisions + boundaries; {STEPS_PER_PASS[args.storage]} "
-                          "steps per pass over memory: the fraction on the bytes of one step may exceed 1)"}
+                          "steps per pass over memory, whose bytes count once)"}
 
     twin = Solver(case.params, storage=args.storage, device=dev, stream=torch.cuda.Stream(dev))
     launches = count_kernels(twin.stream, lambda: twin.step(args.steps))
