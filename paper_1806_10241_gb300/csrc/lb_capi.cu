@@ -525,7 +525,7 @@ lb_status lb_get_fields(lb_ctx *ctx, double *host_fields)
     if (st != LB_OK) return st;
     if (!host_fields) return fail(ctx, LB_ERR_ARG, "host_fields is NULL");
     return exchange(ctx, host_fields, false, "fields", [&](double *stage, int r0, int r1) {
-        return lbk::launch_fields(ctx->hp, ctx->dist[ctx->cur], stage, r0, r1, ctx->stream);
+        return lbk::launch_fields(ctx->hp, ctx->dist[ctx->cur], stage, r0, r1, false, ctx->stream);
     });
 }
 
@@ -553,8 +553,8 @@ lb_status lb_stream_function(lb_ctx *ctx, double *host_psi, double *psi_max)
     for (int r0 = 0; r0 < nz; r0 += rows) {
         const int r1 = r0 + rows < nz ? r0 + rows : nz;
         const size_t n = (size_t)(r1 - r0) * nr;
-        // fields into planes 0..4 of the stage; Psi over plane 0, row maxima over plane 2
-        cudaError_t e = lbk::launch_fields(ctx->hp, ctx->dist[ctx->cur], stage, r0, r1, ctx->stream);
+        // u_x into plane 1 of the stage, Psi into plane 0, row maxima into plane 2
+        cudaError_t e = lbk::launch_fields(ctx->hp, ctx->dist[ctx->cur], stage, r0, r1, true, ctx->stream);
         if (e == cudaSuccess)
             e = lbk::launch_psi(stage + n, stage, stage + 2 * n, r1 - r0, nr, ctx->hp.r0, ctx->stream);
         if (e == cudaSuccess && host_psi)

@@ -93,8 +93,10 @@ inline int64_t pass_count(int64_t n, int T)
 // lattice's device word for it (k_tiles).
 cudaError_t launch_tile(const HostParams &p, const TileLaunch &l, const void *tmap, void *dst, unsigned long long step,
                         int *status, unsigned *begun, unsigned pass, cudaStream_t s);
-// Pre-collision fields of rows [row0, row1) into out[5][row1-row0][nr] (double).
-cudaError_t launch_fields(const HostParams &p, const void *src, double *out, int row0, int row1, cudaStream_t s);
+// Pre-collision fields of rows [row0, row1) into out[5][row1-row0][nr] (double);
+// only_ux: plane 1 alone.
+cudaError_t launch_fields(const HostParams &p, const void *src, double *out, int row0, int row1, bool only_ux,
+                          cudaStream_t s);
 // Bounded-wait self-test: a warp polls an mbarrier nothing arrives at,
 // `polls` times, and sets *status to LB_ERR_TIMEOUT.
 cudaError_t launch_wait_selftest(int *status, int polls, cudaStream_t s);

@@ -1080,16 +1080,17 @@ __device__ __forceinline__ void block_fields(const KP<C> &k, const S *__restrict
 
 // Registers for four of these blocks on an SM, where an FP32 kernel has two by
 // itself, as they wait for their loads: fields of 2048 x 2048 FP32 290 us in all
-// as lb_stream_function takes them, 267 with three, 251 so; diagnostics of 1024 x
+// as lb_stream_function took them, 267 with three, 251 so (238 storing u_x alone); diagnostics of 1024 x
 // 2048 FP32 128, 122 and 110 us, of 64 annuli in one FP16 batch, whose kernel also
 // takes the lattice's parameters from shared memory, 538, 464 and 445 us.
 template <typename C> constexpr int kBlocksPerSm = std::is_same<C, float>::value ? 4 : 1;
 
-// Pre-collision fields of rows [row0, row1) as doubles, out[5][row1 - row0][nr]:
-// a block per `rows` rows.
+// Pre-collision fields of rows [row0, row1) as doubles, out[5][row1 - row0][nr],
+// or u_x alone (plane 1): a block per `rows` rows.
 template <typename S, typename C>
 __global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<C>) k_fields(const __grid_constant__ KP<C> k, const S *__restrict__ src,
-                                                          double *__restrict__ out, int row0, int row1, int nbx, int rows)
+                                                          double *__restrict__ out, int row0, int row1, int nbx, int rows,
+                                                          int only_ux)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     const int s = row0 + (int)(blockIdx.x / nbx) * rows;
@@ -1099,8 +1100,9 @@ __global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<C>) k_fields(const
         [](int, int, const PM<C> &) {},
         [&](int i, int c, const NodeOut<C> &o) {
             double *p = out + (long long)(i - row0) * k.nr + c;
-            p[0] = (double)o.rho;
             p[n] = (double)o.ux;
+            if (only_ux) return;
+            p[0] = (double)o.rho;
             p[2 * n] = (double)o.uy;
             p[3 * n] = (double)o.ut;
             p[4 * n] = (double)o.T;
@@ -1879,7 +1881,7 @@ cudaError_t step_t(const HostParams &h, const Launch &l, const void *src, void *
 }
 
 template <typename S, typename C>
-cudaError_t fields_t(const HostParams &h, const void *src, double *out, int row0, int row1, cudaStream_t s)
+cudaError_t fields_t(const HostParams &h, const void *src, double *out, int row0, int row1, int only_ux, cudaStream_t s)
 {
     const int nbx = (h.nr + kBlockCols - 1) / kBlockCols;
     // 16 rows, 8 on few blocks (1024 x 2048 FP64: 941 us as lb_stream_function takes
@@ -1889,7 +1891,7 @@ cudaError_t fields_t(const HostParams &h, const void *src, double *out, int row0
     while (rows > kBlockChunk && blocks() < 4 * sm_count()) rows /= 2;
     if (blocks() > INT_MAX) return cudaErrorInvalidValue;
     k_fields<S, C><<<(unsigned)blocks(), kBlockThreads, kBlockSmem<C>, s>>>(make_kp<C>(h), (const S *)src, out, row0, row1,
-                                                                            nbx, rows);
+                                                                            nbx, rows, only_ux);
     return cudaGetLastError();
 }
 
@@ -2258,9 +2260,10 @@ cudaError_t launch_psi(const double *ux, double *psi, double *rowmax, int nrows,
     return cudaGetLastError();
 }
 
-cudaError_t launch_fields(const HostParams &p, const void *src, double *out, int row0, int row1, cudaStream_t s)
+cudaError_t launch_fields(const HostParams &p, const void *src, double *out, int row0, int row1, bool only_ux,
+                          cudaStream_t s)
 {
-    DISPATCH(p, (fields_t<S, C>(p, src, out, row0, row1, s)));
+    DISPATCH(p, (fields_t<S, C>(p, src, out, row0, row1, only_ux, s)));
 }
 
 // Blocks of 32 rows, fewer while there would be less than two blocks per SM,
