@@ -348,6 +348,7 @@ lb_status lb_set_params(lb_ctx *ctx, const lb_params *p)
 namespace {
 
 constexpr size_t kOverlapBytes = (size_t)4 << 20;  // exchanges below this are copied in one piece
+constexpr size_t kStridedBytes = (size_t)1 << 20;  // and below this by one strided copy from and to any memory
 
 cudaError_t copy_stream(lb_ctx *ctx)
 {
@@ -394,12 +395,12 @@ cudaError_t copy_planes(double *stage, double *host, size_t n, size_t N, bool to
 // chunk with the kernels of its neighbours: the copies go to a second stream,
 // ordered against the context's stream by events, in up to four parts of the
 // staging area (512 x 1024 FP32: fields in and out 480 us before, 285 us
-// now; the copies alone take 233 us).  A large array that is not page-locked is
-// filled with one copy per plane instead, as many rows at a time as the staging
-// area holds: strided copies into it are slow in chunks (1024 x 2048 FP32: 827
-// us into memory used before, 577 so) and where its pages are new (72 ms, mostly
-// 8 ms so).  kernel(stage, r0, r1) queues the work of a chunk on the context's
-// stream.
+// now; the copies alone take 233 us).  An array that is not page-locked is
+// copied plane by plane instead, as many rows at a time as the staging area
+// holds: strided copies are slow where its pages are new, as in fields at rest
+// from a zeroed array (272 x 272: 1.1 ms in and 2.8 ms out, plane by plane 0.48 and
+// 0.72) and, out, in chunks (1024 x 2048 FP32: 827 us into memory used before, 563
+// so).  kernel(stage, r0, r1) queues the work of a chunk on the context's stream.
 template <typename Kernel>
 lb_status exchange(lb_ctx *ctx, double *host, bool to_device, const char *what, Kernel kernel)
 {
@@ -410,7 +411,7 @@ lb_status exchange(lb_ctx *ctx, double *host, bool to_device, const char *what, 
     const int nr = ctx->hp.nr, nz = ctx->hp.nz;
     const size_t N = (size_t)nr * nz, total = 5 * N * sizeof(double);
     int chunk = rows, parts = 1;
-    const bool paged = !to_device && total >= kOverlapBytes && !page_locked(host);
+    const bool paged = total >= kStridedBytes && !page_locked(host);
     const bool large = total >= kOverlapBytes && rows >= 2 && !paged, overlap = large && copy_stream(ctx) == cudaSuccess;
     if (large && !overlap) cudaGetLastError();  // without a copy stream the chunks follow each other
     if (overlap) {
@@ -439,7 +440,7 @@ lb_status exchange(lb_ctx *ctx, double *host, bool to_device, const char *what, 
         double *at = stage + q * part;
         if (to_device) {
             if (i >= parts && parts > 1) e = cudaStreamWaitEvent(c, ctx->ev_kernel[q], 0);
-            if (e == cudaSuccess) e = copy_planes(at, host + (size_t)r0 * nr, n, N, true, true, c);
+            if (e == cudaSuccess) e = copy_planes(at, host + (size_t)r0 * nr, n, N, true, !paged, c);
             then(ctx->ev_copy[q], c, s);
             if (e == cudaSuccess) e = kernel(at, r0, r1);
             if (e == cudaSuccess && parts > 1) e = cudaEventRecord(ctx->ev_kernel[q], s);
