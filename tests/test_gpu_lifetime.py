@@ -33,28 +33,41 @@ def _solver(stream):
     return s
 
 
+def _while_busy(attempt):
+    """attempt() -> (whether its work was still queued, whether its memory was apart), until the first holds."""
+    for _ in range(5):
+        busy, apart = attempt()
+        torch.cuda.synchronize()
+        if busy:
+            return apart
+    pytest.skip("the work was done too soon")
+
+
 def test_lattice_dropped_with_work_queued():
-    stream = torch.cuda.Stream()
-    s = _solver(stream)
-    s.step(20000)  # some ten milliseconds are still queued on return
-    old, n = _range(s.buffer), s.buffer.numel()
-    del s
-    again = torch.empty(n, dtype=torch.uint8, device="cuda")
-    assert not stream.query()
-    assert _apart(again, old)
-    torch.cuda.synchronize()
+    def attempt():
+        stream = torch.cuda.Stream()
+        s = _solver(stream)
+        s.step(20000)  # some ten milliseconds are still queued on return
+        old, n = _range(s.buffer), s.buffer.numel()
+        del s
+        again = torch.empty(n, dtype=torch.uint8, device="cuda")
+        return not stream.query(), _apart(again, old)
+
+    assert _while_busy(attempt)
 
 
 def test_batch_dropped_with_work_queued():
     from paper_1806_10241_gb300.batch import Batch
-    stream = torch.cuda.Stream()
-    sols = [_solver(torch.cuda.current_stream()) for _ in range(2)]
-    b = Batch(sols, stream=stream)
-    b.step(20000)
-    buffers = [b.buffer] + [s.buffer for s in sols]
-    old, sizes = [_range(t) for t in buffers], [t.numel() for t in buffers]
-    del b, sols, buffers
-    again = [torch.empty(n, dtype=torch.uint8, device="cuda") for n in sizes]
-    assert not stream.query()
-    assert all(_apart(t, o) for t in again for o in old)
-    torch.cuda.synchronize()
+
+    def attempt():
+        stream = torch.cuda.Stream()
+        sols = [_solver(torch.cuda.current_stream()) for _ in range(2)]
+        b = Batch(sols, stream=stream)
+        b.step(20000)
+        buffers = [b.buffer] + [s.buffer for s in sols]
+        old, sizes = [_range(t) for t in buffers], [t.numel() for t in buffers]
+        del b, sols, buffers
+        again = [torch.empty(n, dtype=torch.uint8, device="cuda") for n in sizes]
+        return not stream.query(), all(_apart(t, o) for t in again for o in old)
+
+    assert _while_busy(attempt)
