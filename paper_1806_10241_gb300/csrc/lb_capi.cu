@@ -1054,8 +1054,8 @@ lb_status lb_batch_step(lb_batch *b, int32_t nsteps)
     unsigned long long t = b->counter;  // batch step of the next launch
     const int n = (int)b->ctxs.size();
     auto step_others = [&](unsigned long long at, int from_counter) {
-        return lbk::launch_batch(b->storage, b->automatic() ? one_step_fetch(b) : b->row_fetch, b->d_desc, b->d_prefix, n, b->total, b->d_ctl, b->wpb,
-                                 b->blocks, at, from_counter, b->stream);
+        return lbk::launch_batch(b->storage, b->automatic() ? one_step_fetch(b) : b->row_fetch, b->d_desc, b->d_prefix,
+                                 n, b->total, b->d_ctl, b->wpb, b->blocks, at, from_counter, b->stream);
     };
     auto step_pinned = [&](unsigned long long at, int from_counter) {
         return lbk::launch_batch_pinned(b->storage, b->d_desc, b->d_prefix, n, b->total, b->d_ctl, b->wpb, at,

@@ -1080,17 +1080,18 @@ __device__ __forceinline__ void block_fields(const KP<C> &k, const S *__restrict
 
 // Registers for four of these blocks on an SM, where an FP32 kernel has two by
 // itself, as they wait for their loads: fields of 2048 x 2048 FP32 290 us in all
-// as lb_stream_function took them, 267 with three, 251 so (238 storing u_x alone); diagnostics of 1024 x
-// 2048 FP32 128, 122 and 110 us, of 64 annuli in one FP16 batch, whose kernel also
-// takes the lattice's parameters from shared memory, 538, 464 and 445 us.
+// as lb_stream_function took them, 267 with three, 251 so (238 storing u_x
+// alone); diagnostics of 1024 x 2048 FP32 128, 122 and 110 us, of 64 annuli in one
+// FP16 batch, whose kernel also takes the lattice's parameters from shared memory,
+// 538, 464 and 445 us.
 template <typename C> constexpr int kBlocksPerSm = std::is_same<C, float>::value ? 4 : 1;
 
 // Pre-collision fields of rows [row0, row1) as doubles, out[5][row1 - row0][nr],
 // or u_x alone (plane 1): a block per `rows` rows.
 template <typename S, typename C>
-__global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<C>) k_fields(const __grid_constant__ KP<C> k, const S *__restrict__ src,
-                                                          double *__restrict__ out, int row0, int row1, int nbx, int rows,
-                                                          int only_ux)
+__global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<C>)
+    k_fields(const __grid_constant__ KP<C> k, const S *__restrict__ src, double *__restrict__ out, int row0, int row1,
+             int nbx, int rows, int only_ux)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     const int s = row0 + (int)(blockIdx.x / nbx) * rows;
@@ -1196,9 +1197,9 @@ __device__ __forceinline__ void diag_block(const KP<C> &k, const S *__restrict__
 }
 
 template <typename S, typename C>
-__global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<C>) k_diag(const __grid_constant__ KP<C> k, const S *__restrict__ src,
-                                                        double *__restrict__ partial, double *__restrict__ strips,
-                                                        int seg_rows, int gx)
+__global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<C>)
+    k_diag(const __grid_constant__ KP<C> k, const S *__restrict__ src, double *__restrict__ partial,
+           double *__restrict__ strips, int seg_rows, int gx)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     diag_block<S, C>(k, src, partial, strips, seg_rows, blockIdx.x % gx, blockIdx.x / gx, gx, reinterpret_cast<C *>(smem));
@@ -1639,9 +1640,9 @@ struct BatchDiag {
 };
 
 template <typename S>
-__global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<float>) k_batch_diag(const BatchDesc *__restrict__ d,
-                                                    const BatchDiag *__restrict__ dd, const int *__restrict__ prefix,
-                                                    int n, unsigned long long t)
+__global__ void __launch_bounds__(kBlockThreads, kBlocksPerSm<float>)
+    k_batch_diag(const BatchDesc *__restrict__ d, const BatchDiag *__restrict__ dd, const int *__restrict__ prefix, int n,
+                 unsigned long long t)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     // the lattice of this block: the last m with prefix[m] <= blockIdx.x
@@ -2160,10 +2161,10 @@ TileLaunch plan_tiles(const Lattices &ls, int T)
 // - Strips beyond (512 x 512 FP32: 7.5 us, tiles 8.0).  FP32: two steps (1024 x
 //   2048: 39.4 us as one launch; three 45.2, four 42.5; 512 x 1024: 12.5, 12.7,
 //   12.8).  16-bit: four (1024 x 2048 FP16: 41.5 us; three 43.0, two 43.1; 512 x
-//   1024: 12.2, 12.8, 12.8; with cheaper rounding words, 44.6 and 13.4 now).  Six (eight) warps per block while the strips are
-//   short, four and one more block per SM from 40 (60) rows on (512 x 1024
-//   FP32: 12.5 against 13.1 us; 1024 x 2048: 42.4 against 39.4; two, three or
-//   five warps: 8-20 % slower).
+//   1024: 12.2, 12.8, 12.8; all with cheaper rounding words, 44.6 and 13.4 now).
+//   Six (eight) warps per block while the strips are short, four and one more
+//   block per SM from 40 (60) rows on (512 x 1024 FP32: 12.5 against 13.1 us; 1024
+//   x 2048: 42.4 against 39.4; two, three or five warps: 8-20 % slower).
 // - FP32 strips of more than 64 rows go out as two launches, half of the strips
 //   each, cut for two waves in all (k_tiles; 1024 x 2048: 40.6 us per step, as one
 //   launch of two waves 41.2; 768 x 1536: 23.9, 24.3; 2048 x 2048: 76.1, 77.6).
